@@ -167,8 +167,10 @@ int gp_graph_info_get(const gp_graph *g, gp_graph_info *info);
 
 /* Tunables (the autotuner writes these).  Correctness never depends on them. */
 typedef struct gp_options {
-    int32_t pull_light_max;   /* in-degree <= this: 32 vertices per warp, merged edge stream */
-    int32_t push_light_max;   /* out-degree <= this: same for the push scatter and top-down BFS */
+    int32_t pull_light_max;   /* in-degree <= this: one lane per vertex (pull steps of SSSP and
+                                 Frontier-Exploit PageRank, bottom-up BFS; the pull PageRank
+                                 sweep cuts the edge list in equal tiles at any degree) */
+    int32_t push_light_max;   /* out-degree <= this: 32 vertices per warp (push scatter, adjoint) */
     int32_t chunk_edges;      /* edges per warp chunk for vertices above the light limits */
     int32_t blocks_per_sm;    /* resident blocks per SM for the grid-stride sweep kernels */
     int32_t poll_interval;    /* PageRank sweeps enqueued between convergence read-backs (at
@@ -186,7 +188,8 @@ typedef struct gp_options {
                                  the L2 cache and no vertex takes more than 4096 updates per
                                  sweep (then FP32, whose array stays in L2) */
     int32_t pull_hot_slots;   /* pull PageRank: contributions of this many highest out-degree
-                                 vertices are served from shared memory (0 = off, <= 49152) */
+                                 vertices are served from shared memory (0 = off, <= 49152;
+                                 also off where they hold less than a 32nd of the edges) */
     int32_t push_hot_slots;   /* push PageRank: updates to this many highest in-degree vertices are
                                  summed in shared memory per block, then flushed with one atomic
                                  per vertex and block (0 = off, <= 49152) */
@@ -217,7 +220,7 @@ int gp_graph_get_options(const gp_graph *g, gp_options *opt);
 
 /* ------------------------------------------------------------------ autotuning */
 
-#define GP_TUNE_PULL 0x1u /* pull_light_max, chunk_edges, pull_hot_slots */
+#define GP_TUNE_PULL 0x1u /* pull_hot_slots */
 #define GP_TUNE_PUSH 0x2u /* push_light_max, blocks_per_sm, push_hot_slots */
 #define GP_TUNE_AUTO 0x4u /* pr_auto_mode: the faster of pull and push for this graph */
 #define GP_TUNE_BFS 0x8u  /* bfs_light_max, bfs_alpha, bfs_beta, then bfs_groups */

@@ -3,11 +3,10 @@
 // Correctness never depends on the options; only speed does.  The tuner runs
 // coordinate descent over small candidate sets, timing each candidate with
 // CUDA events on the caller's stream (the faster of two timings), and repeats
-// the pull and the push descent once when a pass changed something (the
-// coordinates interact: the best resident-block count depends on the size of
+// the push descent once when a pass changed something (the coordinates interact: the best resident-block count depends on the size of
 // the shared-memory accumulators, for instance):
-//   pull PageRank: pull_light_max, then chunk_edges, then pull_hot_slots
-//                  (a few sweeps of gp_pagerank(GP_PULL) per candidate);
+//   pull PageRank: pull_hot_slots (a few sweeps of gp_pagerank(GP_PULL) per
+//                  candidate; its tiles do not depend on the degree limits);
 //   push PageRank: push_light_max, then blocks_per_sm, then push_hot_slots;
 //   AUTO:          pr_auto_mode = whichever of pull and push sweeps faster
 //                  (the per-graph push/pull choice of the Generic-Switch idea, Section 5);
@@ -149,15 +148,9 @@ extern "C" int gp_autotune(gp_graph *g, unsigned what, const int32_t *sources, i
     if (st == GP_OK && (what & GP_TUNE_PULL)) {
         st = pull(pull_ms);
         ++evaluated;
-        for (int pass = 0; pass < TUNE_PASSES && st == GP_OK; ++pass) {
-            const gp_options before = best;
-            st = try_values<int32_t>(g, best, pull_ms, &gp_options::pull_light_max, {8, 16, 32}, s, pull, evaluated);
-            if (st == GP_OK) st = try_values<int32_t>(g, best, pull_ms, &gp_options::chunk_edges, {128, 256, 512}, s, pull, evaluated);
-            if (st == GP_OK)
-                st = try_values<int32_t>(g, best, pull_ms, &gp_options::pull_hot_slots, {0, 8192, 16384, 20480, 24576}, s, pull,
-                                         evaluated);
-            if (!memcmp(&before, &best, sizeof(best))) break;
-        }
+        if (st == GP_OK)
+            st = try_values<int32_t>(g, best, pull_ms, &gp_options::pull_hot_slots, {0, 8192, 16384, 20480, 24576}, s, pull,
+                                     evaluated);
     }
     if (st == GP_OK && (what & GP_TUNE_PUSH)) {
         st = push(push_ms);

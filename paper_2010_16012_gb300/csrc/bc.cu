@@ -898,7 +898,7 @@ static int ensure_bc_work(gp_graph *g, cudaStream_t s) {
     GP_TRY(w.mem.alloc(w.med_in, n, s));
     GP_TRY(build_bins(g, w.hub_out, g->csr_off, BC_HUB, BC_CHUNK, s));
     GP_TRY(build_bins(g, w.hub_in, g->csc_off, BC_HUB, BC_CHUNK, s));
-    GP_TRY(build_hot(g, w.hot, BC_HOT, g->csr_off, g->csc_idx, s));
+    GP_TRY(build_hot(g, w.hot, BC_HOT, g->csr_off, g->csc_idx, INT32_MAX, s));
     GP_TRY(select_by_degree(g->csc_off, g->n, BC_LIGHT + 1, BC_HUB, w.mem, w.med_in_all, w.n_med_in_all, INT64_MAX,
                             nullptr, s));
     GP_TRY(w.mem.alloc(w.sigma, n, s));

@@ -131,9 +131,30 @@ constexpr uint32_t HOT_BIT = 0x80000000u;
 struct HotSet {
     int32_t slots = 0;  // requested H (0 = off)
     int64_t nhot = 0;
-    int32_t *hot_id = nullptr;   // [nhot] vertex of each slot
+    int32_t *hot_id = nullptr;   // [nhot] vertex of each slot, ascending
     float *c_hot = nullptr;      // [nhot]
     int32_t *enc_idx = nullptr;  // [m]
+    uint32_t *bits = nullptr;    // [n/32] bit v: v is hot
+    int32_t *prefix = nullptr;   // [n/32] slot of the first hot vertex of each word
+    Arena mem;
+};
+
+// An adjacency cut into tiles of TILE_EDGES consecutive edges, one warp each,
+// whatever the vertices' degrees (the pull sweep's unit of work).  Rows are the
+// vertices with at least one edge, ascending; a row may span tiles.
+constexpr int TILE_EDGES = 256;
+constexpr int64_t TILE_LONG = 16;  // a row over more tiles than this is summed by a whole warp
+struct EdgeTiles {
+    bool ready = false;
+    int64_t ntiles = 0;           // ceil(m / TILE_EDGES)
+    int64_t nrows = 0;            // vertices with edges
+    int64_t nlong = 0;            // rows over more than TILE_LONG tiles
+    uint8_t *heads = nullptr;     // [ntiles * TILE_EDGES / 8] bit e: edge e is the first of its row
+    int32_t *tile_row = nullptr;  // [ntiles] row holding the edge before the tile's first (-1: none)
+    int32_t *rows = nullptr;      // [n] vertex of each row (HOT_BIT set: the row spans tiles), then the vertices without edges
+    int32_t *long_rows = nullptr; // [nlong] rows over more than TILE_LONG tiles
+    float *acc = nullptr;         // [nrows] sweep workspace: sum of the row's edges in the tile it starts in
+    float *carry = nullptr;       // [ntiles] sum of the tile's edges that belong to a row of an earlier tile
     Arena mem;
 };
 
@@ -146,7 +167,7 @@ struct PrWork {
     float *x0_dev = nullptr;       // start vector copy (host input)
     float *out_dev = nullptr;      // output buffer when ranks_out is host memory
     double *partials = nullptr;    // per-block residual partials
-    float *chunk_part = nullptr;   // per-chunk partial sums (pull, big vertices)
+    float *chunk_part = nullptr;   // per-chunk partial sums (adjoint pull, long rows)
     double *acc64 = nullptr;       // FP64 accumulator of the push scatter
     float *lam = nullptr;          // adjoint solution
     float *gw_dev = nullptr;       // weight gradient when the output is host memory
@@ -220,6 +241,7 @@ struct gp_graph {
     gp::BigBins bfs_bins;   // by out-degree at bfs_light_max (BFS top-down), when it differs from push_light_max
     gp::HotSet pull_hot;    // shared-memory contribution cache of the pull sweep
     gp::HotSet push_hot;    // shared-memory accumulators of the push scatter
+    gp::EdgeTiles tiles;    // of the CSC (pull sweep); built by the first sweep
     gp::PrWork pr;
     gp::BfsWork bfs;
     gp_sssp_work *sssp = nullptr;
@@ -235,8 +257,9 @@ int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, i
                cudaStream_t s);
 // The `slots` vertices of largest degree by sel_off, and enc_src (an index array
 // of m entries) with each of them replaced by HOT_BIT | slot.
-int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, const int32_t *enc_src,
+int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, const int32_t *enc_src, int min_share,
               cudaStream_t s);
+int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s);
 int build_pull_hot(gp_graph *g, int32_t slots, cudaStream_t s);
 int build_push_hot(gp_graph *g, int32_t slots, cudaStream_t s);
 int select_by_degree(const int64_t *off, int64_t n, int64_t lo, int64_t hi, Arena &mem, int32_t *&list,

@@ -7,17 +7,13 @@
 // and edge factor w_uv (1 when unweighted).
 //
 // Pull (owner-only writes, no atomics; Section 4.1 "Atomics/Locks"):
-//   k_pull_big    -- vertices whose in-degree exceeds pull_light_max: their
-//                    in-edge lists are cut into chunks of <= chunk_edges edges,
-//                    one warp per chunk, coalesced index loads, warp tree sum
-//                    (Section 4's CREW binary merge-tree) into a per-chunk slot.
-//   k_pull_light  -- blocks [0, light_blocks): one warp per tile of 32
-//                    consecutive vertices; each lane sums its own light
-//                    vertex's in-list with 8 loads in flight (no shuffles: the
-//                    kernel is issue-bound, and light lists are short).  Blocks
-//                    after that: one thread per big vertex adds its chunk
-//                    slots.  Every vertex's y, c' = y*inv_deg and |y - x| are
-//                    written by its owner.
+//   k_pull_tiles  -- the edge list in tiles of 256 consecutive edges, one warp
+//                    each, whatever the vertices' degrees; a segmented warp sum
+//                    (Section 4's CREW binary merge-tree) gives one partial per
+//                    row and tile.
+//   k_pull_finish -- one thread per row adds its tiles' partials (a warp where
+//                    the row spans many) and writes the vertex's y,
+//                    c' = y*inv_deg and |y - x|; every vertex has one writer.
 // Push (scatter with atomics; Section 4.1: O(Lm) write conflicts):
 //   k_push_scatter   -- each source adds d*c[u]*w_uv into y[v] for its
 //                       out-edges with FP32 atomicAdd (RED), big sources in
@@ -74,13 +70,21 @@ struct PrArgs {
     int32_t k;  // sweep number, 1-based
     int32_t nprev;
     double *partials;
-    float *chunk_part;
     double *acc64;  // FP64 push accumulator (or nullptr)
-    const float *c_hot;  // hot contributions (pull, HOT kernels)
+    float *c_hot;   // hot contributions (pull, HOT kernels)
     const int32_t *hot_id;  // hot vertices (push HOT kernels)
+    const uint32_t *hot_bits;    // pull: which vertices are hot, and
+    const int32_t *hot_prefix;   // the slot of the first hot vertex of each word
     int64_t nhot;
+    // pull: the edge tiles (see EdgeTiles)
+    const uint8_t *heads;
+    const int32_t *tile_row, *rows, *long_rows;
+    float *acc, *carry;
+    float *chunk_part;     // adjoint pull: the long rows' chunk sums
+    int32_t split_blocks;  // adjoint pull: blocks of short rows (the others add the long rows' chunks)
+    int64_t m, ntiles, nrows, nlong;
+    int32_t vec_tiles;  // the leading tiles that may be read 32 bytes at a time: full, arrays on 32-byte boundaries
     PrStatus *status;
-    int32_t split_blocks;  // pull: light-tile blocks; push: big-chunk blocks
 };
 
 __device__ __forceinline__ float base_term(const PrArgs &a, int64_t v) {
@@ -130,15 +134,24 @@ __device__ bool pr_gate(const PrArgs &a, int k) {
     return stop != 0;
 }
 
+// c_hot[slot of v] = c where v is hot (see HotSet).
+__device__ __forceinline__ void store_hot(const uint32_t *bits, const int32_t *prefix, float *c_hot, int64_t v, float c) {
+    const uint32_t word = bits[v >> 5], bit = 1u << (v & 31);
+    if (word & bit) c_hot[prefix[v >> 5] + __popc(word & (bit - 1u))] = c;
+}
+
 // x = x0 (or 1/n), c = x * cmul, and the push accumulators zeroed.
 __global__ void k_pr_init(int64_t n, const float *x0, const float *cmul, float *r0, float *c, float *r_push,
-                          double *acc64, PrStatus *status) {
+                          double *acc64, const uint32_t *hot_bits, const int32_t *hot_prefix, float *c_hot,
+                          PrStatus *status) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const float x_uniform = 1.0f / (float)n;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const float x = x0 ? x0[v] : x_uniform;
+        const float cv = cmul ? x * cmul[v] : x;
         r0[v] = x;
-        c[v] = cmul ? x * cmul[v] : x;
+        c[v] = cv;
+        if (hot_bits) store_hot(hot_bits, hot_prefix, c_hot, v, cv);
         if (r_push) r_push[v] = 0.f;
         if (acc64) acc64[v] = 0.0;
     }
@@ -190,35 +203,190 @@ __device__ __forceinline__ float gather_c(const float *__restrict__ c, const flo
     return __ldg(c + u);
 }
 
-// The same gather with the hot contributions read from their compact global
-// copy (pull_light: its few hot gathers do not pay for a shared-memory copy,
-// whose size would also cut the light kernel's resident blocks).
-template <bool HOT>
-__device__ __forceinline__ float gather_c_glob(const float *__restrict__ c, const float *__restrict__ c_hot, int32_t u) {
-    if (HOT && u < 0) return __ldg(c_hot + (u & 0x7fffffff));
-    return __ldg(c + u);
+#ifndef GP_TILE_THREADS
+#define GP_TILE_THREADS 768
+#endif
+constexpr int TILE_THREADS = GP_TILE_THREADS;  // threads per block of the tile kernel, two blocks per SM
+constexpr int LANE_EDGES = TILE_EDGES / 32;  // consecutive edges of a tile that one lane sums
+static_assert(LANE_EDGES == 8, "one head byte and one 32-byte index load per lane");
+
+// Eight consecutive 32-bit words.  The index and weight arrays are streamed
+// once per sweep: evict-first in L2 and not kept in L1, so that they do not
+// push the gathered contributions out.
+__device__ __forceinline__ void ld_stream8(const void *p, uint32_t (&v)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "l"(p));
 }
 
+// One sweep's sums: tile t's edges are gathered eight to a lane and summed by
+// row.  A row that starts in the tile leaves its sum there in acc[row]; edges
+// of a row started in an earlier tile leave theirs in carry[t].
+template <bool W, bool HOT>
+__device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh, int warp, int nwarps) {
+    const int lane = lane_id();
+    const unsigned below = (1u << lane) - 1u;
+    const int32_t *__restrict__ idx = a.idx;
+    const float *__restrict__ c = a.c;
+    const int ntiles = (int)a.ntiles;
+    for (int t = warp; t < ntiles; t += nwarps) {
+        const int64_t e0 = (int64_t)t * TILE_EDGES + lane * LANE_EDGES;
+        const unsigned h = a.heads[(int64_t)t * 32 + lane];  // bit q: edge e0 + q is the first of its row
+        const int32_t row0 = a.tile_row[t];
+        float f[8];
+        if (t < a.vec_tiles) {
+            uint32_t u[8];
+            ld_stream8(idx + e0, u);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f[q] = gather_c<HOT>(c, sh, (int32_t)u[q]);
+            if (W) {
+                ld_stream8(a.w + e0, u);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) f[q] *= __uint_as_float(u[q]);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                f[q] = 0.f;
+                if (e0 + q < a.m) {
+                    f[q] = gather_c<HOT>(c, sh, __ldg(idx + e0 + q));
+                    if (W) f[q] *= __ldg(a.w + e0 + q);
+                }
+            }
+        }
+        const unsigned starts = __ballot_sync(FULL, h != 0);  // lanes where a row starts
+        if (starts == 0) {  // the inside of one long row
+            float s = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
+            s = warp_sum(s);
+            if (lane == 0) a.carry[t] = s;
+            continue;
+        }
+        // rows started in the lanes below: prefix sum of popc(h) <= 8, by its binary digits
+        const unsigned cnt = __popc(h);
+        int before = 0, all = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const unsigned digit = __ballot_sync(FULL, (cnt >> b) & 1u);
+            before += __popc(digit & below) << b;
+            all += __popc(digit) << b;
+        }
+        const int32_t row = row0 + before;  // the row open at the lane's first edge
+        float open = 0.f, s = 0.f;
+        int32_t r = row;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            if ((h >> q) & 1u) {
+                if (r == row)
+                    open = s;  // what the lane adds to the row open at its start
+                else
+                    a.acc[r] = s;  // a row that starts and ends in the lane
+                ++r;
+                s = 0.f;
+            }
+            s += f[q];
+        }
+        // segmented inclusive scan over the lanes: s becomes the sum of the row
+        // open at the lane's end, back to the lane where it starts
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float up = __shfl_up_sync(FULL, s, o);
+            // lanes lane-o+1 .. lane start no row
+            if (lane >= o && (starts & (below + below + 1u) & ~((1u << (lane - o + 1)) - 1u)) == 0) s += up;
+        }
+        float in = __shfl_up_sync(FULL, s, 1);
+        if (lane == 0) in = 0.f;
+        if (h) {
+            if ((starts & below) == 0)
+                a.carry[t] = in + open;
+            else
+                a.acc[row] = in + open;
+        }
+        if (lane == 31) a.acc[row0 + all] = s;
+    }
+}
+
+// Bound by the random 4-byte gathers (one per edge; L1 tags and L2 sectors:
+// ~300 G/s from L2).  Equal tiles keep every lane's eight gathers in use at any
+// degree, where a warp per long list and a lane per short one left most of them
+// idle at degrees near 16: a sweep of a uniform graph (n = 8.0M, m = 128M) took
+// 555 + 335 us split that way and takes 458 + 62 us; R-MAT 22 (m = 128M) 295 +
+// 84 + 4 us, now 280 + 25 us (40 or 32 registers, 768 or 1024 threads a block:
+// within 1% there; 768 is 10% faster on a graph of 16K vertices).
+template <bool W, bool HOT>
+__global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_tiles(PrArgs a) {
+    extern __shared__ float sh_hot[];
+    if (pr_gate(a, a.k)) return;
+    load_hot<HOT>(a, sh_hot);
+    pull_tiles_step<W, HOT>(a, sh_hot, (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                            (int)(gridDim.x * blockDim.x) >> 5);
+}
+
+// The vertex's new iterate from its gathered sum.
+template <bool HOT>
+__device__ __forceinline__ void pull_write(const PrArgs &a, int64_t v, float sum, ResSum &res) {
+    const float y = base_term(a, v) + a.d * (post_factor(a, v) * sum);
+    const float cn = y * c_factor(a, v);
+    res.add(y, a.x[v]);
+    a.y[v] = y;
+    a.c_next[v] = cn;
+    if (HOT) store_hot(a.hot_bits, a.hot_prefix, a.c_hot, v, cn);
+}
+
+// Rows, then, in the first two sweeps, the vertices without in-edges: theirs is
+// the base term in every sweep, so both iterate buffers hold it from then on.
+template <bool HOT>
+__device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread, int64_t nthreads, ResSum &res) {
+    const int64_t count = a.k <= 2 ? a.n : a.nrows;
+    for (int64_t r = thread; r < count; r += nthreads) {
+        const uint32_t code = (uint32_t)a.rows[r];
+        const int64_t v = code & ~HOT_BIT;
+        float sum = r < a.nrows ? a.acc[r] : 0.f;
+        if (code & HOT_BIT) {  // the row spans tiles
+            const int64_t t0 = a.off[v] / TILE_EDGES, t1 = (a.off[v + 1] - 1) / TILE_EDGES;
+            if (t1 - t0 > TILE_LONG) continue;  // below
+            for (int64_t t = t0 + 1; t <= t1; ++t) sum += a.carry[t];
+        }
+        pull_write<HOT>(a, v, sum, res);
+    }
+    const int lane = lane_id();
+    for (int64_t i = thread >> 5; i < a.nlong; i += nthreads >> 5) {
+        const int32_t r = a.long_rows[i];
+        const int64_t v = (uint32_t)a.rows[r] & ~HOT_BIT;
+        const int64_t t0 = a.off[v] / TILE_EDGES, t1 = (a.off[v + 1] - 1) / TILE_EDGES;
+        float sum = 0.f;
+        for (int64_t t = t0 + 1 + lane; t <= t1; t += 32) sum += a.carry[t];
+        sum = warp_sum(sum);
+        if (lane == 0) pull_write<HOT>(a, v, a.acc[r] + sum, res);
+    }
+}
+
+template <bool HOT>
+__global__ void __launch_bounds__(256) k_pull_finish(PrArgs a) {
+    __shared__ double sm[32];
+    if (pr_stopped(a.status)) return;
+    ResSum res;
+    pull_finish_step<HOT>(a, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, res);
+    const double r = block_residual(res, sm);
+    if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
+}
+
+// The adjoint's pull sweep sums a row in a fixed order of its own, whatever the
+// rows around it: a short row's edges one after another in its lane, a long
+// row's in warp chunks and the chunks one after another.  The gradient of a
+// normalised weight is (x_u / S_u)(d lambda_v - lambda_u + g_u), and where u's
+// edges are few and light the bracket cancels while the factor is large: there
+// the order of summation, not only its error, shows in the result (two orders
+// differ by up to 1e-3 of the gradients' RMS on R-MAT 18 with weights in (0, 1]),
+// so gradients keep the order that they have always had.
 constexpr int BIG_UNROLL = 8;
 
 // Index arrays are streamed once per sweep: loaded with the evict-first hint so
 // they do not push the gathered contribution vector out of L2.
-#ifndef GP_IDX_STREAMING
-#define GP_IDX_STREAMING 1
-#endif
-__device__ __forceinline__ int32_t ld_idx(const int32_t *p) {
-#if GP_IDX_STREAMING
-    return __ldcs(p);
-#else
-    return __ldg(p);
-#endif
-}
+__device__ __forceinline__ int32_t ld_idx(const int32_t *p) { return __ldcs(p); }
 
-template <bool W, bool HOT>
-__global__ void __launch_bounds__(1024) k_pull_big(PrArgs a) {
-    extern __shared__ float sh_hot[];
+template <bool W>
+__global__ void __launch_bounds__(1024) k_adj_big(PrArgs a) {
     if (pr_gate(a, a.k)) return;
-    load_hot<HOT>(a, sh_hot);
     const int lane = lane_id();
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -244,7 +412,7 @@ __global__ void __launch_bounds__(1024) k_pull_big(PrArgs a) {
                 const int i = i0 + q * 32 + lane;
                 f[q] = 0.f;
                 if (i < ch.len) {
-                    f[q] = gather_c<HOT>(c, sh_hot, u[q]);
+                    f[q] = __ldg(c + u[q]);
                     if (W) f[q] *= __ldg(wp + i);
                 }
             }
@@ -256,25 +424,10 @@ __global__ void __launch_bounds__(1024) k_pull_big(PrArgs a) {
     }
 }
 
-#ifndef GP_LIGHT_MIN_BLOCKS
-#define GP_LIGHT_MIN_BLOCKS 3
-#endif
-// Owner lane of virtual edge `eid` in a tile: the last lane k with excl[k] <= eid
-// (zero-degree lanes share their successor's excl, so the last one is non-empty).
-__device__ __forceinline__ int tile_owner(int excl, int eid) {
-    int k = 0;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-        const int ex = __shfl_sync(FULL, excl, k + s);
-        if (ex <= eid) k += s;
-    }
-    return k;
-}
-
 constexpr int LIGHT_UNROLL = 8;  // in-edges of a light vertex in flight per lane
 
-template <bool W, bool HOT>
-__global__ void __launch_bounds__(512, GP_LIGHT_MIN_BLOCKS) k_pull_light(PrArgs a) {
+template <bool W>
+__global__ void __launch_bounds__(512, 3) k_adj_light(PrArgs a) {
     __shared__ double sm[32];
     if (pr_stopped(a.status)) return;
     const int lane = lane_id();
@@ -325,7 +478,7 @@ __global__ void __launch_bounds__(512, GP_LIGHT_MIN_BLOCKS) k_pull_light(PrArgs 
                 for (int q = 0; q < LIGHT_UNROLL; ++q) {
                     f[q] = 0.f;
                     if (p0 + q < e1) {
-                        f[q] = gather_c_glob<HOT>(c, a.c_hot, u[q]);
+                        f[q] = __ldg(c + u[q]);
                         if (W) f[q] *= __ldg(wv + p0 + q);
                     }
                 }
@@ -355,12 +508,16 @@ __global__ void __launch_bounds__(512, GP_LIGHT_MIN_BLOCKS) k_pull_light(PrArgs 
     if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
 }
 
-// c_hot[slot] = c[hot_id[slot]] for the sweep that reads c next (none once
-// the iteration has stopped: the launches enqueued past that point return).
-__global__ void k_hot_gather(const int32_t *hot_id, int64_t nhot, const float *c, float *c_hot, const PrStatus *status) {
-    if (status && pr_stopped(status)) return;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nhot; i += stride) c_hot[i] = c[hot_id[i]];
+// Owner lane of virtual edge `eid` in a tile: the last lane k with excl[k] <= eid
+// (zero-degree lanes share their successor's excl, so the last one is non-empty).
+__device__ __forceinline__ int tile_owner(int excl, int eid) {
+    int k = 0;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const int ex = __shfl_sync(FULL, excl, k + s);
+        if (ex <= eid) k += s;
+    }
+    return k;
 }
 
 // ------------------------------------------------------------------ push
@@ -642,14 +799,12 @@ static int ensure_pr_work(gp_graph *g, cudaStream_t s) {
     if (w.ready) return GP_OK;
     const size_t n = (size_t)std::max<int64_t>(g->n, 1);
     const int64_t nbig = std::max(g->pull_bins.nbig, g->push_bins.nbig);
-    const int64_t epi = (nbig + 255) / 256;
-    // covers any grid: at most 32 resident blocks per SM, plus the epilogue blocks
-    w.max_blocks = (int)(std::max(g->num_sms * 32, grid_blocks(g, 256)) + epi + 64);
+    // covers any grid: at most 32 resident blocks per SM, plus the blocks that add the adjoint's chunks
+    w.max_blocks = (int)(std::max(g->num_sms * 32, grid_blocks(g, 256)) + (nbig + 511) / 512 + 64);
     GP_TRY(w.mem.alloc(w.r1, n, s));
     GP_TRY(w.mem.alloc(w.c0, n, s));
     GP_TRY(w.mem.alloc(w.c1, n, s));
     GP_TRY(w.mem.alloc(w.partials, (size_t)w.max_blocks, s));
-    GP_TRY(w.mem.alloc(w.chunk_part, (size_t)std::max<int64_t>(std::max(g->pull_bins.nchunks, g->push_bins.nchunks), 1), s));
     PrStatus *st = nullptr;
     GP_TRY(w.mem.alloc(st, 1, s));
     w.status = st;
@@ -696,7 +851,8 @@ struct IterSpec {
     const int64_t *off;
     const int32_t *idx;
     const float *w;
-    const BigBins *bins;
+    const BigBins *bins;  // push and adjoint pull: the chunks of the long lists
+    EdgeTiles *tiles;     // forward pull: the adjacency's tiles (built on first use); nullptr: adjoint pull
     const float *s;   // base vector (nullable: uniform base_uniform)
     float s_scale, base_uniform, d;
     const float *x0;  // start vector (nullable: 1/n)
@@ -737,29 +893,43 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     a.d = sp.d;
     a.tol = sp.tol;
     a.partials = w.partials;
-    a.chunk_part = w.chunk_part;
     a.status = status;
 
     const int gb = grid_blocks(g, 256);
     const int64_t ntiles = (n + 31) / 32;
     bool hot = false;
-    int tbp = 256, tbl = 256;  // threads per block of pull_big / pull_light
     size_t smem = 0;
-    if (!push && sp.hot) {
-        if (g->pull_hot.slots != g->opt.pull_hot_slots) GP_TRY(build_pull_hot(g, g->opt.pull_hot_slots, s));
-        hot = g->pull_hot.nhot > 0;
+    const bool tiled = !push && sp.tiles;
+    if (!push && !tiled) {
+        if (!w.chunk_part) GP_TRY(w.mem.alloc(w.chunk_part, (size_t)std::max<int64_t>(bins.nchunks, 1), s));
+        a.chunk_part = w.chunk_part;
+    }
+    if (tiled) {
+        GP_TRY(build_tiles(g, *sp.tiles, sp.off, s));
+        const EdgeTiles &t = *sp.tiles;
+        a.m = g->m;
+        a.heads = t.heads;
+        a.tile_row = t.tile_row;
+        a.rows = t.rows;
+        a.long_rows = t.long_rows;
+        a.acc = t.acc;
+        a.carry = t.carry;
+        a.ntiles = t.ntiles;
+        a.nrows = t.nrows;
+        a.nlong = t.nlong;
+        if (sp.hot) {
+            if (g->pull_hot.slots != g->opt.pull_hot_slots) GP_TRY(build_pull_hot(g, g->opt.pull_hot_slots, s));
+            hot = g->pull_hot.nhot > 0;
+        }
         if (hot) {
-            tbp = 1024;
-            tbl = 512;
             smem = (size_t)((g->pull_hot.nhot + 3) & ~int64_t(3)) * sizeof(float);
             a.c_hot = g->pull_hot.c_hot;
+            a.hot_bits = g->pull_hot.bits;
+            a.hot_prefix = g->pull_hot.prefix;
             a.nhot = g->pull_hot.nhot;
             a.idx = g->pull_hot.enc_idx;
         }
-    }
-    if (!push && !hot) {
-        tbp = 1024;
-        tbl = 512;
+        a.vec_tiles = ((uintptr_t)a.idx | (uintptr_t)a.w) % 32 == 0 ? (int32_t)(a.m / TILE_EDGES) : 0;
     }
     if (push && sp.hot) {
         if (g->push_hot.slots != g->opt.push_hot_slots) GP_TRY(build_push_hot(g, g->opt.push_hot_slots, s));
@@ -771,19 +941,24 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
             a.idx = g->push_hot.enc_idx;
         }
     }
-    int g1, g2, split;
-    if (!push) {
+    int g1, g2;
+    const int tpt = TILE_THREADS;
+    if (!push && !tiled) {
         int ob = 0, ol = 0;
-        const void *kb_ = W ? (hot ? (const void *)k_pull_big<true, true> : (const void *)k_pull_big<true, false>)
-                            : (hot ? (const void *)k_pull_big<false, true> : (const void *)k_pull_big<false, false>);
-        const void *kl_ = W ? (hot ? (const void *)k_pull_light<true, true> : (const void *)k_pull_light<true, false>)
-                            : (hot ? (const void *)k_pull_light<false, true> : (const void *)k_pull_light<false, false>);
-        GP_TRY(occupancy(kb_, tbp, smem, ob));
-        GP_TRY(occupancy(kl_, tbl, 0, ol));
-        const int wpb = tbp / 32, wpl = tbl / 32;
-        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (bins.nchunks + wpb - 1) / wpb));
-        split = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ol * g->num_sms, (ntiles + wpl - 1) / wpl));
-        g2 = split + (int)((bins.nbig + tbl - 1) / tbl);
+        GP_TRY(occupancy(W ? (const void *)k_adj_big<true> : (const void *)k_adj_big<false>, 1024, 0, ob));
+        GP_TRY(occupancy(W ? (const void *)k_adj_light<true> : (const void *)k_adj_light<false>, 512, 0, ol));
+        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (bins.nchunks + 31) / 32));
+        a.split_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ol * g->num_sms, (ntiles + 15) / 16));
+        g2 = a.split_blocks + (int)((bins.nbig + 511) / 512);
+    } else if (!push) {
+        int ob = 0, of = 0;
+        const void *kb_ = W ? (hot ? (const void *)k_pull_tiles<true, true> : (const void *)k_pull_tiles<true, false>)
+                            : (hot ? (const void *)k_pull_tiles<false, true> : (const void *)k_pull_tiles<false, false>);
+        GP_TRY(occupancy(kb_, tpt, smem, ob));
+        GP_TRY(occupancy(hot ? (const void *)k_pull_finish<true> : (const void *)k_pull_finish<false>, 256, 0, of));
+        const int wpb = tpt / 32;
+        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (a.ntiles + wpb - 1) / wpb));
+        g2 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)of * g->num_sms, (n + 255) / 256));
     } else {
         // one grid for big chunks and light tiles; as many resident blocks as fit,
         // capped by blocks_per_sm (256-thread units)
@@ -792,29 +967,19 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         GP_TRY(occupancy(ks, 1024, smem, os));
         const int cap = std::max(1, g->opt.blocks_per_sm / 4) * g->num_sms;
         const int64_t work = std::max<int64_t>((bins.nchunks + 31) / 32, (ntiles + 31) / 32);
-        split = 0;
         g1 = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>((int64_t)os * g->num_sms, cap), work));
         g2 = (int)std::max<int64_t>(1, std::min<int64_t>(gb, (n + 255) / 256));
     }
     if (g2 > w.max_blocks) return set_error(GP_ERR_INVALID, "internal: partials too small");
     a.nprev = g2;
-    a.split_blocks = split;
 
     const int ib = (int)std::max<int64_t>(1, std::min<int64_t>(gb, (n + 255) / 256));
     const bool fp64 = push && push_fp64(g, sp.max_updates);
     if (fp64 && !w.acc64) GP_TRY(w.mem.alloc(w.acc64, (size_t)n, s));
     a.acc64 = fp64 ? w.acc64 : nullptr;
     GP_LAUNCH("pr_init", s, (k_pr_init<<<ib, 256, 0, s>>>(n, sp.x0, sp.cmul, R[0], C[0], (push && !fp64) ? R[1] : nullptr,
-                                                          a.acc64, status)));
+                                                          a.acc64, a.hot_bits, a.hot_prefix, a.c_hot, status)));
     GP_TRY(check_launch("pr_init"));
-    auto enqueue_hot_gather = [&](const float *c_src) -> int {
-        const int hb = (int)std::max<int64_t>(1, std::min<int64_t>((g->pull_hot.nhot + 255) / 256, 4096));
-        GP_LAUNCH("hot_gather", s, (k_hot_gather<<<hb, 256, 0, s>>>(g->pull_hot.hot_id, g->pull_hot.nhot, c_src,
-                                                                    g->pull_hot.c_hot, status)));
-        return check_launch("hot_gather");
-    };
-    if (hot && !push) GP_TRY(enqueue_hot_gather(C[0]));
-
     auto enqueue_sweep = [&](int k) -> int {
         PrArgs b = a;
         b.k = k;
@@ -823,20 +988,28 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         if (!push) {
             b.c = C[(k - 1) & 1];
             b.c_next = C[k & 1];
-            if (W && hot) {
-                GP_LAUNCH("pull_big", s, (k_pull_big<true, true><<<g1, tbp, smem, s>>>(b)));
-                GP_LAUNCH("pull_light", s, (k_pull_light<true, true><<<g2, tbl, 0, s>>>(b)));
-            } else if (W) {
-                GP_LAUNCH("pull_big", s, (k_pull_big<true, false><<<g1, tbp, 0, s>>>(b)));
-                GP_LAUNCH("pull_light", s, (k_pull_light<true, false><<<g2, tbl, 0, s>>>(b)));
-            } else if (hot) {
-                GP_LAUNCH("pull_big", s, (k_pull_big<false, true><<<g1, tbp, smem, s>>>(b)));
-                GP_LAUNCH("pull_light", s, (k_pull_light<false, true><<<g2, tbl, 0, s>>>(b)));
-            } else {
-                GP_LAUNCH("pull_big", s, (k_pull_big<false, false><<<g1, tbp, 0, s>>>(b)));
-                GP_LAUNCH("pull_light", s, (k_pull_light<false, false><<<g2, tbl, 0, s>>>(b)));
+            if (!tiled && W) {
+                GP_LAUNCH("adj_big", s, (k_adj_big<true><<<g1, 1024, 0, s>>>(b)));
+                GP_LAUNCH("adj_light", s, (k_adj_light<true><<<g2, 512, 0, s>>>(b)));
+                return check_launch("adjoint sweep");
             }
-            if (hot) GP_TRY(enqueue_hot_gather(b.c_next));
+            if (!tiled) {
+                GP_LAUNCH("adj_big", s, (k_adj_big<false><<<g1, 1024, 0, s>>>(b)));
+                GP_LAUNCH("adj_light", s, (k_adj_light<false><<<g2, 512, 0, s>>>(b)));
+                return check_launch("adjoint sweep");
+            }
+            if (W && hot)
+                GP_LAUNCH("pull_tiles", s, (k_pull_tiles<true, true><<<g1, tpt, smem, s>>>(b)));
+            else if (W)
+                GP_LAUNCH("pull_tiles", s, (k_pull_tiles<true, false><<<g1, tpt, 0, s>>>(b)));
+            else if (hot)
+                GP_LAUNCH("pull_tiles", s, (k_pull_tiles<false, true><<<g1, tpt, smem, s>>>(b)));
+            else
+                GP_LAUNCH("pull_tiles", s, (k_pull_tiles<false, false><<<g1, tpt, 0, s>>>(b)));
+            if (hot)
+                GP_LAUNCH("pull_finish", s, (k_pull_finish<true><<<g2, 256, 0, s>>>(b)));
+            else
+                GP_LAUNCH("pull_finish", s, (k_pull_finish<false><<<g2, 256, 0, s>>>(b)));
         } else {
             b.c = C[0];
             b.c_next = C[0];
@@ -1035,7 +1208,8 @@ extern "C" int gp_pagerank(const gp_graph *gc, int mode, float damping, int iter
     sp.off = push ? g->csr_off : g->csc_off;
     sp.idx = push ? g->csr_idx : g->csc_idx;
     sp.w = g->weighted ? (push ? g->csr_w : g->csc_w) : nullptr;
-    sp.bins = push ? &g->push_bins : &g->pull_bins;
+    sp.bins = &g->push_bins;
+    sp.tiles = &g->tiles;
     sp.s = S;
     sp.s_scale = 1.0f - damping;
     sp.base_uniform = (float)((1.0 - (double)damping) / (double)n);
@@ -1108,6 +1282,7 @@ extern "C" int gp_pagerank_backward(const gp_graph *gc, int mode, float damping,
     sp.idx = push ? g->csc_idx : g->csr_idx;
     sp.w = g->weighted ? (push ? g->csc_w : g->csr_w) : nullptr;
     sp.bins = push ? &g->pull_bins : &g->push_bins;
+    sp.tiles = nullptr;
     sp.s = G;
     sp.s_scale = 1.0f;
     sp.base_uniform = 0.f;

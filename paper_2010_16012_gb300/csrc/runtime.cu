@@ -588,24 +588,65 @@ __global__ void k_deg_hist(const int64_t *off, int64_t n, unsigned long long *hi
         if (sh[i]) atomicAdd(hist + i, (unsigned long long)sh[i]);
 }
 
-__global__ void k_fill_slots(const int32_t *hot_id, int64_t nhot, int32_t *slot) {
+// bits: the vertices with more than `above` edges, one warp per word.
+__global__ void k_hot_bits(const int64_t *off, int64_t n, int64_t above, uint32_t *bits) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nhot; i += stride) slot[hot_id[i]] = (int32_t)i;
+    const int64_t npad = (n + 31) & ~int64_t(31);
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < npad; v += stride) {
+        const unsigned word = __ballot_sync(FULL, v < n && off[v + 1] - off[v] > above);
+        if (lane_id() == 0) bits[v >> 5] = word;
+    }
 }
 
-__global__ void k_encode_hot(const int32_t *idx, int64_t m, const int32_t *slot, int32_t *enc) {
+__global__ void k_hot_mark(const int32_t *list, int64_t count, uint32_t *bits) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-        const int32_t u = idx[e];
-        const int32_t sl = slot[u];
-        enc[e] = sl >= 0 ? (int32_t)(HOT_BIT | (uint32_t)sl) : u;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride)
+        atomicOr(bits + (list[i] >> 5), 1u << (list[i] & 31));
+}
+
+__global__ void k_hot_counts(const uint32_t *bits, int64_t nwords, int64_t *counts) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nwords; i += stride) counts[i] = __popc(bits[i]);
+}
+
+__global__ void k_hot_slots(const uint32_t *bits, int64_t nwords, const int64_t *scan, int32_t *prefix, int32_t *hot_id) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nwords; i += stride) {
+        int32_t sl = (int32_t)scan[i];
+        prefix[i] = sl;
+        for (uint32_t x = bits[i]; x; x &= x - 1) hot_id[sl++] = (int32_t)(i * 32 + __ffs(x) - 1);
+    }
+}
+
+// Latency-bound with one edge per thread in flight (R-MAT 22, 128M edges:
+// 387 us), so eight are; the bitmap is read first: n/8 bytes, most of whose hot
+// words stay in L1.
+__global__ void k_encode_hot(const int32_t *idx, int64_t m, const uint32_t *bits, const int32_t *prefix, int32_t *enc) {
+    constexpr int U = 8;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < m; e0 += U * stride) {
+        int32_t u[U];
+        uint32_t word[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) u[q] = e0 + q * stride < m ? __ldcs(idx + e0 + q * stride) : 0;
+#pragma unroll
+        for (int q = 0; q < U; ++q) word[q] = __ldg(bits + (u[q] >> 5));
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const uint32_t bit = 1u << (u[q] & 31);
+            int32_t code = u[q];
+            if (word[q] & bit)
+                code = (int32_t)(HOT_BIT | (uint32_t)(__ldg(prefix + (u[q] >> 5)) + __popc(word[q] & (bit - 1u))));
+            if (e0 + q * stride < m) enc[e0 + q * stride] = code;
+        }
     }
 }
 
 // Picks the `slots` vertices with the largest degree by `sel_off` (ties: lowest
-// ids), builds the copy of `enc_src` (an index array of the graph) with those
-// vertices encoded as HOT_BIT | slot, and the slot -> vertex table.
-int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, const int32_t *enc_src,
+// ids), gives them slots in ascending order of vertex, and builds the copy of
+// `enc_src` (an index array of the graph) with those vertices encoded as
+// HOT_BIT | slot.  None when they hold less than 1/min_share of the edges.
+int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, const int32_t *enc_src, int min_share,
               cudaStream_t s) {
     h.mem.release(s);
     h = HotSet();
@@ -616,17 +657,17 @@ int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, con
     unsigned long long *hist = nullptr;
     int st = tmp.alloc(hist, HOT_HIST, s);
     std::vector<unsigned long long> hh(HOT_HIST);
+    const int vb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)g->num_sms * 8));
     if (st == GP_OK) {
         cudaError_t e = cudaMemsetAsync(hist, 0, HOT_HIST * sizeof(unsigned long long), s);
-        int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)g->num_sms * 8));
         if (e == cudaSuccess) {
-            GP_LAUNCH("deg_hist", s, (k_deg_hist<<<blocks, 256, 0, s>>>(sel_off, n, hist)));
+            GP_LAUNCH("deg_hist", s, (k_deg_hist<<<vb, 256, 0, s>>>(sel_off, n, hist)));
             e = read_mapped(hh.data(), hist, HOT_HIST * sizeof(unsigned long long), s);
         }
         if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "hot-set histogram: %s", cudaGetErrorString(e));
     }
     // bucket B: every vertex above B is taken, then the lowest ids of bucket B until `slots`
-    int64_t above = 0;
+    int64_t above = 0, edges = 0;
     int B = 0;
     if (st == GP_OK) {
         for (int b = HOT_HIST - 1; b >= 1; --b) {
@@ -635,41 +676,44 @@ int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, con
                 break;
             }
             above += (int64_t)hh[b];
+            edges += (int64_t)hh[b] * b;
         }
     }
-    int32_t *list1 = nullptr, *list2 = nullptr;
-    int64_t c1 = 0, c2 = 0;
-    const int64_t top_lo = B > 0 ? (int64_t)B + 1 : 1;
-    if (st == GP_OK && top_lo <= HOT_HIST - 1)
-        st = select_by_degree(sel_off, n, top_lo, INT64_MAX, tmp, list1, c1, slots, nullptr, s);
-    if (st == GP_OK && B > 0) {
-        const int64_t hi = B == HOT_HIST - 1 ? INT64_MAX : (int64_t)B;
-        st = select_by_degree(sel_off, n, B, hi, tmp, list2, c2, slots - c1, nullptr, s);
+    // ties of bucket B; the last bucket holds every degree from HOT_HIST - 1 up
+    int32_t *ties = nullptr;
+    int64_t ntie = 0;
+    const bool top = B == HOT_HIST - 1;
+    if (st == GP_OK && B > 0 && above < slots) {
+        const int64_t lo = B, hi = top ? INT64_MAX : (int64_t)B;
+        edges += (slots - above) * (int64_t)B;
+        if (edges >= m / min_share) st = select_by_degree(sel_off, n, lo, hi, tmp, ties, ntie, slots - above, nullptr, s);
     }
-    const int64_t nhot = c1 + c2;
-    int32_t *slot = nullptr;
-    if (st == GP_OK) st = h.mem.alloc(h.hot_id, (size_t)std::max<int64_t>(nhot, 1), s);
+    if (st != GP_OK || edges < m / min_share) {
+        tmp.release(s);
+        return st;
+    }
+    const int64_t nhot = above + ntie, nwords = (n + 31) >> 5;
+    int64_t *counts = nullptr;
+    st = h.mem.alloc(h.hot_id, (size_t)std::max<int64_t>(nhot, 1), s);
     if (st == GP_OK) st = h.mem.alloc(h.c_hot, (size_t)std::max<int64_t>(nhot, 4), s);
     if (st == GP_OK) st = h.mem.alloc(h.enc_idx, (size_t)m, s);
-    if (st == GP_OK) st = tmp.alloc(slot, (size_t)n, s);
+    if (st == GP_OK) st = h.mem.alloc(h.bits, (size_t)nwords, s);
+    if (st == GP_OK) st = h.mem.alloc(h.prefix, (size_t)nwords, s);
+    if (st == GP_OK) st = tmp.alloc(counts, (size_t)nwords + 1, s);
     if (st == GP_OK) {
-        cudaError_t e = cudaSuccess;
-        if (c1) e = cudaMemcpyAsync(h.hot_id, list1, c1 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess && c2)
-            e = cudaMemcpyAsync(h.hot_id + c1, list2, c2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(slot, 0xff, (size_t)n * sizeof(int32_t), s);
-        if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "hot-set copy: %s", cudaGetErrorString(e));
-    }
-    if (st == GP_OK && nhot > 0) {
-        int b1 = (int)std::max<int64_t>(1, std::min<int64_t>((nhot + 255) / 256, 65535));
-        GP_LAUNCH("fill_slots", s, (k_fill_slots<<<b1, 256, 0, s>>>(h.hot_id, nhot, slot)));
-        int b2 = (int)std::max<int64_t>(1, std::min<int64_t>((m + 255) / 256, (int64_t)g->num_sms * 8));
-        GP_LAUNCH("encode_hot", s, (k_encode_hot<<<b2, 256, 0, s>>>(enc_src, m, slot, h.enc_idx)));
-        st = check_launch("encode_hot");
-    }
-    if (st == GP_OK) {
-        cudaError_t e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "hot-set build: %s", cudaGetErrorString(e));
+        const int wb = (int)std::max<int64_t>(1, std::min<int64_t>((nwords + 255) / 256, (int64_t)g->num_sms * 8));
+        const int64_t more_than = top ? INT64_MAX : (int64_t)B;  // B == 0: every vertex with edges
+        GP_LAUNCH("hot_bits", s, (k_hot_bits<<<vb, 256, 0, s>>>(sel_off, n, more_than, h.bits)));
+        if (ntie > 0)
+            GP_LAUNCH("hot_mark", s, (k_hot_mark<<<(unsigned)std::min<int64_t>((ntie + 255) / 256, 1024), 256, 0, s>>>(ties, ntie, h.bits)));
+        GP_LAUNCH("hot_counts", s, (k_hot_counts<<<wb, 256, 0, s>>>(h.bits, nwords, counts)));
+        st = exclusive_scan(counts, counts, nwords, tmp, s);
+        if (st == GP_OK) {
+            GP_LAUNCH("hot_slots", s, (k_hot_slots<<<wb, 256, 0, s>>>(h.bits, nwords, counts, h.prefix, h.hot_id)));
+            const int eb = (int)std::max<int64_t>(1, std::min<int64_t>((m + 255) / 256, (int64_t)g->num_sms * 8));
+            GP_LAUNCH("encode_hot", s, (k_encode_hot<<<eb, 256, 0, s>>>(enc_src, m, h.bits, h.prefix, h.enc_idx)));
+            st = check_launch("encode_hot");
+        }
     }
     tmp.release(s);
     if (st != GP_OK) {
@@ -682,15 +726,82 @@ int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, con
 }
 
 // Pull: the most gathered contributions are those of the largest out-degrees;
-// the gathered index array is CSC.
+// the gathered index array is CSC.  On a graph without skew they are no more
+// gathered than the others: below a 32nd of the edges the set is left out.
+constexpr int PULL_HOT_SHARE = 32;
 int build_pull_hot(gp_graph *g, int32_t slots, cudaStream_t s) {
-    return build_hot(g, g->pull_hot, slots, g->csr_off, g->csc_idx, s);
+    return build_hot(g, g->pull_hot, slots, g->csr_off, g->csc_idx, PULL_HOT_SHARE, s);
 }
 
 // Push: the most updated vertices are those of the largest in-degrees; the
 // scattered index array is CSR.
 int build_push_hot(gp_graph *g, int32_t slots, cudaStream_t s) {
-    return build_hot(g, g->push_hot, slots, g->csc_off, g->csr_idx, s);
+    return build_hot(g, g->push_hot, slots, g->csc_off, g->csr_idx, INT32_MAX, s);
+}
+
+// The list of rows: their first edges marked, the tiles told the row that
+// reaches over their start, rows over several tiles flagged.
+__global__ void k_tile_rows(int32_t *rows, int64_t nrows, const int64_t *off, int64_t ntiles, uint32_t *heads,
+                            int32_t *tile_row, int32_t *long_rows, unsigned long long *nlong) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nrows; r += stride) {
+        const int32_t v = rows[r];
+        const int64_t b = off[v], e = off[v + 1];
+        atomicOr(heads + (b >> 5), 1u << (b & 31));
+        // tiles t with b < t * TILE_EDGES <= e: the edge before their first one is this row's
+        for (int64_t t = b / TILE_EDGES + 1; t <= e / TILE_EDGES && t < ntiles; ++t) tile_row[t] = (int32_t)r;
+        if (r == 0) tile_row[0] = -1;
+        const int64_t span = (e - 1) / TILE_EDGES - b / TILE_EDGES;
+        if (span > 0) rows[r] = (int32_t)(HOT_BIT | (uint32_t)v);
+        if (span > TILE_LONG) long_rows[atomicAdd(nlong, 1ull)] = (int32_t)r;
+    }
+}
+
+int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s) {
+    if (t.ready) return GP_OK;
+    const int64_t n = g->n, m = g->m;
+    const int64_t nt = (m + TILE_EDGES - 1) / TILE_EDGES;
+    Arena tmp;
+    int32_t *full = nullptr, *empty = nullptr;
+    int64_t nfull = 0, nempty = 0;
+    unsigned long long *nl = nullptr, hl = 0;
+    // rows of over TILE_LONG tiles hold over (TILE_LONG - 1) * TILE_EDGES edges each
+    const int64_t cap_long = m / ((TILE_LONG - 1) * TILE_EDGES) + 1;
+    int st = select_by_degree(off, n, 1, INT64_MAX, tmp, full, nfull, INT64_MAX, nullptr, s);
+    if (st == GP_OK) st = select_by_degree(off, n, 0, 0, tmp, empty, nempty, INT64_MAX, nullptr, s);
+    if (st == GP_OK) st = tmp.alloc(nl, 1, s);
+    if (st == GP_OK) st = t.mem.alloc(t.rows, (size_t)n, s);
+    if (st == GP_OK) st = t.mem.alloc(t.heads, (size_t)nt * (TILE_EDGES / 8), s);
+    if (st == GP_OK) st = t.mem.alloc(t.tile_row, (size_t)nt, s);
+    if (st == GP_OK) st = t.mem.alloc(t.long_rows, (size_t)cap_long, s);
+    if (st == GP_OK) st = t.mem.alloc(t.acc, (size_t)nfull, s);
+    if (st == GP_OK) st = t.mem.alloc(t.carry, (size_t)nt, s);
+    if (st == GP_OK) {
+        cudaError_t e = cudaMemsetAsync(nl, 0, sizeof(*nl), s);
+        if (e == cudaSuccess && nt) e = cudaMemsetAsync(t.heads, 0, (size_t)nt * (TILE_EDGES / 8), s);
+        if (e == cudaSuccess && nfull) e = cudaMemcpyAsync(t.rows, full, nfull * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess && nempty)
+            e = cudaMemcpyAsync(t.rows + nfull, empty, nempty * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess && nfull) {
+            const int b = (int)std::min<int64_t>((nfull + 255) / 256, (int64_t)g->num_sms * 8);
+            GP_LAUNCH("tile_rows", s, (k_tile_rows<<<b, 256, 0, s>>>(t.rows, nfull, off, nt, (uint32_t *)t.heads, t.tile_row,
+                                                                    t.long_rows, nl)));
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = read_mapped(&hl, nl, sizeof(hl), s);
+        if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "edge tiles: %s", cudaGetErrorString(e));
+    }
+    tmp.release(s);
+    if (st != GP_OK) {
+        t.mem.release(s);
+        t = EdgeTiles();
+        return st;
+    }
+    t.ntiles = nt;
+    t.nrows = nfull;
+    t.nlong = (int64_t)hl;
+    t.ready = true;
+    return GP_OK;
 }
 
 int grid_blocks(const gp_graph *g, int threads_per_block) {
@@ -1117,6 +1228,7 @@ int gp_graph_free(gp_graph *g) {
     g->bfs_bins.mem.release(s);
     g->pull_hot.mem.release(s);
     g->push_hot.mem.release(s);
+    g->tiles.mem.release(s);
     g->mem.release(s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (dev != g->device && dev >= 0) cudaSetDevice(dev);
@@ -1141,7 +1253,8 @@ int gp_graph_info_get(const gp_graph *g, gp_graph_info *info) {
     info->symmetric = g->symmetric;
     info->weighted = g->weighted;
     info->device_bytes = (int64_t)(g->mem.total + g->pull_bins.mem.total + g->push_bins.mem.total +
-                                   g->bfs_bins.mem.total + g->pr.mem.total + g->bfs.mem.total + g->bfs.mmem.total);
+                                   g->bfs_bins.mem.total + g->tiles.mem.total + g->pr.mem.total +
+                                   g->bfs.mem.total + g->bfs.mmem.total);
     return GP_OK;
 }
 

@@ -1,0 +1,90 @@
+"""The pull sweep's edge tiles (256 edges each, whatever the degrees) at the
+places where they can go wrong: rows that end on, one before and one after a
+tile's edge, rows over several and over more than sixteen tiles, vertices
+without in-edges between them, one-edge rows, a last tile of one edge, index and
+weight arrays that do not start on a 32-byte boundary.  Against the same sweeps
+in FP64; tolerance of the method's contract (max-abs 1e-6, L1 1e-5)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+MAX_ABS, L1 = 1e-6, 1e-5
+T = 256
+
+
+@pytest.fixture(scope="module")
+def gp():
+    import torch
+
+    import paper_2010_16012_gb300 as gp
+
+    assert torch.cuda.is_available()
+    gp.load()
+    return gp
+
+
+DEGREES = {
+    "one edge": [1],
+    "one tile": [T],
+    "tile and one": [T, 1],
+    "short of a tile": [T - 1],
+    "over the edge": [T - 1, 2, T - 1, 1],
+    "aligned rows": [T, 0, T, 2 * T, 0, 0, T],
+    "one-edge rows": [1] * (3 * T + 1),
+    "lanes": [8] * 40 + [7, 9, 0, 1] * 30,
+    "sixteen tiles and more": [3, 16 * T, 5, 17 * T, 0, 18 * T + 1, 1, 40 * T - 9],
+    "none": [0, 0, 0],
+    "holes": [0, 0, 5, 0, 300, 0, 0, 1, 0],
+}
+
+
+def make(degrees, seed):
+    """CSC with the given in-degrees over at least 64 vertices, its CSR and weights (some sources repeat)."""
+    rng = np.random.default_rng(seed)
+    n = max(64, len(degrees))
+    deg = np.zeros(n, dtype=np.int64)
+    deg[:len(degrees)] = degrees
+    heads = np.repeat(np.arange(n), deg)
+    tails = np.sort(rng.integers(0, n, heads.size) * (rng.random(heads.size) < 0.8))
+    rng.shuffle(tails)
+    csc_off = np.concatenate([[0], np.cumsum(deg)])
+    order = np.argsort(tails, kind="stable")
+    csr_off = np.concatenate([[0], np.cumsum(np.bincount(tails, minlength=n))])
+    total = np.bincount(tails, minlength=n)[tails].astype(np.float64)
+    w = rng.uniform(0.2, 1.0, heads.size) / np.maximum(total, 1)
+    return n, csr_off, heads[order], w[order], csc_off, tails, w
+
+
+def sweeps(n, csr_off, csc_off, tails, w, iters, d=float(np.float32(0.85))):
+    heads = np.repeat(np.arange(n), np.diff(csc_off))
+    scale = w if w is not None else 1.0 / np.maximum(np.diff(csr_off), 1)[tails]
+    x = np.full(n, 1.0 / n)
+    for _ in range(iters):
+        x = (1 - d) / n + d * np.bincount(heads, weights=scale * x[tails], minlength=n)
+    return x
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("slots", [0, 5])
+@pytest.mark.parametrize("name", list(DEGREES))
+def test_tiles(gp, name, slots, weighted, shift):
+    import torch
+
+    n, csr_off, csr_idx, csr_w, csc_off, csc_idx, csc_w = make(DEGREES[name], seed=len(name))
+
+    def dev(a, dt):  # a view that starts `shift` elements into its storage
+        return torch.cat([torch.zeros(shift, dtype=dt), torch.from_numpy(np.ascontiguousarray(a)).to(dt)]).cuda()[shift:]
+
+    w = [dev(csr_w, torch.float32), dev(csc_w, torch.float32)] if weighted else [None, None]
+    G = gp.Graph(n, dev(csr_off, torch.int64), dev(csr_idx, torch.int32), dev(csc_off, torch.int64),
+                 dev(csc_idx, torch.int32), *w, validate=True)
+    G.set_options(pull_hot_slots=slots)
+    wx = csc_w.astype(np.float32).astype(np.float64) if weighted else None
+    for iters in (1, 2, 3, 8):
+        ref = sweeps(n, csr_off, csc_off, csc_idx, wx, iters)
+        x, st = gp.pagerank(G, gp.PULL, 0.85, iters)
+        err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
+        assert st["iters_done"] == iters
+        assert err.max() <= MAX_ABS and err.sum() <= L1, (name, iters, float(err.max()), float(err.sum()))
