@@ -497,7 +497,9 @@ __global__ void __launch_bounds__(512, 3) k_adj_light(PrArgs a) {
         for (int64_t r = (int64_t)(blockIdx.x - a.split_blocks) * blockDim.x + threadIdx.x; r < a.nbig; r += nth) {
             const int32_t v = a.big[r];
             float acc = 0.f;
-            for (int64_t j = a.cstart[r]; j < a.cstart[r + 1]; ++j) acc += a.chunk_part[j];
+            const int64_t c1 = a.cstart[r + 1];
+#pragma unroll 8
+            for (int64_t j = a.cstart[r]; j < c1; ++j) acc += a.chunk_part[j];
             const float y = base_term(a, v) + a.d * (post_factor(a, v) * acc);
             res.add(y, a.x[v]);
             a.y[v] = y;
@@ -1144,24 +1146,6 @@ static int pr_validate(const gp_graph *g, int mode, float damping, int iters, do
     return GP_OK;
 }
 
-__global__ void k_recompute_inv(const int64_t *csr_off, const float *csr_w, int64_t n, int normalize, float *inv_deg) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += stride) {
-        const int64_t b = csr_off[u], e = csr_off[u + 1];
-        float inv = 0.f;
-        if (e > b) {
-            if (normalize) {
-                double sw = 0.0;
-                for (int64_t j = b; j < e; ++j) sw += (double)csr_w[j];
-                inv = sw > 0.0 ? (float)(1.0 / sw) : 0.f;
-            } else {
-                inv = 1.f;
-            }
-        }
-        inv_deg[u] = inv;
-    }
-}
-
 }  // namespace gp
 
 using namespace gp;
@@ -1367,11 +1351,6 @@ extern "C" int gp_graph_set_weights(gp_graph *g, const float *csr_w, const float
     cudaStream_t s = (cudaStream_t)stream;
     g->csr_w = csr_w;
     g->csc_w = shared ? csr_w : csc_w;
-    const int64_t n = g->n;
-    if (n > 0) {
-        const int b = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)g->num_sms * 8));
-        GP_LAUNCH("recompute_inv", s, (k_recompute_inv<<<b, 256, 0, s>>>(g->csr_off, g->csr_w, n, g->normalized, g->inv_deg)));
-        GP_TRY(check_launch("recompute_inv"));
-    }
-    return GP_OK;
+    // weights as given: the scale is 1 (0 where there are no edges) whatever they are
+    return g->normalized ? weight_scale(g, s) : GP_OK;
 }
