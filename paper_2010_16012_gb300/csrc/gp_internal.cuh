@@ -400,45 +400,49 @@ __device__ __forceinline__ int nth_set_bit(uint32_t x, int j) {
 // ------------------------------------------------------------------ grid barrier
 
 // Grid-wide barrier for cooperative launches (all blocks co-resident).  The
-// spin-wait has an iteration limit: a block that gives up sets `err`, every
-// other waiting block sees it and gives up too, and all of them return false so
-// the kernel can return; the host then reports GP_ERR_TIMEOUT.
+// spin-wait has an iteration limit: a block that gives up sets `err` and marks
+// the count, every other waiting block sees the mark and gives up too, and all
+// of them return false so the kernel can return; the host then reports
+// GP_ERR_TIMEOUT.
 struct GridSync {
-    unsigned count;
-    unsigned gen;
+    unsigned long long count;  // arrivals since the launch's reset (GRID_GAVE_UP: a wait ran out)
     int err;
     int pad;
 };
 
-constexpr unsigned long long GRID_SPIN_LIMIT = 1ull << 24;  // ~2 s of 128 ns sleeps
+constexpr unsigned long long GRID_SPIN_LIMIT = 1ull << 24;  // polls of ~0.7 us
+constexpr unsigned long long GRID_GAVE_UP = 1ull << 63;
 
 // Returns false (and sets gs->err for every block) when a wait runs past
-// `limit` sleeps or another block has already given up.
+// `limit` polls or another block has already given up.
+//
+// Latency-bound: an arrival is one atomic on a count that only grows, and a
+// waiter polls that same word until the whole generation is in, so a barrier
+// costs about one trip to L2 for the last arrival and one for the poll that sees
+// it.  (A last arriver that resets the count and then publishes a generation, as
+// it was before, puts two more dependent trips and their fences in between.)
+// Polls are relaxed loads, and the one acquire fence follows them: an acquire
+// per poll would empty the L1 under the SM's other blocks.
 __device__ __forceinline__ bool grid_sync(GridSync *gs, unsigned nblocks, unsigned long long limit = GRID_SPIN_LIMIT) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned *vgen = &gs->gen;
-        volatile int *verr = &gs->err;
-        const unsigned g0 = *vgen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(&gs->count, 1u);
-        if (arrived == nblocks - 1) {
-            atomicExch(&gs->count, 0u);
-            __threadfence();
-            atomicAdd(&gs->gen, 1u);
-        } else {
-            unsigned long long spins = 0;
-            while (*vgen == g0) {
-                if (*verr || ++spins > limit) {
-                    atomicExch(&gs->err, 1);
-                    break;
-                }
-                __nanosleep(128);
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        const unsigned long long old = atomicAdd(&gs->count, 1ull) & ~GRID_GAVE_UP;
+        const unsigned long long gen = old >> 32 ? old / nblocks : (unsigned long long)((unsigned)old / nblocks);
+        const unsigned long long target = (gen + 1) * nblocks;
+        unsigned long long spins = 0, c;
+        while (true) {
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(&gs->count) : "memory");
+            if (c >= target) break;  // (a mark also ends the wait)
+            if (++spins > limit) {
+                atomicExch(&gs->err, 1);
+                c = atomicOr(&gs->count, GRID_GAVE_UP) | GRID_GAVE_UP;
+                break;
             }
         }
-        __threadfence();
-        s_ok = *verr == 0;
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        s_ok = (c & GRID_GAVE_UP) == 0;
     }
     __syncthreads();
     return s_ok != 0;
