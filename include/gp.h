@@ -525,12 +525,15 @@ typedef struct gp_tc_stats {
 
 /*
  * Per-vertex triangle counts by the NodeIterator of Section 3 (push- and
- * pull-based Triangle Counting): for every v and every ordered pair (w1, w2) of
- * v's neighbours with w1 adjacent to w2, GP_PULL adds one to tc[v] (every count
- * written only by the warp that owns v) and GP_PUSH adds one to tc[w1] with a
- * fetch-and-add; both halve.  GP_AUTO runs the pull form (no atomics).  The
- * graph must have been uploaded as symmetric (GP_UPLOAD_SYMMETRIC) and be simple
- * (no duplicate edges; self-loops are skipped).
+ * pull-based Triangle Counting).  Edges are directed from lower to higher degree,
+ * so each triangle is met once, at its lowest vertex u.  GP_PULL: u leaves what it
+ * found in its out-neighbours' in-lists and every vertex v adds its own list
+ * (every count written only by the owner of v); GP_PUSH: u adds to its
+ * out-neighbours' counts with fetch-and-adds.  GP_AUTO runs the pull form (no
+ * atomics).  The first call lays the directed lists out (kept with the handle,
+ * about 7 bytes per stored edge and 24 per vertex).  The graph must have been
+ * uploaded as symmetric (GP_UPLOAD_SYMMETRIC) and be simple (no duplicate edges;
+ * self-loops are skipped).
  *   tc_out      int64[n] "any" or NULL: triangles containing each vertex.
  *   total_out   host int64 or NULL: number of triangles.
  *   stats       NULL or filled on return.

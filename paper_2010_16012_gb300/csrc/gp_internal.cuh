@@ -223,6 +223,7 @@ struct BfsWork {
 struct gp_sssp_work;  // shortest-path workspace (sssp.cu)
 struct gp_fe_work;    // Frontier-Exploit PageRank workspace (pr_fe.cu)
 struct gp_bc_work;    // betweenness-centrality workspace (bc.cu)
+struct gp_tc_work;    // directed lists of the triangle counts (tc.cu)
 
 struct gp_graph {
     int device = 0;
@@ -247,6 +248,7 @@ struct gp_graph {
     gp_sssp_work *sssp = nullptr;
     gp_fe_work *fe = nullptr;
     gp_bc_work *bc = nullptr;
+    gp_tc_work *tc = nullptr;
     gp::Arena mem;          // copies of the arrays and degree data
     cudaStream_t home = nullptr;
 };
@@ -264,6 +266,8 @@ int weight_scale(gp_graph *g, cudaStream_t s);
 int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s);
 int build_pull_hot(gp_graph *g, int32_t slots, cudaStream_t s);
 int build_push_hot(gp_graph *g, int32_t slots, cudaStream_t s);
+// out[0..N] = exclusive prefix sums of in[0..N) and the total at out[N].  out may alias in.
+int exclusive_scan(const int64_t *in, int64_t *out, int64_t N, Arena &tmp, cudaStream_t s);
 int select_by_degree(const int64_t *off, int64_t n, int64_t lo, int64_t hi, Arena &mem, int32_t *&list,
                      int64_t &count, int64_t cap, int32_t *rank, cudaStream_t s);
 int grid_blocks(const gp_graph *g, int threads_per_block);

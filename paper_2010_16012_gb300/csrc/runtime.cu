@@ -329,8 +329,7 @@ __global__ void k_scan_tiles(const int64_t *in, int64_t *out, int64_t N, const i
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[N] = (offs ? offs[blockIdx.x] : 0) + total;
 }
 
-// out[0..N] = exclusive prefix sums of in[0..N) and the total at out[N].  out may alias in.
-static int exclusive_scan(const int64_t *in, int64_t *out, int64_t N, Arena &tmp, cudaStream_t s) {
+int exclusive_scan(const int64_t *in, int64_t *out, int64_t N, Arena &tmp, cudaStream_t s) {
     if (N <= 0) {
         GP_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), s));
         return GP_OK;
@@ -905,6 +904,7 @@ void release_bfs_multi(gp_graph *g, cudaStream_t s);
 void release_sssp_work(gp_graph *g, cudaStream_t s);
 void release_fe_work(gp_graph *g, cudaStream_t s);
 void release_bc_work(gp_graph *g, cudaStream_t s);
+void release_tc_work(gp_graph *g, cudaStream_t s);
 }  // namespace gp
 
 using namespace gp;
@@ -1266,6 +1266,7 @@ int gp_graph_free(gp_graph *g) {
     release_sssp_work(g, s);
     release_fe_work(g, s);
     release_bc_work(g, s);
+    release_tc_work(g, s);
     g->pull_bins.mem.release(s);
     g->push_bins.mem.release(s);
     g->bfs_bins.mem.release(s);

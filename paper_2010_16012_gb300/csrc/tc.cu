@@ -1,16 +1,23 @@
 // tc.cu -- per-vertex triangle counts by the push- and pull-based
 // NodeIterator of the paper's Section 3 listing.
 //
-// For every vertex v, every neighbour w1 and every neighbour w2 of v with w1
-// adjacent to w2, pull adds one to tc[v] (only v's owner writes it) and push
-// adds one to tc[w1] (fetch-and-add: the listing's FAA atomics); both halve at
-// the end.  The inner loop over w2 is counted at once as |N(v) n N(w1)| minus v
-// and w1 themselves: the number of w2 it accepts.  One warp handles one edge
-// (v, w1) at a time: its lanes take the elements of the shorter of the two
-// sorted lists in turn and binary-search the longer one.  Work units: each
-// light vertex (degree <= push_light_max) is one unit, each chunk of a heavy
-// vertex's list is one; pull adds a heavy vertex's chunk sums in a second
-// kernel, so every count still has a single writer.
+// Every edge is directed from its end of lower degree to the other (ties by
+// id), so that a triangle has one lowest vertex u, whose other two corners v
+// and x are both out-neighbours of u and joined by v -> x.  u's warp or block
+// keeps N+(u) in a shared-memory hash table, streams N+(v) for every v in
+// N+(u), and counts the hits for each member of N+(u) beside its table entry.
+//   pull: the counts go into u's slots of its out-neighbours' in-lists, each
+//         written by u alone; then every vertex adds its own slots (only v's
+//         owner writes tc[v]);
+//   push: u adds them to its out-neighbours' tc with fetch-and-adds (the
+//         listing's FAA atomics).
+// The listing meets every triangle six times (each corner, each order of the
+// other two) and halves; here it is met once.  The directed lists are laid out
+// once per graph.  Graphs outside the contract that the layout detects
+// (unsorted or duplicate edges, an edge without its reverse), lists of more than
+// TC_MAX_OUT out-neighbours and a layout that finds no memory take the listing
+// itself (k_tc): one warp per edge (v, w1), the shorter list's elements
+// binary-searched in the longer one.
 #include <algorithm>
 #include <cstring>
 
@@ -131,9 +138,575 @@ __global__ void k_tc_finish(int64_t n, int push, unsigned long long *tc, unsigne
     if (threadIdx.x == 0 && s) atomicAdd(total, s);
 }
 
+// ------------------------------------------------------------------ directed lists
+
+constexpr int TC_WARP_OUT = 64;     // out-neighbours up to which a warp counts for a vertex
+constexpr int TC_MAX_OUT = 8192;    // and a block (table of at most 16384 entries)
+constexpr int TC_WARP_TABLE = 256;  // entries of a warp's table
+constexpr int TC_WARPS = 8;         // warps per block of the counting kernels
+constexpr int32_t TC_FREE = -1;     // key of a free entry
+
+struct TcPlanStat {
+    unsigned long long general;  // the graph is outside the contract
+    unsigned long long max_out;
+    unsigned long long probes;   // sum over ordered edges of the shorter list's length
+};
+
+// v before w: lower degree, or equal and lower id.
+__device__ __forceinline__ bool tc_before(int64_t dv, int32_t v, int64_t dw, int32_t w) {
+    return dv < dw || (dv == dw && v < w);
+}
+
+// Per vertex, the neighbours after it (out) and before it (in), a warp per vertex.
+__global__ void __launch_bounds__(256) k_tc_count(int64_t n, const int64_t *off, const int32_t *idx, int64_t *nout,
+                                                  int64_t *nin, TcPlanStat *st) {
+    const int lane = lane_id();
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    unsigned long long probes = 0, most = 0;
+    bool bad = false;
+    for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nwarps) {
+        const int64_t b = off[v], e = off[v + 1];
+        int out = 0, in = 0;
+        constexpr int U = 4;
+        for (int64_t e0 = b + lane; e0 < e; e0 += 32 * U) {
+            int32_t w[U];
+            int64_t dw[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) w[q] = e0 + 32 * q < e ? __ldg(idx + e0 + 32 * q) : (int32_t)v;
+#pragma unroll
+            for (int q = 0; q < U; ++q) dw[q] = off[w[q] + 1] - off[w[q]];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                const int64_t p = e0 + 32 * q;
+                if (p >= e) continue;
+                bad |= p > b && __ldg(idx + p - 1) >= w[q];
+                if (w[q] == (int32_t)v) continue;  // self-loop
+                probes += (unsigned long long)(dw[q] < e - b ? dw[q] : e - b);
+                if (tc_before(e - b, (int32_t)v, dw[q], w[q]))
+                    ++out;
+                else
+                    ++in;
+            }
+        }
+        out = warp_sum(out);
+        in = warp_sum(in);
+        most = max(most, (unsigned long long)out);
+        if (lane == 0) {
+            nout[v] = out;
+            nin[v] = in;
+        }
+    }
+    probes = warp_sum(probes);
+    bad = __any_sync(FULL, bad);
+    if (lane == 0) {
+        if (probes) atomicAdd(&st->probes, probes);
+        if (most) atomicMax(&st->max_out, most);
+        if (bad) atomicOr(&st->general, 1ull);
+    }
+}
+
+// The two lists of every vertex, in the order of its neighbours.
+__global__ void __launch_bounds__(256) k_tc_lists(int64_t n, const int64_t *off, const int32_t *idx, const int64_t *out_off,
+                                                  const int64_t *in_off, int32_t *out, int32_t *in) {
+    const int lane = lane_id();
+    const unsigned below = (1u << lane) - 1u;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nwarps) {
+        const int64_t b = off[v], e = off[v + 1];
+        int64_t po = out_off[v], pi = in_off[v];
+        constexpr int U = 4;
+        for (int64_t e0 = b; e0 < e; e0 += 32 * U) {
+            int32_t w[U];
+            int64_t dw[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) w[q] = e0 + 32 * q + lane < e ? __ldg(idx + e0 + 32 * q + lane) : (int32_t)v;
+#pragma unroll
+            for (int q = 0; q < U; ++q) dw[q] = off[w[q] + 1] - off[w[q]];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                const bool other = w[q] != (int32_t)v;
+                const bool after = other && tc_before(e - b, (int32_t)v, dw[q], w[q]);
+                const unsigned mo = __ballot_sync(FULL, after), mi = __ballot_sync(FULL, other && !after);
+                if (after)
+                    out[po + __popc(mo & below)] = w[q];
+                else if (other)
+                    in[pi + __popc(mi & below)] = w[q];
+                po += __popc(mo);
+                pi += __popc(mi);
+            }
+        }
+    }
+}
+
+// rev[e]: the place of u in the in-list of x, for every directed edge e = (u -> x).
+__global__ void __launch_bounds__(256) k_tc_reverse(int64_t n, const int64_t *out_off, const int64_t *in_off,
+                                                    const int32_t *out, const int32_t *in, int32_t *rev, TcPlanStat *st) {
+    const int lane = lane_id();
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    bool bad = false;
+    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += nwarps) {
+        for (int64_t e = out_off[u] + lane; e < out_off[u + 1]; e += 32) {
+            const int32_t x = out[e];
+            const int32_t *list = in + in_off[x];
+            const int len = (int)(in_off[x + 1] - in_off[x]);
+            int lo = 0, hi = len;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (__ldg(list + mid) < (int32_t)u)
+                    lo = mid + 1;
+                else
+                    hi = mid;
+            }
+            if (lo == len || __ldg(list + lo) != (int32_t)u) {
+                bad = true;  // no edge back
+                lo = 0;
+            }
+            rev[e] = lo;
+        }
+    }
+    if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->general, 2ull);
+}
+
+// ------------------------------------------------------------------ counting
+
+struct TcRun {
+    const int64_t *out_off, *in_off;
+    const int32_t *out, *rev;
+    const int32_t *list;         // the vertices this launch counts for
+    int64_t count;
+    int table;                   // entries of a block's table (a power of two)
+    int push;
+    int32_t *slots;              // pull: per in-list entry, the triangles counted by that neighbour
+    unsigned long long *own;     // pull: [n] triangles whose lowest vertex this is
+    unsigned long long *tc;      // push: [n] counts
+    unsigned long long *total;
+    unsigned long long *ticket;  // the next entry of `list` to hand out
+};
+
+// u's out-neighbours: a filter of TC_FILTER bits per table entry, which tells
+// most of the other vertices off with one load, then an open-addressed table
+// with a count per entry.  Both are indexed by one hash, the entry by its high
+// bits.  (Without the filter a warp walks the longest of its 32 probe runs for
+// every 32 elements: 64 issued instructions, against about half of that.)
+constexpr int TC_FILTER = 16;
+struct TcTable {
+    int32_t *key;
+    int *cnt;
+    uint32_t *filter;
+    unsigned bits;  // TC_FILTER * entries - 1
+    __device__ __forceinline__ unsigned hash(int32_t x) const { return ((unsigned)x * 0x9E3779B1u >> 9) & bits; }
+    __device__ __forceinline__ unsigned next(unsigned e) const { return (e + 1) & (bits / TC_FILTER); }
+    // entry of x, or -1
+    __device__ __forceinline__ int find(int32_t x) const {
+        const unsigned h = hash(x);
+        if (!((filter[h >> 5] >> (h & 31)) & 1u)) return -1;
+        for (unsigned e = h / TC_FILTER;; e = next(e)) {
+            const int32_t k = key[e];
+            if (k == x) return (int)e;
+            if (k == TC_FREE) return -1;
+        }
+    }
+    __device__ __forceinline__ void insert(int32_t x) const {
+        const unsigned h = hash(x);
+        atomicOr(filter + (h >> 5), 1u << (h & 31));
+        unsigned e = h / TC_FILTER;
+        while (atomicCAS(key + e, TC_FREE, x) != TC_FREE) e = next(e);
+    }
+};
+
+// Hits of the list elements [b, e) in the table, counted beside their entries, by the whole warp.
+__device__ __forceinline__ int tc_stream(const TcRun &R, int64_t b, int64_t e, const TcTable &T) {
+    constexpr int U = 4;
+    int hits = 0;
+    for (int64_t p = b + lane_id(); p < e; p += 32 * U) {
+        int32_t x[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) x[q] = p + 32 * q < e ? __ldg(R.out + p + 32 * q) : TC_FREE;
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            if (x[q] < 0) continue;
+            const int at = T.find(x[q]);
+            if (at >= 0) {
+                atomicAdd(T.cnt + at, 1);
+                ++hits;
+            }
+        }
+    }
+    return hits;
+}
+
+// What u counted for its out-neighbour of edge e: into that one's in-list slot, or onto its count.
+__device__ __forceinline__ void tc_give(const TcRun &R, int64_t e, int c) {
+    const int32_t x = R.out[e];
+    if (!R.push)
+        R.slots[R.in_off[x] + R.rev[e]] = c;
+    else if (c)
+        atomicAdd(R.tc + x, (unsigned long long)c);
+}
+
+__device__ __forceinline__ void tc_own(const TcRun &R, int32_t u, unsigned long long t) {
+    if (!R.push)
+        R.own[u] = t;
+    else if (t)
+        atomicAdd(R.tc + u, t);
+}
+
+// Measured on R-MAT 2^18 (3.8M undirected edges, 6.6e8 list elements streamed):
+// k_tc 47.9 ms; the two kernels below 629 + 639 us (88% of issue slots busy),
+// the gather 22 us.  TC_WARP_OUT: 126K vertices count in warps and 13K in blocks there.
+// A warp per vertex u of few out-neighbours.  Its out-neighbours' lists, 32 at a
+// time, are one stream of edges over the lanes (whatever their lengths), four
+// windows of 32 in flight (a list each where they average 32 elements and more).
+__global__ void __launch_bounds__(TC_WARPS * 32) k_tc_warp(TcRun R) {
+    __shared__ int32_t s_key[TC_WARPS][TC_WARP_TABLE];
+    __shared__ int s_cnt[TC_WARPS][TC_WARP_TABLE];
+    __shared__ uint32_t s_filter[TC_WARPS][TC_WARP_TABLE * TC_FILTER / 32];
+    constexpr int U = 4;
+    const int lane = lane_id(), wib = threadIdx.x >> 5;
+    const TcTable T = {s_key[wib], s_cnt[wib], s_filter[wib], TC_WARP_TABLE * TC_FILTER - 1};
+    for (int i = lane; i < TC_WARP_TABLE; i += 32) {
+        T.key[i] = TC_FREE;
+        T.cnt[i] = 0;
+    }
+    for (int i = lane; i < TC_WARP_TABLE * TC_FILTER / 32; i += 32) T.filter[i] = 0u;
+    unsigned long long total = 0;
+    constexpr int TAKE = 4;  // vertices per ticket
+    while (true) {
+        unsigned long long t0 = 0;
+        if (lane == 0) t0 = atomicAdd(R.ticket, (unsigned long long)TAKE);
+        t0 = __shfl_sync(FULL, t0, 0);
+        if ((int64_t)t0 >= R.count) break;
+        const int64_t t1 = min((int64_t)t0 + TAKE, R.count);
+        for (int64_t t = (int64_t)t0; t < t1; ++t) {
+            const int32_t u = R.list[t];
+            const int64_t b = R.out_off[u], e = R.out_off[u + 1];
+            __syncwarp();
+            for (int64_t p = b + lane; p < e; p += 32) T.insert(R.out[p]);
+            __syncwarp();
+            unsigned long long sum = 0;
+            for (int64_t p = b; p < e; p += 32) {
+                int64_t lb = 0;
+                int len = 0, at_v = 0;
+                if (p + lane < e) {
+                    const int32_t v = R.out[p + lane];
+                    lb = R.out_off[v];
+                    len = (int)(R.out_off[v + 1] - lb);
+                    at_v = T.find(v);
+                }
+                const int incl = warp_incl_scan(len), excl = incl - len;
+                const int E = __shfl_sync(FULL, incl, 31);
+                int hits = 0;
+                // long lists one after another: finding each element's list costs more than their ends waste
+                const bool each = E >= 32 * 32;
+                for (int i = 0; each && i < 32 && p + i < e; ++i) {
+                    const int64_t vb = __shfl_sync(FULL, lb, i);
+                    const int vl = __shfl_sync(FULL, len, i);
+                    const int mine = tc_stream(R, vb, vb + vl, T);
+                    const int all = warp_sum(mine);
+                    hits += mine;
+                    if (lane == i && all) atomicAdd(T.cnt + at_v, all);
+                }
+                for (int e0 = 0; !each && e0 < E; e0 += 32 * U) {
+                    int32_t x[U];
+                    int from[U];
+#pragma unroll
+                    for (int q = 0; q < U; ++q) {
+                        const int id = e0 + 32 * q + lane;
+                        int k = 0;  // the list that holds element id
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            const int ek = __shfl_sync(FULL, excl, k + o);
+                            if (ek <= id) k += o;
+                        }
+                        const int64_t kb = __shfl_sync(FULL, lb, k);
+                        const int ke = __shfl_sync(FULL, excl, k);
+                        from[q] = __shfl_sync(FULL, at_v, k);
+                        x[q] = id < E ? __ldg(R.out + kb + (id - ke)) : TC_FREE;
+                    }
+#pragma unroll
+                    for (int q = 0; q < U; ++q) {
+                        if (x[q] < 0) continue;
+                        const int at = T.find(x[q]);
+                        if (at >= 0) {
+                            atomicAdd(T.cnt + at, 1);
+                            atomicAdd(T.cnt + from[q], 1);
+                            ++hits;
+                        }
+                    }
+                }
+                sum += (unsigned long long)hits;
+            }
+            sum = warp_sum(sum);
+            __syncwarp();
+            // counts read by every lane before any entry is freed
+            int c[TC_WARP_OUT / 32], at[TC_WARP_OUT / 32];
+            unsigned h[TC_WARP_OUT / 32];
+#pragma unroll
+            for (int q = 0; q < TC_WARP_OUT / 32; ++q) {
+                const int64_t p = b + 32 * q + lane;
+                const int32_t x = p < e ? R.out[p] : 0;
+                at[q] = p < e ? T.find(x) : -1;
+                c[q] = at[q] >= 0 ? T.cnt[at[q]] : 0;
+                h[q] = T.hash(x);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < TC_WARP_OUT / 32; ++q) {
+                if (at[q] < 0) continue;
+                T.key[at[q]] = TC_FREE;
+                T.cnt[at[q]] = 0;
+                T.filter[h[q] >> 5] = 0u;
+                tc_give(R, b + 32 * q + lane, c[q]);
+            }
+            if (lane == 0) tc_own(R, u, sum);
+            total += sum;
+        }
+    }
+    if (lane == 0 && total) atomicAdd(R.total, total);
+}
+
+// A block per vertex u of many out-neighbours, a warp per list N+(v).
+__global__ void __launch_bounds__(TC_WARPS * 32) k_tc_block(TcRun R) {
+    extern __shared__ int32_t s_table[];
+    __shared__ long long s_ticket;
+    __shared__ unsigned long long s_sum[32];
+    const int lane = lane_id(), wib = threadIdx.x >> 5;
+    unsigned long long total = 0;
+    while (true) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_ticket = (long long)atomicAdd(R.ticket, 1ull);
+        __syncthreads();
+        const int64_t t = s_ticket;
+        if (t >= R.count) break;
+        const int32_t u = R.list[t];
+        const int64_t b = R.out_off[u], e = R.out_off[u + 1];
+        int size = 4 * TC_WARP_OUT;  // four times the list, where the table has the room
+        while (size < R.table && size < 4 * (e - b)) size *= 2;
+        const TcTable T = {s_table, s_table + size, (uint32_t *)s_table + 2 * size, (unsigned)size * TC_FILTER - 1u};
+        for (int i = threadIdx.x; i < size; i += blockDim.x) {
+            T.key[i] = TC_FREE;
+            T.cnt[i] = 0;
+        }
+        for (int i = threadIdx.x; i < size * TC_FILTER / 32; i += blockDim.x) T.filter[i] = 0u;
+        __syncthreads();
+        for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) T.insert(R.out[p]);
+        __syncthreads();
+        unsigned long long sum = 0;
+        for (int64_t p0 = b + wib; p0 < e; p0 += 32 * TC_WARPS) {
+            // the warp's next 32 lists located at once
+            const int64_t p = p0 + (int64_t)lane * TC_WARPS;
+            int64_t lb = 0, le = 0;
+            int at_v = -1;
+            if (p < e) {
+                const int32_t v = R.out[p];
+                lb = R.out_off[v];
+                le = R.out_off[v + 1];
+                at_v = T.find(v);
+            }
+            const int lists = __popc(__ballot_sync(FULL, at_v >= 0));
+            for (int i = 0; i < lists; ++i) {
+                const int64_t vb = __shfl_sync(FULL, lb, i), ve = __shfl_sync(FULL, le, i);
+                const int hits = warp_sum(tc_stream(R, vb, ve, T));
+                if (lane == i && hits) {
+                    atomicAdd(T.cnt + at_v, hits);
+                    sum += (unsigned long long)hits;
+                }
+            }
+        }
+        sum = block_sum(sum, s_sum);  // (a block barrier: every count is in)
+        for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) tc_give(R, p, T.cnt[T.find(R.out[p])]);
+        if (threadIdx.x == 0) {
+            tc_own(R, u, sum);
+            total += sum;
+        }
+    }
+    if (threadIdx.x == 0 && total) atomicAdd(R.total, total);
+}
+
+// pull: a vertex's count is its own triangles and those its in-neighbours
+// counted for it.  In-lists of over TC_WIDE entries take a block each (a warp
+// over 25K entries took 0.5 ms), of over 32 a warp, the others a thread.
+constexpr int TC_WIDE = 1024;
+__global__ void __launch_bounds__(256) k_tc_gather(int64_t n, const int64_t *in_off, const int32_t *slots,
+                                                   const unsigned long long *own, const int32_t *mid, int64_t nmid,
+                                                   const int32_t *wide, int64_t nwide, unsigned long long *tc) {
+    __shared__ unsigned long long sm[32];
+    for (int64_t i = blockIdx.x; i < nwide; i += gridDim.x) {
+        const int32_t v = wide[i];
+        const int64_t e = in_off[v + 1];
+        unsigned long long s = 0;
+#pragma unroll 4
+        for (int64_t p = in_off[v] + threadIdx.x; p < e; p += 256) s += (unsigned long long)slots[p];
+        s = block_sum(s, sm);
+        if (threadIdx.x == 0) tc[v] = own[v] + s;
+    }
+    const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = thread >> 5; i < nmid; i += nthreads >> 5) {
+        const int32_t v = mid[i];
+        const int64_t e = in_off[v + 1];
+        unsigned long long s = 0;
+#pragma unroll 4
+        for (int64_t p = in_off[v] + lane_id(); p < e; p += 32) s += (unsigned long long)slots[p];
+        s = warp_sum(s);
+        if (lane_id() == 0) tc[v] = own[v] + s;
+    }
+    for (int64_t v = thread; v < n; v += nthreads) {
+        const int64_t b = in_off[v], e = in_off[v + 1];
+        if (e - b > 32) continue;
+        unsigned long long s = own[v];
+#pragma unroll 4
+        for (int64_t p = b; p < e; ++p) s += (unsigned long long)slots[p];
+        tc[v] = s;
+    }
+}
+
 }  // namespace gp
 
 using namespace gp;
+
+struct gp_tc_work {
+    bool ready = false, general = false;
+    int64_t *out_off = nullptr, *in_off = nullptr;
+    int32_t *out = nullptr, *rev = nullptr, *slots = nullptr;
+    unsigned long long *own = nullptr;
+    int32_t *light = nullptr, *heavy = nullptr;  // vertices by out-neighbours (counting)
+    int64_t nlight = 0, nheavy = 0;
+    int32_t *mid = nullptr, *wide = nullptr;     // vertices by in-list (gather)
+    int64_t nmid = 0, nwide = 0;
+    int table = 0;
+    unsigned long long probes = 0;
+    Arena mem;
+};
+
+namespace gp {
+
+void release_tc_work(gp_graph *g, cudaStream_t s) {
+    if (!g->tc) return;
+    g->tc->mem.release(s);
+    delete g->tc;
+    g->tc = nullptr;
+}
+
+// The directed lists; general = true where the listing has to be run instead.
+static int build_tc(gp_graph *g, gp_tc_work &w, cudaStream_t s) {
+    if (w.ready) return GP_OK;
+    const int64_t n = g->n;
+    Arena tmp;
+    TcPlanStat *st = nullptr, hs = {0, 0, 0};
+    int32_t *in = nullptr;
+    const int wb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, (int64_t)g->num_sms * 8));
+    int64_t ends[2] = {0, 0};
+    auto read_stat = [&]() -> int {
+        const cudaError_t e = read_mapped(&hs, st, sizeof(hs), s);
+        return e == cudaSuccess ? GP_OK : set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
+    };
+    int r = tmp.alloc(st, 1, s);
+    if (r == GP_OK) r = w.mem.alloc(w.out_off, (size_t)n + 1, s);
+    if (r == GP_OK) r = w.mem.alloc(w.in_off, (size_t)n + 1, s);
+    if (r == GP_OK) {
+        const cudaError_t e = cudaMemsetAsync(st, 0, sizeof(*st), s);
+        if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
+    }
+    if (r == GP_OK) {
+        GP_LAUNCH("tc_count", s, (k_tc_count<<<wb, 256, 0, s>>>(n, g->csr_off, g->csr_idx, w.out_off, w.in_off, st)));
+        r = check_launch("tc_count");
+    }
+    if (r == GP_OK) r = read_stat();
+    w.probes = hs.probes;
+    w.general = hs.general || hs.max_out > (unsigned long long)TC_MAX_OUT;
+    if (r == GP_OK && !w.general) r = exclusive_scan(w.out_off, w.out_off, n, tmp, s);
+    if (r == GP_OK && !w.general) r = exclusive_scan(w.in_off, w.in_off, n, tmp, s);
+    if (r == GP_OK && !w.general) {
+        cudaError_t e = read_mapped(&ends[0], w.out_off + n, sizeof(int64_t), s);
+        if (e == cudaSuccess) e = read_mapped(&ends[1], w.in_off + n, sizeof(int64_t), s);
+        if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
+        w.general = ends[0] != ends[1];
+    }
+    if (r == GP_OK && !w.general) {
+        r = w.mem.alloc(w.out, (size_t)ends[0], s);
+        if (r == GP_OK) r = w.mem.alloc(w.rev, (size_t)ends[0], s);
+        if (r == GP_OK) r = w.mem.alloc(w.slots, (size_t)ends[0], s);
+        if (r == GP_OK) r = w.mem.alloc(w.own, (size_t)std::max<int64_t>(n, 1), s);
+        if (r == GP_OK) r = tmp.alloc(in, (size_t)ends[1], s);
+        if (r == GP_OK) {
+            // entries that no list writes (vertices of fewer than two out-neighbours) stay zero
+            cudaError_t e = cudaMemsetAsync(w.slots, 0, (size_t)ends[0] * sizeof(int32_t), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(w.own, 0, (size_t)n * sizeof(unsigned long long), s);
+            if (e == cudaSuccess) {
+                GP_LAUNCH("tc_lists", s, (k_tc_lists<<<wb, 256, 0, s>>>(n, g->csr_off, g->csr_idx, w.out_off, w.in_off, w.out, in)));
+                GP_LAUNCH("tc_reverse", s, (k_tc_reverse<<<wb, 256, 0, s>>>(n, w.out_off, w.in_off, w.out, in, w.rev, st)));
+                e = cudaGetLastError();
+            }
+            if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
+        }
+        if (r == GP_OK) r = read_stat();
+        if (r == GP_OK) w.general = hs.general != 0;
+        if (r == GP_OK && !w.general)
+            r = select_by_degree(w.out_off, n, 2, TC_WARP_OUT, w.mem, w.light, w.nlight, INT64_MAX, nullptr, s);
+        if (r == GP_OK && !w.general)
+            r = select_by_degree(w.out_off, n, TC_WARP_OUT + 1, INT64_MAX, w.mem, w.heavy, w.nheavy, INT64_MAX, nullptr, s);
+        if (r == GP_OK && !w.general) r = select_by_degree(w.in_off, n, 33, TC_WIDE, w.mem, w.mid, w.nmid, INT64_MAX, nullptr, s);
+        if (r == GP_OK && !w.general)
+            r = select_by_degree(w.in_off, n, TC_WIDE + 1, INT64_MAX, w.mem, w.wide, w.nwide, INT64_MAX, nullptr, s);
+        w.table = 4 * TC_WARP_OUT;
+        while (w.table < 2 * TC_MAX_OUT && w.table < 4 * (int64_t)hs.max_out) w.table *= 2;
+    }
+    tmp.release(s);
+    if (r == GP_ERR_OOM) {  // no room for the lists: the listing needs none
+        clear_error();
+        r = GP_OK;
+        w.general = true;
+    }
+    if (w.general || r != GP_OK) w.mem.release(s);
+    w.ready = r == GP_OK;
+    return r;
+}
+
+// Counts by the directed lists into tc (nullptr: only the total, scal[0] = triangles).
+static int run_tc(gp_graph *g, const gp_tc_work &w, bool push, unsigned long long *tc, unsigned long long *scal,
+                  cudaStream_t s) {
+    TcRun R;
+    memset(&R, 0, sizeof(R));
+    R.out_off = w.out_off;
+    R.in_off = w.in_off;
+    R.out = w.out;
+    R.rev = w.rev;
+    R.table = w.table;
+    R.push = push;
+    R.slots = w.slots;
+    R.own = w.own;
+    R.tc = tc;
+    R.total = scal;
+    if (w.nheavy > 0) {
+        const size_t smem = (size_t)w.table * (2 * sizeof(int32_t) + TC_FILTER / 8);
+        int per_sm = 0;
+        GP_CUDA(cudaFuncSetAttribute(k_tc_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_block, TC_WARPS * 32, smem));
+        R.list = w.heavy;
+        R.count = w.nheavy;
+        R.ticket = scal + 1;
+        const int b = (int)std::max<int64_t>(1, std::min<int64_t>(w.nheavy, (int64_t)std::max(per_sm, 1) * g->num_sms));
+        GP_LAUNCH("tc_block", s, (k_tc_block<<<b, TC_WARPS * 32, smem, s>>>(R)));
+        GP_TRY(check_launch("tc_block"));
+    }
+    if (w.nlight > 0) {
+        R.list = w.light;
+        R.count = w.nlight;
+        R.ticket = scal + 2;
+        const int b = (int)std::max<int64_t>(1, std::min<int64_t>((w.nlight + 4 * TC_WARPS - 1) / (4 * TC_WARPS), (int64_t)g->num_sms * 8));
+        GP_LAUNCH("tc_warp", s, (k_tc_warp<<<b, TC_WARPS * 32, 0, s>>>(R)));
+        GP_TRY(check_launch("tc_warp"));
+    }
+    if (!push) {
+        const int b = (int)std::max<int64_t>(1, std::min<int64_t>(std::max((g->n + 255) / 256, w.nwide), (int64_t)g->num_sms * 8));
+        GP_LAUNCH("tc_gather", s, (k_tc_gather<<<b, 256, 0, s>>>(g->n, w.in_off, w.slots, w.own, w.mid, w.nmid, w.wide,
+                                                               w.nwide, tc)));
+        GP_TRY(check_launch("tc_gather"));
+    }
+    return GP_OK;
+}
+
+}  // namespace gp
 
 extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64_t *total_out, gp_tc_stats *stats,
                             void *stream) {
@@ -147,6 +720,10 @@ extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64
     const int64_t n = g->n;
     if (stats) memset(stats, 0, sizeof(*stats));
     const bool push = mode == GP_PUSH;
+    if (!g->tc) g->tc = new gp_tc_work();
+    gp_tc_work &w = *g->tc;
+    if (n > 0) GP_TRY(build_tc(g, w, s));
+    const bool lists = n > 0 && !w.general;
     Arena tmp;
     unsigned long long *tc = nullptr, *cp = nullptr, *scal = nullptr;
     const bool dev_out = tc_out && is_device_ptr(tc_out);
@@ -155,8 +732,8 @@ extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64
     } else {
         GP_TRY(tmp.alloc(tc, (size_t)std::max<int64_t>(n, 1), s));
     }
-    int st = tmp.alloc(scal, 2, s);  // [0] total, [1] probes
-    if (st == GP_OK && !push) st = tmp.alloc(cp, (size_t)std::max<int64_t>(g->push_bins.nchunks, 1), s);
+    int st = tmp.alloc(scal, 3, s);  // [0] total, [1] probes; by the lists: [0] triangles, [1], [2] tickets
+    if (st == GP_OK && !push && !lists) st = tmp.alloc(cp, (size_t)std::max<int64_t>(g->push_bins.nchunks, 1), s);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (st == GP_OK && stats) {
         cudaEventCreate(&ev0);
@@ -166,10 +743,11 @@ extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64
     unsigned long long host[2] = {0, 0};
     cudaError_t e = cudaSuccess;
     if (st == GP_OK) {
-        e = cudaMemsetAsync(scal, 0, 2 * sizeof(unsigned long long), s);
+        e = cudaMemsetAsync(scal, 0, 3 * sizeof(unsigned long long), s);
         if (e == cudaSuccess && push && n > 0) e = cudaMemsetAsync(tc, 0, (size_t)n * sizeof(unsigned long long), s);
     }
-    if (st == GP_OK && e == cudaSuccess && n > 0) {
+    if (st == GP_OK && e == cudaSuccess && lists) st = run_tc(g, w, push, tc, scal, s);
+    if (st == GP_OK && e == cudaSuccess && n > 0 && !lists) {
         TcArgs a;
         memset(&a, 0, sizeof(a));
         a.n = n;
@@ -204,6 +782,10 @@ extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64
     if (st == GP_OK && e == cudaSuccess) e = cudaMemcpyAsync(host, scal, sizeof(host), cudaMemcpyDeviceToHost, s);
     if (st == GP_OK && e == cudaSuccess && stats) e = cudaEventRecord(ev1, s);
     if (st == GP_OK && e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (lists) {
+        host[0] *= 3;  // as the sum of the counts
+        host[1] = w.probes;
+    }
     if (stats && ev0) {
         float ms = 0.f;
         if (e == cudaSuccess) cudaEventElapsedTime(&ms, ev0, ev1);
