@@ -55,12 +55,13 @@ struct BGraph {  // per-graph device descriptor
     int32_t *levels;         // MS-BFS output [n][64]
     int64_t big0, nbig;      // big in-degree vertices of this graph in the big list
     int64_t chunk0, nchunk;  // their in-edge chunks in the chunk list
+    int64_t ochunk0, nochunk;  // out-edge chunks of the vertices of big out-degree (the in-edge ones where the orders are one)
 };
 
-struct BChunk {  // warp work item: a piece of a big vertex's in-edge list
+struct BChunk {  // warp work item: a piece of a big vertex's edge list
     int64_t beg;
     int32_t len;
-    int32_t graph;
+    int32_t v;
 };
 
 struct BJob {  // one graph and the column slice [c0, c0 + 32 * kpl)
@@ -96,6 +97,7 @@ struct BatchDev {
     const int32_t *seeds;   // [ngraphs][K]
     int32_t *iters_done;    // [ngraphs][K]
     const int32_t *sources; // [ngraphs][64] (MS-BFS)
+    int32_t *const *lev_out;  // [ngraphs] where this call's levels go (MS-BFS)
     int32_t *counters;      // [0] most PPR sweeps of any column, [1] BFS levels, [2] packed columns
     int32_t pack_max;       // a job stops once at most this many of its columns iterate (0: never)
     BPend *pend;            // [ngraphs * K] the columns left iterating, in job order
@@ -427,8 +429,48 @@ __global__ void __launch_bounds__(BT_THREADS, GP_BT_MINB) k_ppr_persistent(Batch
 
 // ------------------------------------------------------------------ batched multi-source BFS
 
+// Latency-bound: few bytes per level, so what counts is the longest chain of
+// dependent loads.  Lists above big_min edges are cut in chunks that warps over
+// the whole grid take (one warp walking a hub's 25K edges, 32 at a time, set the
+// time of a level), and every list is read BF_U edges at a time.
+constexpr int BF_U = 4;
+
+// Top-down over the edges [b, e), from `first`, every `step`: f into the out-neighbours' N.
+__device__ __forceinline__ void msbfs_scatter(const BGraph &G, uint64_t f, int64_t first, int64_t e, int step) {
+    for (int64_t j = first; j < e; j += BF_U * step) {
+        int32_t w[BF_U];
+        uint64_t nb[BF_U];
+#pragma unroll
+        for (int q = 0; q < BF_U; ++q) w[q] = j + q * step < e ? __ldg(G.csr_idx + j + q * step) : -1;
+#pragma unroll
+        for (int q = 0; q < BF_U; ++q) nb[q] = w[q] >= 0 ? f & ~G.V[w[q]] : 0ull;
+#pragma unroll
+        for (int q = 0; q < BF_U; ++q)
+            if (nb[q]) atomicOr((unsigned long long *)G.N + w[q], (unsigned long long)nb[q]);
+    }
+}
+
+// All graphs' work of a phase is one range of units (32 vertices, or a chunk)
+// that the warps share, so that a batch of small graphs does not line up behind
+// its first warps; a unit's graph is found in the prefix sums of their counts.
+constexpr int BF_MAX_GRAPHS = 256;
+
+__device__ __forceinline__ int msbfs_graph(const int64_t *prefix, int ng, int64_t unit) {
+    int lo = 0, hi = ng;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (prefix[mid] <= unit)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
 __global__ void __launch_bounds__(BT_THREADS) k_msbfs_persistent(BatchDev B) {
-    __shared__ int s_dir[256];  // per graph: 0 top-down, 1 bottom-up for the current level
+    __shared__ int s_dir[BF_MAX_GRAPHS];  // per graph: 0 top-down, 1 bottom-up for the current level
+    __shared__ int64_t s_tile[BF_MAX_GRAPHS + 1], s_out[BF_MAX_GRAPHS + 1], s_in[BF_MAX_GRAPHS + 1];
+    __shared__ unsigned long long s_count[BF_MAX_GRAPHS][4];
     const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     const int64_t gwarp = gthread >> 5, nwarps = nthreads >> 5;
@@ -436,148 +478,219 @@ __global__ void __launch_bounds__(BT_THREADS) k_msbfs_persistent(BatchDev B) {
     const int nsrc = B.nsrc;
     const uint64_t full = nsrc == 64 ? ~0ull : ((1ull << nsrc) - 1ull);
     const int ng = B.ngraphs;
-    for (int gi = 0; gi < ng; ++gi) {
-        const BGraph &G = B.graphs[gi];
-        for (int64_t v = gthread; v < G.n; v += nthreads) {
-            G.F[v] = 0;
-            G.V[v] = 0;
-            G.N[v] = 0;
+    for (int gi = threadIdx.x; gi < ng; gi += blockDim.x) {
+        s_tile[gi + 1] = (B.graphs[gi].n + 31) >> 5;
+        s_out[gi + 1] = B.graphs[gi].nochunk;
+        s_in[gi + 1] = B.graphs[gi].nchunk;
+        s_dir[gi] = 0;  // a few sources: top-down
+        for (int q = 0; q < 4; ++q) s_count[gi][q] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_tile[0] = s_out[0] = s_in[0] = 0;
+        for (int gi = 0; gi < ng; ++gi) {
+            s_tile[gi + 1] += s_tile[gi];
+            s_out[gi + 1] += s_out[gi];
+            s_in[gi + 1] += s_in[gi];
         }
-        for (int64_t i = gthread; i < G.n * 64; i += nthreads) G.levels[i] = -1;
+    }
+    __syncthreads();
+    const int64_t ntiles = s_tile[ng];
+    for (int64_t u = gwarp; u < ntiles; u += nwarps) {
+        const int gi = msbfs_graph(s_tile, ng, u);
+        const BGraph &G = B.graphs[gi];
+        const int64_t v = (u - s_tile[gi]) * 32 + lane;
+        if (v >= G.n) continue;
+        G.F[v] = 0;
+        G.V[v] = 0;
+        G.N[v] = 0;
     }
     if (gthread < 8 * (int64_t)ng) B.mcount[gthread] = 0;
     if (!grid_sync(B.sync, gridDim.x)) return;
-    if (gthread < (int64_t)ng) {  // one thread per graph seeds its searches
-        const BGraph &G = B.graphs[gthread];
-        for (int j = 0; j < nsrc; ++j) {
-            const int32_t s = B.sources[gthread * 64 + j];
-            G.F[s] |= 1ull << j;
-            G.V[s] |= 1ull << j;
-            G.levels[(int64_t)s * 64 + j] = 0;
-        }
+    for (int64_t i = gthread; i < (int64_t)ng * 64; i += nthreads) {  // a thread per search
+        const int j = (int)(i & 63);
+        if (j >= nsrc) continue;
+        const BGraph &G = B.graphs[i >> 6];
+        const int32_t s = B.sources[i];
+        atomicOr((unsigned long long *)G.F + s, 1ull << j);
+        atomicOr((unsigned long long *)G.V + s, 1ull << j);
+        B.lev_out[i >> 6][(int64_t)s * 64 + j] = 0;
     }
-    for (int gi = threadIdx.x; gi < ng; gi += blockDim.x) s_dir[gi] = 0;  // a few sources: top-down
     if (!grid_sync(B.sync, gridDim.x)) return;
     int L = 0;
     for (;; ++L) {
-        for (int gi = 0; gi < ng; ++gi) {
+        // light vertices, a lane each.  Top-down: a frontier vertex's masks into its
+        // out-neighbours' N; bottom-up: the in-neighbours' masks, until covered
+        for (int64_t u = gwarp; u < ntiles; u += nwarps) {
+            const int gi = msbfs_graph(s_tile, ng, u);
             const BGraph &G = B.graphs[gi];
+            const int64_t v = (u - s_tile[gi]) * 32 + lane;
+            if (v >= G.n) continue;
             if (s_dir[gi] == 0) {
-                // top-down: a lane per frontier vertex of light out-degree scans its
-                // out-edges; heavy frontier vertices are scanned by the whole warp
-                for (int64_t v0 = gwarp * 32; v0 < G.n; v0 += nwarps * 32) {
-                    const int64_t v = v0 + lane;
-                    uint64_t f = 0;
-                    int64_t b = 0, e = 0;
-                    if (v < G.n) {
-                        f = G.F[v];
-                        if (f) {
-                            b = G.csr_off[v];
-                            e = G.csr_off[v + 1];
-                        }
-                    }
-                    const bool heavy = f && e - b > 32;
-                    if (f && !heavy)
-                        for (int64_t j = b; j < e; ++j) {
-                            const int32_t w = __ldg(G.csr_idx + j);
-                            const uint64_t nb = f & ~G.V[w];
-                            if (nb) atomicOr((unsigned long long *)G.N + w, (unsigned long long)nb);
-                        }
-                    for (unsigned hm = __ballot_sync(FULL, heavy); hm; hm &= hm - 1) {
-                        const int hl = __ffs(hm) - 1;
-                        const uint64_t hf = __shfl_sync(FULL, f, hl);
-                        const int64_t hb = __shfl_sync(FULL, b, hl), he = __shfl_sync(FULL, e, hl);
-                        for (int64_t j = hb + lane; j < he; j += 32) {
-                            const int32_t w = __ldg(G.csr_idx + j);
-                            const uint64_t nb = hf & ~G.V[w];
-                            if (nb) atomicOr((unsigned long long *)G.N + w, (unsigned long long)nb);
-                        }
-                    }
-                }
+                const uint64_t f = G.F[v];
+                if (!f) continue;
+                const int64_t b = G.csr_off[v], e = G.csr_off[v + 1];
+                if (e - b <= B.big_min) msbfs_scatter(G, f, b, e, 1);
             } else {
-                // bottom-up: pull the frontier masks of in-neighbours (early exit once
-                // covered); high in-degree vertices are scanned by a whole warp
-                for (int64_t v = gthread; v < G.n; v += nthreads) {
-                    const uint64_t vis = G.V[v];
-                    if (vis == full) continue;
-                    const int64_t b = G.csc_off[v], e = G.csc_off[v + 1];
-                    if (e - b > B.big_min) continue;
-                    uint64_t acc = 0;
-                    for (int64_t j = b; j < e; ++j) {
-                        acc |= G.F[__ldg(G.csc_idx + j)];
-                        if ((acc | vis) == full) break;
-                    }
-                    G.N[v] = acc & ~vis;
+                const uint64_t vis = G.V[v];
+                if (vis == full) continue;
+                const int64_t b = G.csc_off[v], e = G.csc_off[v + 1];
+                if (e - b > B.big_min) continue;
+                uint64_t acc = 0;
+                for (int64_t j = b; j < e && (acc | vis) != full; j += BF_U) {
+                    int32_t w[BF_U];
+#pragma unroll
+                    for (int q = 0; q < BF_U; ++q) w[q] = j + q < e ? __ldg(G.csc_idx + j + q) : -1;
+#pragma unroll
+                    for (int q = 0; q < BF_U; ++q) acc |= w[q] >= 0 ? G.F[w[q]] : 0ull;
                 }
-                for (int64_t r = gwarp; r < G.nbig; r += nwarps) {
-                    const int64_t v = B.big[G.big0 + r];
-                    const uint64_t vis = G.V[v];
-                    if (vis == full) continue;
-                    const int64_t b = G.csc_off[v], e = G.csc_off[v + 1];
-                    uint64_t acc = 0;
-                    for (int64_t j0 = b; j0 < e; j0 += 32) {
-                        const int64_t j = j0 + lane;
-                        uint64_t f = j < e ? G.F[__ldg(G.csc_idx + j)] : 0ull;
-                        const unsigned lo = __reduce_or_sync(FULL, (unsigned)f);
-                        const unsigned hi = __reduce_or_sync(FULL, (unsigned)(f >> 32));
-                        acc |= ((uint64_t)hi << 32) | lo;
-                        if ((acc | vis) == full) break;
-                    }
-                    if (lane == 0) G.N[v] = acc & ~vis;
+                G.N[v] = acc & ~vis;
+            }
+        }
+        // top-down chunks: a lane looks at every nwarps-th one, the warp takes those in the frontier
+        for (int64_t c0 = gwarp; c0 < s_out[ng]; c0 += 32 * nwarps) {
+            const int64_t c = c0 + lane * nwarps;
+            BChunk ch = {0, 0, 0};
+            uint64_t f = 0;
+            int gi = 0;
+            if (c < s_out[ng]) {
+                gi = msbfs_graph(s_out, ng, c);
+                if (s_dir[gi] == 0) {
+                    ch = B.chunks[B.graphs[gi].ochunk0 + (c - s_out[gi])];
+                    f = B.graphs[gi].F[ch.v];
                 }
+            }
+            for (unsigned hm = __ballot_sync(FULL, f != 0); hm; hm &= hm - 1) {
+                const int hl = __ffs(hm) - 1;
+                const uint64_t hf = __shfl_sync(FULL, f, hl);
+                const int64_t hb = __shfl_sync(FULL, ch.beg, hl);
+                const int len = __shfl_sync(FULL, ch.len, hl);
+                msbfs_scatter(B.graphs[__shfl_sync(FULL, gi, hl)], hf, hb + lane, hb + len, 32);
+            }
+        }
+        // bottom-up chunks: what a chunk finds is added to its vertex's N
+        for (int64_t c0 = gwarp; c0 < s_in[ng]; c0 += 32 * nwarps) {
+            const int64_t c = c0 + lane * nwarps;
+            BChunk ch = {0, 0, 0};
+            uint64_t vis = full;
+            int gi = 0;
+            if (c < s_in[ng]) {
+                gi = msbfs_graph(s_in, ng, c);
+                if (s_dir[gi] == 1) {
+                    const BGraph &G = B.graphs[gi];
+                    ch = B.chunks[G.chunk0 + (c - s_in[gi])];
+                    // (other chunks of the vertex may have found some already: less to look for)
+                    vis = G.V[ch.v] | *(volatile uint64_t *)(G.N + ch.v);
+                }
+            }
+            for (unsigned hm = __ballot_sync(FULL, vis != full); hm; hm &= hm - 1) {
+                const int hl = __ffs(hm) - 1;
+                const BGraph &G = B.graphs[__shfl_sync(FULL, gi, hl)];
+                const uint64_t hv = __shfl_sync(FULL, vis, hl);
+                const int64_t hb = __shfl_sync(FULL, ch.beg, hl);
+                const int64_t he = hb + __shfl_sync(FULL, ch.len, hl);
+                uint64_t acc = 0;
+                for (int64_t j = hb + lane; j < he; j += 32 * BF_U) {
+                    int32_t w[BF_U];
+#pragma unroll
+                    for (int q = 0; q < BF_U; ++q) w[q] = j + 32 * q < he ? __ldg(G.csc_idx + j + 32 * q) : -1;
+#pragma unroll
+                    for (int q = 0; q < BF_U; ++q) acc |= w[q] >= 0 ? G.F[w[q]] : 0ull;
+                }
+                const unsigned lo = __reduce_or_sync(FULL, (unsigned)acc);
+                const unsigned hi = __reduce_or_sync(FULL, (unsigned)(acc >> 32));
+                acc = (((uint64_t)hi << 32) | lo) & ~hv;
+                if (lane == hl && acc) atomicOr((unsigned long long *)G.N + ch.v, (unsigned long long)acc);
             }
         }
         if (!grid_sync(B.sync, gridDim.x)) return;
         // update: owner-only writes of V, F and the levels of newly reached
         // searches, and the counters of the next level's direction rule
         unsigned long long *mc = B.mcount + (L & 1) * 4 * ng;
-        for (int gi = 0; gi < ng; ++gi) {
+        for (int64_t u = gwarp; u < ntiles; u += nwarps) {
+            const int gi = msbfs_graph(s_tile, ng, u);
             const BGraph &G = B.graphs[gi];
-            unsigned long long nf = 0, mf = 0, mu = 0, bits = 0;
-            for (int64_t v = gthread; v < G.n; v += nthreads) {
-                const uint64_t vis = G.V[v];
-                const uint64_t nw = G.N[v] & ~vis;
+            const int64_t v0 = (u - s_tile[gi]) * 32, v = v0 + lane;
+            uint64_t nw = 0;
+            unsigned nf = 0, bits = 0;
+            unsigned long long mf = 0, mu = 0;
+            if (v < G.n) {
+                const uint64_t vis = G.V[v], found = G.N[v];
+                nw = found & ~vis;
                 G.F[v] = nw;
+                if (found) G.N[v] = 0;
                 if (nw) {
                     G.V[v] = vis | nw;
-                    G.N[v] = 0;
-                    bits += __popcll(nw);
-                    nf += 1;
-                    mf += (unsigned long long)(G.csr_off[v + 1] - G.csr_off[v]);
-                    for (uint64_t bb = nw; bb; bb &= bb - 1) G.levels[v * 64 + (__ffsll((long long)bb) - 1)] = L + 1;
-                } else if (G.N[v]) {
-                    G.N[v] = 0;
+                    bits = __popcll(nw);
+                    nf = 1;
+                    mf = (unsigned long long)(G.csr_off[v + 1] - G.csr_off[v]);
                 }
-                if ((vis | nw) != full) mu += (unsigned long long)(G.csc_off[v + 1] - G.csc_off[v]);
+                if ((vis | nw) != full) mu = (unsigned long long)(G.csc_off[v + 1] - G.csc_off[v]);
             }
-            nf = warp_sum(nf);
-            mf = warp_sum(mf);
+            // a vertex's 64 levels are one row: written by the warp, two searches to a lane
+            int32_t *lev = B.lev_out[gi];
+            const unsigned rows = __ballot_sync(FULL, nw != 0);
+            for (unsigned m = rows; m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                const uint64_t row = __shfl_sync(FULL, nw, l);
+                int32_t *at = lev + (v0 + l) * 64 + lane;
+                if ((row >> lane) & 1ull) at[0] = L + 1;
+                if ((row >> (lane + 32)) & 1ull) at[32] = L + 1;
+            }
+            if (rows) {
+                nf = __reduce_add_sync(FULL, nf);
+                bits = __reduce_add_sync(FULL, bits);
+                mf = warp_sum(mf);
+            }
             mu = warp_sum(mu);
-            bits = warp_sum(bits);
             if (lane == 0) {
-                if (nf) atomicAdd(mc + 4 * gi + 0, nf);
-                if (mf) atomicAdd(mc + 4 * gi + 1, mf);
-                if (mu) atomicAdd(mc + 4 * gi + 2, mu);
-                if (bits) atomicAdd(mc + 4 * gi + 3, bits);
+                if (rows) {
+                    atomicAdd(&s_count[gi][0], (unsigned long long)nf);
+                    atomicAdd(&s_count[gi][1], mf);
+                    atomicAdd(&s_count[gi][3], (unsigned long long)bits);
+                }
+                if (mu) atomicAdd(&s_count[gi][2], mu);
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 4 * ng; i += blockDim.x) {
+            const unsigned long long c = s_count[i >> 2][i & 3];
+            if (c) {
+                atomicAdd(mc + i, c);
+                s_count[i >> 2][i & 3] = 0;
             }
         }
         if (!grid_sync(B.sync, gridDim.x)) return;
         // every block reads the same counters: next directions, and whether any search moved
-        unsigned long long total = 0;
+        unsigned long long moved = 0;
         const volatile unsigned long long *vmc = mc;
-        for (int gi = 0; gi < ng; ++gi) total += vmc[4 * gi + 3];
         for (int gi = threadIdx.x; gi < ng; gi += blockDim.x) {
             const unsigned long long nf = vmc[4 * gi], mf = vmc[4 * gi + 1], mu = vmc[4 * gi + 2];
+            moved |= vmc[4 * gi + 3];
             const int64_t n = B.graphs[gi].n;
             if (s_dir[gi] == 0)
                 s_dir[gi] = ((float)mf * B.alpha > (float)mu) ? 1 : 0;
             else
                 s_dir[gi] = ((float)nf * B.beta < (float)n) ? 0 : 1;
         }
-        __syncthreads();
         // the other parity's record, last read two barriers ago, is cleared for the next level
         if (gthread < 4 * (int64_t)ng) B.mcount[((L + 1) & 1) * 4 * ng + gthread] = 0;
-        if (total == 0) break;
+        if (!__syncthreads_or(moved != 0)) break;
+    }
+    // what no search reached (with the levels above, every entry is written once)
+    for (int64_t u = gwarp; u < ntiles; u += nwarps) {
+        const int gi = msbfs_graph(s_tile, ng, u);
+        const BGraph &G = B.graphs[gi];
+        const int64_t v0 = (u - s_tile[gi]) * 32, v = v0 + lane;
+        int32_t *lev = B.lev_out[gi];
+        const uint64_t vis = v < G.n ? G.V[v] : ~0ull;
+        for (unsigned m = __ballot_sync(FULL, vis != ~0ull); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const uint64_t row = __shfl_sync(FULL, vis, l);
+            int32_t *at = lev + (v0 + l) * 64 + lane;
+            if (!((row >> lane) & 1ull)) at[0] = -1;
+            if (!((row >> (lane + 32)) & 1ull)) at[32] = -1;
+        }
     }
     if (gthread == 0) B.counters[1] = L + 1;
 }
@@ -601,6 +714,8 @@ struct gp_batch {
     int32_t *seeds = nullptr, *sources = nullptr;
     int32_t *counters = nullptr;
     int32_t *hcounters = nullptr;  // pinned
+    int32_t **lev_out = nullptr;   // device table of the levels' destinations
+    int32_t **hlev_out = nullptr;  // pinned: the call's, before they are copied there
     cudaStream_t home = nullptr;
     cudaGraphExec_t ppr_exec = nullptr, bfs_exec = nullptr;
     bool ppr_stale = true, bfs_stale = true;
@@ -688,16 +803,34 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
             if (d <= big_min) continue;
             big.push_back((int32_t)v);
             for (int64_t p = off[v]; p < off[v + 1]; p += C)
-                chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), gi});
+                chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v});
             bcstart.push_back((int64_t)chunks.size());
         }
         G.nbig = (int64_t)big.size() - G.big0;
         G.nchunk = (int64_t)chunks.size() - G.chunk0;
         max_chunks = std::max(max_chunks, G.nchunk);
+        G.ochunk0 = G.chunk0;
+        G.nochunk = G.nchunk;
         // the widest slice whose two iterates fit the budget (at least 32 columns)
         int ks = std::min(K, BT_MAX_KS);
         while (ks > 32 && 2 * g->n * (int64_t)ks * 4 > budget) ks /= 2;
         for (int c0 = 0; c0 < K; c0 += ks) b->jobs.push_back(BJob{gi, c0, ks / 32, 0});
+    }
+    // after every graph's in-edge chunks (bcstart numbers those): the out-edge ones where the orders differ
+    for (int gi = 0; gi < b->ngraphs; ++gi) {
+        gp_graph *g = b->graphs[gi];
+        if (g->csr_off == g->csc_off) continue;
+        std::vector<int64_t> off((size_t)g->n + 1);
+        cudaError_t e = cudaMemcpyAsync(off.data(), g->csr_off, off.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout: %s", cudaGetErrorString(e));
+        BGraph &G = b->hg[gi];
+        G.ochunk0 = (int64_t)chunks.size();
+        for (int64_t v = 0; v < g->n; ++v)
+            if (off[v + 1] - off[v] > big_min)
+                for (int64_t p = off[v]; p < off[v + 1]; p += C)
+                    chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v});
+        G.nochunk = (int64_t)chunks.size() - G.ochunk0;
     }
     b->layout.release(s);
     BatchDev &D = b->dev;
@@ -772,6 +905,7 @@ extern "C" int gp_batch_create(gp_batch **out, gp_graph *const *graphs, int ngra
         b->layout.release(s);
         b->mem.release(s);
         pinned_free(b->hcounters, 8 * sizeof(int32_t));
+        pinned_free(b->hlev_out, ngraphs * sizeof(int32_t *));
         delete b;
         return st;
     };
@@ -821,6 +955,7 @@ extern "C" int gp_batch_create(gp_batch **out, gp_graph *const *graphs, int ngra
     if (st == GP_OK) st = b->mem.alloc(D.pend, (size_t)ngraphs * K, s);
     if (st == GP_OK) st = b->mem.alloc(D.XP0, (size_t)nmax * 32, s);
     if (st == GP_OK) st = b->mem.alloc(D.XP1, (size_t)nmax * 32, s);
+    if (st == GP_OK) st = b->mem.alloc(b->lev_out, (size_t)ngraphs, s);
     GridSync *sync = nullptr;
     if (st == GP_OK) st = b->mem.alloc(sync, 1, s);
     if (st != GP_OK) return fail(st);
@@ -829,11 +964,15 @@ extern "C" int gp_batch_create(gp_batch **out, gp_graph *const *graphs, int ngra
         st = pinned_alloc(&h, 8 * sizeof(int32_t));
         if (st != GP_OK) return fail(st);
         b->hcounters = (int32_t *)h;
+        st = pinned_alloc(&h, ngraphs * sizeof(int32_t *));
+        if (st != GP_OK) return fail(st);
+        b->hlev_out = (int32_t **)h;
     }
     D.graphs = b->dgraphs;
     D.seeds = b->seeds;
     D.sources = b->sources;
     D.counters = b->counters;
+    D.lev_out = b->lev_out;
     D.sync = sync;
     st = batch_layout(b, s);
     if (st != GP_OK) return fail(st);
@@ -877,6 +1016,7 @@ extern "C" int gp_batch_free(gp_batch *b) {
     b->layout.release(b->home);
     b->mem.release(b->home);
     pinned_free(b->hcounters, 8 * sizeof(int32_t));
+    pinned_free(b->hlev_out, b->ngraphs * sizeof(int32_t *));
     cudaError_t e = cudaStreamSynchronize(b->home);
     delete b;
     if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "gp_batch_free: %s", cudaGetErrorString(e));
@@ -965,6 +1105,10 @@ extern "C" int gp_msbfs_batched(gp_batch *b, const int32_t *sources, int nsrc, i
         GP_CUDA(cudaEventCreate(&ev1));
     }
     GP_CUDA(cudaMemcpyAsync(b->sources, src.data(), src.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    // device outputs are written by the kernel, the others copied from the batch's own buffers
+    for (int gi = 0; gi < b->ngraphs; ++gi)
+        b->hlev_out[gi] = levels_out && levels_out[gi] && is_device_ptr(levels_out[gi]) ? levels_out[gi] : b->hg[gi].levels;
+    GP_CUDA(cudaMemcpyAsync(b->lev_out, b->hlev_out, b->ngraphs * sizeof(int32_t *), cudaMemcpyHostToDevice, s));
     const bool rebuild = b->bfs_stale || b->bfs_nsrc != nsrc;
     int grid = 0;
     GP_TRY(batch_grid(b, (const void *)k_msbfs_persistent, grid));
@@ -979,7 +1123,7 @@ extern "C" int gp_msbfs_batched(gp_batch *b, const int32_t *sources, int nsrc, i
     GP_TRY(st);
     if (stats) GP_CUDA(cudaEventRecord(ev1, s));
     for (int gi = 0; gi < b->ngraphs; ++gi)
-        if (levels_out && levels_out[gi])
+        if (levels_out && levels_out[gi] && b->hlev_out[gi] == b->hg[gi].levels)
             GP_CUDA(cudaMemcpyAsync(levels_out[gi], b->hg[gi].levels, (size_t)b->hg[gi].n * 64 * sizeof(int32_t),
                                     cudaMemcpyDefault, s));
     GP_CUDA(cudaMemcpyAsync(b->hcounters, b->counters, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
