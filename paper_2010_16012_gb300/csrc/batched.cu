@@ -39,6 +39,9 @@
 namespace gp {
 
 constexpr int BT_THREADS = 512;  // threads per block of the persistent kernels
+#ifndef GP_BT_MINB
+#define GP_BT_MINB 2
+#endif
 constexpr int BT_SEG = 8;        // vertices per warp work unit (light rows)
 constexpr int BT_MAX_KS = 128;   // widest column slice of one PageRank job (a float4 per lane)
 
@@ -62,6 +65,8 @@ struct BChunk {  // warp work item: a piece of a big vertex's edge list
     int64_t beg;
     int32_t len;
     int32_t v;
+    int32_t r;    // in-edge chunks: the vertex's place among the big ones,
+    int32_t nch;  // and its chunks
 };
 
 struct BJob {  // one graph and the column slice [c0, c0 + 32 * kpl)
@@ -92,29 +97,54 @@ struct BatchDev {
     const int32_t *big;     // [nbig_total] vertex ids, grouped by graph
     const int64_t *bcstart; // [nbig_total + 1] chunk range of each big vertex
     const BChunk *chunks;
+    unsigned *bdone;        // [nbig_total] chunks of each big vertex summed in this sweep
     float *part;            // [max chunks of one graph][K] chunk partial rows
     double *res_acc;        // [3][K] per-sweep column residuals (a ring)
     const int32_t *seeds;   // [ngraphs][K]
     int32_t *iters_done;    // [ngraphs][K]
     const int32_t *sources; // [ngraphs][64] (MS-BFS)
     int32_t *const *lev_out;  // [ngraphs] where this call's levels go (MS-BFS)
-    int32_t *counters;      // [0] most PPR sweeps of any column, [1] BFS levels, [2] packed columns
+    int32_t *counters;      // [0] most PPR sweeps of any column, [1] BFS levels, [2] packed columns, [3], [4] those left to narrower jobs
     int32_t pack_max;       // a job stops once at most this many of its columns iterate (0: never)
-    BPend *pend;            // [ngraphs * K] the columns left iterating, in job order
-    float *XP0, *XP1;       // [max n][32] iterates of a packed job
+    BPend *pend;            // [3][ngraphs * K] the columns left iterating, in job order: for jobs of 32, 8 and 4
+    float *XP0, *XP1;       // [max n][32] iterates of a packed job (rows as wide as the job)
     unsigned long long *mcount;  // MS-BFS [2][ngraphs][4]: frontier vertices, their out-edges, open in-edges, new bits
     GridSync *sync;
 };
 
 // ------------------------------------------------------------------ batched PPR
 
-// Compensated (Kahan) accumulation: a column sums up to thousands of terms one
-// after another, so the running rounding error is carried in `comp`.
-__device__ __forceinline__ void kahan_add(float &acc, float &comp, float x) {
-    const float y = x - comp;
-    const float t = acc + y;
-    comp = (t - acc) - y;
-    acc = t;
+// Pairs of FP32 values, added (and so on) by one instruction, rounded as the scalar operations are.
+__device__ __forceinline__ uint64_t pk(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpk(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {  // a - b as b * -1 + a, rounded once
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+    return r;
+}
+
+// Compensated (Kahan) accumulation of f * r: a column sums up to thousands of
+// terms one after another, so the running rounding error is carried in `lo`,
+// negated: the sum is hi + lo.
+__device__ __forceinline__ void kahan_add2(uint64_t &hi, uint64_t &lo, uint64_t f, uint64_t r) {
+    uint64_t y;  // f * r + lo, rounded once
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(y) : "l"(f), "l"(r), "l"(lo));
+    const uint64_t t = add2(hi, y);
+    lo = sub2(y, sub2(t, hi));
+    hi = t;
 }
 
 // A job of KS columns maps a warp onto NG = 32 / (KS / 4) edge groups of
@@ -129,9 +159,12 @@ struct Lanes {
 };
 
 #ifndef GP_BT_INFLIGHT
-#define GP_BT_INFLIGHT 8
+#define GP_BT_INFLIGHT 6
 #endif
-constexpr int BT_INFLIGHT = GP_BT_INFLIGHT;  // row segments in flight per lane
+// Row segments in flight per lane: 6 of 4 registers each fit the 64 registers a
+// thread has at two blocks per SM with few spills (R-MAT 2^17, 128 columns: 219
+// us a sweep; 8 in flight 237, 4 in flight 247, 4 at three blocks per SM 254).
+constexpr int BT_INFLIGHT = GP_BT_INFLIGHT;
 
 // Row segments are read through L2 (ld.global.cg): the iterates are rewritten
 // by the kernel itself between sweeps, so the non-coherent read-only path may
@@ -140,57 +173,56 @@ __device__ __forceinline__ float4 ld_seg(const float *X, int K, int32_t u, int c
     return __ldcg(reinterpret_cast<const float4 *>(X + (int64_t)u * K) + c4);
 }
 
-// Compensated partial sums of a lane's four columns: the value is hi - lo.
+// Compensated partial sums of a lane's four columns, in pairs: the value is hi + lo.
 struct Sum4 {
-    float hi[4], lo[4];
+    uint64_t hi[2] = {0, 0}, lo[2] = {0, 0};
+    __device__ __forceinline__ void add(uint64_t f, const float4 &r) {
+        kahan_add2(hi[0], lo[0], f, pk(r.x, r.y));
+        kahan_add2(hi[1], lo[1], f, pk(r.z, r.w));
+    }
 };
+
+// BT_INFLIGHT edges from e on, every `step`; those from `end` on add zero (FULL_W: there are none).
+template <bool FULL_W>
+__device__ __forceinline__ void gather_window(const BGraph &G, const float *X, int K, int64_t e, int64_t end, int step,
+                                              int c4, Sum4 &a) {
+    int32_t u[BT_INFLIGHT];
+    float f[BT_INFLIGHT];
+    float4 r[BT_INFLIGHT];
+#pragma unroll
+    for (int q = 0; q < BT_INFLIGHT; ++q) u[q] = FULL_W || e + q * step < end ? __ldg(G.csc_idx + e + q * step) : -1;
+#pragma unroll
+    for (int q = 0; q < BT_INFLIGHT; ++q) {
+        if (!FULL_W) r[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (FULL_W || u[q] >= 0) r[q] = ld_seg(X, K, u[q], c4);
+    }
+#pragma unroll
+    for (int q = 0; q < BT_INFLIGHT; ++q) {
+        f[q] = FULL_W || u[q] >= 0 ? __ldg(G.inv_deg + u[q]) : 0.f;
+        if (G.csc_w && (FULL_W || u[q] >= 0)) f[q] *= __ldg(G.csc_w + e + q * step);
+    }
+#pragma unroll
+    for (int q = 0; q < BT_INFLIGHT; ++q) a.add(pk(f[q], f[q]), r[q]);
+}
 
 // Sum over in-edges beg, beg + step, beg + 2 step, ... < end of the rows' four
 // columns at c4 (X points at column c0 of row 0; rows are K floats apart), each
 // product folded into a compensated (Kahan) sum: a column sums up to
 // thousands of terms, and a hub's FP32 rounding feeds back into every sweep.
+// The last window is predicated, not walked edge by edge: most lists are shorter
+// than one window, and their edges' loads would wait for one another.
 __device__ __forceinline__ Sum4 gather_seg(const BGraph &G, const float *X, int K, int64_t beg, int64_t end, int step,
                                            int c4) {
     Sum4 a;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a.hi[i] = a.lo[i] = 0.f;
     int64_t e = beg;
-    for (; e + (BT_INFLIGHT - 1) * step < end; e += BT_INFLIGHT * step) {
-        int32_t u[BT_INFLIGHT];
-        float f[BT_INFLIGHT];
-#pragma unroll
-        for (int q = 0; q < BT_INFLIGHT; ++q) u[q] = __ldg(G.csc_idx + e + q * step);
-        float4 r[BT_INFLIGHT];
-#pragma unroll
-        for (int q = 0; q < BT_INFLIGHT; ++q) r[q] = ld_seg(X, K, u[q], c4);
-#pragma unroll
-        for (int q = 0; q < BT_INFLIGHT; ++q) {
-            f[q] = __ldg(G.inv_deg + u[q]);
-            if (G.csc_w) f[q] *= __ldg(G.csc_w + e + q * step);
-        }
-#pragma unroll
-        for (int q = 0; q < BT_INFLIGHT; ++q) {
-            kahan_add(a.hi[0], a.lo[0], f[q] * r[q].x);
-            kahan_add(a.hi[1], a.lo[1], f[q] * r[q].y);
-            kahan_add(a.hi[2], a.lo[2], f[q] * r[q].z);
-            kahan_add(a.hi[3], a.lo[3], f[q] * r[q].w);
-        }
-    }
-    for (; e < end; e += step) {
-        const int32_t u = __ldg(G.csc_idx + e);
-        float f = __ldg(G.inv_deg + u);
-        if (G.csc_w) f *= __ldg(G.csc_w + e);
-        const float4 r = ld_seg(X, K, u, c4);
-        kahan_add(a.hi[0], a.lo[0], f * r.x);
-        kahan_add(a.hi[1], a.lo[1], f * r.y);
-        kahan_add(a.hi[2], a.lo[2], f * r.z);
-        kahan_add(a.hi[3], a.lo[3], f * r.w);
-    }
+    for (; e + (BT_INFLIGHT - 1) * step < end; e += BT_INFLIGHT * step) gather_window<true>(G, X, K, e, end, step, c4, a);
+    if (e < end) gather_window<false>(G, X, K, e, end, step, c4, a);
     return a;
 }
 
 __device__ __forceinline__ float4 value4(const Sum4 &a) {
-    return make_float4(a.hi[0] - a.lo[0], a.hi[1] - a.lo[1], a.hi[2] - a.lo[2], a.hi[3] - a.lo[3]);
+    const float2 x = unpk(add2(a.hi[0], a.lo[0])), y = unpk(add2(a.hi[1], a.lo[1]));
+    return make_float4(x.x, x.y, y.x, y.y);
 }
 
 // Adds the groups' compensated sums of a warp (every group then holds the
@@ -198,25 +230,23 @@ __device__ __forceinline__ float4 value4(const Sum4 &a) {
 template <int KS>
 __device__ __forceinline__ float4 groups_total(Sum4 a) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) a.lo[i] = -a.lo[i];  // value = hi + lo from here on
-#pragma unroll
     for (int o = Lanes<KS>::LPR; o < 32; o <<= 1) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float ohi = __shfl_xor_sync(FULL, a.hi[i], o), olo = __shfl_xor_sync(FULL, a.lo[i], o);
-            const float t = a.hi[i] + ohi;
-            const float bp = t - a.hi[i];
-            const float err = (a.hi[i] - (t - bp)) + (ohi - bp);
+        for (int i = 0; i < 2; ++i) {
+            const uint64_t ohi = __shfl_xor_sync(FULL, a.hi[i], o), olo = __shfl_xor_sync(FULL, a.lo[i], o);
+            const uint64_t t = add2(a.hi[i], ohi);
+            const uint64_t bp = sub2(t, a.hi[i]);
+            const uint64_t err = add2(sub2(a.hi[i], sub2(t, bp)), sub2(ohi, bp));
             a.hi[i] = t;
-            a.lo[i] = a.lo[i] + olo + err;
+            a.lo[i] = add2(add2(a.lo[i], olo), err);
         }
     }
-    return make_float4(a.hi[0] + a.lo[0], a.hi[1] + a.lo[1], a.hi[2] + a.lo[2], a.hi[3] + a.lo[3]);
+    return value4(a);
 }
 
 // The columns one PageRank job iterates: a slice of a graph's own iterates
 // (pend == nullptr: columns c0 .. c0 + KS - 1 of X0/X1, rows K apart), or a
-// packed job over the batch's packed iterates (rows 32 apart), whose column j
+// packed job over the batch's packed iterates (rows KS apart), whose column j
 // continues the graph's column pend[j].col after pend[j].kdone sweeps.
 struct PView {
     int graph;
@@ -225,25 +255,36 @@ struct PView {
     int c0;
     const BPend *pend;  // packed job, or nullptr
     int cnt;            // packed job: columns in use (the rest idle)
-    __device__ int col(int c) const { return pend ? pend[c].col : c0 + c; }
-    __device__ int kbase(int c) const { return pend ? pend[c].kdone : 0; }
+    // columns still iterating when at most `leave` are left go to `list`, whose length is *count
+    int leave;
+    BPend *list;
+    int32_t *count;
+};
+
+// A job's columns in shared memory: the graph's column and the seed of each,
+// the sweeps it has had before, and whether it still iterates.
+struct PCols {
+    __align__(16) int col[BT_MAX_KS], seed[BT_MAX_KS], kbase[BT_MAX_KS], active[BT_MAX_KS];
+    int next[2];                              // by sweep parity: the block's next unit
+    float res[BT_THREADS / 32][32][4];        // per lane: |y - x| of its four columns
+    double wres[BT_THREADS / 32][8];          // narrow jobs: a warp's sums
 };
 
 // Writes the lane's four columns of row v of the slice of Y from the gathered
-// sum, carrying stopped columns forward; adds |y - x| of the columns still
-// iterating to the lane's residual slots (shared memory, one owner each).
-__device__ __forceinline__ void finish_seg(const BatchDev &B, const PView &V, const float *Xc, float *Y, int64_t v,
-                                           int c4, float4 sum, float *my_res, const int *s_active) {
-    const int64_t o = v * V.ld + V.c0 + 4 * c4;
-    const float4 x = __ldcg(reinterpret_cast<const float4 *>(Xc + o));
+// sum and the row x of the current iterate, carrying stopped columns forward;
+// adds |y - x| of the columns still iterating to the lane's residual slots
+// (shared memory, one owner each).
+__device__ __forceinline__ void finish_seg(const BatchDev &B, float *Y, int64_t o, int64_t v, int c4, const float4 &x,
+                                           const float4 &sum, float *my_res, const PCols &C) {
     const float xs[4] = {x.x, x.y, x.z, x.w}, ss[4] = {sum.x, sum.y, sum.z, sum.w};
+    const int4 a4 = *reinterpret_cast<const int4 *>(C.active + 4 * c4), s4 = *reinterpret_cast<const int4 *>(C.seed + 4 * c4);
+    const int act[4] = {a4.x, a4.y, a4.z, a4.w}, seed[4] = {s4.x, s4.y, s4.z, s4.w};
     float ys[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const int c = 4 * c4 + q;
         ys[q] = xs[q];
-        if (s_active[c]) {
-            const float base = (B.seeds[V.graph * B.K + V.col(c)] == (int32_t)v) ? B.one_minus_d : 0.f;
+        if (act[q]) {
+            const float base = seed[q] == (int32_t)v ? B.one_minus_d : 0.f;
             ys[q] = base + B.d * ss[q];
             my_res[q] += fabsf(ys[q] - xs[q]);
         }
@@ -251,12 +292,36 @@ __device__ __forceinline__ void finish_seg(const BatchDev &B, const PView &V, co
     *reinterpret_cast<float4 *>(Y + o) = make_float4(ys[0], ys[1], ys[2], ys[3]);
 }
 
-// One job: the slice's sweeps from the start vector to convergence, or, for a
-// slice of the graph's own iterates, until at most B.pack_max of its columns
-// still iterate (those are then left, at their latest iterate, to a packed job).
-// Returns false when a grid barrier gave up.
+// Sum of partial rows first, first + NG, ... < end (the row's columns at `part`), over the warp's groups.
 template <int KS>
-__device__ bool ppr_job(const BatchDev &B, const PView &J, float (*s_res)[32][4], int *s_active) {
+__device__ __forceinline__ float4 sum_parts(const float *part, int64_t first, int64_t end) {
+    constexpr int NG = Lanes<KS>::NG;
+    Sum4 a;
+    const uint64_t one = pk(1.f, 1.f);
+    for (int64_t c = first; c < end; c += BT_INFLIGHT * NG) {
+        float4 p[BT_INFLIGHT];
+#pragma unroll
+        for (int q = 0; q < BT_INFLIGHT; ++q) {
+            p[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c + q * NG < end) p[q] = __ldcg(reinterpret_cast<const float4 *>(part + (c + q * NG) * KS));
+        }
+#pragma unroll
+        for (int q = 0; q < BT_INFLIGHT; ++q) a.add(one, p[q]);
+    }
+    return groups_total<KS>(a);
+}
+
+// One job: the slice's sweeps from the start vector to convergence, or until at
+// most J.leave of its columns still iterate (those are then left, at their
+// latest iterate, to a packed job).  Returns false when a grid barrier gave up.
+// Bound by the L2 row gathers on large graphs (R-MAT 2^17, 128 columns: 305 ->
+// 219 us a sweep, 8.7 TB/s of gathered rows), by the chains of loads per vertex
+// and the barrier on small ones (8,155 vertices: 39 -> 29 us).  What the warps
+// waited for before was one another: equal shares of unequal units, and a
+// second phase with a barrier of its own for the big vertices' partial rows.
+// Not inlined: the widths' loops share no registers.
+template <int KS>
+__device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C) {
     constexpr int LPR = Lanes<KS>::LPR, NG = Lanes<KS>::NG;
     const int K = B.K;
     const int ld = J.ld;
@@ -266,108 +331,154 @@ __device__ bool ppr_job(const BatchDev &B, const PView &J, float (*s_res)[32][4]
     const int wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int64_t gwarp = gthread >> 5, nwarps = nthreads >> 5;
+    const int64_t nwarps = nthreads >> 5;
+    if (threadIdx.x < 2) C.next[threadIdx.x] = 0;
+    for (int c = threadIdx.x; c < KS; c += blockDim.x) {
+        const bool used = !J.pend || c < J.cnt;
+        C.col[c] = !used ? 0 : J.pend ? J.pend[c].col : J.c0 + c;
+        C.kbase[c] = J.pend && used ? J.pend[c].kdone : 0;
+        C.seed[c] = B.seeds[J.graph * K + C.col[c]];
+        C.active[c] = used && C.kbase[c] < B.iters;
+    }
+    __syncthreads();
     if (!J.pend) {
         // start: every column at 1/n, or at its seed's one-hot vector
         const float x0 = 1.0f / (float)n;
         for (int64_t i = gthread; i < n * KS; i += nthreads) {
             const int64_t v = i / KS;
             const int c = (int)(i % KS);
-            J.X0[v * ld + J.c0 + c] =
-                B.one_hot_start ? (B.seeds[J.graph * K + J.c0 + c] == (int32_t)v ? 1.0f : 0.0f) : x0;
+            J.X0[v * ld + J.c0 + c] = B.one_hot_start ? (C.seed[c] == (int32_t)v ? 1.0f : 0.0f) : x0;
         }
     } else {
         // start: the packed columns' latest iterates (idle columns at zero)
         for (int64_t i = gthread; i < n * KS; i += nthreads) {
             const int64_t v = i / KS;
             const int c = (int)(i % KS);
-            J.X0[v * ld + c] = c < J.cnt ? __ldcg(G.X0 + v * K + J.pend[c].col) : 0.f;
+            J.X0[v * ld + c] = c < J.cnt ? __ldcg(G.X0 + v * K + C.col[c]) : 0.f;
         }
     }
-    for (int c = threadIdx.x; c < KS; c += blockDim.x) s_active[c] = !J.pend || (c < J.cnt && J.kbase(c) < B.iters);
     if (gthread < 3 * KS) B.res_acc[(gthread / KS) * K + (gthread % KS)] = 0.0;
     if (!grid_sync(B.sync, gridDim.x)) return false;
-    const int64_t nseg = (n + BT_SEG - 1) / BT_SEG;
-    const float *Xj0 = J.X0 + J.c0, *Xj1 = J.X1 + J.c0;
+    // vertices per warp unit: few where the graph has few, so that every warp gets some
+    int seg = BT_SEG;
+    while (seg > NG && (n + seg - 1) / seg < nwarps) seg /= 2;
+    seg = max(seg, NG);
+    const int64_t nseg = (n + seg - 1) / seg;
     int k = 1, last = 0;
     for (; k <= B.iters; ++k) {
         const float *Xc = (k & 1) ? J.X0 : J.X1;
-        const float *Xs = (k & 1) ? Xj0 : Xj1;  // column c0 of the current iterate
+        const float *Xs = Xc + J.c0;  // column c0 of the current iterate
         float *Y = (k & 1) ? J.X1 : J.X0;
         double *racc = B.res_acc + (k % 3) * K;
         if (blockIdx.x == 0)  // the ring slot of sweep k + 1 (last read two sweeps ago)
             for (int c = threadIdx.x; c < KS; c += blockDim.x) B.res_acc[((k + 1) % 3) * K + c] = 0.0;
-        float *my_res = s_res[wib][lane];
+        float *my_res = C.res[wib][lane];
 #pragma unroll
         for (int q = 0; q < 4; ++q) my_res[q] = 0.f;
-        // phase A: light rows (BT_SEG vertices per warp unit, a vertex per group)
-        // and chunks of big vertices (split over the groups)
-        for (int64_t u = gwarp; u < nseg + G.nchunk; u += nwarps) {
-            if (u < nseg) {
-                const int64_t v1 = min(n, (u + 1) * BT_SEG);
-                for (int64_t v = u * BT_SEG + grp; v < v1; v += NG) {
-                    const int64_t b = G.csc_off[v], e = G.csc_off[v + 1];
-                    if (e - b > B.big_min) continue;  // big vertex: finished in phase B
-                    const float4 sum = value4(gather_seg(G, Xs, ld, b, e, 1, c4));
-                    finish_seg(B, J, Xc, Y, v, c4, sum, my_res, s_active);
+        if (threadIdx.x == 0) C.next[(k + 1) & 1] = 0;
+        // The block's units, each to the warp that is free (equal shares of them left the warps
+        // waiting for one another most of the time on small graphs): chunks of big vertices,
+        // split over the groups, then light rows, a vertex per group.
+        while (true) {
+            int i = 0;
+            if (lane == 0) i = atomicAdd(&C.next[k & 1], 1);
+            i = __shfl_sync(FULL, i, 0);
+            const int64_t u = (int64_t)i * gridDim.x + blockIdx.x;
+            if (u >= G.nchunk + nseg) break;
+            if (u < G.nchunk) {
+                const BChunk ch = B.chunks[G.chunk0 + u];
+                const int64_t v = ch.v;
+                const int64_t o = v * ld + J.c0 + 4 * c4;
+                float4 sum = groups_total<KS>(gather_seg(G, Xs, ld, ch.beg + grp, ch.beg + ch.len, NG, c4));
+                if (ch.nch > 1) {
+                    // the last of the vertex's chunks to finish adds the partial rows, in their order
+                    if (grp == 0) *reinterpret_cast<float4 *>(B.part + u * KS + 4 * c4) = sum;
+                    __syncwarp();
+                    unsigned done = 0;
+                    if (lane == 0) {
+                        __threadfence();
+                        done = atomicInc(B.bdone + ch.r, (unsigned)ch.nch - 1u);  // back at 0 after the last
+                        __threadfence();
+                    }
+                    if (__shfl_sync(FULL, done, 0) != (unsigned)ch.nch - 1u) continue;
+                    const int64_t cb = B.bcstart[ch.r] - G.chunk0;
+                    sum = sum_parts<KS>(B.part + 4 * c4, cb + grp, cb + ch.nch);
+                }
+                if (grp == 0) {
+                    const float4 x = __ldcg(reinterpret_cast<const float4 *>(Xc + o));
+                    finish_seg(B, Y, o, v, c4, x, sum, my_res, C);
                 }
             } else {
-                const int64_t c = u - nseg;
-                const BChunk ch = B.chunks[G.chunk0 + c];
-                const float4 sum = groups_total<KS>(gather_seg(G, Xs, ld, ch.beg + grp, ch.beg + ch.len, NG, c4));
-                if (grp == 0) *reinterpret_cast<float4 *>(B.part + c * KS + 4 * c4) = sum;
+                const int64_t v0 = (u - G.nchunk) * seg;
+                int64_t ob = 0;  // the unit's lists, a vertex per lane
+                int len = 0;
+                if (lane < seg && v0 + lane < n) {
+                    ob = G.csc_off[v0 + lane];
+                    const int64_t d = G.csc_off[v0 + lane + 1] - ob;
+                    // big vertices are done above; without in-edges a row is its base in every
+                    // sweep, so both iterates hold it after two
+                    len = d > B.big_min || (d == 0 && k > 2) ? -1 : (int)d;
+                } else {
+                    len = -1;
+                }
+                for (int i2 = 0; i2 < seg; i2 += NG) {
+                    const int64_t b = __shfl_sync(FULL, ob, i2 + grp);
+                    const int dl = __shfl_sync(FULL, len, i2 + grp);
+                    if (dl < 0) continue;
+                    const int64_t v = v0 + i2 + grp, o = v * ld + J.c0 + 4 * c4;
+                    const float4 sum = value4(gather_seg(G, Xs, ld, b, b + dl, 1, c4));
+                    const float4 x = __ldcg(reinterpret_cast<const float4 *>(Xc + o));
+                    finish_seg(B, Y, o, v, c4, x, sum, my_res, C);
+                }
             }
-        }
-        if (!grid_sync(B.sync, gridDim.x)) return false;
-        // phase B: big vertices add their chunks' partial rows (chunks split over the groups)
-        for (int64_t r = gwarp; r < G.nbig; r += nwarps) {
-            const int64_t v = B.big[G.big0 + r];
-            Sum4 a;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a.hi[i] = a.lo[i] = 0.f;
-            for (int64_t c = B.bcstart[G.big0 + r] - G.chunk0 + grp; c < B.bcstart[G.big0 + r + 1] - G.chunk0; c += NG) {
-                const float4 p = __ldcg(reinterpret_cast<const float4 *>(B.part + c * KS + 4 * c4));
-                kahan_add(a.hi[0], a.lo[0], p.x);
-                kahan_add(a.hi[1], a.lo[1], p.y);
-                kahan_add(a.hi[2], a.lo[2], p.z);
-                kahan_add(a.hi[3], a.lo[3], p.w);
-            }
-            const float4 sum = groups_total<KS>(a);
-            if (grp == 0) finish_seg(B, J, Xc, Y, v, c4, sum, my_res, s_active);
         }
         // the block's column residuals: the slots of every warp and group added
         // in a fixed order, then one FP64 atomic per column into the sweep's ring slot
+        if (KS < 32) {  // many groups per column: a warp's are added first
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                double r = my_res[q];
+#pragma unroll
+                for (int o = LPR; o < 32; o <<= 1) r += __shfl_xor_sync(FULL, r, o);
+                if (grp == 0) C.wres[wib][(4 * c4 + q) % 8] = r;
+            }
+        }
         __syncthreads();
         for (int c = threadIdx.x; c < KS; c += blockDim.x) {
-            if (!s_active[c]) continue;
-            ResSum t;
-            for (int i = 0; i < wpb; ++i)
-                for (int g = 0; g < NG; ++g) t.push(s_res[i][g * LPR + c / 4][c % 4]);
-            const double r = t.get();
+            if (!C.active[c]) continue;
+            double r = 0.0;
+            if (KS < 32) {
+                for (int i = 0; i < wpb; ++i) r += C.wres[i][c % 8];
+            } else {
+                ResSum t;
+                for (int i = 0; i < wpb; ++i)
+                    for (int g = 0; g < NG; ++g) t.push(C.res[i][g * LPR + c / 4][c % 4]);
+                r = t.get();
+            }
             if (r != 0.0) atomicAdd(racc + c, r);
         }
         if (!grid_sync(B.sync, gridDim.x)) return false;
         // every block takes the same decision from the same totals
         int any = 0;
         for (int c = threadIdx.x; c < KS; c += blockDim.x) {
-            if (!s_active[c]) continue;
+            if (!C.active[c]) continue;
             const double r = __ldcg(racc + c);
-            const int kc = J.kbase(c) + k;  // the column's sweeps
-            if (blockIdx.x == 0) B.iters_done[J.graph * K + J.col(c)] = kc;
+            const int kc = C.kbase[c] + k;  // the column's sweeps
+            if (blockIdx.x == 0) B.iters_done[J.graph * K + C.col[c]] = kc;
             if (r < B.tol || kc >= B.iters)
-                s_active[c] = 0;
+                C.active[c] = 0;
             else
                 any = 1;
         }
         const int nact = __syncthreads_count(any);  // one column per thread (KS <= blockDim)
         last = k;
         if (!nact) break;
-        if (!J.pend && nact <= B.pack_max) {
-            // the few columns left go to a packed job; block 0 lists them in column order
+        if (nact <= J.leave) {
+            // the few columns left go to a narrower job; block 0 lists them in column order
             if (blockIdx.x == 0 && threadIdx.x == 0) {
-                int at = atomicAdd(B.counters + 2, nact);
+                int at = atomicAdd(J.count, nact);
                 for (int c = 0; c < KS; ++c)
-                    if (s_active[c]) B.pend[at++] = BPend{J.graph, J.c0 + c, k, 0};
+                    if (C.active[c]) J.list[at++] = BPend{J.graph, C.col[c], C.kbase[c] + k, 0};
             }
             break;
         }
@@ -384,47 +495,57 @@ __device__ bool ppr_job(const BatchDev &B, const PView &J, float (*s_res)[32][4]
         for (int64_t i = gthread; i < n * KS; i += nthreads) {
             const int64_t v = i / KS;
             const int c = (int)(i % KS);
-            if (c < J.cnt) G.X0[v * K + J.pend[c].col] = __ldcg(J.X0 + v * ld + c);
+            if (c < J.cnt) G.X0[v * K + C.col[c]] = __ldcg(J.X0 + v * ld + c);
         }
     }
     if (gthread == 0) {
         // packed columns: their own counts (written by this block's threads before the last block barrier)
         int most = J.pend ? 0 : last;
-        for (int c = 0; J.pend && c < J.cnt; ++c) most = max(most, B.iters_done[J.graph * K + J.pend[c].col]);
+        for (int c = 0; J.pend && c < J.cnt; ++c) most = max(most, B.iters_done[J.graph * K + C.col[c]]);
         B.counters[0] = max(B.counters[0], most);
     }
     return grid_sync(B.sync, gridDim.x);  // the next job reuses part and res_acc
 }
 
-#ifndef GP_BT_MINB
-#define GP_BT_MINB 2
-#endif
-__global__ void __launch_bounds__(BT_THREADS, GP_BT_MINB) k_ppr_persistent(BatchDev B) {
-    __shared__ float s_res[BT_THREADS / 32][32][4];  // per lane: |y - x| of its four columns
-    __shared__ int s_active[BT_MAX_KS];
+// Packed jobs over a list of columns, up to 32 of one graph at a time (the list
+// is in job order, so a graph's columns are adjacent).  Few columns take a
+// narrow job, whose sweeps gather 16 or 32 bytes per edge instead of 128 (R-MAT
+// 2^17: 97 us a sweep of 32 columns): one slow column can need five times the
+// sweeps of the others.
+template <int KS>
+__device__ bool ppr_packed(const BatchDev &B, const BPend *list, int count, int leave, BPend *next, int32_t *next_count,
+                           PCols &C) {
+    for (int i = 0; i < count;) {
+        const int g = list[i].graph;
+        int j = i + 1;
+        while (j < count && j - i < KS && list[j].graph == g) ++j;
+        const PView J = {g, B.XP0, B.XP1, KS, 0, list + i, j - i, leave, next, next_count};
+        if (!ppr_job<KS>(B, J, C)) return false;
+        i = j;
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(BT_THREADS, GP_BT_MINB) k_ppr_persistent(const __grid_constant__ BatchDev B) {
+    __shared__ PCols C;
     for (int ji = 0; ji < B.njobs; ++ji) {
         const BJob Jb = B.jobs[ji];
         const BGraph &G = B.graphs[Jb.graph];
-        const PView J = {Jb.graph, G.X0, G.X1, B.K, Jb.c0, nullptr, 0};
+        const PView J = {Jb.graph, G.X0, G.X1, B.K, Jb.c0, nullptr, 0, B.pack_max, B.pend, B.counters + 2};
         bool ok;
         switch (Jb.kpl) {
-            case 1: ok = ppr_job<32>(B, J, s_res, s_active); break;
-            case 2: ok = ppr_job<64>(B, J, s_res, s_active); break;
-            default: ok = ppr_job<128>(B, J, s_res, s_active); break;
+            case 1: ok = ppr_job<32>(B, J, C); break;
+            case 2: ok = ppr_job<64>(B, J, C); break;
+            default: ok = ppr_job<128>(B, J, C); break;
         }
         if (!ok) return;
     }
-    // the columns the jobs left: packed 32 at a time, a packed job never
-    // mixing graphs (the list is in job order, so a graph's columns are adjacent)
-    const int np = *(volatile int32_t *)(B.counters + 2);
-    for (int i = 0; i < np;) {
-        const int g = B.pend[i].graph;
-        int j = i + 1;
-        while (j < np && j - i < 32 && B.pend[j].graph == g) ++j;
-        const PView J = {g, B.XP0, B.XP1, 32, 0, B.pend + i, j - i};
-        if (!ppr_job<32>(B, J, s_res, s_active)) return;
-        i = j;
-    }
+    // the columns the jobs left, 32 to a job; what those leave 8 to a job, then 4
+    const int64_t most = (int64_t)B.ngraphs * B.K;
+    volatile int32_t *count = B.counters;
+    if (!ppr_packed<32>(B, B.pend, count[2], 8, B.pend + most, B.counters + 3, C)) return;
+    if (!ppr_packed<8>(B, B.pend + most, count[3], 4, B.pend + 2 * most, B.counters + 4, C)) return;
+    ppr_packed<4>(B, B.pend + 2 * most, count[4], 0, nullptr, nullptr, C);
 }
 
 // ------------------------------------------------------------------ batched multi-source BFS
@@ -711,6 +832,7 @@ struct gp_batch {
     gp::Arena mem;     // iterates, masks, levels and per-batch records
     gp::Arena layout;  // work lists that depend on the options
     gp::BGraph *dgraphs = nullptr;
+    int64_t nbig = 0;  // big vertices of all graphs
     int32_t *seeds = nullptr, *sources = nullptr;
     int32_t *counters = nullptr;
     int32_t *hcounters = nullptr;  // pinned
@@ -747,7 +869,8 @@ static int coop_launch(gp_batch *b, const void *kernel, cudaGraphExec_t &exec, b
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->dev.sync, 0, sizeof(GridSync), cap);
-        if (e == cudaSuccess) e = cudaMemsetAsync(b->counters, 0, 4 * sizeof(int32_t), cap);
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->counters, 0, 8 * sizeof(int32_t), cap);
+        if (e == cudaSuccess && b->nbig) e = cudaMemsetAsync(b->dev.bdone, 0, b->nbig * sizeof(unsigned), cap);
         if (e == cudaSuccess) {
             cudaLaunchConfig_t cfg;
             memset(&cfg, 0, sizeof(cfg));
@@ -777,12 +900,22 @@ static int coop_launch(gp_batch *b, const void *kernel, cudaGraphExec_t &exec, b
     return GP_OK;
 }
 
+// Edges per chunk of a graph of m edges: the option's, halved while that leaves
+// a warp of the grid without a chunk's worth of edges (a chunk's windows of loads
+// follow one another: at 128 edges they are a small graph's whole sweep).
+static int64_t chunk_size(const gp_batch *b, int64_t m) {
+    const int64_t warps = (int64_t)b->num_sms * GP_BT_MINB * (BT_THREADS / 32);
+    int64_t c = b->opt.chunk_edges;
+    while (c >= 64 && c * warps > m) c /= 2;
+    return c;
+}
+
 // Work lists for the current options: big in-degree vertices and their chunks,
 // big out-degree vertices, and the PPR jobs (column slices sized to the L2
 // budget).  Reads the offsets once; synchronises the stream.
 static int batch_layout(gp_batch *b, cudaStream_t s) {
     const int K = b->K;
-    const int64_t big_min = b->opt.big_in_degree, C = b->opt.chunk_edges;
+    const int64_t big_min = b->opt.big_in_degree;
     std::vector<int32_t> big;
     std::vector<int64_t> bcstart(1, 0);
     std::vector<BChunk> chunks;
@@ -795,15 +928,17 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
         cudaError_t e = cudaMemcpyAsync(off.data(), g->csc_off, off.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout: %s", cudaGetErrorString(e));
+        const int64_t C = chunk_size(b, g->m);
         BGraph &G = b->hg[gi];
         G.big0 = (int64_t)big.size();
         G.chunk0 = (int64_t)chunks.size();
         for (int64_t v = 0; v < g->n; ++v) {
             const int64_t d = off[v + 1] - off[v];
             if (d <= big_min) continue;
+            const int32_t r = (int32_t)big.size(), nch = (int32_t)((d + C - 1) / C);
             big.push_back((int32_t)v);
             for (int64_t p = off[v]; p < off[v + 1]; p += C)
-                chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v});
+                chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v, r, nch});
             bcstart.push_back((int64_t)chunks.size());
         }
         G.nbig = (int64_t)big.size() - G.big0;
@@ -824,12 +959,13 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
         cudaError_t e = cudaMemcpyAsync(off.data(), g->csr_off, off.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout: %s", cudaGetErrorString(e));
+        const int64_t C = chunk_size(b, g->m);
         BGraph &G = b->hg[gi];
         G.ochunk0 = (int64_t)chunks.size();
         for (int64_t v = 0; v < g->n; ++v)
             if (off[v + 1] - off[v] > big_min)
                 for (int64_t p = off[v]; p < off[v + 1]; p += C)
-                    chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v});
+                    chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v, 0, 0});
         G.nochunk = (int64_t)chunks.size() - G.ochunk0;
     }
     b->layout.release(s);
@@ -844,7 +980,9 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
     if (st == GP_OK) st = b->layout.alloc(dch, std::max<size_t>(chunks.size(), 1), s);
     if (st == GP_OK) st = b->layout.alloc(djobs, b->jobs.size(), s);
     if (st == GP_OK) st = b->layout.alloc(D.part, (size_t)max_chunks * K, s);
+    if (st == GP_OK) st = b->layout.alloc(D.bdone, std::max<size_t>(big.size(), 1), s);
     if (st != GP_OK) return st;
+    b->nbig = (int64_t)big.size();
     cudaError_t e = cudaMemcpyAsync(b->dgraphs, b->hg.data(), b->ngraphs * sizeof(BGraph), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && !big.empty()) e = cudaMemcpyAsync(dbig, big.data(), big.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dbc, bcstart.data(), bcstart.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
@@ -952,7 +1090,7 @@ extern "C" int gp_batch_create(gp_batch **out, gp_graph *const *graphs, int ngra
     if (st == GP_OK) st = b->mem.alloc(D.iters_done, (size_t)ngraphs * K, s);
     if (st == GP_OK) st = b->mem.alloc(b->counters, 8, s);
     if (st == GP_OK) st = b->mem.alloc(D.mcount, (size_t)ngraphs * 8, s);
-    if (st == GP_OK) st = b->mem.alloc(D.pend, (size_t)ngraphs * K, s);
+    if (st == GP_OK) st = b->mem.alloc(D.pend, (size_t)3 * ngraphs * K, s);
     if (st == GP_OK) st = b->mem.alloc(D.XP0, (size_t)nmax * 32, s);
     if (st == GP_OK) st = b->mem.alloc(D.XP1, (size_t)nmax * 32, s);
     if (st == GP_OK) st = b->mem.alloc(b->lev_out, (size_t)ngraphs, s);
