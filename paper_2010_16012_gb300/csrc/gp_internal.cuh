@@ -158,6 +158,8 @@ struct EdgeTiles {
     Arena mem;
 };
 
+struct GridSync;
+
 // Cached PageRank workspace (sized for the graph; reused across calls).
 struct PrWork {
     bool ready = false;
@@ -171,10 +173,19 @@ struct PrWork {
     double *acc64 = nullptr;       // FP64 accumulator of the push scatter
     float *lam = nullptr;          // adjoint solution
     float *gw_dev = nullptr;       // weight gradient when the output is host memory
+    GridSync *sync = nullptr;      // barrier of the sweeps in one launch
     void *status = nullptr;        // device PrStatus
     void *status_host = nullptr;   // pinned mirror (written by the kernels)
     void *status_mirror = nullptr; // its device-side address
     int max_blocks = 0;
+    cudaEvent_t ev[2] = {nullptr, nullptr};  // start and end of a timed call
+    struct Fit {
+        const void *kernel;
+        int threads;
+        size_t smem;
+        int blocks;
+    };
+    std::vector<Fit> fits;  // resident blocks per SM, by kernel and shape
     Arena mem;
 };
 

@@ -143,7 +143,7 @@ __device__ __forceinline__ void store_hot(const uint32_t *bits, const int32_t *p
 // x = x0 (or 1/n), c = x * cmul, and the push accumulators zeroed.
 __global__ void k_pr_init(int64_t n, const float *x0, const float *cmul, float *r0, float *c, float *r_push,
                           double *acc64, const uint32_t *hot_bits, const int32_t *hot_prefix, float *c_hot,
-                          PrStatus *status) {
+                          PrStatus *status, GridSync *sync) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const float x_uniform = 1.0f / (float)n;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
@@ -161,6 +161,7 @@ __global__ void k_pr_init(int64_t n, const float *x0, const float *cmul, float *
         status->residual = 0.0;
         status->converged = 0;
         status->upd_l2 = status->upd_shared = status->upd_merged = status->flush_l2 = 0;
+        *sync = GridSync();
     }
 }
 
@@ -197,10 +198,15 @@ __device__ __forceinline__ void load_hot(const PrArgs &a, float *sh) {
     __syncthreads();
 }
 
-template <bool HOT>
-__device__ __forceinline__ float gather_c(const float *__restrict__ c, const float *sh, int32_t u) {
+// LOOP: the contributions are rewritten by the same launch, so they may be kept
+// in L1 between barriers but not taken through the read-only path.
+template <bool HOT, bool LOOP>
+__device__ __forceinline__ float gather_c(const float *c, const float *sh, int32_t u) {
     if (HOT && u < 0) return sh[u & 0x7fffffff];
-    return __ldg(c + u);
+    if (!LOOP) return __ldg(c + u);
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(c + u));
+    return v;
 }
 
 #ifndef GP_TILE_THREADS
@@ -219,15 +225,69 @@ __device__ __forceinline__ void ld_stream8(const void *p, uint32_t (&v)[8]) {
                  : "l"(p));
 }
 
-// One sweep's sums: tile t's edges are gathered eight to a lane and summed by
-// row.  A row that starts in the tile leaves its sum there in acc[row]; edges
-// of a row started in an earlier tile leave theirs in carry[t].
-template <bool W, bool HOT>
-__device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh, int warp, int nwarps) {
+// A tile's sums by row, from its lanes' products f (eight consecutive edges
+// each), row-start bits h and the row open at its start.  A row that starts in
+// the tile leaves its sum there in acc[row]; edges of a row started in an
+// earlier tile leave theirs in carry[t].  Called by the whole warp.
+__device__ __forceinline__ void tile_sums(const PrArgs &a, int64_t t, unsigned h, int32_t row0, const float (&f)[8]) {
     const int lane = lane_id();
     const unsigned below = (1u << lane) - 1u;
+    const unsigned starts = __ballot_sync(FULL, h != 0);  // lanes where a row starts
+    if (starts == 0) {  // the inside of one long row
+        float s = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
+        s = warp_sum(s);
+        if (lane == 0) a.carry[t] = s;
+        return;
+    }
+    // rows started in the lanes below: prefix sum of popc(h) <= 8, by its binary digits
+    const unsigned cnt = __popc(h);
+    int before = 0, all = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const unsigned digit = __ballot_sync(FULL, (cnt >> b) & 1u);
+        before += __popc(digit & below) << b;
+        all += __popc(digit) << b;
+    }
+    const int32_t row = row0 + before;  // the row open at the lane's first edge
+    float open = 0.f, s = 0.f;
+    int32_t r = row;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        if ((h >> q) & 1u) {
+            if (r == row)
+                open = s;  // what the lane adds to the row open at its start
+            else
+                a.acc[r] = s;  // a row that starts and ends in the lane
+            ++r;
+            s = 0.f;
+        }
+        s += f[q];
+    }
+    // segmented inclusive scan over the lanes: s becomes the sum of the row
+    // open at the lane's end, back to the lane where it starts
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float up = __shfl_up_sync(FULL, s, o);
+        // lanes lane-o+1 .. lane start no row
+        if (lane >= o && (starts & (below + below + 1u) & ~((1u << (lane - o + 1)) - 1u)) == 0) s += up;
+    }
+    float in = __shfl_up_sync(FULL, s, 1);
+    if (lane == 0) in = 0.f;
+    if (h) {
+        if ((starts & below) == 0)
+            a.carry[t] = in + open;
+        else
+            a.acc[row] = in + open;
+    }
+    if (lane == 31) a.acc[row0 + all] = s;
+}
+
+// One sweep's sums: tiles warp, warp + nwarps, ...
+template <bool W, bool HOT, bool LOOP>
+__device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh, int warp, int nwarps) {
+    const int lane = lane_id();
     const int32_t *__restrict__ idx = a.idx;
-    const float *__restrict__ c = a.c;
+    const float *c = a.c;
     const int ntiles = (int)a.ntiles;
     for (int t = warp; t < ntiles; t += nwarps) {
         const int64_t e0 = (int64_t)t * TILE_EDGES + lane * LANE_EDGES;
@@ -238,7 +298,7 @@ __device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh
             uint32_t u[8];
             ld_stream8(idx + e0, u);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) f[q] = gather_c<HOT>(c, sh, (int32_t)u[q]);
+            for (int q = 0; q < 8; ++q) f[q] = gather_c<HOT, LOOP>(c, sh, (int32_t)u[q]);
             if (W) {
                 ld_stream8(a.w + e0, u);
 #pragma unroll
@@ -249,59 +309,12 @@ __device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh
             for (int q = 0; q < 8; ++q) {
                 f[q] = 0.f;
                 if (e0 + q < a.m) {
-                    f[q] = gather_c<HOT>(c, sh, __ldg(idx + e0 + q));
+                    f[q] = gather_c<HOT, LOOP>(c, sh, __ldg(idx + e0 + q));
                     if (W) f[q] *= __ldg(a.w + e0 + q);
                 }
             }
         }
-        const unsigned starts = __ballot_sync(FULL, h != 0);  // lanes where a row starts
-        if (starts == 0) {  // the inside of one long row
-            float s = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
-            s = warp_sum(s);
-            if (lane == 0) a.carry[t] = s;
-            continue;
-        }
-        // rows started in the lanes below: prefix sum of popc(h) <= 8, by its binary digits
-        const unsigned cnt = __popc(h);
-        int before = 0, all = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const unsigned digit = __ballot_sync(FULL, (cnt >> b) & 1u);
-            before += __popc(digit & below) << b;
-            all += __popc(digit) << b;
-        }
-        const int32_t row = row0 + before;  // the row open at the lane's first edge
-        float open = 0.f, s = 0.f;
-        int32_t r = row;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            if ((h >> q) & 1u) {
-                if (r == row)
-                    open = s;  // what the lane adds to the row open at its start
-                else
-                    a.acc[r] = s;  // a row that starts and ends in the lane
-                ++r;
-                s = 0.f;
-            }
-            s += f[q];
-        }
-        // segmented inclusive scan over the lanes: s becomes the sum of the row
-        // open at the lane's end, back to the lane where it starts
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float up = __shfl_up_sync(FULL, s, o);
-            // lanes lane-o+1 .. lane start no row
-            if (lane >= o && (starts & (below + below + 1u) & ~((1u << (lane - o + 1)) - 1u)) == 0) s += up;
-        }
-        float in = __shfl_up_sync(FULL, s, 1);
-        if (lane == 0) in = 0.f;
-        if (h) {
-            if ((starts & below) == 0)
-                a.carry[t] = in + open;
-            else
-                a.acc[row] = in + open;
-        }
-        if (lane == 31) a.acc[row0 + all] = s;
+        tile_sums(a, t, h, row0, f);
     }
 }
 
@@ -317,7 +330,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_tiles(PrArgs a) {
     extern __shared__ float sh_hot[];
     if (pr_gate(a, a.k)) return;
     load_hot<HOT>(a, sh_hot);
-    pull_tiles_step<W, HOT>(a, sh_hot, (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+    pull_tiles_step<W, HOT, false>(a, sh_hot, (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
                             (int)(gridDim.x * blockDim.x) >> 5);
 }
 
@@ -368,6 +381,165 @@ __global__ void __launch_bounds__(256) k_pull_finish(PrArgs a) {
     pull_finish_step<HOT>(a, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, res);
     const double r = block_residual(res, sm);
     if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
+}
+
+// All sweeps of a small graph in one cooperative launch: two barriers a sweep
+// instead of two launches, and the convergence test on the device.  Without a
+// hot set: on such graphs most of the contribution vector stays in L1.
+struct PrLoop {
+    PrArgs a;  // sweep k from R[(k-1)&1], C[(k-1)&1] to R[k&1], C[k&1]
+    float *R[2], *C[2];
+    int32_t iters;
+    PrStatus *mirror;
+    GridSync *sync;
+};
+
+// The end of sweep k, called by every block: true when it was the last one.
+__device__ __forceinline__ bool loop_end(const PrLoop &P, int k, double *sm, double &residual) {
+    __shared__ double s_res;
+    if (P.a.tol <= 0.0 && k < P.iters) return false;
+    double t = 0.0;  // the same sum in the same order in every block
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) t += P.a.partials[i];
+    t = block_sum(t, sm);
+    if (threadIdx.x == 0) s_res = t;
+    __syncthreads();
+    residual = s_res;
+    return residual < P.a.tol || k == P.iters;
+}
+
+__device__ __forceinline__ void loop_status(const PrLoop &P, int k, double residual) {
+    PrStatus *st = P.a.status;
+    st->done = st->converged = residual < P.a.tol;
+    st->iters_done = k;
+    st->residual = residual;
+    *P.mirror = *st;
+    __threadfence_system();
+}
+
+template <bool W>
+__global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_loop(const __grid_constant__ PrLoop P) {
+    __shared__ double sm[32];
+    PrArgs a = P.a;
+    const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
+    double residual = 0.0;
+    int k = 1;
+    for (;; ++k) {
+        a.k = k;
+        a.x = P.R[(k - 1) & 1];
+        a.y = P.R[k & 1];
+        a.c = P.C[(k - 1) & 1];
+        a.c_next = P.C[k & 1];
+        pull_tiles_step<W, false, true>(a, nullptr, (int)(thread >> 5), (int)(nthreads >> 5));
+        if (!grid_sync(P.sync, gridDim.x)) return;
+        ResSum res;
+        pull_finish_step<false>(a, thread, nthreads, res);
+        const double r = block_residual(res, sm);
+        if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
+        if (!grid_sync(P.sync, gridDim.x)) return;
+        if (loop_end(P, k, sm, residual)) break;
+    }
+    if (k & 1)  // the caller's buffer is R[0]
+        for (int64_t v = thread; v < a.n; v += nthreads) P.R[0][v] = P.R[1][v];
+    if (thread == 0) loop_status(P, k, residual);
+}
+
+// The same with a tile to a warp and a row to a thread, for graphs that the grid
+// holds that way: what does not change between sweeps (indices, weights, row
+// numbers and places, the vertex's factors) and the iterate itself stay in
+// registers, and a sweep is two chains of one load each between its barriers:
+// 5 us a sweep at R-MAT 2^14, where the loop above takes 9 and launches 17.
+template <bool W>
+__global__ void __launch_bounds__(TILE_THREADS, 1) k_pull_loop_regs(const __grid_constant__ PrLoop P) {
+    __shared__ double sm[32];
+    const PrArgs &a = P.a;
+    const int lane = lane_id();
+    const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // the warp's tile
+    const int64_t t = thread >> 5;
+    const bool tile = t < a.ntiles;
+    const int64_t e0 = t * TILE_EDGES + lane * LANE_EDGES;
+    const unsigned h = tile ? a.heads[t * 32 + lane] : 0u;
+    const int32_t row0 = tile ? a.tile_row[t] : 0;
+    int32_t u[8];
+    float w[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const bool edge = tile && e0 + q < a.m;
+        u[q] = edge ? __ldg(a.idx + e0 + q) : -1;
+        w[q] = W && edge ? __ldg(a.w + e0 + q) : 0.f;
+    }
+    // the thread's row, or vertex without in-edges (acc: its sum's place; long rows are a warp's)
+    const bool has = thread < a.n, filled = thread < a.nrows;
+    int64_t v = 0, c0 = 0, c1 = 0;  // the carries to add: [c0, c1)
+    bool mine = has;
+    if (has) {
+        const uint32_t code = (uint32_t)a.rows[thread];
+        v = code & ~HOT_BIT;
+        if (code & HOT_BIT) {
+            c0 = a.off[v] / TILE_EDGES + 1;
+            c1 = (a.off[v + 1] - 1) / TILE_EDGES + 1;
+            mine = c1 - c0 <= TILE_LONG;
+        }
+    }
+    // the warp's long row
+    const bool longrow = t < a.nlong;
+    int32_t lr = 0;
+    int64_t lv = 0, l0 = 0, l1 = 0;
+    if (longrow) {
+        lr = a.long_rows[t];
+        lv = (uint32_t)a.rows[lr] & ~HOT_BIT;
+        l0 = a.off[lv] / TILE_EDGES + 1;
+        l1 = (a.off[lv + 1] - 1) / TILE_EDGES + 1;
+    }
+    const bool leader = longrow && lane == 0;
+    const float base = has ? base_term(a, v) : 0.f, cm = has ? c_factor(a, v) : 0.f;
+    const float lbase = leader ? base_term(a, lv) : 0.f, lcm = leader ? c_factor(a, lv) : 0.f;
+    float x = has ? P.R[0][v] : 0.f, lx = leader ? P.R[0][lv] : 0.f;
+    double residual = 0.0;
+    int k = 1;
+    for (;; ++k) {
+        const float *c = P.C[(k - 1) & 1];
+        float *c_next = P.C[k & 1];
+        if (tile) {
+            float f[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                f[q] = u[q] >= 0 ? gather_c<false, true>(c, nullptr, u[q]) : 0.f;
+                if (W) f[q] *= w[q];
+            }
+            tile_sums(a, t, h, row0, f);
+        }
+        if (!grid_sync(P.sync, gridDim.x)) return;
+        ResSum res;
+        if (mine) {
+            float sum = filled ? a.acc[thread] : 0.f;
+            for (int64_t i = c0; i < c1; ++i) sum += a.carry[i];
+            const float y = base + a.d * sum;
+            res.add(y, x);
+            x = y;
+            c_next[v] = y * cm;
+        }
+        if (longrow) {
+            float sum = 0.f;
+            for (int64_t i = l0 + lane; i < l1; i += 32) sum += a.carry[i];
+            sum = warp_sum(sum);
+            if (lane == 0) {
+                const float y = lbase + a.d * (a.acc[lr] + sum);
+                res.add(y, lx);
+                lx = y;
+                c_next[lv] = y * lcm;
+            }
+        }
+        if (a.tol > 0.0 || k == P.iters) {
+            const double r = block_residual(res, sm);
+            if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
+        }
+        if (!grid_sync(P.sync, gridDim.x)) return;
+        if (loop_end(P, k, sm, residual)) break;
+    }
+    if (mine) P.R[0][v] = x;
+    if (leader) P.R[0][lv] = lx;
+    if (thread == 0) loop_status(P, k, residual);
 }
 
 // The adjoint's pull sweep sums a row in a fixed order of its own, whatever the
@@ -781,18 +953,27 @@ __global__ void __launch_bounds__(256) k_grad_w(GradArgs a) {
 // ------------------------------------------------------------------ driver
 
 void release_pr_work(gp_graph *g, cudaStream_t s) {
+    for (cudaEvent_t e : g->pr.ev)
+        if (e) cudaEventDestroy(e);
     pinned_free(g->pr.status_host, 4 * sizeof(PrStatus));
     g->pr.status_host = nullptr;
     g->pr.mem.release(s);
     g->pr = PrWork();
 }
 
-// Resident blocks per SM of `kernel` (raising its dynamic shared-memory limit first).
-static int occupancy(const void *kernel, int threads, size_t smem, int &blocks) {
+// Resident blocks per SM of `kernel` (raising its dynamic shared-memory limit
+// first), asked once per graph and shape: the two queries cost a call 5 us.
+static int occupancy(PrWork &w, const void *kernel, int threads, size_t smem, int &blocks) {
+    for (const PrWork::Fit &f : w.fits)
+        if (f.kernel == kernel && f.threads == threads && f.smem == smem) {
+            blocks = f.blocks;
+            return GP_OK;
+        }
     // the opt-in is needed whenever dynamic + static shared memory exceeds 48 KiB; set it for any size
     if (smem > 0) GP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem));
     if (blocks < 1) return set_error(GP_ERR_UNSUPPORTED, "kernel does not fit on an SM (%zu B shared memory)", smem);
+    w.fits.push_back({kernel, threads, smem, blocks});
     return GP_OK;
 }
 
@@ -810,8 +991,10 @@ static int ensure_pr_work(gp_graph *g, cudaStream_t s) {
     PrStatus *st = nullptr;
     GP_TRY(w.mem.alloc(st, 1, s));
     w.status = st;
+    GP_TRY(w.mem.alloc(w.sync, 1, s));
     GP_TRY(pinned_alloc(&w.status_host, 4 * sizeof(PrStatus)));
     GP_TRY(pinned_device_ptr(w.status_host, &w.status_mirror));
+    for (cudaEvent_t &e : w.ev) GP_CUDA(cudaEventCreate(&e));
     w.ready = true;
     return GP_OK;
 }
@@ -838,6 +1021,13 @@ static const void *push_kernel(bool W, bool fp64, bool hot) {
 // PUSH_FP32_MAX_UPDATES updates per sweep (FP32 order noise at such hubs sets a
 // residual floor near 1e-7).
 constexpr int64_t PUSH_FP32_MAX_UPDATES = 4096;
+
+// Pull graphs of at most this many edge tiles run all sweeps in one launch.
+// Measured per call of 20 sweeps, a launch per step and one launch: R-MAT 2^14
+// (1.7K tiles) 360 and 168 us, 2^16 (7.1K) 460 and 288, 2^18 (30K) 624 and 574,
+// uniform 2^18 (16K) 732 and 606; above, the hot set that the launches keep in
+// shared memory wins on skewed graphs (R-MAT 2^20, 123K tiles: 1480 and 1810).
+constexpr int64_t LOOP_TILES = 32768;
 static bool push_fp64(const gp_graph *g, int64_t max_updates) {
     if (g->opt.push_fp64_accum >= 0) return g->opt.push_fp64_accum != 0;
     const bool fits = 8 * g->n <= g->l2_bytes / 2;
@@ -902,6 +1092,7 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     bool hot = false;
     size_t smem = 0;
     const bool tiled = !push && sp.tiles;
+    bool loop = false;  // all sweeps in one launch
     if (!push && !tiled) {
         if (!w.chunk_part) GP_TRY(w.mem.alloc(w.chunk_part, (size_t)std::max<int64_t>(bins.nchunks, 1), s));
         a.chunk_part = w.chunk_part;
@@ -919,7 +1110,8 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         a.ntiles = t.ntiles;
         a.nrows = t.nrows;
         a.nlong = t.nlong;
-        if (sp.hot) {
+        loop = t.ntiles <= LOOP_TILES;
+        if (sp.hot && !loop) {
             if (g->pull_hot.slots != g->opt.pull_hot_slots) GP_TRY(build_pull_hot(g, g->opt.pull_hot_slots, s));
             hot = g->pull_hot.nhot > 0;
         }
@@ -945,19 +1137,34 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     }
     int g1, g2;
     const int tpt = TILE_THREADS;
+    const void *kl = nullptr;  // the kernel of all sweeps
     if (!push && !tiled) {
         int ob = 0, ol = 0;
-        GP_TRY(occupancy(W ? (const void *)k_adj_big<true> : (const void *)k_adj_big<false>, 1024, 0, ob));
-        GP_TRY(occupancy(W ? (const void *)k_adj_light<true> : (const void *)k_adj_light<false>, 512, 0, ol));
+        GP_TRY(occupancy(w, W ? (const void *)k_adj_big<true> : (const void *)k_adj_big<false>, 1024, 0, ob));
+        GP_TRY(occupancy(w, W ? (const void *)k_adj_light<true> : (const void *)k_adj_light<false>, 512, 0, ol));
         g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (bins.nchunks + 31) / 32));
         a.split_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ol * g->num_sms, (ntiles + 15) / 16));
         g2 = a.split_blocks + (int)((bins.nbig + 511) / 512);
+    } else if (loop) {
+        // a warp per tile and a thread per row where the grid holds that many, and no
+        // more blocks than that to wait for
+        constexpr int wpb = TILE_THREADS / 32;
+        const int64_t regs = std::max((a.ntiles + wpb - 1) / wpb, (n + TILE_THREADS - 1) / TILE_THREADS);
+        int ob = 0;
+        kl = W ? (const void *)k_pull_loop_regs<true> : (const void *)k_pull_loop_regs<false>;
+        GP_TRY(occupancy(w, kl, TILE_THREADS, 0, ob));
+        if (regs > (int64_t)ob * g->num_sms || a.nlong > regs * wpb) {
+            kl = W ? (const void *)k_pull_loop<true> : (const void *)k_pull_loop<false>;
+            GP_TRY(occupancy(w, kl, TILE_THREADS, 0, ob));
+        }
+        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, regs));
+        g2 = g1;
     } else if (!push) {
         int ob = 0, of = 0;
         const void *kb_ = W ? (hot ? (const void *)k_pull_tiles<true, true> : (const void *)k_pull_tiles<true, false>)
                             : (hot ? (const void *)k_pull_tiles<false, true> : (const void *)k_pull_tiles<false, false>);
-        GP_TRY(occupancy(kb_, tpt, smem, ob));
-        GP_TRY(occupancy(hot ? (const void *)k_pull_finish<true> : (const void *)k_pull_finish<false>, 256, 0, of));
+        GP_TRY(occupancy(w, kb_, tpt, smem, ob));
+        GP_TRY(occupancy(w, hot ? (const void *)k_pull_finish<true> : (const void *)k_pull_finish<false>, 256, 0, of));
         const int wpb = tpt / 32;
         g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (a.ntiles + wpb - 1) / wpb));
         g2 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)of * g->num_sms, (n + 255) / 256));
@@ -966,7 +1173,7 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         // capped by blocks_per_sm (256-thread units)
         const void *ks = push_kernel(W, push_fp64(g, sp.max_updates), hot);
         int os = 0;
-        GP_TRY(occupancy(ks, 1024, smem, os));
+        GP_TRY(occupancy(w, ks, 1024, smem, os));
         const int cap = std::max(1, g->opt.blocks_per_sm / 4) * g->num_sms;
         const int64_t work = std::max<int64_t>((bins.nchunks + 31) / 32, (ntiles + 31) / 32);
         g1 = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>((int64_t)os * g->num_sms, cap), work));
@@ -980,7 +1187,7 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     if (fp64 && !w.acc64) GP_TRY(w.mem.alloc(w.acc64, (size_t)n, s));
     a.acc64 = fp64 ? w.acc64 : nullptr;
     GP_LAUNCH("pr_init", s, (k_pr_init<<<ib, 256, 0, s>>>(n, sp.x0, sp.cmul, R[0], C[0], (push && !fp64) ? R[1] : nullptr,
-                                                          a.acc64, a.hot_bits, a.hot_prefix, a.c_hot, status)));
+                                                          a.acc64, a.hot_bits, a.hot_prefix, a.c_hot, status, w.sync)));
     GP_TRY(check_launch("pr_init"));
     auto enqueue_sweep = [&](int k) -> int {
         PrArgs b = a;
@@ -1035,6 +1242,28 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         return check_launch("pr_finish");
     };
 
+    if (loop) {
+        PrLoop P;
+        P.a = a;
+        P.R[0] = R[0];
+        P.R[1] = R[1];
+        P.C[0] = C[0];
+        P.C[1] = C[1];
+        P.iters = sp.iters;
+        P.mirror = (PrStatus *)w.status_mirror + 2;
+        P.sync = w.sync;
+        volatile PrStatus *host = (PrStatus *)w.status_host + 2;
+        host->iters_done = -1;  // the launch's last block of work replaces it
+        {
+            ProfScope ps("pull_loop", s);
+            void *args[] = {&P};
+            GP_CUDA(cudaLaunchCooperativeKernel(kl, dim3((unsigned)g1), dim3(TILE_THREADS), args, 0, s));
+        }
+        GP_CUDA(cudaStreamSynchronize(s));
+        if (host->iters_done < 0) return set_error(GP_ERR_TIMEOUT, "PageRank: a grid barrier wait ran out");
+        memcpy(&fin, (const PrStatus *)w.status_host + 2, sizeof(fin));
+        return GP_OK;
+    }
     const int poll = std::max(1, g->opt.poll_interval);
     const int iters = sp.iters;
     int issued = 0;
@@ -1172,8 +1401,8 @@ extern "C" int gp_pagerank(const gp_graph *gc, int mode, float damping, int iter
     PrWork &w = g->pr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (stats) {
-        GP_CUDA(cudaEventCreate(&ev0));
-        GP_CUDA(cudaEventCreate(&ev1));
+        ev0 = w.ev[0];
+        ev1 = w.ev[1];
         GP_CUDA(cudaEventRecord(ev0, s));
     }
     const bool out_dev = is_device_ptr(ranks_out);
@@ -1212,8 +1441,6 @@ extern "C" int gp_pagerank(const gp_graph *gc, int mode, float damping, int iter
         GP_CUDA(cudaEventSynchronize(ev1));
         float ms = 0.f;
         cudaEventElapsedTime(&ms, ev0, ev1);
-        cudaEventDestroy(ev0);
-        cudaEventDestroy(ev1);
         stats->iters_done = fin.iters_done;
         stats->mode_used = mode;
         stats->residual = fin.residual;
@@ -1248,8 +1475,8 @@ extern "C" int gp_pagerank_backward(const gp_graph *gc, int mode, float damping,
     PrWork &w = g->pr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (stats) {
-        GP_CUDA(cudaEventCreate(&ev0));
-        GP_CUDA(cudaEventCreate(&ev1));
+        ev0 = w.ev[0];
+        ev1 = w.ev[1];
         GP_CUDA(cudaEventRecord(ev0, s));
     }
     const float *X = nullptr, *G = nullptr;
@@ -1325,8 +1552,6 @@ extern "C" int gp_pagerank_backward(const gp_graph *gc, int mode, float damping,
         GP_CUDA(cudaEventSynchronize(ev1));
         float ms = 0.f;
         cudaEventElapsedTime(&ms, ev0, ev1);
-        cudaEventDestroy(ev0);
-        cudaEventDestroy(ev1);
         stats->iters_done = fin.iters_done;
         stats->mode_used = mode;
         stats->residual = fin.residual;

@@ -88,3 +88,36 @@ def test_tiles(gp, name, slots, weighted, shift):
         err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
         assert st["iters_done"] == iters
         assert err.max() <= MAX_ABS and err.sum() <= L1, (name, iters, float(err.max()), float(err.sum()))
+
+
+@pytest.mark.parametrize("weighted,slots,shift", [(False, 20480, 0), (True, 20480, 1), (False, 0, 1)])
+@pytest.mark.parametrize("bulk", [1_200_000, 8_600_000])
+def test_tiles_of_larger_graphs(gp, bulk, weighted, slots, shift):
+    """The same rows in graphs that the one-launch loop holds a tile to a warp no
+    longer (1.2M edges) and that run a launch per step (8.6M edges, above 32768
+    tiles): before and after a bulk of other rows, and a last tile cut short."""
+    import torch
+
+    rng = np.random.default_rng(bulk)
+    edges = [d for name in DEGREES for d in DEGREES[name]]
+    fill = rng.integers(0, 33, bulk // 16).tolist()
+    n, csr_off, csr_idx, csr_w, csc_off, csc_idx, csc_w = make(edges + fill + edges, seed=3)
+
+    def dev(a, dt):
+        return torch.cat([torch.zeros(shift, dtype=dt), torch.from_numpy(np.ascontiguousarray(a)).to(dt)]).cuda()[shift:]
+
+    w = [dev(csr_w, torch.float32), dev(csc_w, torch.float32)] if weighted else [None, None]
+    G = gp.Graph(n, dev(csr_off, torch.int64), dev(csr_idx, torch.int32), dev(csc_off, torch.int64),
+                 dev(csc_idx, torch.int32), *w)
+    G.set_options(pull_hot_slots=slots)
+    wx = csc_w.astype(np.float32).astype(np.float64) if weighted else None
+    for iters in (1, 2, 5):
+        ref = sweeps(n, csr_off, csc_off, csc_idx, wx, iters)
+        x, st = gp.pagerank(G, gp.PULL, 0.85, iters)
+        err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
+        assert st["iters_done"] == iters
+        assert err.max() <= MAX_ABS and err.sum() <= L1, (iters, float(err.max()), float(err.sum()))
+    ref = sweeps(n, csr_off, csc_off, csc_idx, wx, 200)
+    x, st = gp.pagerank(G, gp.PULL, 0.85, 200, 1e-6)  # stopped by the residual, within its bound of the fixed point
+    err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
+    assert st["converged"] and st["residual"] < 1e-6 and st["iters_done"] < 200 and err.sum() <= 1e-6 / 0.15 + L1
