@@ -33,6 +33,7 @@ namespace gp {
 
 constexpr int SS_WARPS = 32;
 constexpr int SS_THREADS = SS_WARPS * 32;
+constexpr int SS_WORDS = 512;  // bitmap words of a block's pass over the active set
 constexpr unsigned long long SS_NONE = ~0ull;  // key of an unreached vertex: (+inf, 0xffffffff)
 
 __device__ __forceinline__ unsigned long long ss_pack(float d, uint32_t pred) {
@@ -50,7 +51,7 @@ struct SsCtr {
     unsigned long long examined;
     unsigned long long settled_in;  // in-degree of the vertices settled at an epoch end
     unsigned long long nb_key;      // epoch end: max of (~0 - bucket) over pending vertices; 0 = none
-    unsigned long long pad;
+    unsigned long long heavy;       // vertices of the active set above the push light limit
 };
 
 struct SsIterStat {
@@ -70,6 +71,7 @@ struct SsRun {
     const int64_t *csr_off, *csc_off;
     const int32_t *csr_idx, *csc_idx;
     const float *csr_w, *csc_w;  // nullptr: unit weights
+    int64_t push_light_max;
     const int32_t *push_rank;    // [n] rank among vertices with out-degree > push light limit, -1 if light
     const int64_t *push_cstart;
     const Chunk *push_chunks;
@@ -99,6 +101,18 @@ __device__ __forceinline__ unsigned long long ss_bucket(float d, float delta) {
     return q < 4.0e18f ? (unsigned long long)q : 4000000000000000000ull;
 }
 
+// The least distance whose bucket lies above b (infinity: none does).  A new
+// distance is never below its source's bucket, so one comparison tells whether
+// it stays in bucket b, where the quotient costs a third of an edge's instructions.
+__device__ __forceinline__ float ss_bucket_end(unsigned long long b, float delta) {
+    const float inf = __int_as_float(0x7f800000);
+    if (!(ss_bucket(inf, delta) > b)) return inf;
+    float x = (float)(b + 1) * delta;
+    while (x > 0.f && ss_bucket(x, delta) > b) x = __uint_as_float(__float_as_uint(x) - 1u);
+    while (ss_bucket(x, delta) <= b) x = __uint_as_float(__float_as_uint(x) + 1u);
+    return x;
+}
+
 __device__ __forceinline__ unsigned long long ss_now() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -110,42 +124,72 @@ __device__ __forceinline__ unsigned long long ss_now() {
 
 struct SsLocal {  // per-thread counter contributions of an iteration
     unsigned long long nact = 0, mact = 0, npend = 0, examined = 0;
+    unsigned heavy = 0;
 };
 
-// Offer (nd, u) to w, whose key was read as `seen`; on a strict distance
-// improvement mark w active (same bucket) or pending (later bucket), counting
-// first marks only.  Keys only decrease, so a `seen` that is not above the
-// offer (a plain, possibly stale, read is never below the current key) means
-// the atomic could not change anything.
-__device__ __forceinline__ void ss_offer_seen(const SsRun &R, uint32_t *act_next, unsigned long long b, float nd,
-                                              int32_t u, int32_t w, unsigned long long seen, SsLocal &c) {
-    if (w == R.src) return;  // (0, src) is final; a zero-weight edge into it must not change its predecessor
-    const unsigned long long cand = ss_pack(nd, (uint32_t)u);
-    if (cand >= seen) return;
-    const unsigned long long old = atomicMin(R.key + w, cand);
-    if (!(nd < ss_dist(old))) return;
-    const uint32_t bit = 1u << (w & 31);
-    if (ss_bucket(nd, R.delta) == b) {
-        atomicOr(R.members + (w >> 5), bit);
-        if (!(atomicOr(act_next + (w >> 5), bit) & bit)) {
-            c.nact += 1;
-            c.mact += (unsigned long long)(R.csr_off[w + 1] - R.csr_off[w]);
+__device__ __forceinline__ void ss_count_active(const SsRun &R, int64_t v, SsLocal &c) {
+    const int64_t deg = R.csr_off[v + 1] - R.csr_off[v];
+    c.nact += 1;
+    c.mact += (unsigned long long)deg;
+    c.heavy += deg > R.push_light_max;
+}
+
+// Offer (nd, u) to w, whose key was read as `seen`, for up to U edges of a lane
+// (w < 0: none); on a strict distance improvement mark w active (same bucket)
+// or pending (later bucket), counting first marks only.  Keys only decrease, so
+// a `seen` that is not above the offer (a plain, possibly stale, read is never
+// below the current key) means the atomic could not change anything.  All
+// minima are issued before the first answer is looked at, then all marks: an
+// offer is two dependent trips to L2, and U of them one after another were most
+// of an iteration's time.
+template <int U>
+__device__ __forceinline__ void ss_offers(const SsRun &R, uint32_t *act_next, float end, const float (&nd)[U],
+                                          const int32_t (&u)[U], const int32_t (&w)[U],
+                                          const unsigned long long (&seen)[U], SsLocal &c) {
+    unsigned long long old[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+        const unsigned long long cand = ss_pack(nd[q], (uint32_t)u[q]);
+        old[q] = 0;
+        // (0, src) is final; a zero-weight edge into the source must not change its predecessor
+        if (w[q] >= 0 && w[q] != R.src && cand < seen[q]) old[q] = atomicMin(R.key + w[q], cand);
+    }
+    uint32_t was[U];
+    bool same[U], later[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+        const bool better = old[q] != 0 && nd[q] < ss_dist(old[q]);  // (a reached key is never 0 off the source)
+        same[q] = better && nd[q] < end;
+        later[q] = better && !same[q];
+        const uint32_t bit = 1u << (w[q] & 31);
+        was[q] = bit;
+        if (better) was[q] = atomicOr((same[q] ? act_next : R.pend) + (w[q] >> 5), bit);
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+        if ((was[q] >> (w[q] & 31)) & 1u) continue;
+        if (later[q]) {
+            c.npend += 1;
+        } else {
+            ss_count_active(R, w[q], c);
         }
-    } else if (!(atomicOr(R.pend + (w >> 5), bit) & bit)) {
-        c.npend += 1;
     }
 }
 
-__device__ __forceinline__ void ss_offer(const SsRun &R, uint32_t *act_next, unsigned long long b, float nd, int32_t u,
-                                         int32_t w, SsLocal &c) {
-    ss_offer_seen(R, act_next, b, nd, u, w, R.key[w], c);
+__device__ __forceinline__ void ss_offer(const SsRun &R, uint32_t *act_next, float end, float nd, int32_t u, int32_t w, SsLocal &c) {
+    const float n1[1] = {nd};
+    const int32_t u1[1] = {u}, w1[1] = {w};
+    const unsigned long long s1[1] = {R.key[w]};
+    ss_offers<1>(R, act_next, end, n1, u1, w1, s1, c);
 }
 
 __device__ void ss_flush(SsCtr *nx, const SsLocal &c) {
     __shared__ unsigned long long sm[32];
     const unsigned long long a = block_sum(c.nact, sm), b = block_sum(c.mact, sm), p = block_sum(c.npend, sm),
                              e = block_sum(c.examined, sm);
+    const int h = __syncthreads_or(c.heavy != 0);  // (only whether there are any is asked)
     if (threadIdx.x == 0) {
+        if (h) atomicAdd(&nx->heavy, 1ull);
         if (a) atomicAdd(&nx->nact, a);
         if (b) atomicAdd(&nx->mact, b);
         if (p) atomicAdd(&nx->npend, p);
@@ -153,104 +197,179 @@ __device__ void ss_flush(SsCtr *nx, const SsLocal &c) {
     }
 }
 
-// Push, phase A: a warp ranks the active vertices of 32 bitmap words; light
-// ones relax their out-edges as one merged edge stream over the warp, heavy
-// ones queue their chunk ids for phase B.
+constexpr int SS_U = 4;  // relaxations in flight per lane
+
+// Push, phase A: a block gathers the active vertices of its words (eight
+// neighbouring words to a block in turn, since they lie dense among the low ids
+// of a power-law graph) into shared memory; its warps take them 32 at a time,
+// as they get free.  Light ones relax their out-edges as one merged edge stream
+// over the warp, heavy ones queue their chunk ids for phase B.
 __device__ void ss_push_a(const SsRun &R, const uint32_t *act_cur, uint32_t *act_next, SsCtr *cur,
-                          unsigned long long b, SsLocal &c) {
-    const int lane = lane_id();
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+                          float end, uint16_t *s_queue, SsLocal &c) {
+    __shared__ int s_warp[SS_WARPS];
+    __shared__ int s_next;
+    const int lane = lane_id(), wib = threadIdx.x >> 5;
     const int64_t nwords = (R.n + 31) >> 5;
-    for (int64_t base = warp * 32; base < nwords; base += nwarps * 32) {
-        const int64_t wd = base + lane;
-        const uint32_t word = wd < nwords ? act_cur[wd] : 0u;
+    for (int64_t pass = 0; pass * gridDim.x * SS_WORDS < nwords; ++pass) {
+        auto word_of = [&](int i) {
+            return ((pass * (SS_WORDS / 8) + i / 8) * gridDim.x + blockIdx.x) * 8 + i % 8;
+        };
+        const int64_t wd = word_of(threadIdx.x);
+        uint32_t word = (int)threadIdx.x < SS_WORDS && wd < nwords ? act_cur[wd] : 0u;
         const int cnt = __popc(word);
         const int incl = warp_incl_scan(cnt);
-        const int excl = incl - cnt;
-        const int total = __shfl_sync(FULL, incl, 31);
-        for (int r = 0; r < total; r += 32) {
-            const int id = r + lane;
-            int k = 0;
-#pragma unroll
-            for (int st = 16; st > 0; st >>= 1) {
-                const int ek = __shfl_sync(FULL, excl, k + st);
-                if (ek <= id) k += st;
-            }
-            const uint32_t kw = __shfl_sync(FULL, word, k);
-            const int kex = __shfl_sync(FULL, excl, k);
+        __syncthreads();  // the previous pass is done with the queue
+        if (lane == 31) s_warp[wib] = incl;
+        if (threadIdx.x == 0) s_next = 0;
+        __syncthreads();
+        int at = incl - cnt, total = 0;
+        for (int i = 0; i < SS_WARPS; ++i) {
+            at += i < wib ? s_warp[i] : 0;
+            total += s_warp[i];
+        }
+        for (; word; word &= word - 1) s_queue[at++] = (uint16_t)(threadIdx.x * 32 + __ffs(word) - 1);
+        __syncthreads();
+        while (true) {
+            int id = 0;
+            if (lane == 0) id = atomicAdd(&s_next, 32);
+            id = __shfl_sync(FULL, id, 0);
+            if (id >= total) break;
+            id += lane;
             int32_t u = -1;
             int deg = 0;
             int64_t eb = 0;
             float du = 0.f;
             if (id < total) {
-                u = (int32_t)((base + k) * 32 + nth_set_bit(kw, id - kex));
+                const int code = s_queue[id];
+                u = (int32_t)(word_of(code >> 5) * 32 + (code & 31));
                 const int32_t rk = R.push_rank[u];
+                eb = R.csr_off[u];
+                deg = (int)(R.csr_off[u + 1] - eb);
+                du = ss_dist(R.key[u]);
                 if (rk >= 0) {  // heavy: its chunks go to phase B
+                    deg = 0;
                     const int64_t c0 = R.push_cstart[rk], c1 = R.push_cstart[rk + 1];
                     const unsigned long long pos = atomicAdd(&cur->h_len, (unsigned long long)(c1 - c0));
                     for (int64_t j = c0; j < c1; ++j) R.hq[pos + (j - c0)] = (int32_t)j;
-                } else {
-                    eb = R.csr_off[u];
-                    deg = (int)(R.csr_off[u + 1] - eb);
-                    du = ss_dist(R.key[u]);
                 }
             }
             const int dincl = warp_incl_scan(deg);
             const int dexcl = dincl - deg;
             const int E = __shfl_sync(FULL, dincl, 31);
-            for (int eb0 = 0; eb0 < E; eb0 += 32) {
-                const int eid = eb0 + lane;
-                int o = 0;
+            for (int eb0 = 0; eb0 < E; eb0 += 32 * SS_U) {
+                float nd[SS_U];
+                int32_t ou[SS_U], w[SS_U];
+                unsigned long long seen[SS_U];
 #pragma unroll
-                for (int st = 16; st > 0; st >>= 1) {
-                    const int ek = __shfl_sync(FULL, dexcl, o + st);
-                    if (ek <= eid) o += st;
+                for (int q = 0; q < SS_U; ++q) {
+                    const int eid = eb0 + 32 * q + lane;
+                    int o = 0;
+#pragma unroll
+                    for (int st = 16; st > 0; st >>= 1) {
+                        const int ek = __shfl_sync(FULL, dexcl, o + st);
+                        if (ek <= eid) o += st;
+                    }
+                    const int64_t ob = __shfl_sync(FULL, eb, o);
+                    const int oex = __shfl_sync(FULL, dexcl, o);
+                    ou[q] = __shfl_sync(FULL, u, o);
+                    nd[q] = __shfl_sync(FULL, du, o);
+                    w[q] = -1;
+                    if (eid < E) {
+                        const int64_t pos = ob + (eid - oex);
+                        w[q] = __ldcs(R.csr_idx + pos);
+                        nd[q] += R.csr_w ? __ldcs(R.csr_w + pos) : 1.f;
+                        ++c.examined;
+                    }
                 }
-                const int64_t ob = __shfl_sync(FULL, eb, o);
-                const int oex = __shfl_sync(FULL, dexcl, o);
-                const int32_t ou = __shfl_sync(FULL, u, o);
-                const float odu = __shfl_sync(FULL, du, o);
-                if (eid < E) {
-                    const int64_t pos = ob + (eid - oex);
-                    const int32_t w = __ldcs(R.csr_idx + pos);
-                    const float wt = R.csr_w ? __ldcs(R.csr_w + pos) : 1.f;
-                    ++c.examined;
-                    ss_offer(R, act_next, b, odu + wt, ou, w, c);
-                }
+#pragma unroll
+                for (int q = 0; q < SS_U; ++q) seen[q] = w[q] >= 0 ? R.key[w[q]] : 0ull;
+                ss_offers<SS_U>(R, act_next, end, nd, ou, w, seen, c);
             }
         }
     }
 }
 
-// Push, phase B: the queued chunks of heavy active vertices, one warp each.
-__device__ void ss_push_b(const SsRun &R, uint32_t *act_next, int64_t h_len, unsigned long long b, SsLocal &c) {
-    const int lane = lane_id();
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    constexpr int U = 4;  // relaxations in flight per lane
-    for (int64_t j = warp; j < h_len; j += nwarps) {
-        const Chunk ch = R.push_chunks[R.hq[j]];
-        const float du = ss_dist(R.key[ch.v]);
-        for (int i0 = lane; i0 < ch.len; i0 += 32 * U) {
-            int32_t w[U];
-            float wt[U];
-            unsigned long long seen[U];
-#pragma unroll
-            for (int q = 0; q < U; ++q) {
-                const int i = i0 + 32 * q;
-                w[q] = i < ch.len ? __ldcs(R.csr_idx + ch.beg + i) : -1;
-                wt[q] = i < ch.len && R.csr_w ? __ldcs(R.csr_w + ch.beg + i) : 1.f;
-            }
-#pragma unroll
-            for (int q = 0; q < U; ++q) seen[q] = w[q] >= 0 ? R.key[w[q]] : 0ull;
-#pragma unroll
-            for (int q = 0; q < U; ++q)
-                if (w[q] >= 0) {
-                    ++c.examined;
-                    ss_offer_seen(R, act_next, b, du + wt[q], ch.v, w[q], seen[q], c);
+// Push, phase B: the queued chunks of heavy active vertices, one to a warp, each
+// block's share by demand.  A window of 32 * SS_U edges is three dependent trips
+// to memory (indices, keys, offers); the next window's indices and keys are
+// loaded before the offers of this one.
+struct SsWindow {
+    int32_t u = -1;  // the window's source (-1: there is no window)
+    int32_t w[SS_U];
+    float nd[SS_U];
+};
+
+constexpr int SS_TAKE = 4;  // chunks a warp takes at a time, looked up together
+
+struct SsChunks {  // the warp's walk over its chunks
+    Chunk mine = {0, 0, -1};  // lane i: the i-th of those taken, with its source's distance
+    float mine_du = 0.f;
+    int which = SS_TAKE;
+    int64_t beg = 0;
+    int32_t v = -1, len = 0, at = 0;
+    float du = 0.f;
+    // the next window of the walk, indices and weights loaded
+    __device__ __forceinline__ void next(const SsRun &R, int64_t h_len, int *s_next, SsWindow &n, SsLocal &c) {
+        const int lane = lane_id();
+        n.u = -1;
+        if (at >= len) {
+            if (++which >= SS_TAKE) {
+                int i = 0;
+                if (lane == 0) i = atomicAdd(s_next, SS_TAKE);
+                i = __shfl_sync(FULL, i, 0);
+                const int64_t j = (int64_t)(i + lane) * gridDim.x + blockIdx.x;
+                mine.v = -1;
+                if (lane < SS_TAKE && j < h_len) {
+                    mine = R.push_chunks[R.hq[j]];
+                    mine_du = ss_dist(R.key[mine.v]);
                 }
+                which = 0;
+            }
+            v = __shfl_sync(FULL, mine.v, which);
+            if (v < 0) {
+                which = SS_TAKE;
+                len = at = 0;
+                return;
+            }
+            beg = __shfl_sync(FULL, mine.beg, which);
+            len = __shfl_sync(FULL, mine.len, which);
+            du = __shfl_sync(FULL, mine_du, which);
+            at = 0;
         }
+        n.u = v;
+#pragma unroll
+        for (int q = 0; q < SS_U; ++q) {
+            const int e = at + 32 * q + lane;
+            n.w[q] = e < len ? __ldcs(R.csr_idx + beg + e) : -1;
+            n.nd[q] = e < len && R.csr_w ? __ldcs(R.csr_w + beg + e) : 1.f;
+            c.examined += e < len;
+        }
+        at += 32 * SS_U;
+    }
+};
+
+__device__ void ss_push_b(const SsRun &R, uint32_t *act_next, int64_t h_len, float end, SsLocal &c) {
+    __shared__ int s_next;
+    if (threadIdx.x == 0) s_next = 0;
+    __syncthreads();
+    SsChunks walk;
+    SsWindow n;
+    walk.next(R, h_len, &s_next, n, c);
+    float du = walk.du;
+    while (n.u >= 0) {
+        float nd[SS_U];
+        int32_t u[SS_U], w[SS_U];
+        unsigned long long seen[SS_U];
+#pragma unroll
+        for (int q = 0; q < SS_U; ++q) {
+            u[q] = n.u;
+            w[q] = n.w[q];
+            nd[q] = du + n.nd[q];
+            seen[q] = w[q] >= 0 ? R.key[w[q]] : 0ull;
+        }
+        walk.next(R, h_len, &s_next, n, c);
+        du = walk.du;
+        ss_offers<SS_U>(R, act_next, end, nd, u, w, seen, c);
     }
 }
 
@@ -265,7 +384,7 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
 
 // Pull: heavy unsettled vertices by chunks (warp minimum, atomicMin into the
 // key), then the light unsettled vertices, one lane each over all in-edges.
-__device__ void ss_pull(const SsRun &R, const uint32_t *act_cur, uint32_t *act_next, unsigned long long b, SsLocal &c) {
+__device__ void ss_pull(const SsRun &R, const uint32_t *act_cur, uint32_t *act_next, float end, SsLocal &c) {
     const int lane = lane_id();
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -283,7 +402,7 @@ __device__ void ss_pull(const SsRun &R, const uint32_t *act_cur, uint32_t *act_n
             }
         }
         best = warp_min_u64(best);
-        if (lane == 0 && best != SS_NONE) ss_offer(R, act_next, b, ss_dist(best), (int32_t)(uint32_t)best, ch.v, c);
+        if (lane == 0 && best != SS_NONE) ss_offer(R, act_next, end, ss_dist(best), (int32_t)(uint32_t)best, ch.v, c);
     }
     const int64_t nwords = (R.n + 31) >> 5;
     for (int64_t base = warp * 32; base < nwords; base += nwarps * 32) {
@@ -323,12 +442,8 @@ __device__ void ss_pull(const SsRun &R, const uint32_t *act_cur, uint32_t *act_n
                 const float nd = ss_dist(best);
                 if (nd < ss_dist(own)) {
                     const uint32_t bit = 1u << (v & 31);
-                    if (ss_bucket(nd, R.delta) == b) {
-                        atomicOr(R.members + (v >> 5), bit);
-                        if (!(atomicOr(act_next + (v >> 5), bit) & bit)) {
-                            c.nact += 1;
-                            c.mact += (unsigned long long)(R.csr_off[v + 1] - R.csr_off[v]);
-                        }
+                    if (nd < end) {
+                        if (!(atomicOr(act_next + (v >> 5), bit) & bit)) ss_count_active(R, v, c);
                     } else if (!(atomicOr(R.pend + (v >> 5), bit) & bit)) {
                         c.npend += 1;
                     }
@@ -338,7 +453,26 @@ __device__ void ss_pull(const SsRun &R, const uint32_t *act_cur, uint32_t *act_n
     }
 }
 
+// Calls f(key of v, bit) for the vertices of the set bits of word i, four keys in flight.
+template <class F>
+__device__ __forceinline__ void ss_each_key(const SsRun &R, int64_t i, uint32_t word, F f) {
+    while (word) {
+        int bit[4];
+        unsigned long long k[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            bit[q] = word ? __ffs(word) - 1 : -1;
+            k[q] = word ? R.key[i * 32 + bit[q]] : 0ull;
+            word &= word - 1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (bit[q] >= 0) f(k[q], bit[q]);
+    }
+}
+
 __global__ void __launch_bounds__(SS_THREADS) k_sssp_persistent(SsRun R) {
+    __shared__ uint16_t s_queue[32 * SS_WORDS];  // active vertices of a pass: word of the pass, bit
     const unsigned long long t_start = ss_now();
     const int64_t n = R.n;
     const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -378,6 +512,8 @@ __global__ void __launch_bounds__(SS_THREADS) k_sssp_persistent(SsRun R) {
     int64_t it = 0, epochs = 1, examined = 0, pushes = 0, pulls = 0;
     read_ctr(0);
     unsigned long long nact = s_c[0], mact = s_c[1];
+    float end = ss_bucket_end(b, R.delta);
+    bool heavy = true;  // the active set may hold vertices above the light limit
     while (true) {
         if (nact == 0) {
             // epoch end: settle bucket b, find the smallest pending bucket above b
@@ -388,19 +524,19 @@ __global__ void __launch_bounds__(SS_THREADS) k_sssp_persistent(SsRun R) {
                 if (mw) {
                     R.unset[i] &= ~mw;
                     R.members[i] = 0u;
+#pragma unroll 4
                     for (uint32_t x = mw; x; x &= x - 1) {
                         const int64_t v = i * 32 + (__ffs(x) - 1);
                         settled_in += (unsigned long long)(R.csc_off[v + 1] - R.csc_off[v]);
                     }
                 }
-                for (uint32_t x = R.pend[i]; x; x &= x - 1) {
-                    const int64_t v = i * 32 + (__ffs(x) - 1);
-                    const unsigned long long bv = ss_bucket(ss_dist(R.key[v]), R.delta);
+                ss_each_key(R, i, R.pend[i], [&](unsigned long long key, int) {
+                    const unsigned long long bv = ss_bucket(ss_dist(key), R.delta);
                     if (bv > b) {
                         const unsigned long long kb = ~0ull - bv;
                         best = kb > best ? kb : best;
                     }
-                }
+                });
             }
             {
                 __shared__ unsigned long long sm[32];
@@ -433,30 +569,27 @@ __global__ void __launch_bounds__(SS_THREADS) k_sssp_persistent(SsRun R) {
                 const uint32_t pw = R.pend[i];
                 if (!pw) continue;
                 uint32_t moved = 0, stale = 0;
-                for (uint32_t x = pw; x; x &= x - 1) {
-                    const int bit = __ffs(x) - 1;
+                ss_each_key(R, i, pw, [&](unsigned long long key, int bit) {
                     const int64_t v = i * 32 + bit;
-                    const unsigned long long bv = ss_bucket(ss_dist(R.key[v]), R.delta);
+                    const unsigned long long bv = ss_bucket(ss_dist(key), R.delta);
                     if (bv == nb) {
                         moved |= 1u << bit;
-                        c.nact += 1;
-                        c.mact += (unsigned long long)(R.csr_off[v + 1] - R.csr_off[v]);
+                        ss_count_active(R, v, c);
                     } else if (bv <= b) {
                         stale |= 1u << bit;
                     }
-                }
+                });
                 R.pend[i] = pw & ~(moved | stale);
-                if (moved) {
-                    R.act[cur][i] |= moved;
-                    R.members[i] |= moved;
-                }
+                if (moved) R.act[cur][i] |= moved;
             }
             ss_flush(R.ctr + cur, c);
             if (!grid_sync(R.sync, gridDim.x)) return;
             read_ctr(cur);
             nact = s_c[0];
             mact = s_c[1];
+            heavy = s_c[7] != 0;
             b = nb;
+            end = ss_bucket_end(b, R.delta);
             ++epochs;
             continue;
         }
@@ -476,19 +609,23 @@ __global__ void __launch_bounds__(SS_THREADS) k_sssp_persistent(SsRun R) {
         const uint32_t *act_cur = R.act[cur];
         uint32_t *act_next = R.act[nxt];
         if (gthread < CW) ((unsigned long long *)(R.ctr + spare))[gthread] = 0;
-        for (int64_t i = gthread; i < nwords; i += nthreads) R.act[spare][i] = 0u;
+        // an epoch's members are the vertices that were active in its iterations
+        for (int64_t i = gthread; i < nwords; i += nthreads) {
+            R.act[spare][i] = 0u;
+            const uint32_t word = act_cur[i];
+            if (word) R.members[i] |= word;
+        }
         SsLocal c;
         if (dir == GP_PUSH) {
-            ss_push_a(R, act_cur, act_next, R.ctr + cur, b, c);
-            if (!grid_sync(R.sync, gridDim.x)) return;
-            read_ctr(cur);
-            const int64_t h_len = (int64_t)s_c[3];
-            if (h_len > 0) {
-                ss_push_b(R, act_next, h_len, b, c);
+            ss_push_a(R, act_cur, act_next, R.ctr + cur, end, s_queue, c);
+            if (heavy) {
+                if (!grid_sync(R.sync, gridDim.x)) return;
+                read_ctr(cur);
+                ss_push_b(R, act_next, (int64_t)s_c[3], end, c);
             }
             ++pushes;
         } else {
-            ss_pull(R, act_cur, act_next, b, c);
+            ss_pull(R, act_cur, act_next, end, c);
             ++pulls;
         }
         ss_flush(R.ctr + nxt, c);
@@ -506,6 +643,7 @@ __global__ void __launch_bounds__(SS_THREADS) k_sssp_persistent(SsRun R) {
         examined += (int64_t)s_c[4];
         nact = s_c[0];
         mact = s_c[1];
+        heavy = s_c[7] != 0;
         ++it;
     }
     // outputs
@@ -711,6 +849,7 @@ extern "C" int gp_sssp(const gp_graph *gc, int32_t src, float delta, int mode, c
     R.csc_idx = g->csc_idx;
     R.csr_w = g->csr_w;
     R.csc_w = g->csc_w;
+    R.push_light_max = g->push_bins.light_max;
     R.push_rank = g->push_bins.rank;
     R.push_cstart = g->push_bins.cstart;
     R.push_chunks = g->push_bins.chunks;
