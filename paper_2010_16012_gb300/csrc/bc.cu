@@ -49,6 +49,12 @@
 namespace gp {
 
 constexpr int BC_THREADS = 512;
+// Sources at a time, by the graph's edges.  Measured per source with 1, 4, 8 and
+// 16 groups: R-MAT 2^20 (31M edges) 480, 256, 243 and 277 us; uniform 300K
+// vertices (4.8M) 404, 124, 97 and 72; R-MAT 2^16 (1.8M) 247, 67, 42 and 32; 2^13
+// 211, 52, 28 and 17.
+constexpr int64_t BC_GROUPS = 16, BC_GROUPS_LARGE = 8, BC_LARGE = int64_t(1) << 24;
+constexpr int64_t BC_GROUP_BYTES = int64_t(4) << 30;  // memory for their workspaces (81 bytes per vertex each)
 constexpr int64_t BC_BATCH = 4096;  // sources per launch
 constexpr int BC_W = 4;             // 32-edge windows of a merged stream in flight per lane
 constexpr int BC_WL = 8;            // list entries in flight per lane (chunks, medium and light lists)
@@ -106,7 +112,6 @@ struct BcRun {
     BcCum *lev;          // [n + 2]
     BcCtr *ctr;          // [3]
     const int32_t *sources;
-    int64_t nsrc;
     int32_t mode, ndirs;
     const int8_t *dirs;
     float alpha;
@@ -114,6 +119,22 @@ struct BcRun {
     BcStepStat *stats;
     BcSummary *summary;
     GridSync *sync;
+    int32_t block0, blocks;  // the blocks that run the source: blockIdx block0 .. block0 + blocks - 1
+};
+
+// The sources of a launch: the grid is cut into groups of blocks, each with its
+// own workspace and barrier, that draw sources from a shared counter.  A
+// source's steps are latency more than work (half of its time went to steps of
+// a few microseconds' worth of edges, and in the others warps waited at the
+// barrier longer than for memory), so groups that share the SMs fill each
+// other's waits.
+constexpr int BC_MAX_GROUPS = (int)BC_GROUPS;
+struct BcMulti {
+    BcRun runs[BC_MAX_GROUPS];
+    int32_t groups, bpg;
+    int64_t nsrc;
+    unsigned long long *next;  // the next source to hand out (zero at launch)
+    long long *slot;           // [2 * groups]: the source a group's leader drew, by draw parity
 };
 
 struct BcLocal {  // per-thread contributions of a step
@@ -128,8 +149,13 @@ __device__ __forceinline__ unsigned long long bc_now() {
 
 __device__ __forceinline__ bool bit_of(const uint32_t *bits, int32_t v) { return (bits[v >> 5] >> (v & 31)) & 1u; }
 
-__device__ __forceinline__ int64_t warp_id_global() { return ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
-__device__ __forceinline__ int64_t warps_total() { return ((int64_t)gridDim.x * blockDim.x) >> 5; }
+// This thread and warp within the blocks that run the source, and their numbers.
+__device__ __forceinline__ int64_t group_thread(const BcRun &R) {
+    return (int64_t)((int)blockIdx.x - R.block0) * blockDim.x + threadIdx.x;
+}
+__device__ __forceinline__ int64_t group_threads(const BcRun &R) { return (int64_t)R.blocks * blockDim.x; }
+__device__ __forceinline__ int64_t group_warp(const BcRun &R) { return group_thread(R) >> 5; }
+__device__ __forceinline__ int64_t group_warps(const BcRun &R) { return group_threads(R) >> 5; }
 
 __device__ void bc_flush(BcCtr *nx, const BcLocal &c) {
     __shared__ unsigned long long sm[32];
@@ -266,8 +292,8 @@ __device__ __forceinline__ double group_gather(const int32_t *__restrict__ idx, 
 // The items [b, e) of a list, 32/G per warp at once: group g of the warp gets
 // item it or -1 (all lanes call work together).
 template <int G, class F>
-__device__ __forceinline__ void warp_groups_each(long long b, long long e, F work) {
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+__device__ __forceinline__ void warp_groups_each(const BcRun &R, long long b, long long e, F work) {
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     constexpr int NG = 32 / G;
     const int g = lane_id() / G;
     for (long long i0 = b + warp * NG; i0 < e; i0 += nwarps * NG) {
@@ -279,9 +305,9 @@ __device__ __forceinline__ void warp_groups_each(long long b, long long e, F wor
 // As warp_select_each, the selected items taken 32/G at a time, one per group
 // of G lanes (-1 for a group without one; all lanes call work together).
 template <int G, class P, class F>
-__device__ __forceinline__ void warp_select_groups(int64_t count, P pred, F work) {
+__device__ __forceinline__ void warp_select_groups(const BcRun &R, int64_t count, P pred, F work) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     constexpr int NG = 32 / G;
     const int g = lane / G;
     for (int64_t k0 = 0; warp + nwarps * k0 < count; k0 += 32) {
@@ -303,9 +329,9 @@ __device__ __forceinline__ void warp_select_groups(int64_t count, P pred, F work
 // pred (32 tests per load round, consecutive items on different warps); the
 // selected items are then taken one by one by the whole warp.
 template <class P, class F>
-__device__ __forceinline__ void warp_select_each(int64_t count, P pred, F work) {
+__device__ __forceinline__ void warp_select_each(const BcRun &R, int64_t count, P pred, F work) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     for (int64_t k0 = 0; warp + nwarps * k0 < count; k0 += 32) {
         const int64_t i = warp + nwarps * (k0 + lane);
         const bool sel = i < count && pred(i);
@@ -336,12 +362,12 @@ __device__ __forceinline__ void bc_visit(const BcRun &R, const int32_t *w, const
 
 __device__ void bc_fwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcCum &b, BcLocal &c) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     const int32_t l1 = l + 1;
     const uint32_t *fb = R.lbits[l & 3];
     uint32_t *nb = R.lbits[l1 & 3];
     // hubs of the frontier: every hub chunk whose vertex is in Q_l
-    warp_select_each(R.n_hub_out, [&](int64_t j) { return bit_of(fb, R.hub_out[j].v); }, [&](int64_t j) {
+    warp_select_each(R, R.n_hub_out, [&](int64_t j) { return bit_of(fb, R.hub_out[j].v); }, [&](int64_t j) {
         const Chunk ch = R.hub_out[j];
         double su[BC_WL];
         su[0] = R.sigma[ch.v];
@@ -353,7 +379,7 @@ __device__ void bc_fwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcC
     // medium lists: BC_G lanes per vertex when there are enough of them, else a warp each
     auto med_push = [&](auto gsz) {
         constexpr int G = decltype(gsz)::value;
-        warp_groups_each<G>(a.med_out, b.med_out, [&](long long i) {
+        warp_groups_each<G>(R, a.med_out, b.med_out, [&](long long i) {
             if (i < 0) return;
             const int32_t u = R.med_out[i];
             double su[BC_WL];
@@ -396,13 +422,13 @@ __device__ void bc_fwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcC
 
 __device__ void bc_fwd_pull(const BcRun &R, int32_t l, BcLocal &c) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     const int32_t l1 = l + 1;
     const uint32_t *fb = R.lbits[l & 3];
     uint32_t *nb = R.lbits[l1 & 3];
     // the candidate set (unvis) does not change during the step
     // hub in-lists by chunks, sums added atomically, claimed by CAS
-    warp_select_each(R.n_hub_in, [&](int64_t j) { return bit_of(R.unvis, R.hub_in[j].v); }, [&](int64_t j) {
+    warp_select_each(R, R.n_hub_in, [&](int64_t j) { return bit_of(R.unvis, R.hub_in[j].v); }, [&](int64_t j) {
         const Chunk ch = R.hub_in[j];
         const double s = list_gather(R.csc_idx, ch.beg, ch.beg + ch.len, fb, R.sigma);
         if (lane == 0) {
@@ -414,7 +440,7 @@ __device__ void bc_fwd_pull(const BcRun &R, int32_t l, BcLocal &c) {
         }
     });
     // medium in-lists: BC_G lanes per vertex
-    warp_select_groups<BC_G>(R.n_med_in_all, [&](int64_t i) { return bit_of(R.unvis, R.med_in_all[i]); }, [&](int64_t i) {
+    warp_select_groups<BC_G>(R, R.n_med_in_all, [&](int64_t i) { return bit_of(R.unvis, R.med_in_all[i]); }, [&](int64_t i) {
         const int32_t v = i >= 0 ? R.med_in_all[i] : 0;
         const int64_t eb = i >= 0 ? R.csc_off[v] : 0, ee = i >= 0 ? R.csc_off[v + 1] : 0;
         const double s = group_gather<BC_G>(R.csc_idx, eb, ee, fb, R.sigma);
@@ -429,7 +455,7 @@ __device__ void bc_fwd_pull(const BcRun &R, int32_t l, BcLocal &c) {
     });
     // light in-lists: one candidate word (32 vertices) at a time per warp, as one stream
     const int64_t nwords = (R.n + 31) >> 5;
-    warp_select_each(nwords, [&](int64_t wd) { return R.unvis[wd] != 0u; }, [&](int64_t wd) {
+    warp_select_each(R, nwords, [&](int64_t wd) { return R.unvis[wd] != 0u; }, [&](int64_t wd) {
         const uint32_t word = R.unvis[wd];
         const int32_t v = (int32_t)(wd * 32 + lane);
         int deg = 0;
@@ -456,7 +482,7 @@ __device__ void bc_fwd_pull(const BcRun &R, int32_t l, BcLocal &c) {
 // warp and 32 words), take them out of the pull candidates and count degrees.
 __device__ void bc_compact(const BcRun &R, const uint32_t *bits, BcCtr *nx, const BcCum &cur, BcLocal &c) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     const int64_t nwords = (R.n + 31) >> 5;
     for (int64_t base = warp * 32; base < nwords; base += nwarps * 32) {
         const int64_t wd = base + lane;
@@ -503,7 +529,7 @@ __device__ void bc_compact(const BcRun &R, const uint32_t *bits, BcCtr *nx, cons
 __device__ void bc_bwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcCum &b, bool scatter, bool store_coef,
                             double *acc, BcLocal &c) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     const uint32_t *qb = R.lbits[l & 3];        // Q_l
     const uint32_t *pb = R.lbits[(l - 1) & 3];  // Q_{l-1}
     // N entries u[q] of the encoded CSC (-1: none) receive cw[q] when in Q_{l-1}
@@ -527,7 +553,7 @@ __device__ void bc_bwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcC
     if (scatter) {
         for (int i = threadIdx.x; i < R.nhot; i += blockDim.x) acc[i] = 0.0;
         __syncthreads();
-        warp_select_each(R.n_hub_in, [&](int64_t j) { return bit_of(qb, R.hub_in[j].v); }, [&](int64_t j) {
+        warp_select_each(R, R.n_hub_in, [&](int64_t j) { return bit_of(qb, R.hub_in[j].v); }, [&](int64_t j) {
             const Chunk ch = R.hub_in[j];
             double cw[BC_WL];
             cw[0] = 1.0 / R.sigma[ch.v] + R.S[ch.v];
@@ -539,7 +565,7 @@ __device__ void bc_bwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcC
         });
         auto med_scatter = [&](auto gsz) {
             constexpr int G = decltype(gsz)::value;
-            warp_groups_each<G>(a.med_in, b.med_in, [&](long long i) {
+            warp_groups_each<G>(R, a.med_in, b.med_in, [&](long long i) {
                 if (i < 0) return;
                 const int32_t w = R.med_in[i];
                 double cw[BC_WL];
@@ -566,7 +592,7 @@ __device__ void bc_bwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcC
             const int32_t w = R.order[qi];
             const double sg = R.sigma[w], sw = R.S[w];
             cw = 1.0 / sg + sw;
-            R.bc[w] += sg * sw;
+            atomicAdd(R.bc + w, sg * sw);  // (other groups add for their sources)
             if (store_coef) R.coef[w] = cw;
             eb = R.csc_off[w];
             const int64_t d = R.csc_off[w + 1] - eb;
@@ -592,10 +618,10 @@ __device__ void bc_bwd_push(const BcRun &R, int32_t l, const BcCum &a, const BcC
 // out-neighbours in Q_l.
 __device__ void bc_bwd_pull(const BcRun &R, int32_t l, const BcCum &p, const BcCum &a, BcLocal &c) {
     const int lane = lane_id();
-    const int64_t warp = warp_id_global(), nwarps = warps_total();
+    const int64_t warp = group_warp(R), nwarps = group_warps(R);
     const uint32_t *qb = R.lbits[l & 3];        // Q_l
     const uint32_t *pb = R.lbits[(l - 1) & 3];  // Q_{l-1}
-    warp_select_each(R.n_hub_out, [&](int64_t j) { return bit_of(pb, R.hub_out[j].v); }, [&](int64_t j) {
+    warp_select_each(R, R.n_hub_out, [&](int64_t j) { return bit_of(pb, R.hub_out[j].v); }, [&](int64_t j) {
         const Chunk ch = R.hub_out[j];
         const double s = list_gather(R.csr_idx, ch.beg, ch.beg + ch.len, qb, R.coef);
         if (lane == 0) {
@@ -605,7 +631,7 @@ __device__ void bc_bwd_pull(const BcRun &R, int32_t l, const BcCum &p, const BcC
     });
     auto med_gather = [&](auto gsz) {
         constexpr int G = decltype(gsz)::value;
-        warp_groups_each<G>(p.med_out, a.med_out, [&](long long i) {
+        warp_groups_each<G>(R, p.med_out, a.med_out, [&](long long i) {
             const int32_t u = i >= 0 ? R.med_out[i] : 0;
             const int64_t eb = i >= 0 ? R.csr_off[u] : 0, ee = i >= 0 ? R.csr_off[u + 1] : 0;
             const double s = group_gather<G>(R.csr_idx, eb, ee, qb, R.coef);
@@ -639,17 +665,15 @@ __device__ void bc_bwd_pull(const BcRun &R, int32_t l, const BcCum &p, const BcC
 
 // Set the bits of order[b, e) in `bits` (one level's bitmap, from its vertex range).
 __device__ __forceinline__ void bc_mark(const BcRun &R, long long b, long long e, uint32_t *bits) {
-    const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+    const int64_t gthread = group_thread(R), nthreads = group_threads(R);
     for (long long i = b + gthread; i < e; i += nthreads) {
         const int32_t v = R.order[i];
         atomicOr(bits + (v >> 5), 1u << (v & 31));
     }
 }
 
-__device__ __forceinline__ void bc_clear(uint32_t *bits, int64_t nwords) {
-    const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+__device__ __forceinline__ void bc_clear(const BcRun &R, uint32_t *bits, int64_t nwords) {
+    const int64_t gthread = group_thread(R), nthreads = group_threads(R);
     for (int64_t i = gthread; i < nwords; i += nthreads) bits[i] = 0u;
 }
 
@@ -663,9 +687,11 @@ __device__ __forceinline__ BcCum bc_load_lev(const BcCum *p) {
     return a;
 }
 
-__global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(BcRun R) {
-    const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
+__global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(const __grid_constant__ BcMulti M) {
+    const int grp = blockIdx.x / M.bpg;
+    if (grp >= M.groups) return;
+    const BcRun &R = M.runs[grp];
+    const int64_t gthread = group_thread(R), nthreads = group_threads(R);
     const int64_t nwords = (R.n + 31) >> 5;
     constexpr int CW = (int)(sizeof(BcCtr) / sizeof(unsigned long long));
     __shared__ unsigned long long s_c[CW];
@@ -678,17 +704,24 @@ __global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(BcRun R) {
         R.unvis[i] = R.nzin[i];
         for (int q = 0; q < 4; ++q) R.lbits[q][i] = 0u;
     }
-    if (!grid_sync(R.sync, gridDim.x)) return;
     int64_t levels = 0, reached = 0, examined = 0, pushes = 0, pulls = 0;
-    for (int64_t k = 0; k < R.nsrc; ++k) {
+    for (int draw = 0;; ++draw) {
+        // the leader draws a source and the group's barrier publishes it; the same
+        // barrier ends the previous source's reset in every block.  Two slots by
+        // turns: one is rewritten only after every block has read it
+        long long *slot = M.slot + 2 * grp + (draw & 1);
+        if (gthread == 0) *slot = (long long)atomicAdd(M.next, 1ull);
+        if (!grid_sync(R.sync, R.blocks)) return;
+        const int64_t k = *(volatile long long *)slot;
+        if (k >= M.nsrc) break;
         const int32_t src = R.sources[k];
-        if (src < 0 || (int64_t)src >= R.n) {  // every block reads the same source: all return here
+        if (src < 0 || (int64_t)src >= R.n) {  // every block of the group reads the same source: all return here
             if (gthread == 0) atomicExch(&R.sync->err, 3);
             return;
         }
         const bool rec = R.record && k == 0;
         // the source: level 0, one path; its record goes to ctr[0], the others start at zero
-        if (blockIdx.x == 0) {
+        if (gthread < blockDim.x) {
             const int64_t dout = R.csr_off[src + 1] - R.csr_off[src], din = R.csc_off[src + 1] - R.csc_off[src];
             const bool mo = dout > BC_LIGHT && dout <= BC_HUB, mi = din > BC_LIGHT && din <= BC_HUB;
             if (threadIdx.x < 3 * CW) {
@@ -710,7 +743,7 @@ __global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(BcRun R) {
                 R.lbits[0][src >> 5] |= 1u << (src & 31);
             }
         }
-        if (!grid_sync(R.sync, gridDim.x)) return;
+        if (!grid_sync(R.sync, R.blocks)) return;
         read_ctr(0);
         BcCum prev = {0, 0, 0, 0, 0};
         BcCum cur = {(long long)s_c[0], (long long)s_c[1], (long long)s_c[2], (long long)s_c[3], (long long)s_c[4]};
@@ -751,16 +784,16 @@ __global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(BcRun R) {
             const int dir = decide((double)mf * R.alpha > (double)(mu > 0 ? mu : 0));
             BcCtr *nx = R.ctr + (t + 1) % 3;
             if (gthread < CW) ((unsigned long long *)(R.ctr + (t + 2) % 3))[gthread] = 0;
-            bc_clear(R.lbits[(l + 2) & 3], nwords);  // Q_{l-2}: no longer read
+            bc_clear(R, R.lbits[(l + 2) & 3], nwords);  // Q_{l-2}: no longer read
             BcLocal c;
             if (dir == GP_PUSH)
                 bc_fwd_push(R, l, prev, cur, c);
             else
                 bc_fwd_pull(R, l, c);
-            if (!grid_sync(R.sync, gridDim.x)) return;
+            if (!grid_sync(R.sync, R.blocks)) return;
             bc_compact(R, R.lbits[(l + 1) & 3], nx, cur, c);
             bc_flush(nx, c);
-            if (!grid_sync(R.sync, gridDim.x)) return;
+            if (!grid_sync(R.sync, R.blocks)) return;
             read_ctr((int)((t + 1) % 3));
             const BcCum nxt = {cur.start + (long long)s_c[0], cur.med_out + (long long)s_c[1],
                                cur.med_in + (long long)s_c[2], cur.in + (long long)s_c[3], cur.out + (long long)s_c[4]};
@@ -781,18 +814,18 @@ __global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(BcRun R) {
             BcCtr *nx = R.ctr + (t + 1) % 3;
             if (gthread < CW) ((unsigned long long *)(R.ctr + (t + 2) % 3))[gthread] = 0;
             // one step ahead: Q_{lb-2}'s bitmap into the slot cleared last step; Q_{lb+1}'s cleared
-            bc_clear(R.lbits[(lb + 1) & 3], nwords);
+            bc_clear(R, R.lbits[(lb + 1) & 3], nwords);
             if (lb >= 2) bc_mark(R, bc_load_lev(R.lev + lb - 2).start, p.start, R.lbits[(lb - 2) & 3]);
             BcLocal c;
             if (dir == GP_PUSH) {
                 bc_bwd_push(R, lb, a, b, true, false, s_acc, c);
             } else {
                 bc_bwd_push(R, lb, a, b, false, true, s_acc, c);
-                if (!grid_sync(R.sync, gridDim.x)) return;
+                if (!grid_sync(R.sync, R.blocks)) return;
                 bc_bwd_pull(R, lb, p, a, c);
             }
             bc_flush(nx, c);
-            if (!grid_sync(R.sync, gridDim.x)) return;
+            if (!grid_sync(R.sync, R.blocks)) return;
             read_ctr((int)((t + 1) % 3));
             end_step(dir, 1, lb, b.start - a.start, s_c[5]);
         }
@@ -808,14 +841,14 @@ __global__ void __launch_bounds__(BC_THREADS, 2) k_bc_persistent(BcRun R) {
             R.unvis[i] = R.nzin[i];
             for (int q = 0; q < 4; ++q) R.lbits[q][i] = 0u;
         }
-        if (!grid_sync(R.sync, gridDim.x)) return;
     }
     if (gthread == 0) {
-        R.summary->levels = levels;
-        R.summary->reached = reached;
-        R.summary->examined = examined;
-        R.summary->pushes = pushes;
-        R.summary->pulls = pulls;
+        auto add = [](int64_t *to, int64_t x) { atomicAdd((unsigned long long *)to, (unsigned long long)x); };
+        add(&R.summary->levels, levels);
+        add(&R.summary->reached, reached);
+        add(&R.summary->examined, examined);
+        add(&R.summary->pushes, pushes);
+        add(&R.summary->pulls, pulls);
     }
 }
 
@@ -840,16 +873,22 @@ using namespace gp;
 
 struct gp_bc_work {
     bool ready = false;
-    int32_t *dist = nullptr, *order = nullptr, *med_out = nullptr, *med_in = nullptr;
+    struct Group {  // what one source's search needs
+        int32_t *dist = nullptr, *order = nullptr, *med_out = nullptr, *med_in = nullptr;
+        double *sigma = nullptr, *S = nullptr, *coef = nullptr;
+        uint32_t *unvis = nullptr, *lbits[4] = {nullptr, nullptr, nullptr, nullptr};
+        BcCum *lev = nullptr;
+        BcCtr *ctr = nullptr;
+    };
+    std::vector<Group> groups;  // as many as the calls so far could use
+    bool dirty = true;          // their per-vertex state may not be clean (at first, and after an aborted launch)
+    unsigned long long *next = nullptr;  // the draw counter, then two slots per group
     int32_t *med_in_all = nullptr;  // every vertex with a medium in-list
     int64_t n_med_in_all = 0;
     BigBins hub_out, hub_in;  // lists above BC_HUB cut into BC_CHUNK-edge chunks
     HotSet hot;               // the BC_HOT largest out-degrees, CSC encoded
-    double *sigma = nullptr, *S = nullptr, *coef = nullptr, *bc = nullptr;
-    uint32_t *unvis = nullptr, *nzin = nullptr;
-    uint32_t *lbits[4] = {nullptr, nullptr, nullptr, nullptr};
-    BcCum *lev = nullptr;
-    BcCtr *ctr = nullptr;
+    double *bc = nullptr;
+    uint32_t *nzin = nullptr;
     BcStepStat *stats = nullptr;
     BcSummary *summary = nullptr;  // [one per launch of a call, up to BC_MAX_LAUNCH_SUMMARIES]
     GridSync *sync = nullptr;
@@ -866,7 +905,7 @@ struct gp_bc_work {
 namespace gp {
 
 // host mirror: summary, per-step statistics, barrier status
-constexpr size_t BC_HOST_BYTES = sizeof(BcSummary) + GP_BC_MAX_STEPS * sizeof(BcStepStat) + sizeof(GridSync);
+constexpr size_t BC_HOST_BYTES = sizeof(BcSummary) + GP_BC_MAX_STEPS * sizeof(BcStepStat) + BC_MAX_GROUPS * sizeof(GridSync);
 
 void release_bc_work(gp_graph *g, cudaStream_t s) {
     if (!g->bc) return;
@@ -892,26 +931,16 @@ static int ensure_bc_work(gp_graph *g, cudaStream_t s) {
     if (w.ready) return GP_OK;
     const size_t n = (size_t)std::max<int64_t>(g->n, 1);
     const size_t words = (n + 31) / 32;
-    GP_TRY(w.mem.alloc(w.dist, n, s));
-    GP_TRY(w.mem.alloc(w.order, n, s));
-    GP_TRY(w.mem.alloc(w.med_out, n, s));
-    GP_TRY(w.mem.alloc(w.med_in, n, s));
     GP_TRY(build_bins(g, w.hub_out, g->csr_off, BC_HUB, BC_CHUNK, s));
     GP_TRY(build_bins(g, w.hub_in, g->csc_off, BC_HUB, BC_CHUNK, s));
     GP_TRY(build_hot(g, w.hot, BC_HOT, g->csr_off, g->csc_idx, INT32_MAX, s));
     GP_TRY(select_by_degree(g->csc_off, g->n, BC_LIGHT + 1, BC_HUB, w.mem, w.med_in_all, w.n_med_in_all, INT64_MAX,
                             nullptr, s));
-    GP_TRY(w.mem.alloc(w.sigma, n, s));
-    GP_TRY(w.mem.alloc(w.S, n, s));
-    GP_TRY(w.mem.alloc(w.coef, n, s));
-    GP_TRY(w.mem.alloc(w.unvis, words, s));
     GP_TRY(w.mem.alloc(w.nzin, words, s));
-    for (int q = 0; q < 4; ++q) GP_TRY(w.mem.alloc(w.lbits[q], words, s));
-    GP_TRY(w.mem.alloc(w.lev, n + 2, s));
-    GP_TRY(w.mem.alloc(w.ctr, 3, s));
+    GP_TRY(w.mem.alloc(w.next, 1 + 2 * BC_MAX_GROUPS, s));
     GP_TRY(w.mem.alloc(w.stats, GP_BC_MAX_STEPS, s));
     GP_TRY(w.mem.alloc(w.summary, 1, s));
-    GP_TRY(w.mem.alloc(w.sync, 1, s));
+    GP_TRY(w.mem.alloc(w.sync, BC_MAX_GROUPS, s));
     GP_TRY(w.mem.alloc(w.dirs, GP_BC_MAX_STEPS, s));
     if (g->n > 0) {
         k_bc_nzin<<<(int)std::min<size_t>((words + 255) / 256, 4096), 256, 0, s>>>(g->n, g->csc_off, w.nzin);
@@ -927,10 +956,53 @@ static int ensure_bc_work(gp_graph *g, cudaStream_t s) {
     return GP_OK;
 }
 
+// Workspaces for up to `want` groups, within the memory set aside for them; one
+// at least (GP_ERR_OOM where not even that is to be had).
+static int ensure_bc_groups(gp_graph *g, int want, cudaStream_t s) {
+    gp_bc_work &w = *g->bc;
+    const size_t n = (size_t)std::max<int64_t>(g->n, 1), words = (n + 31) / 32;
+    const int64_t fit = BC_GROUP_BYTES / (int64_t)(80 * n + 20 * words);
+    want = (int)std::max<int64_t>(1, std::min<int64_t>(want, fit));
+    while ((int)w.groups.size() < want) {
+        gp_bc_work::Group q;
+        Arena mem;
+        int st = mem.alloc(q.dist, n, s);
+        if (st == GP_OK) st = mem.alloc(q.order, n, s);
+        if (st == GP_OK) st = mem.alloc(q.med_out, n, s);
+        if (st == GP_OK) st = mem.alloc(q.med_in, n, s);
+        if (st == GP_OK) st = mem.alloc(q.sigma, n, s);
+        if (st == GP_OK) st = mem.alloc(q.S, n, s);
+        if (st == GP_OK) st = mem.alloc(q.coef, n, s);
+        if (st == GP_OK) st = mem.alloc(q.unvis, words, s);
+        for (int i = 0; i < 4 && st == GP_OK; ++i) st = mem.alloc(q.lbits[i], words, s);
+        if (st == GP_OK) st = mem.alloc(q.lev, n + 2, s);
+        if (st == GP_OK) st = mem.alloc(q.ctr, 3, s);
+        if (st != GP_OK) {
+            mem.release(s);
+            if (st != GP_ERR_OOM || w.groups.empty()) return st;
+            clear_error();  // the groups there are will do
+            break;
+        }
+        for (auto &b : mem.bufs) w.mem.bufs.push_back(b);
+        w.mem.total += mem.total;
+        w.groups.push_back(q);
+        w.dirty = true;
+    }
+    return GP_OK;
+}
+
 static int bc_barrier_status(int err, const char *when) {
     if (err == 3) return set_error(GP_ERR_INVALID, "gp_bc: a source outside [0, n)%s", when);
     if (err) return set_error(GP_ERR_TIMEOUT, "gp_bc: a grid barrier wait ran out%s", when);
     return GP_OK;
+}
+
+// The first error of a launch's groups (a bad source before a wait that ran out).
+static int bc_error(const GridSync *sync, int groups) {
+    int err = 0;
+    for (int q = 0; q < groups; ++q)
+        if (sync[q].err && err != 3) err = sync[q].err;
+    return err;
 }
 
 extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsources, int mode, const int8_t *dirs,
@@ -961,8 +1033,8 @@ extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsource
     if (w.pending) {  // the barrier status of the previous, asynchronous call
         GP_CUDA(cudaEventSynchronize(w.done_ev));
         w.pending = false;
-        const int err = hsync->err;
-        hsync->err = 0;
+        const int err = bc_error(hsync, BC_MAX_GROUPS);
+        w.dirty = w.dirty || err;
         GP_TRY(bc_barrier_status(err, " in the previous asynchronous call"));
     }
     if (stats) memset(stats, 0, sizeof(*stats));
@@ -988,12 +1060,19 @@ extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsource
         GP_CUDA(cudaEventCreate(&ev1));
         GP_CUDA(cudaEventRecord(ev0, s));
     }
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>(nsources, g->m > BC_LARGE ? BC_GROUPS_LARGE : BC_GROUPS));
+    GP_TRY(ensure_bc_groups(g, (int)most, s));
+    const int groups = (int)std::min<int64_t>(most, (int64_t)w.groups.size());
     if (n > 0) {
         GP_CUDA(cudaMemsetAsync(bc, 0, (size_t)n * sizeof(double), s));
-        // clean per-vertex state: every launch leaves it so, this covers an aborted one
-        GP_CUDA(cudaMemsetAsync(w.dist, 0xff, (size_t)n * sizeof(int32_t), s));
-        GP_CUDA(cudaMemsetAsync(w.sigma, 0, (size_t)n * sizeof(double), s));
-        GP_CUDA(cudaMemsetAsync(w.S, 0, (size_t)n * sizeof(double), s));
+        if (w.dirty) {  // clean per-vertex state: every launch that runs to its end leaves it so
+            for (const auto &q : w.groups) {
+                GP_CUDA(cudaMemsetAsync(q.dist, 0xff, (size_t)n * sizeof(int32_t), s));
+                GP_CUDA(cudaMemsetAsync(q.sigma, 0, (size_t)n * sizeof(double), s));
+                GP_CUDA(cudaMemsetAsync(q.S, 0, (size_t)n * sizeof(double), s));
+            }
+            w.dirty = false;
+        }
     }
     BcRun R;
     memset(&R, 0, sizeof(R));
@@ -1008,23 +1087,12 @@ extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsource
     R.nhot = (int32_t)w.hot.nhot;
     R.med_in_all = w.med_in_all;
     R.n_med_in_all = w.n_med_in_all;
-    R.med_out = w.med_out;
-    R.med_in = w.med_in;
     R.hub_out = w.hub_out.chunks;
     R.hub_in = w.hub_in.chunks;
     R.n_hub_out = w.hub_out.nchunks;
     R.n_hub_in = w.hub_in.nchunks;
-    R.dist = w.dist;
-    R.sigma = w.sigma;
-    R.S = w.S;
-    R.coef = w.coef;
     R.bc = bc;
-    R.order = w.order;
-    R.unvis = w.unvis;
     R.nzin = w.nzin;
-    for (int q = 0; q < 4; ++q) R.lbits[q] = w.lbits[q];
-    R.lev = w.lev;
-    R.ctr = w.ctr;
     R.mode = mode;
     R.alpha = g->opt.bc_alpha;
     R.stats = w.stats;
@@ -1036,27 +1104,53 @@ extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsource
         R.dirs = w.dirs;
         R.ndirs = nd;
     }
-    GP_CUDA(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), s));
+    GP_CUDA(cudaMemsetAsync(w.sync, 0, BC_MAX_GROUPS * sizeof(GridSync), s));
+    BcMulti M;
+    memset(&M, 0, sizeof(M));
+    M.groups = groups;
+    M.bpg = w.grid / groups;
+    M.next = w.next;
+    M.slot = (long long *)(w.next + 1);
     BcSummary total;
     memset(&total, 0, sizeof(total));
     const bool wait = stats || !out_dev || (nsources > 0 && !src_dev);
     for (int64_t k0 = 0; k0 < nsources && n > 0; k0 += BC_BATCH) {
         R.sources = src + k0;
-        R.nsrc = std::min<int64_t>(BC_BATCH, nsources - k0);
         R.record = stats && k0 == 0;
+        M.nsrc = std::min<int64_t>(BC_BATCH, nsources - k0);
+        for (int q = 0; q < groups; ++q) {
+            const gp_bc_work::Group &wq = w.groups[(size_t)q];
+            BcRun &r = M.runs[q];
+            r = R;
+            r.dist = wq.dist;
+            r.order = wq.order;
+            r.med_out = wq.med_out;
+            r.med_in = wq.med_in;
+            r.sigma = wq.sigma;
+            r.S = wq.S;
+            r.coef = wq.coef;
+            r.unvis = wq.unvis;
+            for (int i = 0; i < 4; ++i) r.lbits[i] = wq.lbits[i];
+            r.lev = wq.lev;
+            r.ctr = wq.ctr;
+            r.sync = w.sync + q;
+            r.block0 = q * M.bpg;
+            r.blocks = M.bpg;
+        }
+        GP_CUDA(cudaMemsetAsync(w.next, 0, sizeof(*w.next), s));
         GP_CUDA(cudaMemsetAsync(w.summary, 0, sizeof(BcSummary), s));
         {
             ProfScope ps("bc_persistent", s);
-            void *args[] = {&R};
+            void *args[] = {&M};
             GP_CUDA(cudaLaunchCooperativeKernel((const void *)k_bc_persistent, dim3((unsigned)w.grid),
                                                 dim3(BC_THREADS), args, 0, s));
         }
         if (stats) {  // per-launch summaries are summed on the host
             GP_CUDA(cudaMemcpyAsync(hs, w.summary, sizeof(BcSummary), cudaMemcpyDeviceToHost, s));
             if (k0 == 0) GP_CUDA(cudaMemcpyAsync(hl, w.stats, GP_BC_MAX_STEPS * sizeof(BcStepStat), cudaMemcpyDeviceToHost, s));
-            GP_CUDA(cudaMemcpyAsync(hsync, w.sync, sizeof(GridSync), cudaMemcpyDeviceToHost, s));
+            GP_CUDA(cudaMemcpyAsync(hsync, w.sync, groups * sizeof(GridSync), cudaMemcpyDeviceToHost, s));
             GP_CUDA(cudaStreamSynchronize(s));
-            if (hsync->err) break;
+            if (bc_error(hsync, groups)) break;
             if (k0 == 0) total.steps = hs->steps;
             total.levels += hs->levels;
             total.reached += hs->reached;
@@ -1066,7 +1160,7 @@ extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsource
         }
     }
     if (!out_dev && n > 0) GP_CUDA(cudaMemcpyAsync(bc_out, bc, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, s));
-    GP_CUDA(cudaMemcpyAsync(hsync, w.sync, sizeof(GridSync), cudaMemcpyDeviceToHost, s));
+    GP_CUDA(cudaMemcpyAsync(hsync, w.sync, BC_MAX_GROUPS * sizeof(GridSync), cudaMemcpyDeviceToHost, s));
     if (!wait) {
         // nothing for the host to read: return without waiting; the barrier
         // status is checked by the next call on this graph
@@ -1076,8 +1170,8 @@ extern "C" int gp_bc(const gp_graph *gc, const int32_t *sources, int64_t nsource
     }
     if (stats) GP_CUDA(cudaEventRecord(ev1, s));
     GP_CUDA(cudaStreamSynchronize(s));
-    const int err = hsync->err;
-    hsync->err = 0;
+    const int err = bc_error(hsync, BC_MAX_GROUPS);
+    w.dirty = w.dirty || err;
     if (stats) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, ev0, ev1);
