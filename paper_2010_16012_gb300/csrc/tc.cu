@@ -150,6 +150,8 @@ struct TcPlanStat {
     unsigned long long general;  // the graph is outside the contract
     unsigned long long max_out;
     unsigned long long probes;   // sum over ordered edges of the shorter list's length
+    unsigned long long out, in;  // lengths of the two kinds of list, all vertices
+    unsigned long long light, heavy, mid, wide;  // vertices by out-neighbours and by in-list (see TcRun, k_tc_gather)
 };
 
 // v before w: lower degree, or equal and lower id.
@@ -157,12 +159,16 @@ __device__ __forceinline__ bool tc_before(int64_t dv, int32_t v, int64_t dw, int
     return dv < dw || (dv == dw && v < w);
 }
 
+// In-lists of over TC_WIDE entries take a block each in the pull's gather, of over 32 a warp.
+constexpr int TC_WIDE = 1024;
+
 // Per vertex, the neighbours after it (out) and before it (in), a warp per vertex.
 __global__ void __launch_bounds__(256) k_tc_count(int64_t n, const int64_t *off, const int32_t *idx, int64_t *nout,
                                                   int64_t *nin, TcPlanStat *st) {
     const int lane = lane_id();
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long probes = 0, most = 0;
+    unsigned long long probes = 0, most = 0, outs = 0, ins = 0;
+    unsigned kind[4] = {0, 0, 0, 0};
     bool bad = false;
     for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nwarps) {
         const int64_t b = off[v], e = off[v + 1];
@@ -191,6 +197,12 @@ __global__ void __launch_bounds__(256) k_tc_count(int64_t n, const int64_t *off,
         out = warp_sum(out);
         in = warp_sum(in);
         most = max(most, (unsigned long long)out);
+        outs += (unsigned)out;
+        ins += (unsigned)in;
+        kind[0] += out >= 2 && out <= TC_WARP_OUT;
+        kind[1] += out > TC_WARP_OUT;
+        kind[2] += in > 32 && in <= TC_WIDE;
+        kind[3] += in > TC_WIDE;
         if (lane == 0) {
             nout[v] = out;
             nin[v] = in;
@@ -202,6 +214,33 @@ __global__ void __launch_bounds__(256) k_tc_count(int64_t n, const int64_t *off,
         if (probes) atomicAdd(&st->probes, probes);
         if (most) atomicMax(&st->max_out, most);
         if (bad) atomicOr(&st->general, 1ull);
+        if (outs) atomicAdd(&st->out, outs);
+        if (ins) atomicAdd(&st->in, ins);
+        if (kind[0]) atomicAdd(&st->light, (unsigned long long)kind[0]);
+        if (kind[1]) atomicAdd(&st->heavy, (unsigned long long)kind[1]);
+        if (kind[2]) atomicAdd(&st->mid, (unsigned long long)kind[2]);
+        if (kind[3]) atomicAdd(&st->wide, (unsigned long long)kind[3]);
+    }
+}
+
+// The lists of vertices by kind, in any order (at[] counts them).
+__global__ void k_tc_kinds(int64_t n, const int64_t *out_off, const int64_t *in_off, int32_t *light, int32_t *heavy,
+                           int32_t *mid, int32_t *wide, unsigned long long *at) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~int64_t(31); v0 < n; v0 += stride) {
+        const int64_t v = v0 + lane_id();
+        const int64_t out = v < n ? out_off[v + 1] - out_off[v] : 0, in = v < n ? in_off[v + 1] - in_off[v] : 0;
+        const bool is[4] = {out >= 2 && out <= TC_WARP_OUT, out > TC_WARP_OUT, in > 32 && in <= TC_WIDE, in > TC_WIDE};
+        int32_t *list[4] = {light, heavy, mid, wide};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned m = __ballot_sync(FULL, is[k]);
+            if (!m) continue;
+            unsigned long long p = 0;
+            if (lane_id() == __ffs(m) - 1) p = atomicAdd(at + k, (unsigned long long)__popc(m));
+            p = __shfl_sync(FULL, p, __ffs(m) - 1);
+            if (is[k]) list[k][p + __popc(m & ((1u << lane_id()) - 1u))] = (int32_t)v;
+        }
     }
 }
 
@@ -524,9 +563,8 @@ __global__ void __launch_bounds__(TC_WARPS * 32) k_tc_block(TcRun R) {
 }
 
 // pull: a vertex's count is its own triangles and those its in-neighbours
-// counted for it.  In-lists of over TC_WIDE entries take a block each (a warp
-// over 25K entries took 0.5 ms), of over 32 a warp, the others a thread.
-constexpr int TC_WIDE = 1024;
+// counted for it.  Long in-lists take a block each (a warp over 25K entries took
+// 0.5 ms), shorter ones a warp, the others a thread.
 __global__ void __launch_bounds__(256) k_tc_gather(int64_t n, const int64_t *in_off, const int32_t *slots,
                                                    const unsigned long long *own, const int32_t *mid, int64_t nmid,
                                                    const int32_t *wide, int64_t nwide, unsigned long long *tc) {
@@ -566,6 +604,7 @@ using namespace gp;
 
 struct gp_tc_work {
     bool ready = false, general = false;
+    TcPlanStat *fresh = nullptr;  // after the layout, until the first call has read it
     int64_t *out_off = nullptr, *in_off = nullptr;
     int32_t *out = nullptr, *rev = nullptr, *slots = nullptr;
     unsigned long long *own = nullptr;
@@ -592,62 +631,62 @@ static int build_tc(gp_graph *g, gp_tc_work &w, cudaStream_t s) {
     if (w.ready) return GP_OK;
     const int64_t n = g->n;
     Arena tmp;
-    TcPlanStat *st = nullptr, hs = {0, 0, 0};
+    TcPlanStat *st = nullptr, hs;
+    memset(&hs, 0, sizeof(hs));
     int32_t *in = nullptr;
+    unsigned long long *at = nullptr;
     const int wb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, (int64_t)g->num_sms * 8));
-    int64_t ends[2] = {0, 0};
-    auto read_stat = [&]() -> int {
-        const cudaError_t e = read_mapped(&hs, st, sizeof(hs), s);
-        return e == cudaSuccess ? GP_OK : set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
-    };
-    int r = tmp.alloc(st, 1, s);
-    if (r == GP_OK) r = w.mem.alloc(w.out_off, (size_t)n + 1, s);
-    if (r == GP_OK) r = w.mem.alloc(w.in_off, (size_t)n + 1, s);
+    // (few allocations: a dozen of them were a third of a small graph's first call)
+    int64_t *offs = nullptr;
+    int r = w.mem.alloc(offs, 2 * ((size_t)n + 1) + sizeof(TcPlanStat) / sizeof(int64_t), s);
     if (r == GP_OK) {
-        const cudaError_t e = cudaMemsetAsync(st, 0, sizeof(*st), s);
+        w.out_off = offs;
+        w.in_off = offs + n + 1;
+        st = (TcPlanStat *)(offs + 2 * (n + 1));
+    }
+    if (r == GP_OK) {
+        cudaError_t e = cudaMemsetAsync(st, 0, sizeof(*st), s);
+        if (e == cudaSuccess) {
+            GP_LAUNCH("tc_count", s, (k_tc_count<<<wb, 256, 0, s>>>(n, g->csr_off, g->csr_idx, w.out_off, w.in_off, st)));
+            e = read_mapped(&hs, st, sizeof(hs), s);
+        }
         if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
     }
-    if (r == GP_OK) {
-        GP_LAUNCH("tc_count", s, (k_tc_count<<<wb, 256, 0, s>>>(n, g->csr_off, g->csr_idx, w.out_off, w.in_off, st)));
-        r = check_launch("tc_count");
-    }
-    if (r == GP_OK) r = read_stat();
     w.probes = hs.probes;
-    w.general = hs.general || hs.max_out > (unsigned long long)TC_MAX_OUT;
-    if (r == GP_OK && !w.general) r = exclusive_scan(w.out_off, w.out_off, n, tmp, s);
-    if (r == GP_OK && !w.general) r = exclusive_scan(w.in_off, w.in_off, n, tmp, s);
+    w.general = hs.general || hs.max_out > (unsigned long long)TC_MAX_OUT || hs.out != hs.in;
     if (r == GP_OK && !w.general) {
-        cudaError_t e = read_mapped(&ends[0], w.out_off + n, sizeof(int64_t), s);
-        if (e == cudaSuccess) e = read_mapped(&ends[1], w.in_off + n, sizeof(int64_t), s);
-        if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
-        w.general = ends[0] != ends[1];
-    }
-    if (r == GP_OK && !w.general) {
-        r = w.mem.alloc(w.out, (size_t)ends[0], s);
-        if (r == GP_OK) r = w.mem.alloc(w.rev, (size_t)ends[0], s);
-        if (r == GP_OK) r = w.mem.alloc(w.slots, (size_t)ends[0], s);
-        if (r == GP_OK) r = w.mem.alloc(w.own, (size_t)std::max<int64_t>(n, 1), s);
-        if (r == GP_OK) r = tmp.alloc(in, (size_t)ends[1], s);
+        w.nlight = (int64_t)hs.light;
+        w.nheavy = (int64_t)hs.heavy;
+        w.nmid = (int64_t)hs.mid;
+        w.nwide = (int64_t)hs.wide;
+        r = exclusive_scan(w.out_off, w.out_off, n, tmp, s);
+        if (r == GP_OK) r = exclusive_scan(w.in_off, w.in_off, n, tmp, s);
+        const size_t edges = (size_t)hs.out, kinds = (size_t)(hs.light + hs.heavy + hs.mid + hs.wide);
+        unsigned long long *wide = nullptr;  // own, the counters of the kinds, then the 32-bit arrays
+        if (r == GP_OK) r = w.mem.alloc(wide, (size_t)n + 4 + (3 * edges + kinds) / 2 + 1, s);
+        if (r == GP_OK) r = tmp.alloc(in, (size_t)hs.in, s);
         if (r == GP_OK) {
+            w.own = wide;
+            at = wide + n;
+            w.slots = (int32_t *)(wide + n + 4);
+            w.out = w.slots + edges;
+            w.rev = w.out + edges;
+            w.light = w.rev + edges;
+            w.heavy = w.light + hs.light;
+            w.mid = w.heavy + hs.heavy;
+            w.wide = w.mid + hs.mid;
             // entries that no list writes (vertices of fewer than two out-neighbours) stay zero
-            cudaError_t e = cudaMemsetAsync(w.slots, 0, (size_t)ends[0] * sizeof(int32_t), s);
-            if (e == cudaSuccess) e = cudaMemsetAsync(w.own, 0, (size_t)n * sizeof(unsigned long long), s);
+            cudaError_t e = cudaMemsetAsync(wide, 0, ((size_t)n + 4) * sizeof(*wide) + edges * sizeof(int32_t), s);
             if (e == cudaSuccess) {
+                const int vb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)g->num_sms * 8));
+                GP_LAUNCH("tc_kinds", s, (k_tc_kinds<<<vb, 256, 0, s>>>(n, w.out_off, w.in_off, w.light, w.heavy, w.mid, w.wide, at)));
                 GP_LAUNCH("tc_lists", s, (k_tc_lists<<<wb, 256, 0, s>>>(n, g->csr_off, g->csr_idx, w.out_off, w.in_off, w.out, in)));
                 GP_LAUNCH("tc_reverse", s, (k_tc_reverse<<<wb, 256, 0, s>>>(n, w.out_off, w.in_off, w.out, in, w.rev, st)));
                 e = cudaGetLastError();
             }
             if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
         }
-        if (r == GP_OK) r = read_stat();
-        if (r == GP_OK) w.general = hs.general != 0;
-        if (r == GP_OK && !w.general)
-            r = select_by_degree(w.out_off, n, 2, TC_WARP_OUT, w.mem, w.light, w.nlight, INT64_MAX, nullptr, s);
-        if (r == GP_OK && !w.general)
-            r = select_by_degree(w.out_off, n, TC_WARP_OUT + 1, INT64_MAX, w.mem, w.heavy, w.nheavy, INT64_MAX, nullptr, s);
-        if (r == GP_OK && !w.general) r = select_by_degree(w.in_off, n, 33, TC_WIDE, w.mem, w.mid, w.nmid, INT64_MAX, nullptr, s);
-        if (r == GP_OK && !w.general)
-            r = select_by_degree(w.in_off, n, TC_WIDE + 1, INT64_MAX, w.mem, w.wide, w.nwide, INT64_MAX, nullptr, s);
+        w.fresh = st;  // whether every edge has its reverse is read with the first counts
         w.table = 4 * TC_WARP_OUT;
         while (w.table < 2 * TC_MAX_OUT && w.table < 4 * (int64_t)hs.max_out) w.table *= 2;
     }
@@ -741,6 +780,8 @@ extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64
         cudaEventRecord(ev0, s);
     }
     unsigned long long host[2] = {0, 0};
+    TcPlanStat plan;
+    memset(&plan, 0, sizeof(plan));
     cudaError_t e = cudaSuccess;
     if (st == GP_OK) {
         e = cudaMemsetAsync(scal, 0, 3 * sizeof(unsigned long long), s);
@@ -780,8 +821,21 @@ extern "C" int gp_triangles(const gp_graph *gc, int mode, int64_t *tc_out, int64
     if (st == GP_OK && e == cudaSuccess && tc_out && !dev_out && n > 0)
         e = cudaMemcpyAsync(tc_out, tc, (size_t)n * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
     if (st == GP_OK && e == cudaSuccess) e = cudaMemcpyAsync(host, scal, sizeof(host), cudaMemcpyDeviceToHost, s);
+    const bool fresh = lists && w.fresh;
+    if (st == GP_OK && e == cudaSuccess && fresh) e = cudaMemcpyAsync(&plan, w.fresh, sizeof(plan), cudaMemcpyDeviceToHost, s);
     if (st == GP_OK && e == cudaSuccess && stats) e = cudaEventRecord(ev1, s);
     if (st == GP_OK && e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (st == GP_OK && e == cudaSuccess && fresh) {
+        w.fresh = nullptr;
+        if (plan.general) {  // an edge without its reverse: the listing's counts instead
+            w.general = true;
+            w.mem.release(s);
+            tmp.release(s);
+            if (ev0) cudaEventDestroy(ev0);
+            if (ev1) cudaEventDestroy(ev1);
+            return gp_triangles(gc, mode, tc_out, total_out, stats, stream);
+        }
+    }
     if (lists) {
         host[0] *= 3;  // as the sum of the counts
         host[1] = w.probes;

@@ -96,3 +96,19 @@ def test_outside_the_contract(gp, mode):
     rows[5] = rows[5][::-1]
     tc, total, st = gp.triangles(upload(gp, 9, rows), mode)  # searched as if sorted: ends, in bounds
     assert 0 <= total <= math.comb(6, 3)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_one_way_edges(gp, mode):
+    """A graph called symmetric whose edge 8 -> 3 has no reverse (and 2 -> 6 none, so that the lists' lengths
+    agree): the listing's answer, on the first call and after."""
+    rows = clique_rows(9, 6)
+    rows[8] = [r for r in rows[8] if r != 3]
+    rows[2] = sorted(rows[2] + [6])
+    ref, probes = listing(9, rows)
+    G = upload(gp, 9, rows)
+    for _ in range(2):
+        tc, total, st = gp.triangles(G, mode)
+        if mode == 1:
+            assert np.array_equal(tc.cpu().numpy(), ref)
+        assert st["probes"] == probes
