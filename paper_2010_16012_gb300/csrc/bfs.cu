@@ -4,8 +4,8 @@
 // Section 3.3 and Algorithm 3 (push- and pull-based BFS, every ready counter
 // equal to one):
 //   top-down  (push): every frontier vertex v scans its out-edges (v->w) and
-//             claims each unvisited w with a compare-and-swap on level[w]
-//             (Section 4.3: O(m) CAS in total); the winner records the parent
+//             claims each unvisited w with an atomic on its bit of the bitmap of
+//             unvisited vertices (Section 4.3: O(m) CAS in total); the winner records the parent
 //             and appends w to the next frontier (the k-filter of Section 4,
 //             here a warp-aggregated queue append).
 //   bottom-up (pull): every unvisited vertex v scans its in-edges (u->v) and
@@ -62,7 +62,10 @@ struct BfsArgs {
     int32_t *h_next;
     const uint32_t *bits_cur;
     uint32_t *bits_next;   // next frontier bitmap (zero on entry)
-    uint32_t *unvis;       // bottom-up candidates; each word owned by one warp of a bottom-up level
+    uint32_t *unvis;       // unvisited vertices with in-edges; each word owned by one warp of a bottom-up level
+    const uint32_t *nzin;  // vertices with in-edges
+    int32_t src;
+    bool fill;             // bottom-up: no earlier level has written the unreached vertices' -1 (see bfs_fill)
     BfsCtr *cur, *nxt;
     int32_t L;           // level being expanded: new vertices get L + 1
     int32_t make_queue;  // top-down: also build the next frontier's queue
@@ -109,15 +112,16 @@ __device__ __forceinline__ void frontier_append(const BfsArgs &a, bool take, int
     }
 }
 
-// Claim w from u at level L+1; returns true for the winner, which also marks w
-// in the next frontier's bitmap and removes it from the bottom-up candidates.
+// Claim w (which has an in-edge: this one) from u at level L+1; returns true for
+// the winner, which also marks w in the next frontier's bitmap.  The claim is on
+// the bitmap of unvisited vertices, n/8 bytes that stay in cache, not on the level.
 __device__ __forceinline__ bool td_claim(const BfsArgs &a, int32_t w, int32_t u) {
-    if (a.level[w] != -1) return false;
-    if (atomicCAS(a.level + w, -1, a.L + 1) != -1) return false;
-    if (a.parent) a.parent[w] = u;
     const uint32_t bit = 1u << (w & 31);
+    if (!(a.unvis[w >> 5] & bit)) return false;
+    if (!(atomicAnd(a.unvis + (w >> 5), ~bit) & bit)) return false;
+    a.level[w] = a.L + 1;
+    if (a.parent) a.parent[w] = u;
     atomicOr(a.bits_next + (w >> 5), bit);
-    atomicAnd(a.unvis + (w >> 5), ~bit);
     return true;
 }
 
@@ -234,9 +238,12 @@ __device__ void bfs_topdown_step(const BfsArgs &a) {
 #endif
 constexpr int BFS_WARPS = GP_BFS_WARPS;  // warps per block of the persistent kernel
 #ifndef GP_BU_SCAN
-#define GP_BU_SCAN 4
+#define GP_BU_SCAN 3
 #endif
-constexpr int BU_SCAN = GP_BU_SCAN;  // in-edges a bottom-up lane checks per step
+// In-edges a bottom-up lane checks per step.  The scan is bound by the sectors it
+// asks for as much as by their latency: 64 searches on R-MAT 2^22 in 5885, 5673,
+// 5521, 5662, 5939 and 6637 us with 1, 2, 3, 4, 6 and 8.
+constexpr int BU_SCAN = GP_BU_SCAN;
 // A candidate with more in-edges than this is a hub: its lane probes only that
 // many, and a hub with no frontier vertex among them is finished by the chunk
 // pass (one lane walking a hub's whole in-list would hold up its warp).
@@ -245,21 +252,67 @@ constexpr int BU_SCAN = GP_BU_SCAN;  // in-edges a bottom-up lane checks per ste
 #endif
 constexpr int64_t BU_PROBE = GP_BU_PROBE;
 
+// Levels and parents are not filled with -1 at the start of a search: the first
+// bottom-up level, which passes over all vertices anyway, writes -1 to every one
+// that is not visited then, in whole lines with what it finds, and a search
+// without such a level does it at its end.  (R-MAT 2^22: the fill was 33 MB of
+// writes, and the later stores into lines that had left the cache as much again.)
+__device__ __forceinline__ void bfs_fill_words(const BfsArgs &a, int64_t base, uint32_t none) {
+    const int lane = lane_id();
+    for (unsigned m = __ballot_sync(FULL, none != 0u); m; m &= m - 1) {
+        const int k = __ffs(m) - 1;
+        const uint32_t word = __shfl_sync(FULL, none, k);
+        if (!((word >> lane) & 1u)) continue;
+        const int64_t v = (base + k) * 32 + lane;
+        a.level[v] = -1;
+        if (a.parent) a.parent[v] = -1;
+    }
+}
+
+// The vertices of word wd that `open` (unvisited with in-edges) and the absence of in-edges leave at -1.
+__device__ __forceinline__ uint32_t bfs_unreached(const BfsArgs &a, int64_t wd, uint32_t open) {
+    uint32_t none = open | ~a.nzin[wd];
+    if (wd == a.src >> 5) none &= ~(1u << (a.src & 31));
+    if (wd * 32 + 32 > a.n) none &= (1u << (a.n & 31)) - 1u;
+    return none;
+}
+
+__device__ void bfs_fill(const BfsArgs &a) {
+    const int64_t nwords = (a.n + 31) >> 5;
+    for (int64_t base = search_warp(a) * 32; base < nwords; base += search_nwarps(a) * 32) {
+        const int64_t wd = base + lane_id();
+        bfs_fill_words(a, base, wd < nwords ? bfs_unreached(a, wd, a.unvis[wd]) : 0u);
+    }
+}
+
 __device__ void bfs_bottomup_step(const BfsArgs &a) {
     __shared__ uint32_t s_found[BFS_WARPS][32];
+    __shared__ int s_next;
     const int lane = lane_id(), wib = threadIdx.x >> 5;
-    const int64_t warp = search_warp(a);
-    const int64_t nwarps = search_nwarps(a);
     const int64_t nwords = (a.n + 31) >> 5;
     unsigned long long nf = 0, mf = 0, mu = 0, ex = 0, deferred = 0;
-    for (int64_t base = warp * 32; base < nwords; base += nwarps * 32) {
+    // A block's warps take units as they get free (equal shares: 6278 against 5515 us for
+    // 64 searches on R-MAT 2^22); words per unit: two units to a warp, so that small
+    // graphs spread over all of them (the largest level of one search on 2^14: 25 -> 6 us).
+    const int words = (int)max((int64_t)1, min((int64_t)32, nwords / (2 * search_nwarps(a))));
+    if (threadIdx.x == 0) s_next = 0;
+    __syncthreads();
+    while (true) {
+        int unit = 0;
+        if (lane == 0) unit = atomicAdd(&s_next, 1);
+        unit = __shfl_sync(FULL, unit, 0);
+        const int64_t base = ((int64_t)unit * a.ngblk + a.gblk) * words;
+        if (base >= nwords) break;
         const int64_t wd = base + lane;
-        const uint32_t cand = wd < nwords ? a.unvis[wd] : 0u;
+        const uint32_t cand = lane < words && wd < nwords ? a.unvis[wd] : 0u;
         const int cnt = __popc(cand);
         const int incl = warp_incl_scan(cnt);
         const int excl = incl - cnt;
         const int total = __shfl_sync(FULL, incl, 31);
-        if (total == 0) continue;  // uniform across the warp
+        if (total == 0) {  // uniform across the warp
+            if (a.fill) bfs_fill_words(a, base, lane < words && wd < nwords ? bfs_unreached(a, wd, 0u) : 0u);
+            continue;
+        }
         s_found[wib][lane] = 0u;
         __syncwarp();
         // Round r's candidate (vertex and in-edge range) is located and its
@@ -339,6 +392,7 @@ __device__ void bfs_bottomup_step(const BfsArgs &a) {
             a.bits_next[wd] = fw;
             a.unvis[wd] = cand & ~fw;
         }
+        if (a.fill) bfs_fill_words(a, base, lane < words && wd < nwords ? bfs_unreached(a, wd, cand & ~fw) : 0u);
         __syncwarp();
     }
     flush_counters(a, nf, mf, mu, ex, deferred);
@@ -348,15 +402,16 @@ __device__ void bfs_bottomup_step(const BfsArgs &a) {
 // in-edge chunks (chunk_edges each) of every hub still unvisited are scanned by
 // warps across the whole grid, so a hub's in-list is spread over many warps.
 // Each chunk stops at its first frontier vertex, or when another chunk has
-// claimed the hub; chunks of one hub settle the claim with one compare-and-swap
-// on its level (the owner-only rule applied to the hub's set of chunks).
+// claimed the hub; chunks of one hub settle the claim with one atomic on its
+// bit (the owner-only rule applied to the hub's set of chunks).
 constexpr int BU_WARP_UNROLL = 8;
 
 __device__ void bfs_bottomup_hubs(const BfsArgs &a) {
     const int lane = lane_id();
     const int64_t warp = search_warp(a);
     const int64_t nwarps = search_nwarps(a);
-    volatile int32_t *vlevel = a.level;
+    volatile uint32_t *vunvis = a.unvis;
+    auto open = [&](int32_t v) { return ((vunvis[v >> 5] >> (v & 31)) & 1u) != 0u; };
     unsigned long long nf = 0, mf = 0, mu = 0, ex = 0;
     for (int64_t base = warp * 32; base < a.pull_nchunks; base += nwarps * 32) {
         const int64_t j = base + lane;
@@ -367,7 +422,7 @@ __device__ void bfs_bottomup_hubs(const BfsArgs &a) {
         bool need = false;
         if (j < a.pull_nchunks) {
             ch = a.pull_chunks[j];
-            if (vlevel[ch.v] == -1) need = a.csc_off[ch.v + 1] - a.csc_off[ch.v] > a.bu_probe;
+            if (open(ch.v)) need = a.csc_off[ch.v + 1] - a.csc_off[ch.v] > a.bu_probe;
         }
         for (unsigned nm = __ballot_sync(FULL, need); nm; nm &= nm - 1) {
             const int hl = __ffs(nm) - 1;
@@ -379,7 +434,7 @@ __device__ void bfs_bottomup_hubs(const BfsArgs &a) {
             int scanned = 0;
             for (int i0 = 0; i0 < cl && hit < 0; i0 += 32 * BU_WARP_UNROLL) {
                 int claimed = 0;
-                if (lane == 0 && i0 > 0) claimed = vlevel[v] != -1;
+                if (lane == 0 && i0 > 0) claimed = !open(v);
                 if (__shfl_sync(FULL, claimed, 0)) break;  // uniform
                 int32_t u[BU_WARP_UNROLL];
 #pragma unroll
@@ -405,11 +460,11 @@ __device__ void bfs_bottomup_hubs(const BfsArgs &a) {
             }
             if (lane == 0) {
                 ex += (unsigned long long)(hit >= 0 ? hit - cb + 1 : scanned);
-                if (hit >= 0 && atomicCAS(a.level + v, -1, a.L + 1) == -1) {
+                const uint32_t bit = 1u << (v & 31);
+                if (hit >= 0 && (atomicAnd(a.unvis + (v >> 5), ~bit) & bit)) {
+                    a.level[v] = a.L + 1;
                     if (a.parent) a.parent[v] = par;
-                    const uint32_t bit = 1u << (v & 31);
                     atomicOr(a.bits_next + (v >> 5), bit);
-                    atomicAnd(a.unvis + (v >> 5), ~bit);
                     const int64_t din = a.csc_off[v + 1] - a.csc_off[v];
                     nf += 1;
                     mf += (unsigned long long)(a.csr_off == a.csc_off ? din : a.csr_off[v + 1] - a.csr_off[v]);
@@ -488,6 +543,7 @@ struct BfsRun {
     BfsLevelStat *stats;  // [GP_BFS_MAX_LEVELS]
     BfsSummary *summary;
     GridSync *sync;
+    BfsSummary *mirror;  // single search: where the host reads the summary and, if there are stats, the levels after it
 };
 
 // 512-thread blocks, two per SM (R-MAT 22, 64 searches: 11.5 ms one launch
@@ -513,14 +569,14 @@ __device__ bool bfs_search(const BfsRun &R, const SearchIO &io, int gblk, int ng
     const int64_t gthread = (int64_t)gblk * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)ngblk * blockDim.x;
     const int64_t nwords = (n + 31) >> 5;
-    // level/parent, counters, bitmaps and candidates set for frontier 0 = {src}
+    // counters, bitmaps and candidates set for frontier 0 = {src}
     const int32_t src = io.src;
     const int32_t s_rank = R.base.push_rank[src];
     const int64_t s_c0 = s_rank >= 0 ? R.base.push_cstart[s_rank] : 0;
     const int64_t s_c1 = s_rank >= 0 ? R.base.push_cstart[s_rank + 1] : 0;
-    for (int64_t v = gthread; v < n; v += nthreads) {
-        io.level[v] = v == src ? 0 : -1;
-        if (io.parent) io.parent[v] = v == src ? src : -1;
+    if (gthread == 0) {
+        io.level[src] = 0;
+        if (io.parent) io.parent[src] = src;
     }
     constexpr int CW = (int)(sizeof(BfsCtr) / sizeof(unsigned long long));
     if (gthread < 3 * CW) {
@@ -549,6 +605,9 @@ __device__ bool bfs_search(const BfsRun &R, const SearchIO &io, int gblk, int ng
     a.parent = io.parent;
     a.gblk = gblk;
     a.ngblk = ngblk;
+    a.nzin = R.nzin;
+    a.src = src;
+    a.fill = true;
     // counter records are read by one thread per block and shared through
     // shared memory: every thread loading the same line would queue tens of
     // thousands of requests on one L2 slice per level
@@ -625,6 +684,7 @@ __device__ bool bfs_search(const BfsRun &R, const SearchIO &io, int gblk, int ng
             in_queue = a.make_queue != 0;
         } else {
             bfs_bottomup_step(a);
+            a.fill = false;
             in_queue = false;
         }
         if (!grid_sync(R.sync, ngblk)) return false;
@@ -656,6 +716,7 @@ __device__ bool bfs_search(const BfsRun &R, const SearchIO &io, int gblk, int ng
         cur = nxt;
         ++L;
     }
+    if (a.fill) bfs_fill(a);
     if (gthread == 0) {
         io.summary->levels = L;
         io.summary->reached = reached;
@@ -669,7 +730,13 @@ __device__ bool bfs_search(const BfsRun &R, const SearchIO &io, int gblk, int ng
 
 __global__ void __launch_bounds__(BFS_THREADS, GP_BFS_MINB) k_bfs_persistent(BfsRun R) {
     const SearchIO io = {R.src, R.base.level, R.base.parent, R.summary};
-    bfs_search(R, io, blockIdx.x, gridDim.x);
+    if (!bfs_search(R, io, blockIdx.x, gridDim.x) || blockIdx.x != 0) return;
+    // the results the host waits for go straight into its mapped block (not level by
+    // level: a barrier's fence would wait for each store's way to the host)
+    __syncthreads();
+    const int words = R.stats ? (int)min(R.summary->levels, (int64_t)GP_BFS_MAX_LEVELS) * (int)(sizeof(BfsLevelStat) / 4) : 0;
+    for (int i = threadIdx.x; i < words; i += blockDim.x) ((uint32_t *)(R.mirror + 1))[i] = ((const uint32_t *)R.stats)[i];
+    if (threadIdx.x == 0) *R.mirror = *R.summary;
 }
 
 // Several searches in one launch: the grid is cut into `groups` groups of
@@ -733,8 +800,8 @@ __global__ void k_nzin_bits(int64_t n, const int64_t *csc_off, uint32_t *bits) {
     }
 }
 
-// host mirror: summary, per-level statistics, barrier status
-constexpr size_t BFS_HOST_BYTES = sizeof(BfsSummary) + GP_BFS_MAX_LEVELS * sizeof(BfsLevelStat) + sizeof(GridSync);
+// host mirror: summary, per-level statistics
+constexpr size_t BFS_HOST_BYTES = sizeof(BfsSummary) + GP_BFS_MAX_LEVELS * sizeof(BfsLevelStat);
 
 void release_bfs_work(gp_graph *g, cudaStream_t s) {
     if (g->bfs.done_ev) {
@@ -745,6 +812,8 @@ void release_bfs_work(gp_graph *g, cudaStream_t s) {
         cudaEventSynchronize(g->bfs.mdone_ev);
         cudaEventDestroy(g->bfs.mdone_ev);
     }
+    for (cudaEvent_t e : g->bfs.ev)
+        if (e) cudaEventDestroy(e);
     pinned_free(g->bfs.ctr_host, BFS_HOST_BYTES);
     pinned_free(g->bfs.mhost, g->bfs.mhost_bytes);
     g->bfs.ctr_host = nullptr;
@@ -830,6 +899,8 @@ static int ensure_bfs_work(gp_graph *g, const BigBins &bins, cudaStream_t s) {
     if (per_sm < 1) return set_error(GP_ERR_UNSUPPORTED, "BFS kernel does not fit on an SM");
     w.grid = per_sm * g->num_sms;
     GP_TRY(pinned_alloc(&w.ctr_host, BFS_HOST_BYTES));
+    GP_TRY(pinned_device_ptr(w.ctr_host, &w.ctr_mirror));
+    for (cudaEvent_t &e : w.ev) GP_CUDA(cudaEventCreate(&e));
     GP_CUDA(cudaEventCreateWithFlags(&w.done_ev, cudaEventDisableTiming));
     w.ready = true;
     return GP_OK;
@@ -871,20 +942,20 @@ static int bfs_run(const gp_graph *gc, int32_t src, int mode, const int8_t *dirs
     char *h = (char *)w.ctr_host;
     BfsSummary *hs = (BfsSummary *)h;
     BfsLevelStat *hl = (BfsLevelStat *)(h + sizeof(BfsSummary));
-    GridSync *hsync = (GridSync *)(h + sizeof(BfsSummary) + GP_BFS_MAX_LEVELS * sizeof(BfsLevelStat));
+    volatile int64_t *ended = &hs->levels;  // -1 until a search has run to its end
     if (w.pending) {  // the barrier status of the previous, asynchronous search
         GP_CUDA(cudaEventSynchronize(w.done_ev));
         w.pending = false;
-        if (hsync->err) {
-            hsync->err = 0;
+        if (*ended < 0) {
+            w.sync_clean = false;
             return set_error(GP_ERR_TIMEOUT, "BFS: a grid barrier wait ran out in the previous asynchronous search");
         }
     }
     if (stats) memset(stats, 0, sizeof(*stats));
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (stats) {
-        GP_CUDA(cudaEventCreate(&ev0));
-        GP_CUDA(cudaEventCreate(&ev1));
+        ev0 = w.ev[0];
+        ev1 = w.ev[1];
         GP_CUDA(cudaEventRecord(ev0, s));
     }
     int32_t *level = level_out, *parent = parent_out;
@@ -910,7 +981,8 @@ static int bfs_run(const gp_graph *gc, int32_t src, int mode, const int8_t *dirs
     R.base.unvis = w.unvis;
     R.ctr = (BfsCtr *)w.ctr;
     R.src = src;
-    R.stats = (BfsLevelStat *)w.stats;
+    R.stats = stats ? (BfsLevelStat *)w.stats : nullptr;
+    R.mirror = (BfsSummary *)w.ctr_mirror;
     R.summary = (BfsSummary *)w.summary;
     R.sync = (GridSync *)w.sync;
     if (dirs) {
@@ -925,7 +997,11 @@ static int bfs_run(const gp_graph *gc, int32_t src, int mode, const int8_t *dirs
         R.dirs = (const int8_t *)w.dirs;
         R.ndirs = ndirs;
     }
-    GP_CUDA(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), s));
+    if (!w.sync_clean) {  // a launch that runs to its end leaves a whole number of generations
+        GP_CUDA(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), s));
+        w.sync_clean = true;
+    }
+    *ended = -1;
     {
         ProfScope ps("bfs_persistent", s);
         void *args[] = {&R};
@@ -934,7 +1010,6 @@ static int bfs_run(const gp_graph *gc, int32_t src, int mode, const int8_t *dirs
     }
     if (!lvl_dev) GP_CUDA(cudaMemcpyAsync(level_out, level, n * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (!par_dev) GP_CUDA(cudaMemcpyAsync(parent_out, parent, n * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    GP_CUDA(cudaMemcpyAsync(hsync, w.sync, sizeof(GridSync), cudaMemcpyDeviceToHost, s));
     if (!stats && lvl_dev && par_dev) {
         // nothing for the host to read: return without waiting; the barrier
         // status is checked by the next search on this graph
@@ -943,14 +1018,10 @@ static int bfs_run(const gp_graph *gc, int32_t src, int mode, const int8_t *dirs
         return GP_OK;
     }
     if (stats) {
-        GP_CUDA(cudaMemcpyAsync(hs, w.summary, sizeof(BfsSummary), cudaMemcpyDeviceToHost, s));
-        GP_CUDA(cudaMemcpyAsync(hl, w.stats, GP_BFS_MAX_LEVELS * sizeof(BfsLevelStat), cudaMemcpyDeviceToHost, s));
         GP_CUDA(cudaEventRecord(ev1, s));
         GP_CUDA(cudaEventSynchronize(ev1));
         float ms = 0.f;
         cudaEventElapsedTime(&ms, ev0, ev1);
-        cudaEventDestroy(ev0);
-        cudaEventDestroy(ev1);
         stats->levels = (int32_t)hs->levels;
         stats->switches = (int32_t)hs->switches;
         stats->reached = hs->reached;
@@ -966,8 +1037,12 @@ static int bfs_run(const gp_graph *gc, int32_t src, int mode, const int8_t *dirs
             stats->level_ns[i] = hl[i].ns;
         }
     }
-    GP_CUDA(cudaStreamSynchronize(s));
-    if (hsync->err) return set_error(GP_ERR_TIMEOUT, "BFS: a grid barrier wait ran out");
+    if (!stats) GP_CUDA(cudaStreamSynchronize(s));
+    if (*ended < 0) {
+        w.sync_clean = false;
+        if (stats) memset(stats, 0, sizeof(*stats));
+        return set_error(GP_ERR_TIMEOUT, "BFS: a grid barrier wait ran out");
+    }
     return GP_OK;
 }
 

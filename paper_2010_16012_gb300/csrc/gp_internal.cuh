@@ -199,10 +199,13 @@ struct BfsWork {
     uint32_t *nzin = nullptr;                // vertices with in-edges (the initial candidates)
     int32_t *level_dev = nullptr, *parent_dev = nullptr;  // when outputs are host memory
     void *ctr = nullptr;                     // device counters
-    void *ctr_host = nullptr;                // pinned mirror of the summary, level stats and barrier word
+    void *ctr_host = nullptr;                // pinned mirror of the summary and level stats (written by the kernel)
+    void *ctr_mirror = nullptr;              // its device-side address
     void *stats = nullptr;                   // per-level statistics (device)
     void *summary = nullptr;                 // search summary (device)
     void *sync = nullptr;                    // grid barrier word
+    bool sync_clean = false;                 // it holds a whole number of generations
+    cudaEvent_t ev[2] = {nullptr, nullptr};  // start and end of a timed call
     int8_t *dirs = nullptr;                  // forced directions (device copy)
     int dirs_cap = 0;                        // entries `dirs` holds
     int grid = 0;                            // blocks of the cooperative launch
