@@ -203,7 +203,7 @@ def pick_sources(g, count: int):
 
 
 KERNEL_SOURCE = {"pull_tiles": "pagerank.cu", "pull_finish": "pagerank.cu", "pull_big": "pagerank.cu",
-                 "pull_light": "pagerank.cu", "push_scatter": "pagerank.cu",
+                 "pull_light": "pagerank.cu", "push_tiles": "pagerank.cu", "push_scatter": "pagerank.cu",
                  "push_epilogue": "pagerank.cu", "bfs_persistent": "bfs.cu", "bfs_multi": "bfs.cu"}
 
 
@@ -265,6 +265,7 @@ def kernel_bytes(g, opt, l2_bytes=None) -> dict:
     fp64 = mode == 1 or (mode == -1 and not (l2_bytes is not None and 8 * n > l2_bytes // 2
                                              and int(din.max(initial=0)) <= 4096))
     rows, tiles = int((din > 0).sum()), (m + 255) // 256
+    sources = int((dout > 0).sum())
     return {
         # indices + row-start bits + c (once) + a sum written per row, a row number read and a carry written per tile
         "pull_tiles": 4 * m + m // 8 + 4 * n + 4 * rows + 8 * tiles,
@@ -275,7 +276,9 @@ def kernel_bytes(g, opt, l2_bytes=None) -> dict:
         "pull_big": 4 * e_big_in + 16 * ch_in + 4 * ch_in,
         # light in-edge lists + offsets + c (once) + x, inv_deg read + y, c' written + big-vertex combine
         "pull_light": 4 * (m - e_big_in) + 8 * (n + 1) + 4 * n * 5 + 4 * ch_in + 12 * nb_in,
-        # all out-edge lists + offsets + c + y read-modify-write + chunk table
+        # out-edge indices + source bits + sources + c + y read-modify-write
+        "push_tiles": 4 * m + m // 8 + 4 * tiles + 8 * sources + 8 * n,
+        # the same with sources found from the offsets and a chunk table (the lists split by degree)
         "push_scatter": 4 * m + 8 * (n + 1) + 4 * n + 8 * n + 16 * ch_out,
         # FP64: the accumulator read and reset, x and inv_deg read, y and c' written;
         # FP32: y, x, inv_deg read, y, c' and the next accumulator (x) written
@@ -329,7 +332,7 @@ def run_ours(args, dist: Dist):
     opt_struct = G0.options()
     G0.free()
     kb = kernel_bytes(g, opt_struct, getattr(torch.cuda.get_device_properties(dev), "L2_cache_size", None))
-    pr_kernels = {gp.PULL: ("pull_tiles", "pull_finish"), gp.PUSH: ("push_scatter", "push_epilogue")}
+    pr_kernels = {gp.PULL: ("pull_tiles", "pull_finish"), gp.PUSH: ("push_tiles", "push_epilogue")}
     bfs_stats = {}
     n_in = int(np.count_nonzero(np.diff(g.csc_off)))  # vertices with in-edges (every reached vertex has one)
 

@@ -170,7 +170,7 @@ typedef struct gp_options {
     int32_t pull_light_max;   /* in-degree <= this: one lane per vertex (pull steps of SSSP and
                                  Frontier-Exploit PageRank, bottom-up BFS; the pull PageRank
                                  sweep cuts the edge list in equal tiles at any degree) */
-    int32_t push_light_max;   /* out-degree <= this: 32 vertices per warp (push scatter, adjoint) */
+    int32_t push_light_max;   /* out-degree <= this: 32 vertices per warp (adjoint, SSSP) */
     int32_t chunk_edges;      /* edges per warp chunk for vertices above the light limits */
     int32_t blocks_per_sm;    /* resident blocks per SM for the grid-stride sweep kernels */
     int32_t poll_interval;    /* PageRank sweeps enqueued between convergence read-backs (at
@@ -221,7 +221,7 @@ int gp_graph_get_options(const gp_graph *g, gp_options *opt);
 /* ------------------------------------------------------------------ autotuning */
 
 #define GP_TUNE_PULL 0x1u /* pull_hot_slots */
-#define GP_TUNE_PUSH 0x2u /* push_light_max, blocks_per_sm, push_hot_slots */
+#define GP_TUNE_PUSH 0x2u /* push_hot_slots */
 #define GP_TUNE_AUTO 0x4u /* pr_auto_mode: the faster of pull and push for this graph */
 #define GP_TUNE_BFS 0x8u  /* bfs_light_max, bfs_alpha, bfs_beta, then bfs_groups */
 #define GP_TUNE_ALL 0xFu

@@ -2,12 +2,10 @@
 //
 // Correctness never depends on the options; only speed does.  The tuner runs
 // coordinate descent over small candidate sets, timing each candidate with
-// CUDA events on the caller's stream (the faster of two timings), and repeats
-// the push descent once when a pass changed something (the coordinates interact: the best resident-block count depends on the size of
-// the shared-memory accumulators, for instance):
+// CUDA events on the caller's stream (the faster of two timings):
 //   pull PageRank: pull_hot_slots (a few sweeps of gp_pagerank(GP_PULL) per
 //                  candidate; its tiles do not depend on the degree limits);
-//   push PageRank: push_light_max, then blocks_per_sm, then push_hot_slots;
+//   push PageRank: push_hot_slots;
 //   AUTO:          pr_auto_mode = whichever of pull and push sweeps faster
 //                  (the per-graph push/pull choice of the Generic-Switch idea, Section 5);
 //   BFS:           bfs_light_max, then bfs_alpha, then bfs_beta (gp_bfs(GP_AUTO)
@@ -36,7 +34,7 @@ struct Timer {
     }
 };
 
-constexpr int TUNE_WARM = 2, TUNE_SWEEPS = 6, TUNE_REPS = 2, TUNE_PASSES = 2;
+constexpr int TUNE_WARM = 2, TUNE_SWEEPS = 6, TUNE_REPS = 2;
 
 // Milliseconds per sweep of gp_pagerank(mode) under the graph's current
 // options: the fastest of TUNE_REPS timed runs.
@@ -155,15 +153,9 @@ extern "C" int gp_autotune(gp_graph *g, unsigned what, const int32_t *sources, i
     if (st == GP_OK && (what & GP_TUNE_PUSH)) {
         st = push(push_ms);
         ++evaluated;
-        for (int pass = 0; pass < TUNE_PASSES && st == GP_OK; ++pass) {
-            const gp_options before = best;
-            st = try_values<int32_t>(g, best, push_ms, &gp_options::push_light_max, {8, 16, 32, 64}, s, push, evaluated);
-            if (st == GP_OK) st = try_values<int32_t>(g, best, push_ms, &gp_options::blocks_per_sm, {4, 8, 12}, s, push, evaluated);
-            if (st == GP_OK)
-                st = try_values<int32_t>(g, best, push_ms, &gp_options::push_hot_slots,
-                                         {0, 8192, 16384, 24576, 32768, 40960, 49152}, s, push, evaluated);
-            if (!memcmp(&before, &best, sizeof(best))) break;
-        }
+        if (st == GP_OK)
+            st = try_values<int32_t>(g, best, push_ms, &gp_options::push_hot_slots,
+                                     {0, 8192, 16384, 24576, 32768, 40960, 49152}, s, push, evaluated);
     }
     if (st == GP_OK && (what & GP_TUNE_AUTO)) {
         if (!(what & GP_TUNE_PULL)) st = pull(pull_ms);

@@ -256,7 +256,8 @@ struct gp_graph {
     gp::BigBins bfs_bins;   // by out-degree at bfs_light_max (BFS top-down), when it differs from push_light_max
     gp::HotSet pull_hot;    // shared-memory contribution cache of the pull sweep
     gp::HotSet push_hot;    // shared-memory accumulators of the push scatter
-    gp::EdgeTiles tiles;    // of the CSC (pull sweep); built by the first sweep
+    gp::EdgeTiles tiles;      // of the CSC (pull sweep); built by the first sweep
+    gp::EdgeTiles out_tiles;  // of the CSR (push sweep), where it is not the same array pair
     gp::PrWork pr;
     gp::BfsWork bfs;
     gp_sssp_work *sssp = nullptr;

@@ -15,9 +15,9 @@
 //                    the row spans many) and writes the vertex's y,
 //                    c' = y*inv_deg and |y - x|; every vertex has one writer.
 // Push (scatter with atomics; Section 4.1: O(Lm) write conflicts):
-//   k_push_scatter   -- each source adds d*c[u]*w_uv into y[v] for its
-//                       out-edges with FP32 atomicAdd (RED), big sources in
-//                       warp chunks, light sources in 32-vertex tiles.
+//   k_push_tiles     -- each source adds d*c[u]*w_uv into y[v] for its
+//                       out-edges with atomics (RED), over tiles of the
+//                       out-edge list like the pull's.
 //   k_push_epilogue  -- per vertex: residual, c' and the (1-d)s reset of the
 //                       buffer the next sweep accumulates into.
 // Convergence (not in the paper, which runs a fixed L): the L1 residual is
@@ -718,90 +718,108 @@ __device__ __forceinline__ void scatter_add(T *y, float *sh, int32_t dst, float 
     }
 }
 
+// Bound by the latency of its chains (indices, row, contribution) and the
+// shared-memory atomics, not by the reductions in L2: without those it is 4%
+// faster.  So what pays is equal work per lane and full occupancy: tiles and two
+// blocks per SM take R-MAT n = 1.0M (30M edges) from PUSH_WAS to PUSH_NOW us a sweep, where a
+// warp walked each 256-edge piece of a long list, a merged stream of the short
+// ones found every edge's source by a search over the warp, and one block of
+// 32768 accumulators filled the SM's shared memory.
 template <bool W, class T, bool HOT>
-__global__ void __launch_bounds__(1024) k_push_scatter(PrArgs a) {
+__global__ void __launch_bounds__(TILE_THREADS, 2) k_push_tiles(PrArgs a) {
     extern __shared__ float sh_acc[];
+    __shared__ float agg[TILE_THREADS];
     if (pr_gate(a, a.k)) return;
     if (HOT) {
         for (int64_t i = threadIdx.x; i < a.nhot; i += blockDim.x) sh_acc[i] = 0.f;
         __syncthreads();
     }
     const int lane = lane_id();
-    const int32_t *__restrict__ idx = a.idx;
-    const float *__restrict__ wv = a.w;
+    const unsigned below = (1u << lane) - 1u;
     T *y = sizeof(T) == 8 ? (T *)a.acc64 : (T *)a.y;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int warp = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * blockDim.x) >> 5;
+    const int ntiles = (int)a.ntiles;
     PushCount cnt;
-    // big sources: one warp per chunk of out-edges
-    for (int64_t j = warp; j < a.nchunks; j += nwarps) {
-        const Chunk ch = a.chunks[j];
-        const float cu = a.d * __ldg(a.c + ch.v);
-        const int32_t *ip = idx + ch.beg;
-        const float *wp = W ? wv + ch.beg : nullptr;
-        int i = lane;
-        for (; i + 96 < ch.len; i += 128) {
-            const int v0 = __ldg(ip + i), v1 = __ldg(ip + i + 32), v2 = __ldg(ip + i + 64), v3 = __ldg(ip + i + 96);
-            scatter_add<T, HOT>(y, sh_acc, v0, W ? cu * __ldg(wp + i) : cu, cnt);
-            scatter_add<T, HOT>(y, sh_acc, v1, W ? cu * __ldg(wp + i + 32) : cu, cnt);
-            scatter_add<T, HOT>(y, sh_acc, v2, W ? cu * __ldg(wp + i + 64) : cu, cnt);
-            scatter_add<T, HOT>(y, sh_acc, v3, W ? cu * __ldg(wp + i + 96) : cu, cnt);
-        }
-        for (; i < ch.len; i += 32) scatter_add<T, HOT>(y, sh_acc, __ldg(ip + i), W ? cu * __ldg(wp + i) : cu, cnt);
-    }
-    // light sources: 32 consecutive sources per warp, one merged edge stream
-    __shared__ float agg[1024];
-    const int64_t n = a.n;
-    const int64_t ntiles = (n + 31) >> 5;
-    for (int64_t t = warp; t < ntiles; t += nwarps) {
-        const int64_t u = t * 32 + lane;
-        int64_t b = 0, e = 0;
-        float cu = 0.f;
-        if (u < n) {
-            b = a.off[u];
-            e = a.off[u + 1];
-        }
-        const int64_t dd = e - b;
-        const bool big = dd > a.light_max;
-        const int deg = big ? 0 : (int)dd;
-        if (deg > 0) cu = a.d * __ldg(a.c + u);
-        const int incl = warp_incl_scan(deg);
-        const int excl = incl - deg;
-        const int E = __shfl_sync(FULL, incl, 31);
-        for (int base = 0; base < E; base += 32) {
-            const int eid = base + lane;
-            int k = 0;
+    for (int t = warp; t < ntiles; t += nwarps) {
+        const int64_t e0 = (int64_t)t * TILE_EDGES + lane * LANE_EDGES;
+        const unsigned h = a.heads[(int64_t)t * 32 + lane];  // bit q: edge e0 + q is the first of its source
+        const int32_t row0 = a.tile_row[t];
+        int32_t dst[8];
+        float val[8];
+        if (t < a.vec_tiles) {
+            uint32_t u[8];
+            ld_stream8(a.idx + e0, u);
 #pragma unroll
-            for (int s = 16; s > 0; s >>= 1) {
-                const int ex = __shfl_sync(FULL, excl, k + s);
-                if (ex <= eid) k += s;
-            }
-            const int64_t kb = __shfl_sync(FULL, b, k);
-            const int kex = __shfl_sync(FULL, excl, k);
-            const float ck = __shfl_sync(FULL, cu, k);
-            // idle lanes get keys no real edge has: positive and >= n is impossible for
-            // plain vertices, and HOT keys are negative
-            int32_t dst = (int32_t)(0x7fffffff - lane);
-            float val = 0.f;
-            if (eid < E) {
-                const int64_t pos = kb + (eid - kex);
-                dst = __ldg(idx + pos);
-                val = W ? ck * __ldg(wv + pos) : ck;
-            }
-            // Updates from different sources of the tile that hit the same vertex
-            // (typically a hub) are summed in the warp first, so the vertex takes one
-            // atomic per window instead of one per edge.
-            const unsigned peers = __match_any_sync(FULL, dst);
-            if (__all_sync(FULL, peers == (1u << lane))) {
-                if (eid < E) scatter_add<T, HOT>(y, sh_acc, dst, val, cnt);
+            for (int q = 0; q < 8; ++q) dst[q] = (int32_t)u[q];
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) dst[q] = e0 + q < a.m ? __ldg(a.idx + e0 + q) : 0;
+        }
+        // the sources' contributions: sources started in the lanes below (as in tile_sums), then in the lane
+        const unsigned nh = __popc(h);
+        int row = row0, sources = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const unsigned digit = __ballot_sync(FULL, (nh >> b) & 1u);
+            row += __popc(digit & below) << b;
+            sources += __popc(digit) << b;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            int32_t v = -1;
+            if (((h >> q) & 1u) || (q == 0 && e0 < a.m)) v = a.rows[row + __popc(h & ((2u << q) - 1u))] & 0x7fffffff;
+            val[q] = __int_as_float(v);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int32_t v = __float_as_int(val[q]);
+            val[q] = v >= 0 ? a.d * __ldg(a.c + v) : 0.f;
+        }
+#pragma unroll
+        for (int q = 1; q < 8; ++q)
+            if (!((h >> q) & 1u)) val[q] = val[q - 1];
+        if (W) {
+            if (t < a.vec_tiles) {
+                uint32_t w[8];
+                ld_stream8(a.w + e0, w);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) val[q] *= __uint_as_float(w[q]);
             } else {
-                agg[threadIdx.x] = val;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) val[q] *= e0 + q < a.m ? __ldg(a.w + e0 + q) : 0.f;
+            }
+        }
+        // Updates of one vertex by different sources (a hub by its leaves) are summed
+        // first: a lane's neighbouring ones, then, where the tile has many sources,
+        // the warp's.  A hub's FP32 accumulator then takes few terms.
+        bool crowd = sources >= 8;
+        if (crowd)  // (most such tiles share no vertex: their first edges tell)
+            crowd = !__all_sync(FULL, __match_any_sync(FULL, e0 < a.m ? dst[0] : (int32_t)(0x7fffffff - lane)) == (1u << lane));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            bool mine = e0 + q < a.m;
+            if (q < 7 && e0 + q + 1 < a.m && dst[q] == dst[q + 1]) {
+                val[q + 1] += val[q];
+                ++cnt.merged;
+                mine = false;
+            }
+            if (!crowd) {
+                if (mine) scatter_add<T, HOT>(y, sh_acc, dst[q], val[q], cnt);
+                continue;
+            }
+            // idle lanes get keys no update has: positive and >= n is impossible for
+            // plain vertices, and HOT keys are negative
+            const unsigned peers = __match_any_sync(FULL, mine ? dst[q] : (int32_t)(0x7fffffff - lane));
+            if (__all_sync(FULL, peers == (1u << lane))) {
+                if (mine) scatter_add<T, HOT>(y, sh_acc, dst[q], val[q], cnt);
+            } else {
+                agg[threadIdx.x] = val[q];
                 __syncwarp();
-                if (eid < E && (peers & ((1u << lane) - 1u)) == 0) {  // lowest lane of its group
-                    float sum = val;
+                if (mine && (peers & below) == 0) {  // lowest lane of its group
+                    float sum = val[q];
                     for (unsigned rest = peers & ~(1u << lane); rest; rest &= rest - 1)
                         sum += agg[(threadIdx.x & ~31u) + (__ffs(rest) - 1)];
-                    scatter_add<T, HOT>(y, sh_acc, dst, sum, cnt);
+                    scatter_add<T, HOT>(y, sh_acc, dst[q], sum, cnt);
                     cnt.merged += __popc(peers) - 1;
                 }
                 __syncwarp();
@@ -1006,11 +1024,11 @@ static int ensure_vec(gp_graph *g, float *&slot, cudaStream_t s) {
 
 static const void *push_kernel(bool W, bool fp64, bool hot) {
     if (fp64) {
-        if (W) return hot ? (const void *)k_push_scatter<true, double, true> : (const void *)k_push_scatter<true, double, false>;
-        return hot ? (const void *)k_push_scatter<false, double, true> : (const void *)k_push_scatter<false, double, false>;
+        if (W) return hot ? (const void *)k_push_tiles<true, double, true> : (const void *)k_push_tiles<true, double, false>;
+        return hot ? (const void *)k_push_tiles<false, double, true> : (const void *)k_push_tiles<false, double, false>;
     }
-    if (W) return hot ? (const void *)k_push_scatter<true, float, true> : (const void *)k_push_scatter<true, float, false>;
-    return hot ? (const void *)k_push_scatter<false, float, true> : (const void *)k_push_scatter<false, float, false>;
+    if (W) return hot ? (const void *)k_push_tiles<true, float, true> : (const void *)k_push_tiles<true, float, false>;
+    return hot ? (const void *)k_push_tiles<false, float, true> : (const void *)k_push_tiles<false, float, false>;
 }
 
 // Width of the push accumulator.  FP64 sums make the scattered result independent
@@ -1034,6 +1052,9 @@ static bool push_fp64(const gp_graph *g, int64_t max_updates) {
     return fits || max_updates > PUSH_FP32_MAX_UPDATES;
 }
 
+// Whether the out- and in-edges are one array pair.
+static bool one_order(const gp_graph *g) { return g->csr_off == g->csc_off; }
+
 // One power iteration y = base + d * post_scale * (gather or scatter over the
 // given adjacency) of a PageRank-type linear system, with on-device
 // convergence; used for the forward pass and for the adjoint.
@@ -1043,8 +1064,8 @@ struct IterSpec {
     const int64_t *off;
     const int32_t *idx;
     const float *w;
-    const BigBins *bins;  // push and adjoint pull: the chunks of the long lists
-    EdgeTiles *tiles;     // forward pull: the adjacency's tiles (built on first use); nullptr: adjoint pull
+    EdgeTiles *tiles;     // the adjacency's tiles (built on first use); nullptr: adjoint pull,
+    const BigBins *bins;  // which takes the chunks of its long lists
     const float *s;   // base vector (nullable: uniform base_uniform)
     float s_scale, base_uniform, d;
     const float *x0;  // start vector (nullable: 1/n)
@@ -1062,7 +1083,6 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     PrStatus *status = (PrStatus *)w.status;
     const bool push = sp.push;
     const bool W = sp.w != nullptr;
-    const BigBins &bins = *sp.bins;
 
     PrArgs a;
     memset(&a, 0, sizeof(a));
@@ -1070,12 +1090,14 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     a.off = sp.off;
     a.idx = sp.idx;
     a.w = sp.w;
-    a.big = bins.big;
-    a.cstart = bins.cstart;
-    a.chunks = bins.chunks;
-    a.nbig = bins.nbig;
-    a.nchunks = bins.nchunks;
-    a.light_max = bins.light_max;
+    if (sp.bins) {
+        a.big = sp.bins->big;
+        a.cstart = sp.bins->cstart;
+        a.chunks = sp.bins->chunks;
+        a.nbig = sp.bins->nbig;
+        a.nchunks = sp.bins->nchunks;
+        a.light_max = sp.bins->light_max;
+    }
     a.s = sp.s;
     a.s_scale = sp.s_scale;
     a.base_uniform = sp.base_uniform;
@@ -1094,10 +1116,10 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     const bool tiled = !push && sp.tiles;
     bool loop = false;  // all sweeps in one launch
     if (!push && !tiled) {
-        if (!w.chunk_part) GP_TRY(w.mem.alloc(w.chunk_part, (size_t)std::max<int64_t>(bins.nchunks, 1), s));
+        if (!w.chunk_part) GP_TRY(w.mem.alloc(w.chunk_part, (size_t)std::max<int64_t>(a.nchunks, 1), s));
         a.chunk_part = w.chunk_part;
     }
-    if (tiled) {
+    if (sp.tiles) {
         GP_TRY(build_tiles(g, *sp.tiles, sp.off, s));
         const EdgeTiles &t = *sp.tiles;
         a.m = g->m;
@@ -1110,7 +1132,9 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         a.ntiles = t.ntiles;
         a.nrows = t.nrows;
         a.nlong = t.nlong;
-        loop = t.ntiles <= LOOP_TILES;
+        loop = !push && t.ntiles <= LOOP_TILES;
+    }
+    if (tiled) {
         if (sp.hot && !loop) {
             if (g->pull_hot.slots != g->opt.pull_hot_slots) GP_TRY(build_pull_hot(g, g->opt.pull_hot_slots, s));
             hot = g->pull_hot.nhot > 0;
@@ -1123,7 +1147,6 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
             a.nhot = g->pull_hot.nhot;
             a.idx = g->pull_hot.enc_idx;
         }
-        a.vec_tiles = ((uintptr_t)a.idx | (uintptr_t)a.w) % 32 == 0 ? (int32_t)(a.m / TILE_EDGES) : 0;
     }
     if (push && sp.hot) {
         if (g->push_hot.slots != g->opt.push_hot_slots) GP_TRY(build_push_hot(g, g->opt.push_hot_slots, s));
@@ -1135,6 +1158,7 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
             a.idx = g->push_hot.enc_idx;
         }
     }
+    a.vec_tiles = ((uintptr_t)a.idx | (uintptr_t)a.w) % 32 == 0 ? (int32_t)(a.m / TILE_EDGES) : 0;
     int g1, g2;
     const int tpt = TILE_THREADS;
     const void *kl = nullptr;  // the kernel of all sweeps
@@ -1142,9 +1166,9 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         int ob = 0, ol = 0;
         GP_TRY(occupancy(w, W ? (const void *)k_adj_big<true> : (const void *)k_adj_big<false>, 1024, 0, ob));
         GP_TRY(occupancy(w, W ? (const void *)k_adj_light<true> : (const void *)k_adj_light<false>, 512, 0, ol));
-        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (bins.nchunks + 31) / 32));
+        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (a.nchunks + 31) / 32));
         a.split_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ol * g->num_sms, (ntiles + 15) / 16));
-        g2 = a.split_blocks + (int)((bins.nbig + 511) / 512);
+        g2 = a.split_blocks + (int)((a.nbig + 511) / 512);
     } else if (loop) {
         // a warp per tile and a thread per row where the grid holds that many, and no
         // more blocks than that to wait for
@@ -1169,14 +1193,11 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (a.ntiles + wpb - 1) / wpb));
         g2 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)of * g->num_sms, (n + 255) / 256));
     } else {
-        // one grid for big chunks and light tiles; as many resident blocks as fit,
-        // capped by blocks_per_sm (256-thread units)
         const void *ks = push_kernel(W, push_fp64(g, sp.max_updates), hot);
         int os = 0;
-        GP_TRY(occupancy(w, ks, 1024, smem, os));
-        const int cap = std::max(1, g->opt.blocks_per_sm / 4) * g->num_sms;
-        const int64_t work = std::max<int64_t>((bins.nchunks + 31) / 32, (ntiles + 31) / 32);
-        g1 = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>((int64_t)os * g->num_sms, cap), work));
+        GP_TRY(occupancy(w, ks, TILE_THREADS, smem, os));
+        const int wpb = TILE_THREADS / 32;
+        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)os * g->num_sms, (a.ntiles + wpb - 1) / wpb));
         g2 = (int)std::max<int64_t>(1, std::min<int64_t>(gb, (n + 255) / 256));
     }
     if (g2 > w.max_blocks) return set_error(GP_ERR_INVALID, "internal: partials too small");
@@ -1224,9 +1245,9 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
             b.c_next = C[0];
             const void *ks = push_kernel(W, fp64, hot);
             {
-                ProfScope ps("push_scatter", s);
+                ProfScope ps("push_tiles", s);
                 void *args[] = {&b};
-                GP_CUDA(cudaLaunchKernel(ks, dim3((unsigned)g1), dim3(1024), args, smem, s));
+                GP_CUDA(cudaLaunchKernel(ks, dim3((unsigned)g1), dim3(TILE_THREADS), args, smem, s));
             }
             if (fp64)
                 GP_LAUNCH("push_epilogue", s, (k_push_epilogue<double><<<g2, 256, 0, s>>>(b)));
@@ -1421,8 +1442,8 @@ extern "C" int gp_pagerank(const gp_graph *gc, int mode, float damping, int iter
     sp.off = push ? g->csr_off : g->csc_off;
     sp.idx = push ? g->csr_idx : g->csc_idx;
     sp.w = g->weighted ? (push ? g->csr_w : g->csc_w) : nullptr;
-    sp.bins = &g->push_bins;
-    sp.tiles = &g->tiles;
+    sp.tiles = push && !one_order(g) ? &g->out_tiles : &g->tiles;
+    sp.bins = nullptr;
     sp.s = S;
     sp.s_scale = 1.0f - damping;
     sp.base_uniform = (float)((1.0 - (double)damping) / (double)n);
@@ -1492,8 +1513,8 @@ extern "C" int gp_pagerank_backward(const gp_graph *gc, int mode, float damping,
     sp.off = push ? g->csc_off : g->csr_off;
     sp.idx = push ? g->csc_idx : g->csr_idx;
     sp.w = g->weighted ? (push ? g->csc_w : g->csr_w) : nullptr;
-    sp.bins = push ? &g->pull_bins : &g->push_bins;
-    sp.tiles = nullptr;
+    sp.tiles = push ? &g->tiles : nullptr;
+    sp.bins = &g->push_bins;
     sp.s = G;
     sp.s_scale = 1.0f;
     sp.base_uniform = 0.f;

@@ -1002,7 +1002,7 @@ int gp_options_default(gp_options *opt) {
     opt->bfs_beta = 24.0f;
     opt->push_fp64_accum = -1;
     opt->pull_hot_slots = 20480;
-    opt->push_hot_slots = 32768;
+    opt->push_hot_slots = 24576;  // two blocks of accumulators per SM
     opt->sssp_alpha = 1.0f;
     opt->fe_alpha = 8.0f;
     opt->bc_alpha = 1.0f;
@@ -1273,6 +1273,7 @@ int gp_graph_free(gp_graph *g) {
     g->pull_hot.mem.release(s);
     g->push_hot.mem.release(s);
     g->tiles.mem.release(s);
+    g->out_tiles.mem.release(s);
     g->mem.release(s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (dev != g->device && dev >= 0) cudaSetDevice(dev);
@@ -1297,7 +1298,7 @@ int gp_graph_info_get(const gp_graph *g, gp_graph_info *info) {
     info->symmetric = g->symmetric;
     info->weighted = g->weighted;
     info->device_bytes = (int64_t)(g->mem.total + g->pull_bins.mem.total + g->push_bins.mem.total +
-                                   g->bfs_bins.mem.total + g->tiles.mem.total + g->pr.mem.total +
+                                   g->bfs_bins.mem.total + g->tiles.mem.total + g->out_tiles.mem.total + g->pr.mem.total +
                                    g->bfs.mem.total + g->bfs.mmem.total);
     return GP_OK;
 }

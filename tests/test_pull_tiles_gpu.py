@@ -121,3 +121,32 @@ def test_tiles_of_larger_graphs(gp, bulk, weighted, slots, shift):
     x, st = gp.pagerank(G, gp.PULL, 0.85, 200, 1e-6)  # stopped by the residual, within its bound of the fixed point
     err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
     assert st["converged"] and st["residual"] < 1e-6 and st["iters_done"] < 200 and err.sum() <= 1e-6 / 0.15 + L1
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("slots", [0, 5])
+@pytest.mark.parametrize("name", list(DEGREES))
+def test_push_tiles(gp, name, slots, weighted, shift):
+    """The same lists as out-edges: the push sweep's tiles, heads that several of a tile's sources share among them."""
+    import torch
+
+    n, csc_off, csc_idx, csc_w, csr_off, csr_idx, csr_w = make(DEGREES[name], seed=len(name))
+    out = np.maximum(np.bincount(np.repeat(np.arange(n), np.diff(csr_off)), minlength=n), 1)
+    csr_w = csr_w / out[np.repeat(np.arange(n), np.diff(csr_off))]  # scaled down: what leaves a source stays below 1
+    csc_w = csr_w[np.argsort(csr_idx, kind="stable")]
+
+    def dev(a, dt):
+        return torch.cat([torch.zeros(shift, dtype=dt), torch.from_numpy(np.ascontiguousarray(a)).to(dt)]).cuda()[shift:]
+
+    w = [dev(csr_w, torch.float32), dev(csc_w, torch.float32)] if weighted else [None, None]
+    G = gp.Graph(n, dev(csr_off, torch.int64), dev(csr_idx, torch.int32), dev(csc_off, torch.int64),
+                 dev(csc_idx, torch.int32), *w, validate=True)
+    G.set_options(push_hot_slots=slots, push_fp64_accum=1)
+    wx = csc_w.astype(np.float32).astype(np.float64) if weighted else None
+    for iters in (1, 3):
+        ref = sweeps(n, csr_off, csc_off, csc_idx, wx, iters)
+        x, st = gp.pagerank(G, gp.PUSH, 0.85, iters)
+        err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
+        assert st["push_updates_l2"] + st["push_updates_shared"] + st["push_updates_merged"] == csr_idx.size * iters
+        assert err.max() <= MAX_ABS and err.sum() <= L1, (name, iters, float(err.max()), float(err.sum()))
