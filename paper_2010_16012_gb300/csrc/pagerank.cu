@@ -106,14 +106,16 @@ __device__ __forceinline__ bool pr_stopped(const PrStatus *status) {
 // Convergence gate at the start of sweep k: every block reduces the residual
 // partials of sweep k-1 in the same order, so all blocks take the same
 // decision; block 0 records it.  Returns true when the iteration has stopped.
-__device__ bool pr_gate(const PrArgs &a, int k) {
+// With tol = 0 there is nothing to decide: only the record after the last sweep
+// (`record`) reduces them, and the sweeps start 2 us earlier.
+__device__ bool pr_gate(const PrArgs &a, int k, bool record = false) {
     __shared__ double sm[32];
     __shared__ int stop;
     volatile PrStatus *st = a.status;
     if (threadIdx.x == 0) stop = st->done;
     __syncthreads();
     if (stop) return true;
-    if (k > 1) {
+    if (k > 1 && (a.tol > 0.0 || record)) {
         double r = 0.0;
         for (int i = threadIdx.x; i < a.nprev; i += blockDim.x) r += a.partials[i];
         r = block_sum(r, sm);
@@ -169,7 +171,7 @@ __global__ void k_pr_init(int64_t n, const float *x0, const float *cmul, float *
 // sweep, and writes the status into the host's mapped mirror slot: the host
 // polls it with no copy, so polling never waits behind other transfers.
 __global__ void k_pr_finish(PrArgs a, PrStatus *mirror) {
-    pr_gate(a, a.k);
+    pr_gate(a, a.k, true);
     if (threadIdx.x == 0) {
         *mirror = *a.status;  // the gate ended with a block barrier
         __threadfence_system();
@@ -556,14 +558,20 @@ constexpr int BIG_UNROLL = 8;
 // they do not push the gathered contribution vector out of L2.
 __device__ __forceinline__ int32_t ld_idx(const int32_t *p) { return __ldcs(p); }
 
-template <bool W>
-__global__ void __launch_bounds__(1024) k_adj_big(PrArgs a) {
-    if (pr_gate(a, a.k)) return;
+// The row's new value.  Rounded as written here, whatever is around it: left to
+// the compiler, the base's product and this one compete for the fused addition,
+// and short and long rows were rounded unlike (fused, and not), which stays.
+__device__ __forceinline__ float adj_value(const PrArgs &a, float base, float ps, float sum, bool long_row) {
+    const float g = __fmul_rn(ps, sum);
+    return long_row ? __fadd_rn(base, __fmul_rn(a.d, g)) : __fmaf_rn(a.d, g, base);
+}
+
+// The long rows' chunks, chunk j by warp j mod nwarps.
+template <bool W, bool LOOP>
+__device__ __forceinline__ void adj_big_step(const PrArgs &a, int64_t warp, int64_t nwarps) {
     const int lane = lane_id();
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int32_t *__restrict__ idx = a.idx;
-    const float *__restrict__ c = a.c;
+    const float *c = a.c;
     const float *__restrict__ w = a.w;
     for (int64_t j = warp; j < a.nchunks; j += nwarps) {
         const Chunk ch = a.chunks[j];
@@ -584,12 +592,12 @@ __global__ void __launch_bounds__(1024) k_adj_big(PrArgs a) {
                 const int i = i0 + q * 32 + lane;
                 f[q] = 0.f;
                 if (i < ch.len) {
-                    f[q] = __ldg(c + u[q]);
-                    if (W) f[q] *= __ldg(wp + i);
+                    f[q] = gather_c<false, LOOP>(c, nullptr, u[q]);
+                    if (W) f[q] = __fmul_rn(f[q], __ldg(wp + i));
                 }
             }
 #pragma unroll
-            for (int q = 0; q < BIG_UNROLL; ++q) acc += f[q];
+            for (int q = 0; q < BIG_UNROLL; ++q) acc = __fadd_rn(acc, f[q]);
         }
         acc = warp_sum(acc);
         if (lane == 0) a.chunk_part[j] = acc;
@@ -598,88 +606,160 @@ __global__ void __launch_bounds__(1024) k_adj_big(PrArgs a) {
 
 constexpr int LIGHT_UNROLL = 8;  // in-edges of a light vertex in flight per lane
 
-template <bool W>
-__global__ void __launch_bounds__(512, 3) k_adj_light(PrArgs a) {
-    __shared__ double sm[32];
-    if (pr_stopped(a.status)) return;
+// The short rows, 32 vertices to a warp.
+template <bool W, bool LOOP>
+__device__ __forceinline__ void adj_light_step(const PrArgs &a, int64_t warp, int64_t nwarps, ResSum &res) {
     const int lane = lane_id();
-    ResSum res;
     const int64_t n = a.n;
-    if ((int)blockIdx.x < a.split_blocks) {
-        const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        const int64_t nwarps = ((int64_t)a.split_blocks * blockDim.x) >> 5;
-        const int64_t ntiles = (n + 31) >> 5;
-        const int32_t *__restrict__ idx = a.idx;
-        const float *__restrict__ c = a.c;
-        const float *__restrict__ wv = a.w;
-        // offsets of the first tile; inside the loop the next tile's are fetched early
-        int64_t t = warp;
-        int64_t nb = 0, ne = 0;
-        if (t < ntiles && t * 32 + lane < n) {
-            nb = a.off[t * 32 + lane];
-            ne = a.off[t * 32 + lane + 1];
+    const int64_t ntiles = (n + 31) >> 5;
+    const int32_t *__restrict__ idx = a.idx;
+    const float *c = a.c;
+    const float *__restrict__ wv = a.w;
+    // offsets of the first tile; inside the loop the next tile's are fetched early
+    int64_t t = warp;
+    int64_t nb = 0, ne = 0;
+    if (t < ntiles && t * 32 + lane < n) {
+        nb = a.off[t * 32 + lane];
+        ne = a.off[t * 32 + lane + 1];
+    }
+    for (; t < ntiles; t += nwarps) {
+        const int64_t v = t * 32 + lane;
+        const int64_t b = nb, e = ne;
+        // per-vertex operands, independent of the edges: issued now
+        float xv = 0.f, cm = 0.f, ps = 0.f, base_v = 0.f;
+        if (v < n) {
+            xv = a.x[v];
+            cm = c_factor(a, v);
+            ps = post_factor(a, v);
+            base_v = base_term(a, v);
         }
-        for (; t < ntiles; t += nwarps) {
-            const int64_t v = t * 32 + lane;
-            const int64_t b = nb, e = ne;
-            // per-vertex operands, independent of the edges: issued now
-            float xv = 0.f, cm = 0.f, ps = 0.f, base_v = 0.f;
-            if (v < n) {
-                xv = a.x[v];
-                cm = c_factor(a, v);
-                ps = post_factor(a, v);
-                base_v = base_term(a, v);
-            }
-            const int64_t tn = t + nwarps, vn = tn * 32 + lane;
-            nb = ne = 0;
-            if (tn < ntiles && vn < n) {
-                nb = a.off[vn];
-                ne = a.off[vn + 1];
-            }
-            const int64_t dd = e - b;
-            const bool big = dd > a.light_max;
-            // a light vertex's own lane sums its in-list, LIGHT_UNROLL loads in flight
-            const int64_t e1 = big ? b : e;
-            float acc = 0.f;
-            for (int64_t p0 = b; p0 < e1; p0 += LIGHT_UNROLL) {
-                int32_t u[LIGHT_UNROLL];
-                float f[LIGHT_UNROLL];
+        const int64_t tn = t + nwarps, vn = tn * 32 + lane;
+        nb = ne = 0;
+        if (tn < ntiles && vn < n) {
+            nb = a.off[vn];
+            ne = a.off[vn + 1];
+        }
+        const int64_t dd = e - b;
+        const bool big = dd > a.light_max;
+        // a light vertex's own lane sums its in-list, LIGHT_UNROLL loads in flight
+        const int64_t e1 = big ? b : e;
+        float acc = 0.f;
+        for (int64_t p0 = b; p0 < e1; p0 += LIGHT_UNROLL) {
+            int32_t u[LIGHT_UNROLL];
+            float f[LIGHT_UNROLL];
 #pragma unroll
-                for (int q = 0; q < LIGHT_UNROLL; ++q) u[q] = p0 + q < e1 ? ld_idx(idx + p0 + q) : 0;
+            for (int q = 0; q < LIGHT_UNROLL; ++q) u[q] = p0 + q < e1 ? ld_idx(idx + p0 + q) : 0;
 #pragma unroll
-                for (int q = 0; q < LIGHT_UNROLL; ++q) {
-                    f[q] = 0.f;
-                    if (p0 + q < e1) {
-                        f[q] = __ldg(c + u[q]);
-                        if (W) f[q] *= __ldg(wv + p0 + q);
-                    }
+            for (int q = 0; q < LIGHT_UNROLL; ++q) {
+                f[q] = 0.f;
+                if (p0 + q < e1) {
+                    f[q] = gather_c<false, LOOP>(c, nullptr, u[q]);
+                    if (W) f[q] = __fmul_rn(f[q], __ldg(wv + p0 + q));
                 }
+            }
 #pragma unroll
-                for (int q = 0; q < LIGHT_UNROLL; ++q) acc += f[q];
-            }
-            if (v < n && !big) {
-                const float y = base_v + a.d * (ps * acc);
-                res.add(y, xv);
-                a.y[v] = y;
-                a.c_next[v] = y * cm;
-            }
+            for (int q = 0; q < LIGHT_UNROLL; ++q) acc = __fadd_rn(acc, f[q]);
         }
-    } else {
-        const int64_t nth = (int64_t)(gridDim.x - a.split_blocks) * blockDim.x;
-        for (int64_t r = (int64_t)(blockIdx.x - a.split_blocks) * blockDim.x + threadIdx.x; r < a.nbig; r += nth) {
-            const int32_t v = a.big[r];
-            float acc = 0.f;
-            const int64_t c1 = a.cstart[r + 1];
-#pragma unroll 8
-            for (int64_t j = a.cstart[r]; j < c1; ++j) acc += a.chunk_part[j];
-            const float y = base_term(a, v) + a.d * (post_factor(a, v) * acc);
+        if (v < n && !big) {
+            const float y = adj_value(a, base_v, ps, acc, false);
+            res.add(y, xv);
+            a.y[v] = y;
+            a.c_next[v] = y * cm;
+        }
+    }
+}
+
+// The long rows' chunk sums, one after another: a warp loads 32 at a time and
+// every lane adds them in their order (a thread that walked a hub's 200 took
+// most of the kernel's time).
+__device__ __forceinline__ void adj_combine_step(const PrArgs &a, int64_t warp, int64_t nwarps, ResSum &res) {
+    const int lane = lane_id();
+    for (int64_t r0 = warp * 32; r0 < a.nbig; r0 += nwarps * 32) {
+        const int64_t r = r0 + lane;
+        int64_t c0 = 0, c1 = 0;
+        int32_t v = 0;
+        if (r < a.nbig) {
+            v = a.big[r];
+            c0 = a.cstart[r];
+            c1 = a.cstart[r + 1];
+        }
+        float acc = 0.f;
+        const bool wide = c1 - c0 > 16;
+        if (!wide) {
+#pragma unroll 4
+            for (int64_t j = c0; j < c1; ++j) acc += a.chunk_part[j];
+        }
+        for (unsigned m = __ballot_sync(FULL, wide); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const int64_t b = __shfl_sync(FULL, c0, l), e = __shfl_sync(FULL, c1, l);
+            float sum = 0.f;
+            for (int64_t j = b; j < e; j += 32) {
+                const float part = j + lane < e ? a.chunk_part[j + lane] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const float p = __shfl_sync(FULL, part, i);
+                    if (j + i < e) sum += p;
+                }
+            }
+            if (lane == l) acc = sum;
+        }
+        if (r < a.nbig) {
+            const float y = adj_value(a, base_term(a, v), post_factor(a, v), acc, true);
             res.add(y, a.x[v]);
             a.y[v] = y;
             a.c_next[v] = y * c_factor(a, v);
         }
     }
+}
+
+template <bool W>
+__global__ void __launch_bounds__(1024) k_adj_big(PrArgs a) {
+    if (pr_gate(a, a.k)) return;
+    adj_big_step<W, false>(a, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((int64_t)gridDim.x * blockDim.x) >> 5);
+}
+
+template <bool W>
+__global__ void __launch_bounds__(512, 3) k_adj_light(PrArgs a) {
+    __shared__ double sm[32];
+    if (pr_stopped(a.status)) return;
+    ResSum res;
+    if ((int)blockIdx.x < a.split_blocks)
+        adj_light_step<W, false>(a, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                                 ((int64_t)a.split_blocks * blockDim.x) >> 5, res);
+    else
+        adj_combine_step(a, ((int64_t)(blockIdx.x - a.split_blocks) * blockDim.x + threadIdx.x) >> 5,
+                         ((int64_t)(gridDim.x - a.split_blocks) * blockDim.x) >> 5, res);
     const double r = block_residual(res, sm);
     if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
+}
+
+// All sweeps of a small graph's adjoint in one cooperative launch, as k_pull_loop.
+template <bool W>
+__global__ void __launch_bounds__(512, 3) k_adj_loop(const __grid_constant__ PrLoop P) {
+    __shared__ double sm[32];
+    PrArgs a = P.a;
+    const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
+    const int64_t warp = thread >> 5, nwarps = nthreads >> 5;
+    double residual = 0.0;
+    int k = 1;
+    for (;; ++k) {
+        a.x = P.R[(k - 1) & 1];
+        a.y = P.R[k & 1];
+        a.c = P.C[(k - 1) & 1];
+        a.c_next = P.C[k & 1];
+        ResSum res;
+        adj_big_step<W, true>(a, warp, nwarps);
+        adj_light_step<W, true>(a, warp, nwarps, res);
+        if (!grid_sync(P.sync, gridDim.x)) return;
+        adj_combine_step(a, warp, nwarps, res);
+        const double r = block_residual(res, sm);
+        if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
+        if (!grid_sync(P.sync, gridDim.x)) return;
+        if (loop_end(P, k, sm, residual)) break;
+    }
+    if (k & 1)  // the caller's buffer is R[0]
+        for (int64_t v = thread; v < a.n; v += nthreads) P.R[0][v] = P.R[1][v];
+    if (thread == 0) loop_status(P, k, residual);
 }
 
 // Owner lane of virtual edge `eid` in a tile: the last lane k with excl[k] <= eid
@@ -721,7 +801,7 @@ __device__ __forceinline__ void scatter_add(T *y, float *sh, int32_t dst, float 
 // Bound by the latency of its chains (indices, row, contribution) and the
 // shared-memory atomics, not by the reductions in L2: without those it is 4%
 // faster.  So what pays is equal work per lane and full occupancy: tiles and two
-// blocks per SM take R-MAT n = 1.0M (30M edges) from PUSH_WAS to PUSH_NOW us a sweep, where a
+// blocks per SM take R-MAT n = 1.0M (30M edges) from 150 to 110 us a sweep, where a
 // warp walked each 256-edge piece of a long list, a merged stream of the short
 // ones found every edge's source by a search over the warp, and one block of
 // 32768 accumulators filled the SM's shared memory.
@@ -1116,6 +1196,7 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     const bool tiled = !push && sp.tiles;
     bool loop = false;  // all sweeps in one launch
     if (!push && !tiled) {
+        loop = g->m <= LOOP_TILES * TILE_EDGES;
         if (!w.chunk_part) GP_TRY(w.mem.alloc(w.chunk_part, (size_t)std::max<int64_t>(a.nchunks, 1), s));
         a.chunk_part = w.chunk_part;
     }
@@ -1160,15 +1241,22 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     }
     a.vec_tiles = ((uintptr_t)a.idx | (uintptr_t)a.w) % 32 == 0 ? (int32_t)(a.m / TILE_EDGES) : 0;
     int g1, g2;
-    const int tpt = TILE_THREADS;
+    int tpt = TILE_THREADS;    // its threads per block
     const void *kl = nullptr;  // the kernel of all sweeps
-    if (!push && !tiled) {
+    if (!push && !tiled && loop) {
+        int ob = 0;
+        kl = W ? (const void *)k_adj_loop<true> : (const void *)k_adj_loop<false>;
+        tpt = 512;
+        GP_TRY(occupancy(w, kl, tpt, 0, ob));
+        g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (std::max(a.nchunks, ntiles) + 15) / 16));
+        g2 = g1;
+    } else if (!push && !tiled) {
         int ob = 0, ol = 0;
         GP_TRY(occupancy(w, W ? (const void *)k_adj_big<true> : (const void *)k_adj_big<false>, 1024, 0, ob));
         GP_TRY(occupancy(w, W ? (const void *)k_adj_light<true> : (const void *)k_adj_light<false>, 512, 0, ol));
         g1 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ob * g->num_sms, (a.nchunks + 31) / 32));
         a.split_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ol * g->num_sms, (ntiles + 15) / 16));
-        g2 = a.split_blocks + (int)((a.nbig + 511) / 512);
+        g2 = a.split_blocks + (int)std::min<int64_t>((a.nbig + 511) / 512, (int64_t)ol * g->num_sms);
     } else if (loop) {
         // a warp per tile and a thread per row where the grid holds that many, and no
         // more blocks than that to wait for
@@ -1276,9 +1364,9 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
         volatile PrStatus *host = (PrStatus *)w.status_host + 2;
         host->iters_done = -1;  // the launch's last block of work replaces it
         {
-            ProfScope ps("pull_loop", s);
+            ProfScope ps(tiled ? "pull_loop" : "adj_loop", s);
             void *args[] = {&P};
-            GP_CUDA(cudaLaunchCooperativeKernel(kl, dim3((unsigned)g1), dim3(TILE_THREADS), args, 0, s));
+            GP_CUDA(cudaLaunchCooperativeKernel(kl, dim3((unsigned)g1), dim3((unsigned)tpt), args, 0, s));
         }
         GP_CUDA(cudaStreamSynchronize(s));
         if (host->iters_done < 0) return set_error(GP_ERR_TIMEOUT, "PageRank: a grid barrier wait ran out");
