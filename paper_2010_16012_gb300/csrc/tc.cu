@@ -140,7 +140,10 @@ __global__ void k_tc_finish(int64_t n, int push, unsigned long long *tc, unsigne
 
 // ------------------------------------------------------------------ directed lists
 
-constexpr int TC_WARP_OUT = 64;     // out-neighbours up to which a warp counts for a vertex
+// Out-neighbours up to which a warp counts for a vertex.  Kernel times at 16, 32
+// and 64: R-MAT 2^18 1070, 1041 and 1188 us, n = 50K 180, 197 and 302, n = 400K 2406,
+// 2143 and 2165; uniform 260K (lists of about 16) 810, 200 and 200.
+constexpr int TC_WARP_OUT = 32;
 constexpr int TC_MAX_OUT = 8192;    // and a block (table of at most 16384 entries)
 constexpr int TC_WARP_TABLE = 256;  // entries of a warp's table
 constexpr int TC_WARPS = 8;         // warps per block of the counting kernels
@@ -391,8 +394,7 @@ __device__ __forceinline__ void tc_own(const TcRun &R, int32_t u, unsigned long 
 }
 
 // Measured on R-MAT 2^18 (3.8M undirected edges, 6.6e8 list elements streamed):
-// k_tc 47.9 ms; the two kernels below 629 + 639 us (88% of issue slots busy),
-// the gather 22 us.  TC_WARP_OUT: 126K vertices count in warps and 13K in blocks there.
+// k_tc 47.9 ms; this kernel and the next but one 290 + 752 us, the gather 16 us.
 // A warp per vertex u of few out-neighbours.  Its out-neighbours' lists, 32 at a
 // time, are one stream of edges over the lanes (whatever their lengths), four
 // windows of 32 in flight (a list each where they average 32 elements and more).
@@ -478,10 +480,10 @@ __global__ void __launch_bounds__(TC_WARPS * 32) k_tc_warp(TcRun R) {
             sum = warp_sum(sum);
             __syncwarp();
             // counts read by every lane before any entry is freed
-            int c[TC_WARP_OUT / 32], at[TC_WARP_OUT / 32];
-            unsigned h[TC_WARP_OUT / 32];
+            int c[(TC_WARP_OUT + 31) / 32], at[(TC_WARP_OUT + 31) / 32];
+            unsigned h[(TC_WARP_OUT + 31) / 32];
 #pragma unroll
-            for (int q = 0; q < TC_WARP_OUT / 32; ++q) {
+            for (int q = 0; q < (TC_WARP_OUT + 31) / 32; ++q) {
                 const int64_t p = b + 32 * q + lane;
                 const int32_t x = p < e ? R.out[p] : 0;
                 at[q] = p < e ? T.find(x) : -1;
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32) k_tc_warp(TcRun R) {
             }
             __syncwarp();
 #pragma unroll
-            for (int q = 0; q < TC_WARP_OUT / 32; ++q) {
+            for (int q = 0; q < (TC_WARP_OUT + 31) / 32; ++q) {
                 if (at[q] < 0) continue;
                 T.key[at[q]] = TC_FREE;
                 T.cnt[at[q]] = 0;
@@ -562,6 +564,91 @@ __global__ void __launch_bounds__(TC_WARPS * 32) k_tc_block(TcRun R) {
     if (threadIdx.x == 0 && total) atomicAdd(R.total, total);
 }
 
+// The same with u's out-neighbours as a bitmap over all vertices, for graphs
+// whose bitmap fits in shared memory: a search is one load and a test, and a
+// hit's place in the list is the word's first place and a bit count, with no
+// probing.  Bound by the bank conflicts of those loads and of the counts (13
+// cycles of an SM per 32 elements): 629 -> 529 us on R-MAT 2^18.
+constexpr int TC_BITS_WARPS = 16;
+constexpr int64_t TC_BITS_MAX = int64_t(1) << 19;  // vertices: two blocks of 96 KB per SM
+
+__global__ void __launch_bounds__(TC_BITS_WARPS * 32) k_tc_bits(TcRun R, int64_t n) {
+    extern __shared__ int32_t s_table[];
+    __shared__ long long s_ticket;
+    __shared__ unsigned long long s_sum[32];
+    const int lane = lane_id(), wib = threadIdx.x >> 5;
+    const int nwords = (int)((n + 31) >> 5);
+    uint32_t *bits = (uint32_t *)s_table;
+    int *cnt = s_table + nwords;                       // [the longest list]
+    uint16_t *first = (uint16_t *)(cnt + R.table);     // place in the list of a word's first vertex
+    for (int i = threadIdx.x; i < nwords; i += blockDim.x) bits[i] = 0u;
+    unsigned long long total = 0;
+    while (true) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_ticket = (long long)atomicAdd(R.ticket, 1ull);
+        __syncthreads();
+        const int64_t t = s_ticket;
+        if (t >= R.count) break;
+        const int32_t u = R.list[t];
+        const int64_t b = R.out_off[u], e = R.out_off[u + 1];
+        for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
+            const int32_t x = R.out[p];
+            if (p == b || R.out[p - 1] >> 5 != x >> 5) first[x >> 5] = (uint16_t)(p - b);
+            atomicOr(bits + (x >> 5), 1u << (x & 31));
+            cnt[p - b] = 0;
+        }
+        __syncthreads();
+        unsigned long long sum = 0;
+        for (int64_t p0 = b + wib; p0 < e; p0 += 32 * TC_BITS_WARPS) {
+            // the warp's next 32 lists located at once
+            const int64_t p = p0 + (int64_t)lane * TC_BITS_WARPS;
+            int64_t lb = 0;
+            int len = 0;
+            if (p < e) {
+                const int32_t v = R.out[p];
+                lb = R.out_off[v];
+                len = (int)(R.out_off[v + 1] - lb);
+            }
+            const int lists = __popc(__ballot_sync(FULL, p < e));
+            for (int i = 0; i < lists; ++i) {
+                const int32_t *list = R.out + __shfl_sync(FULL, lb, i);
+                const int l = __shfl_sync(FULL, len, i);
+                int hits = 0;
+                constexpr int U = 4;
+                for (int j = lane; j < l; j += 32 * U) {
+                    int32_t x[U];
+#pragma unroll
+                    for (int q = 0; q < U; ++q) x[q] = j + 32 * q < l ? __ldg(list + j + 32 * q) : -1;
+#pragma unroll
+                    for (int q = 0; q < U; ++q) {
+                        if (x[q] < 0) continue;
+                        const uint32_t word = bits[x[q] >> 5], bit = 1u << (x[q] & 31);
+                        if (word & bit) {
+                            atomicAdd(cnt + first[x[q] >> 5] + __popc(word & (bit - 1u)), 1);
+                            ++hits;
+                        }
+                    }
+                }
+                hits = __reduce_add_sync(FULL, hits);
+                if (lane == i && hits) {
+                    atomicAdd(cnt + (p - b), hits);
+                    sum += (unsigned)hits;
+                }
+            }
+        }
+        sum = block_sum(sum, s_sum);  // (a block barrier: every count is in)
+        for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
+            tc_give(R, p, cnt[p - b]);
+            bits[R.out[p] >> 5] = 0u;
+        }
+        if (threadIdx.x == 0) {
+            tc_own(R, u, sum);
+            total += sum;
+        }
+    }
+    if (threadIdx.x == 0 && total) atomicAdd(R.total, total);
+}
+
 // pull: a vertex's count is its own triangles and those its in-neighbours
 // counted for it.  Long in-lists take a block each (a warp over 25K entries took
 // 0.5 ms), shorter ones a warp, the others a thread.
@@ -612,7 +699,7 @@ struct gp_tc_work {
     int64_t nlight = 0, nheavy = 0;
     int32_t *mid = nullptr, *wide = nullptr;     // vertices by in-list (gather)
     int64_t nmid = 0, nwide = 0;
-    int table = 0;
+    int table = 0, max_out = 0;
     unsigned long long probes = 0;
     Arena mem;
 };
@@ -687,6 +774,7 @@ static int build_tc(gp_graph *g, gp_tc_work &w, cudaStream_t s) {
             if (e != cudaSuccess) r = set_error(GP_ERR_CUDA, "triangle lists: %s", cudaGetErrorString(e));
         }
         w.fresh = st;  // whether every edge has its reverse is read with the first counts
+        w.max_out = (int)hs.max_out;
         w.table = 4 * TC_WARP_OUT;
         while (w.table < 2 * TC_MAX_OUT && w.table < 4 * (int64_t)hs.max_out) w.table *= 2;
     }
@@ -717,15 +805,25 @@ static int run_tc(gp_graph *g, const gp_tc_work &w, bool push, unsigned long lon
     R.tc = tc;
     R.total = scal;
     if (w.nheavy > 0) {
-        const size_t smem = (size_t)w.table * (2 * sizeof(int32_t) + TC_FILTER / 8);
+        const bool bits = g->n <= TC_BITS_MAX;
+        const size_t words = (size_t)((g->n + 31) >> 5);
+        const size_t smem = bits ? words * (sizeof(uint32_t) + sizeof(uint16_t)) + (size_t)w.max_out * sizeof(int32_t) + 4
+                                 : (size_t)w.table * (2 * sizeof(int32_t) + TC_FILTER / 8);
+        const void *kernel = bits ? (const void *)k_tc_bits : (const void *)k_tc_block;
+        const int threads = (bits ? TC_BITS_WARPS : TC_WARPS) * 32;
         int per_sm = 0;
-        GP_CUDA(cudaFuncSetAttribute(k_tc_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_block, TC_WARPS * 32, smem));
+        GP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
         R.list = w.heavy;
         R.count = w.nheavy;
         R.ticket = scal + 1;
         const int b = (int)std::max<int64_t>(1, std::min<int64_t>(w.nheavy, (int64_t)std::max(per_sm, 1) * g->num_sms));
-        GP_LAUNCH("tc_block", s, (k_tc_block<<<b, TC_WARPS * 32, smem, s>>>(R)));
+        if (bits) {
+            R.table = w.max_out;
+            GP_LAUNCH("tc_bits", s, (k_tc_bits<<<b, threads, smem, s>>>(R, g->n)));
+        } else {
+            GP_LAUNCH("tc_block", s, (k_tc_block<<<b, threads, smem, s>>>(R)));
+        }
         GP_TRY(check_launch("tc_block"));
     }
     if (w.nlight > 0) {

@@ -112,3 +112,25 @@ def test_one_way_edges(gp, mode):
         if mode == 1:
             assert np.array_equal(tc.cpu().numpy(), ref)
         assert st["probes"] == probes
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("n", [(1 << 19) - 1, 1 << 19, (1 << 19) + 1])
+def test_bitmap_and_table(gp, n, mode):
+    """A clique at each end of the ids of a graph at, below and above the vertices whose bitmap fits in shared
+    memory (the hash table from there on), joined by one edge."""
+    import torch
+
+    k = 90
+    a = np.concatenate([np.arange(k), np.arange(n - k, n)])
+    u, v = np.triu_indices(k, 1)
+    src = np.concatenate([a[u], a[k + u], [a[0]]])
+    dst = np.concatenate([a[v], a[k + v], [a[-1]]])
+    src, dst = np.concatenate([src, dst]), np.concatenate([dst, src])
+    order = np.lexsort((dst, src))
+    off = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=n))])
+    G = gp.Graph(n, torch.from_numpy(off).cuda(), torch.from_numpy(dst[order]).int().cuda(), symmetric=True)
+    tc, total, _ = gp.triangles(G, mode)
+    ref = np.zeros(n, dtype=np.int64)
+    ref[a] = math.comb(k - 1, 2)
+    assert total == 2 * math.comb(k, 3) and np.array_equal(tc.cpu().numpy(), ref)
