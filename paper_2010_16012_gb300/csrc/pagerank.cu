@@ -662,7 +662,7 @@ __device__ __forceinline__ void adj_light_step(const PrArgs &a, int64_t warp, in
         }
         if (v < n && !big) {
             const float y = adj_value(a, base_v, ps, acc, false);
-            res.add(y, xv);
+            if (!LOOP) res.add(y, xv);  // (the loop draws its rows in no fixed order)
             a.y[v] = y;
             a.c_next[v] = y * cm;
         }
@@ -734,12 +734,26 @@ __global__ void __launch_bounds__(512, 3) k_adj_light(PrArgs a) {
 }
 
 // All sweeps of a small graph's adjoint in one cooperative launch, as k_pull_loop.
+// A block's warps draw its units -- 32 short rows, or a long row's chunk, short rows
+// first as they take longest -- from a counter in shared memory: units differ
+// severalfold in time, and with a fixed share for every warp (5.4 chunks and 1.1
+// groups of rows at R-MAT 2^18) half of the sweep was waiting for the last ones.
+// 34 -> 26 us a sweep there; the chunks first measured 30, a draw ahead of the work 27.
+// Rows' values don't depend on who computes them; the residual's FP64 sum would, so
+// a sweep that needs it takes the short rows' part in a pass of its own.
 template <bool W>
 __global__ void __launch_bounds__(512, 3) k_adj_loop(const __grid_constant__ PrLoop P) {
     __shared__ double sm[32];
     PrArgs a = P.a;
+    __shared__ int drawn[2];
     const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int64_t warp = thread >> 5, nwarps = nthreads >> 5;
+    const int wib = threadIdx.x >> 5;
+    // the block's groups of rows and chunks: those congruent to its number
+    const int64_t B = gridDim.x, b = blockIdx.x;
+    const int rows = (int)((((a.n + 31) >> 5) - b + B - 1) / B);
+    const int units = rows + (int)((a.nchunks - b + B - 1) / B);
+    if (threadIdx.x < 2) drawn[threadIdx.x] = 0;
+    __syncthreads();
     double residual = 0.0;
     int k = 1;
     for (;; ++k) {
@@ -747,11 +761,23 @@ __global__ void __launch_bounds__(512, 3) k_adj_loop(const __grid_constant__ PrL
         a.y = P.R[k & 1];
         a.c = P.C[(k - 1) & 1];
         a.c_next = P.C[k & 1];
+        if (threadIdx.x == 0) drawn[(k + 1) & 1] = 0;  // the next sweep's, behind two barriers
         ResSum res;
-        adj_big_step<W, true>(a, warp, nwarps);
-        adj_light_step<W, true>(a, warp, nwarps, res);
+        for (;;) {
+            int u = 0;
+            if (lane_id() == 0) u = atomicAdd(&drawn[k & 1], 1);
+            u = __shfl_sync(FULL, u, 0);
+            if (u >= units) break;
+            if (u < rows)
+                adj_light_step<W, true>(a, b + (int64_t)u * B, 1 << 30, res);
+            else
+                adj_big_step<W, true>(a, b + (int64_t)(u - rows) * B, 1 << 30);
+        }
         if (!grid_sync(P.sync, gridDim.x)) return;
-        adj_combine_step(a, warp, nwarps, res);
+        if (a.tol > 0.0 || k == P.iters)
+            for (int64_t v = thread; v < a.n; v += nthreads)
+                if (a.off[v + 1] - a.off[v] <= a.light_max) res.add(a.y[v], a.x[v]);
+        adj_combine_step(a, wib * B + b, nthreads >> 5, res);
         const double r = block_residual(res, sm);
         if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
         if (!grid_sync(P.sync, gridDim.x)) return;

@@ -58,3 +58,28 @@ def test_rows(gp, light, chunk, weighted, bulk):
         assert st["iters_done"] == iters if tol == 0.0 else st["converged"] and st["iters_done"] < 400
         bound = (deg.max() + 4) * 2.0 ** -24 / (1 - d) * np.abs(lam).max()
         assert np.abs(gs.cpu().numpy() - (1 - d) * lam).max() <= (1 - d) * bound + 1e-7
+
+
+@pytest.mark.parametrize("tol", [0.0, 1e-3])
+def test_drawn_units_repeat(gp, tol):
+    """More groups of rows and chunks than warps, drawn in no fixed order: the same
+    bits, sweeps and residual each time (no rounding may depend on who adds)."""
+    import torch
+
+    rng = np.random.default_rng(3)
+    n = 300_000
+    deg = rng.integers(0, 9, n)
+    deg[rng.integers(0, n, 2000)] = rng.integers(33, 900, 2000)
+    src = np.repeat(np.arange(n), deg)
+    dst = rng.integers(0, n, src.size)
+    order = np.argsort(dst, kind="stable")
+    dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(dt).cuda()  # noqa: E731
+    off = lambda x: dev(np.concatenate([[0], np.cumsum(np.bincount(x, minlength=n))]), torch.int64)  # noqa: E731
+    G = gp.Graph(n, off(src), dev(dst, torch.int32), off(dst), dev(src[order], torch.int32))
+    g = dev(rng.standard_normal(n), torch.float32)
+    x = torch.full((n,), 1.0 / n, device="cuda")
+    runs = [gp.pagerank_backward(G, x, g, gp.PULL, 0.85, 12 if tol == 0.0 else 400, tol, want_weights=False)
+            for _ in range(3)]
+    for _, gs, st in runs[1:]:
+        assert torch.equal(gs, runs[0][1])
+        assert (st["iters_done"], st["residual"]) == (runs[0][2]["iters_done"], runs[0][2]["residual"])
