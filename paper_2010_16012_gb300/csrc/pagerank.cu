@@ -324,8 +324,8 @@ __device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh
 // ~300 G/s from L2).  Equal tiles keep every lane's eight gathers in use at any
 // degree, where a warp per long list and a lane per short one left most of them
 // idle at degrees near 16: a sweep of a uniform graph (n = 8.0M, m = 128M) took
-// 555 + 335 us split that way and takes 458 + 62 us; R-MAT 22 (m = 128M) 295 +
-// 84 + 4 us, now 280 + 25 us (40 or 32 registers, 768 or 1024 threads a block:
+// 555 + 335 us split that way and takes 462 + 61 us; R-MAT 22 (m = 128M) 295 +
+// 84 + 4 us, now 252 + 22 us (40 or 32 registers, 768 or 1024 threads a block:
 // within 1% there; 768 is 10% faster on a graph of 16K vertices).
 template <bool W, bool HOT>
 __global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_tiles(PrArgs a) {
@@ -336,12 +336,18 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_tiles(PrArgs a) {
                             (int)(gridDim.x * blockDim.x) >> 5);
 }
 
-// The vertex's new iterate from its gathered sum.
+// What a vertex's new iterate takes beside its gathered sum.
+struct PullRow {
+    float x, base, post, c;
+    __device__ __forceinline__ PullRow(const PrArgs &a, int64_t v)
+        : x(a.x[v]), base(base_term(a, v)), post(post_factor(a, v)), c(c_factor(a, v)) {}
+};
+
 template <bool HOT>
-__device__ __forceinline__ void pull_write(const PrArgs &a, int64_t v, float sum, ResSum &res) {
-    const float y = base_term(a, v) + a.d * (post_factor(a, v) * sum);
-    const float cn = y * c_factor(a, v);
-    res.add(y, a.x[v]);
+__device__ __forceinline__ void pull_write(const PrArgs &a, int64_t v, const PullRow &row, float sum, ResSum &res) {
+    const float y = row.base + a.d * (row.post * sum);
+    const float cn = y * row.c;
+    res.add(y, row.x);
     a.y[v] = y;
     a.c_next[v] = cn;
     if (HOT) store_hot(a.hot_bits, a.hot_prefix, a.c_hot, v, cn);
@@ -349,19 +355,25 @@ __device__ __forceinline__ void pull_write(const PrArgs &a, int64_t v, float sum
 
 // Rows, then, in the first two sweeps, the vertices without in-edges: theirs is
 // the base term in every sweep, so both iterate buffers hold it from then on.
+// Bound by memory, and short of it by latency: the next row's number and a row's
+// operands are fetched before they are needed (n = 8.0M, 36 bytes a row: 68 -> 61
+// us; R-MAT 22: 26 -> 22.5; four rows a thread were slower than one).
 template <bool HOT>
 __device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread, int64_t nthreads, ResSum &res) {
     const int64_t count = a.k <= 2 ? a.n : a.nrows;
+    uint32_t next = thread < count ? (uint32_t)a.rows[thread] : 0u;
     for (int64_t r = thread; r < count; r += nthreads) {
-        const uint32_t code = (uint32_t)a.rows[r];
+        const uint32_t code = next;
+        if (r + nthreads < count) next = (uint32_t)a.rows[r + nthreads];
         const int64_t v = code & ~HOT_BIT;
         float sum = r < a.nrows ? a.acc[r] : 0.f;
+        const PullRow row(a, v);
         if (code & HOT_BIT) {  // the row spans tiles
             const int64_t t0 = a.off[v] / TILE_EDGES, t1 = (a.off[v + 1] - 1) / TILE_EDGES;
             if (t1 - t0 > TILE_LONG) continue;  // below
             for (int64_t t = t0 + 1; t <= t1; ++t) sum += a.carry[t];
         }
-        pull_write<HOT>(a, v, sum, res);
+        pull_write<HOT>(a, v, row, sum, res);
     }
     const int lane = lane_id();
     for (int64_t i = thread >> 5; i < a.nlong; i += nthreads >> 5) {
@@ -371,7 +383,7 @@ __device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread
         float sum = 0.f;
         for (int64_t t = t0 + 1 + lane; t <= t1; t += 32) sum += a.carry[t];
         sum = warp_sum(sum);
-        if (lane == 0) pull_write<HOT>(a, v, a.acc[r] + sum, res);
+        if (lane == 0) pull_write<HOT>(a, v, PullRow(a, v), a.acc[r] + sum, res);
     }
 }
 
