@@ -119,6 +119,7 @@ struct BigBins {
     int64_t *cstart = nullptr;  // [nbig + 1] first chunk of each big vertex
     Chunk *chunks = nullptr;    // [nchunks]
     int32_t *rank = nullptr;    // [n] position of v in `big`, -1 for light vertices
+    double *sums = nullptr;     // [nchunks] weight sums (normalised graphs' out-lists)
     int32_t light_max = 0;
     int32_t chunk_edges = 0;
     Arena mem;

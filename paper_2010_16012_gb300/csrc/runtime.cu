@@ -806,6 +806,7 @@ int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, i
     b.cstart = nullptr;
     b.chunks = nullptr;
     b.rank = nullptr;
+    b.sums = nullptr;
     b.light_max = light_max;
     b.chunk_edges = chunk_edges;
     const int64_t n = g->n;
@@ -838,6 +839,8 @@ int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, i
     }
     tmp.release(s);
     if (st != GP_OK) return st;
+    // (here, so that new weights need no allocation)
+    if (&b == &g->push_bins && g->normalized) GP_TRY(b.mem.alloc(b.sums, (size_t)std::max<int64_t>(nchunks, 1), s));
     b.nbig = nbig;
     b.nchunks = nchunks;
     return GP_OK;
@@ -881,18 +884,15 @@ __global__ void k_weight_scale(const int64_t *off, const float *w, int64_t n, co
 int weight_scale(gp_graph *g, cudaStream_t s) {
     if (g->n == 0) return GP_OK;
     const BigBins &b = g->push_bins;
-    Arena tmp;
-    double *part = nullptr;
-    GP_TRY(tmp.alloc(part, (size_t)std::max<int64_t>(b.nchunks, 1), s));
+    if (!b.sums)  // a rebuild found no memory
+        GP_TRY(build_bins(g, g->push_bins, g->csr_off, g->opt.push_light_max, g->opt.chunk_edges, s));
     if (b.nchunks > 0) {
         const int cb = (int)std::min<int64_t>((b.nchunks + 7) / 8, (int64_t)g->num_sms * 8);
-        GP_LAUNCH("weight_chunks", s, (k_weight_chunks<<<cb, 256, 0, s>>>(b.chunks, b.nchunks, g->csr_w, part)));
+        GP_LAUNCH("weight_chunks", s, (k_weight_chunks<<<cb, 256, 0, s>>>(b.chunks, b.nchunks, g->csr_w, b.sums)));
     }
     const int vb = (int)std::min<int64_t>((g->n + 255) / 256, (int64_t)g->num_sms * 8);
-    GP_LAUNCH("weight_scale", s, (k_weight_scale<<<vb, 256, 0, s>>>(g->csr_off, g->csr_w, g->n, b.rank, b.cstart, part, g->inv_deg)));
-    const int st = check_launch("weight_scale");
-    tmp.release(s);
-    return st;
+    GP_LAUNCH("weight_scale", s, (k_weight_scale<<<vb, 256, 0, s>>>(g->csr_off, g->csr_w, g->n, b.rank, b.cstart, b.sums, g->inv_deg)));
+    return check_launch("weight_scale");
 }
 
 }  // namespace gp
