@@ -1,6 +1,7 @@
 // bc.cu -- betweenness centrality by Brandes' scheme with push- and
 // pull-based steps (the paper's Section 3 BC listing), a batch of sources per
-// persistent cooperative launch.
+// persistent cooperative launch: groups of blocks take sources from one counter
+// and run them side by side, each group with its own workspace and barrier.
 //
 // Forward phase of a source s: a level-synchronous BFS that counts shortest
 // paths, sigma(w) = sum of sigma(u) over the in-neighbours u one level closer.

@@ -16,11 +16,10 @@
 // bitmap (the winner of each claim also sets the vertex's bit), so a switch to
 // bottom-up needs no conversion; a bottom-up level produces only the bitmap,
 // which is compacted into a queue when the search switches back.  Bottom-up
-// levels visit only the 32-vertex words that still hold candidates: a bitmap
-// of vertices with in-edges that may be unvisited, thinned by each bottom-up
-// level (vertices claimed top-down are dropped when a bottom-up level meets
-// them).  Frontier vertices whose out-degree exceeds
-// push_light_max are kept as chunk ids of the push chunk table, so one warp
+// levels visit only the 32-vertex words that still hold candidates: the bitmap
+// of unvisited vertices with in-edges, from which both kinds of level take what
+// they reach.  Frontier vertices whose out-degree exceeds
+// bfs_light_max are kept as chunk ids of the push chunk table, so one warp
 // handles at most chunk_edges of a hub's edges.
 // The direction heuristic (not given in the paper, which cites direction-
 // optimising BFS in Section 1 and describes switching thresholds as

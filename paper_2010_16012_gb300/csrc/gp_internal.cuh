@@ -287,6 +287,7 @@ int exclusive_scan(const int64_t *in, int64_t *out, int64_t N, Arena &tmp, cudaS
 int select_by_degree(const int64_t *off, int64_t n, int64_t lo, int64_t hi, Arena &mem, int32_t *&list,
                      int64_t &count, int64_t cap, int32_t *rank, cudaStream_t s);
 int grid_blocks(const gp_graph *g, int threads_per_block);
+int allow_smem(const void *kernel);
 
 // ------------------------------------------------------------------ device primitives
 

@@ -1106,7 +1106,7 @@ static int occupancy(PrWork &w, const void *kernel, int threads, size_t smem, in
             return GP_OK;
         }
     // the opt-in is needed whenever dynamic + static shared memory exceeds 48 KiB; set it for any size
-    if (smem > 0) GP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 0) GP_TRY(allow_smem(kernel));
     GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem));
     if (blocks < 1) return set_error(GP_ERR_UNSUPPORTED, "kernel does not fit on an SM (%zu B shared memory)", smem);
     w.fits.push_back({kernel, threads, smem, blocks});

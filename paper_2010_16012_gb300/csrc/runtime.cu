@@ -793,6 +793,19 @@ int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s) {
     return GP_OK;
 }
 
+// Raises a kernel's dynamic shared-memory limit to the most a block can have.
+// Always to the same value: the limit is the process's, not the launch's, and
+// another graph (or thread) may be about to launch the kernel with more.
+int allow_smem(const void *kernel) {
+    cudaFuncAttributes at;
+    int dev = 0, most = 0;
+    GP_CUDA(cudaFuncGetAttributes(&at, kernel));
+    GP_CUDA(cudaGetDevice(&dev));
+    GP_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    GP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes));
+    return GP_OK;
+}
+
 int grid_blocks(const gp_graph *g, int threads_per_block) {
     int per_sm = std::max(1, g->opt.blocks_per_sm * 256 / std::max(32, threads_per_block));
     return std::max(1, g->num_sms * per_sm);

@@ -812,7 +812,7 @@ static int run_tc(gp_graph *g, const gp_tc_work &w, bool push, unsigned long lon
         const void *kernel = bits ? (const void *)k_tc_bits : (const void *)k_tc_block;
         const int threads = (bits ? TC_BITS_WARPS : TC_WARPS) * 32;
         int per_sm = 0;
-        GP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        GP_TRY(allow_smem(kernel));
         GP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
         R.list = w.heavy;
         R.count = w.nheavy;

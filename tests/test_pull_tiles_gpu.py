@@ -150,3 +150,28 @@ def test_push_tiles(gp, name, slots, weighted, shift):
         err = np.abs(x.cpu().numpy().astype(np.float64) - ref)
         assert st["push_updates_l2"] + st["push_updates_shared"] + st["push_updates_merged"] == csr_idx.size * iters
         assert err.max() <= MAX_ABS and err.sum() <= L1, (name, iters, float(err.max()), float(err.sum()))
+
+
+@pytest.mark.parametrize("mode", ["PUSH", "PULL"])
+def test_hot_set_sizes_in_turn(gp, mode):
+    """A large hot set, a small one and the large one again, on one graph and with another graph's in between: every
+    size's shared memory is to be had each time.  Equal to the run without a hot set within the orders' rounding."""
+    import torch
+
+    rng = np.random.default_rng(1)
+    n = 60_000
+    deg = rng.integers(0, 300, n)  # over 32768 tiles: a launch per step
+    src = np.repeat(np.arange(n), deg)
+    dst = rng.integers(0, n, src.size)
+    order = np.argsort(dst, kind="stable")
+    off = lambda x: torch.from_numpy(np.concatenate([[0], np.cumsum(np.bincount(x, minlength=n))])).cuda()  # noqa: E731
+    arrays = off(src), torch.from_numpy(dst).int().cuda(), off(dst), torch.from_numpy(src[order]).int().cuda()
+    A, B = gp.Graph(n, *arrays), gp.Graph(n, *arrays)
+    key = mode.lower() + "_hot_slots"
+    ref = None
+    for G, slots in ((A, 0), (A, 40960), (A, 8192), (A, 40960), (B, 4096), (A, 40960), (B, 4096)):
+        G.set_options(**{key: slots})
+        x, _ = gp.pagerank(G, getattr(gp, mode), 0.85, 3)
+        x = x.cpu().numpy().astype(np.float64)
+        ref = x if ref is None else ref
+        assert np.abs(x - ref).max() <= MAX_ABS and np.abs(x - ref).sum() <= L1, (slots,)
