@@ -728,22 +728,24 @@ int build_push_hot(gp_graph *g, int32_t slots, cudaStream_t s) {
     return build_hot(g, g->push_hot, slots, g->csc_off, g->csr_idx, INT32_MAX, s);
 }
 
-// The list of rows: their first edges marked, the tiles told the row that
-// reaches over their start, rows over several tiles flagged.
-__global__ void k_tile_rows(int32_t *rows, int64_t nrows, const int64_t *off, int64_t ntiles, uint32_t *heads,
-                            int32_t *tile_row, int32_t *long_rows, unsigned long long *nlong) {
+// The list of rows, then the vertices without any: rows' first edges marked, the
+// tiles told the row that reaches over their start, rows over several tiles flagged.
+__global__ void k_tile_rows(const int32_t *full, int64_t nrows, const int32_t *empty, int64_t nempty, const int64_t *off,
+                            int64_t ntiles, int32_t *rows, uint32_t *heads, int32_t *tile_row, int32_t *long_rows,
+                            unsigned long long *nlong) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nrows; r += stride) {
-        const int32_t v = rows[r];
+        const int32_t v = full[r];
         const int64_t b = off[v], e = off[v + 1];
         atomicOr(heads + (b >> 5), 1u << (b & 31));
         // tiles t with b < t * TILE_EDGES <= e: the edge before their first one is this row's
         for (int64_t t = b / TILE_EDGES + 1; t <= e / TILE_EDGES && t < ntiles; ++t) tile_row[t] = (int32_t)r;
         if (r == 0) tile_row[0] = -1;
         const int64_t span = (e - 1) / TILE_EDGES - b / TILE_EDGES;
-        if (span > 0) rows[r] = (int32_t)(HOT_BIT | (uint32_t)v);
+        rows[r] = span > 0 ? (int32_t)(HOT_BIT | (uint32_t)v) : v;
         if (span > TILE_LONG) long_rows[atomicAdd(nlong, 1ull)] = (int32_t)r;
     }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nempty; i += stride) rows[nrows + i] = empty[i];
 }
 
 int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s) {
@@ -768,13 +770,10 @@ int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s) {
     if (st == GP_OK) {
         cudaError_t e = cudaMemsetAsync(nl, 0, sizeof(*nl), s);
         if (e == cudaSuccess && nt) e = cudaMemsetAsync(t.heads, 0, (size_t)nt * (TILE_EDGES / 8), s);
-        if (e == cudaSuccess && nfull) e = cudaMemcpyAsync(t.rows, full, nfull * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess && nempty)
-            e = cudaMemcpyAsync(t.rows + nfull, empty, nempty * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess && nfull) {
-            const int b = (int)std::min<int64_t>((nfull + 255) / 256, (int64_t)g->num_sms * 8);
-            GP_LAUNCH("tile_rows", s, (k_tile_rows<<<b, 256, 0, s>>>(t.rows, nfull, off, nt, (uint32_t *)t.heads, t.tile_row,
-                                                                    t.long_rows, nl)));
+        if (e == cudaSuccess && n) {
+            const int b = (int)std::min<int64_t>((n + 255) / 256, (int64_t)g->num_sms * 8);
+            GP_LAUNCH("tile_rows", s, (k_tile_rows<<<b, 256, 0, s>>>(full, nfull, empty, nempty, off, nt, t.rows,
+                                                                    (uint32_t *)t.heads, t.tile_row, t.long_rows, nl)));
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = read_mapped(&hl, nl, sizeof(hl), s);
