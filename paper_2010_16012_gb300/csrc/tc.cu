@@ -4,8 +4,8 @@
 // Every edge is directed from its end of lower degree to the other (ties by
 // id), so that a triangle has one lowest vertex u, whose other two corners v
 // and x are both out-neighbours of u and joined by v -> x.  u's warp or block
-// keeps N+(u) in a shared-memory hash table, streams N+(v) for every v in
-// N+(u), and counts the hits for each member of N+(u) beside its table entry.
+// keeps N+(u) in shared memory (a hash table or a bitmap), streams N+(v) for every v in
+// N+(u), and counts the hits for each member of N+(u) beside its entry.
 //   pull: the counts go into u's slots of its out-neighbours' in-lists, each
 //         written by u alone; then every vertex adds its own slots (only v's
 //         owner writes tc[v]);
@@ -568,7 +568,8 @@ __global__ void __launch_bounds__(TC_WARPS * 32) k_tc_block(TcRun R) {
 // whose bitmap fits in shared memory: a search is one load and a test, and a
 // hit's place in the list is the word's first place and a bit count, with no
 // probing.  Bound by the bank conflicts of those loads and of the counts (13
-// cycles of an SM per 32 elements): 629 -> 529 us on R-MAT 2^18.
+// cycles of an SM per 32 elements): 629 -> 529 us on R-MAT 2^18 with the lists of
+// more than 64, 755 with those of more than 32.
 constexpr int TC_BITS_WARPS = 16;
 constexpr int64_t TC_BITS_MAX = int64_t(1) << 19;  // vertices: two blocks of 96 KB per SM
 

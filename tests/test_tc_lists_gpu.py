@@ -1,5 +1,5 @@
 """Triangle counts by the directed lists at the places where they can go wrong:
-lists at and around the warp/block limit (64 out-neighbours), tables at and
+lists at and around the warp/block limit (32 out-neighbours), tables at and
 around their doublings, one and no out-neighbour, self-loops; and the inputs
 that take the listing instead (a duplicate edge, an unsorted list), against the
 listing itself.  Whole numbers: equal."""
@@ -52,7 +52,7 @@ def listing(n, rows):
 
 
 @pytest.mark.parametrize("mode", [0, 1])
-@pytest.mark.parametrize("k", [2, 3, 64, 65, 66, 129, 257, 600, 2100])
+@pytest.mark.parametrize("k", [2, 3, 32, 33, 34, 64, 65, 66, 129, 257, 600, 2100])
 def test_cliques(gp, k, mode):
     n = k + 5
     G = upload(gp, n, clique_rows(n, k))
