@@ -280,7 +280,8 @@ __global__ void __launch_bounds__(256) k_tc_lists(int64_t n, const int64_t *off,
     }
 }
 
-// rev[e]: the place of u in the in-list of x, for every directed edge e = (u -> x).
+// rev[e]: the place of u in the in-list of x, for every directed edge e = (u -> x)
+// (-1: not there; the counts made so are dropped, but stay in bounds).
 __global__ void __launch_bounds__(256) k_tc_reverse(int64_t n, const int64_t *out_off, const int64_t *in_off,
                                                     const int32_t *out, const int32_t *in, int32_t *rev, TcPlanStat *st) {
     const int lane = lane_id();
@@ -300,8 +301,8 @@ __global__ void __launch_bounds__(256) k_tc_reverse(int64_t n, const int64_t *ou
                     hi = mid;
             }
             if (lo == len || __ldg(list + lo) != (int32_t)u) {
-                bad = true;  // no edge back
-                lo = 0;
+                bad = true;  // no edge back, so no slot
+                lo = -1;
             }
             rev[e] = lo;
         }
@@ -380,10 +381,11 @@ __device__ __forceinline__ int tc_stream(const TcRun &R, int64_t b, int64_t e, c
 // What u counted for its out-neighbour of edge e: into that one's in-list slot, or onto its count.
 __device__ __forceinline__ void tc_give(const TcRun &R, int64_t e, int c) {
     const int32_t x = R.out[e];
-    if (!R.push)
-        R.slots[R.in_off[x] + R.rev[e]] = c;
-    else if (c)
+    if (!R.push) {
+        if (R.rev[e] >= 0) R.slots[R.in_off[x] + R.rev[e]] = c;
+    } else if (c) {
         atomicAdd(R.tc + x, (unsigned long long)c);
+    }
 }
 
 __device__ __forceinline__ void tc_own(const TcRun &R, int32_t u, unsigned long long t) {

@@ -134,3 +134,27 @@ def test_bitmap_and_table(gp, n, mode):
     ref = np.zeros(n, dtype=np.int64)
     ref[a] = math.comb(k - 1, 2)
     assert total == 2 * math.comb(k, 3) and np.array_equal(tc.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_one_way_edge_into_the_last_vertex(gp, mode):
+    """An edge without its reverse into the last vertex, whose in-list is empty and lies at the end of all of them
+    (and another one-way edge, so that the lists' lengths agree): nothing counted for it has a place to go."""
+    k = 6
+    n = k + 3
+    rows = [[] for _ in range(n)]
+    for v in range(2, k + 2):
+        rows[v] = [u for u in range(2, k + 2) if u != v]
+    rows[0] = [4, n - 1]        # one way to n - 1
+    rows[4] = [0] + rows[4]
+    rows[2] = [1] + rows[2]     # one way to 1
+    rows[n - 1] = [2, 3]
+    rows[2].append(n - 1)
+    rows[3].append(n - 1)
+    ref, probes = listing(n, rows)
+    G = upload(gp, n, rows)
+    for _ in range(2):
+        tc, total, st = gp.triangles(G, mode)
+        if mode == 1:
+            assert np.array_equal(tc.cpu().numpy(), ref)
+        assert st["probes"] == probes
