@@ -104,7 +104,7 @@ struct BatchDev {
     int32_t *iters_done;    // [ngraphs][K]
     const int32_t *sources; // [ngraphs][64] (MS-BFS)
     int32_t *const *lev_out;  // [ngraphs] where this call's levels go (MS-BFS)
-    int32_t *counters;      // [0] most PPR sweeps of any column, [1] BFS levels, [2] packed columns, [3], [4] those left to narrower jobs
+    int32_t *counters;      // [0] most PPR sweeps of any column, [1] BFS levels, [2] packed columns, [3], [4] those left to narrower jobs, [5] rows listed, [6] 1: not a closed set, [7] last columns
     int32_t pack_max;       // a job stops once at most this many of its columns iterate (0: never)
     BPend *pend;            // [3][ngraphs * K] the columns left iterating, in job order: for jobs of 32, 8 and 4
     float *XP0, *XP1;       // [max n][32] iterates of a packed job (rows as wide as the job)
@@ -311,6 +311,67 @@ __device__ __forceinline__ float4 sum_parts(const float *part, int64_t first, in
     return groups_total<KS>(a);
 }
 
+// The rows that a graph's last column reaches, where they are few.  The slowest
+// columns are those seeded in a component of a few vertices (their alternating
+// modes decay as d^k: five times the sweeps of the others), and all their other
+// rows are zero and stay so.  A column that has been alone for PPR_ALONE sweeps goes
+// to a job of its own (LAST), which after two sweeps lists the rows in which it is
+// not zero in either iterate (or has its seed), in the room behind the iterates;
+// R.whole stays true unless no out-edge of theirs leaves them, they are at most an
+// eighth of the rows and none has a long in-list (those go by chunks).  The sums of
+// the listed rows are the same ones in the same order, and the others need no
+// writes.  At 131K vertices a sweep of two rows takes about 35 us less than one of
+// all: six R-MAT graphs of up to 2^17 vertices with one such column, of 89 sweeps,
+// 27.4 -> 25.1 ms (handed over after 4 sweeps alone 24.6, but more columns pay for it).
+constexpr int PPR_ALONE = 10;
+struct PRows {
+    bool whole = true;
+    const int32_t *list = nullptr;
+    int64_t count = 0;
+};
+template <int KS>
+__device__ __noinline__ bool ppr_rows(const BatchDev &B, const PView &J, int32_t seed, PRows &R) {
+    const BGraph &G = B.graphs[J.graph];
+    const int64_t n = G.n;
+    const int lane = lane_id();
+    const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
+    int32_t *list = reinterpret_cast<int32_t *>(J.X1 + n * KS);  // of X1's 32 columns the job has KS
+    uint32_t *bits = reinterpret_cast<uint32_t *>(list + n);
+    int32_t *count = B.counters + 5, *out = B.counters + 6;
+    for (int64_t v0 = (gthread >> 5) * 32; v0 < n; v0 += nthreads) {
+        const int64_t v = v0 + lane;
+        const bool in = v < n && (__ldcg(J.X0 + v * KS) != 0.f || __ldcg(J.X1 + v * KS) != 0.f || v == seed);
+        const unsigned m = __ballot_sync(FULL, in);
+        const bool longest = __any_sync(FULL, in && G.csc_off[v + 1] - G.csc_off[v] > B.big_min);
+        int at = 0;
+        if (lane == 0) {
+            bits[v0 >> 5] = m;
+            if (m) at = atomicAdd(count, __popc(m));
+            if (longest) atomicOr(out, 1);
+        }
+        at = __shfl_sync(FULL, at, 0);
+        if (in) list[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
+    }
+    if (!grid_sync(B.sync, gridDim.x)) return false;
+    R.count = __ldcg(count);
+    const bool few = R.count <= n / 8;
+    if (few) {
+        bool leaves = false;
+        for (int64_t i = gthread; i < R.count; i += nthreads) {
+            const int32_t u = __ldcg(list + i);
+            for (int64_t e = G.csr_off[u]; e < G.csr_off[u + 1] && !leaves; ++e) {
+                const int32_t w = __ldg(G.csr_idx + e);
+                leaves = !((__ldcg(bits + (w >> 5)) >> (w & 31)) & 1u);
+            }
+        }
+        if (leaves) atomicOr(out, 1);
+    }
+    if (!grid_sync(B.sync, gridDim.x)) return false;
+    R.whole = !few || __ldcg(out) != 0;
+    R.list = list;
+    return true;
+}
+
 // One job: the slice's sweeps from the start vector to convergence, or until at
 // most J.leave of its columns still iterate (those are then left, at their
 // latest iterate, to a packed job).  Returns false when a grid barrier gave up.
@@ -320,7 +381,7 @@ __device__ __forceinline__ float4 sum_parts(const float *part, int64_t first, in
 // waited for before was one another: equal shares of unequal units, and a
 // second phase with a barrier of its own for the big vertices' partial rows.
 // Not inlined: the widths' loops share no registers.
-template <int KS>
+template <int KS, bool LAST = false>
 __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C) {
     constexpr int LPR = Lanes<KS>::LPR, NG = Lanes<KS>::NG;
     const int K = B.K;
@@ -358,7 +419,10 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
         }
     }
     if (gthread < 3 * KS) B.res_acc[(gthread / KS) * K + (gthread % KS)] = 0.0;
+    if (LAST && gthread == 0) B.counters[5] = B.counters[6] = 0;
     if (!grid_sync(B.sync, gridDim.x)) return false;
+    PRows R;
+    int alone = 0;  // sweeps with one column left
     // vertices per warp unit: few where the graph has few, so that every warp gets some
     int seg = BT_SEG;
     while (seg > NG && (n + seg - 1) / seg < nwarps) seg /= 2;
@@ -384,8 +448,9 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
             if (lane == 0) i = atomicAdd(&C.next[k & 1], 1);
             i = __shfl_sync(FULL, i, 0);
             const int64_t u = (int64_t)i * gridDim.x + blockIdx.x;
-            if (u >= G.nchunk + nseg) break;
-            if (u < G.nchunk) {
+            const bool few = LAST && !R.whole;  // the listed rows
+            if (u >= (few ? (R.count + seg - 1) / seg : G.nchunk + nseg)) break;
+            if (!few && u < G.nchunk) {
                 const BChunk ch = B.chunks[G.chunk0 + u];
                 const int64_t v = ch.v;
                 const int64_t o = v * ld + J.c0 + 4 * c4;
@@ -409,12 +474,14 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
                     finish_seg(B, Y, o, v, c4, x, sum, my_res, C);
                 }
             } else {
-                const int64_t v0 = (u - G.nchunk) * seg;
+                const int64_t v0 = (few ? u : u - G.nchunk) * seg;
                 int64_t ob = 0;  // the unit's lists, a vertex per lane
                 int len = 0;
-                if (lane < seg && v0 + lane < n) {
-                    ob = G.csc_off[v0 + lane];
-                    const int64_t d = G.csc_off[v0 + lane + 1] - ob;
+                int32_t lv = 0;
+                if (lane < seg && v0 + lane < (few ? R.count : n)) {
+                    if (few) lv = __ldcg(R.list + v0 + lane);
+                    ob = G.csc_off[few ? lv : v0 + lane];
+                    const int64_t d = G.csc_off[(few ? lv : v0 + lane) + 1] - ob;
                     // big vertices are done above; without in-edges a row is its base in every
                     // sweep, so both iterates hold it after two
                     len = d > B.big_min || (d == 0 && k > 2) ? -1 : (int)d;
@@ -424,8 +491,9 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
                 for (int i2 = 0; i2 < seg; i2 += NG) {
                     const int64_t b = __shfl_sync(FULL, ob, i2 + grp);
                     const int dl = __shfl_sync(FULL, len, i2 + grp);
+                    const int32_t l = LAST ? __shfl_sync(FULL, lv, i2 + grp) : 0;
                     if (dl < 0) continue;
-                    const int64_t v = v0 + i2 + grp, o = v * ld + J.c0 + 4 * c4;
+                    const int64_t v = few ? l : v0 + i2 + grp, o = v * ld + J.c0 + 4 * c4;
                     const float4 sum = value4(gather_seg(G, Xs, ld, b, b + dl, 1, c4));
                     const float4 x = __ldcg(reinterpret_cast<const float4 *>(Xc + o));
                     finish_seg(B, Y, o, v, c4, x, sum, my_res, C);
@@ -473,7 +541,8 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
         const int nact = __syncthreads_count(any);  // one column per thread (KS <= blockDim)
         last = k;
         if (!nact) break;
-        if (nact <= J.leave) {
+        if constexpr (KS == 4) alone += nact == 1;
+        if (nact <= J.leave && (KS != 4 || alone >= PPR_ALONE)) {
             // the few columns left go to a narrower job; block 0 lists them in column order
             if (blockIdx.x == 0 && threadIdx.x == 0) {
                 int at = atomicAdd(J.count, nact);
@@ -482,6 +551,8 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
             }
             break;
         }
+        if constexpr (LAST)  // both iterates are whole
+            if (k == 2 && !ppr_rows<KS>(B, J, C.seed[0], R)) return false;
     }
     // the slice's last iterate was written by sweep `last`: into X1 when odd
     if (last & 1)
@@ -512,7 +583,7 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
 // narrow job, whose sweeps gather 16 or 32 bytes per edge instead of 128 (R-MAT
 // 2^17: 97 us a sweep of 32 columns): one slow column can need five times the
 // sweeps of the others.
-template <int KS>
+template <int KS, bool LAST = false>
 __device__ bool ppr_packed(const BatchDev &B, const BPend *list, int count, int leave, BPend *next, int32_t *next_count,
                            PCols &C) {
     for (int i = 0; i < count;) {
@@ -520,7 +591,7 @@ __device__ bool ppr_packed(const BatchDev &B, const BPend *list, int count, int 
         int j = i + 1;
         while (j < count && j - i < KS && list[j].graph == g) ++j;
         const PView J = {g, B.XP0, B.XP1, KS, 0, list + i, j - i, leave, next, next_count};
-        if (!ppr_job<KS>(B, J, C)) return false;
+        if (!ppr_job<KS, LAST>(B, J, C)) return false;
         i = j;
     }
     return true;
@@ -540,12 +611,14 @@ __global__ void __launch_bounds__(BT_THREADS, GP_BT_MINB) k_ppr_persistent(const
         }
         if (!ok) return;
     }
-    // the columns the jobs left, 32 to a job; what those leave 8 to a job, then 4
+    // the columns the jobs left, 32 to a job; what those leave 8 to a job, then 4, and a
+    // slow last one by itself
     const int64_t most = (int64_t)B.ngraphs * B.K;
     volatile int32_t *count = B.counters;
     if (!ppr_packed<32>(B, B.pend, count[2], 8, B.pend + most, B.counters + 3, C)) return;
     if (!ppr_packed<8>(B, B.pend + most, count[3], 4, B.pend + 2 * most, B.counters + 4, C)) return;
-    ppr_packed<4>(B, B.pend + 2 * most, count[4], 0, nullptr, nullptr, C);
+    if (!ppr_packed<4>(B, B.pend + 2 * most, count[4], 1, B.pend, B.counters + 7, C)) return;
+    ppr_packed<4, true>(B, B.pend, count[7], 0, nullptr, nullptr, C);
 }
 
 // ------------------------------------------------------------------ batched multi-source BFS
