@@ -311,12 +311,13 @@ __device__ __forceinline__ float4 sum_parts(const float *part, int64_t first, in
     return groups_total<KS>(a);
 }
 
-// The rows that a graph's last column reaches, where they are few.  The slowest
+// The rows that a graph's last columns reach, where they are few.  The slowest
 // columns are those seeded in a component of a few vertices (their alternating
 // modes decay as d^k: five times the sweeps of the others), and all their other
 // rows are zero and stay so.  A column that has been alone for PPR_ALONE sweeps goes
-// to a job of its own (LAST), which after two sweeps lists the rows in which it is
-// not zero in either iterate (or has its seed), in the room behind the iterates;
+// to a last job (LAST), up to four of a graph together where several slices leave
+// one each.  After two sweeps it lists the rows in which any of its columns is not
+// zero in either iterate (or has its seed), in the room behind the iterates;
 // R.whole stays true unless no out-edge of theirs leaves them, they are at most an
 // eighth of the rows and none has a long in-list (those go by chunks).  The sums of
 // the listed rows are the same ones in the same order, and the others need no
@@ -330,7 +331,7 @@ struct PRows {
     int64_t count = 0;
 };
 template <int KS>
-__device__ __noinline__ bool ppr_rows(const BatchDev &B, const PView &J, int32_t seed, PRows &R) {
+__device__ __noinline__ bool ppr_rows(const BatchDev &B, const PView &J, const PCols &C, PRows &R) {
     const BGraph &G = B.graphs[J.graph];
     const int64_t n = G.n;
     const int lane = lane_id();
@@ -340,7 +341,9 @@ __device__ __noinline__ bool ppr_rows(const BatchDev &B, const PView &J, int32_t
     int32_t *count = B.counters + 5, *out = B.counters + 6;
     for (int64_t v0 = (gthread >> 5) * 32; v0 < n; v0 += nthreads) {
         const int64_t v = v0 + lane;
-        const bool in = v < n && (__ldcg(J.X0 + v * KS) != 0.f || __ldcg(J.X1 + v * KS) != 0.f || v == seed);
+        bool in = false;
+        for (int c = 0; c < J.cnt && v < n; ++c)
+            in |= __ldcg(J.X0 + v * KS + c) != 0.f || __ldcg(J.X1 + v * KS + c) != 0.f || v == C.seed[c];
         const unsigned m = __ballot_sync(FULL, in);
         const bool longest = __any_sync(FULL, in && G.csc_off[v + 1] - G.csc_off[v] > B.big_min);
         int at = 0;
@@ -552,7 +555,7 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
             break;
         }
         if constexpr (LAST)  // both iterates are whole
-            if (k == 2 && !ppr_rows<KS>(B, J, C.seed[0], R)) return false;
+            if (k == 2 && !ppr_rows<KS>(B, J, C, R)) return false;
     }
     // the slice's last iterate was written by sweep `last`: into X1 when odd
     if (last & 1)
@@ -611,8 +614,8 @@ __global__ void __launch_bounds__(BT_THREADS, GP_BT_MINB) k_ppr_persistent(const
         }
         if (!ok) return;
     }
-    // the columns the jobs left, 32 to a job; what those leave 8 to a job, then 4, and a
-    // slow last one by itself
+    // the columns the jobs left, 32 to a job; what those leave 8 to a job, then 4, and the
+    // slow last one of each of these on the rows that they reach
     const int64_t most = (int64_t)B.ngraphs * B.K;
     volatile int32_t *count = B.counters;
     if (!ppr_packed<32>(B, B.pend, count[2], 8, B.pend + most, B.counters + 3, C)) return;
