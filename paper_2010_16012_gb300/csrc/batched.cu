@@ -228,7 +228,7 @@ __device__ __forceinline__ float4 value4(const Sum4 &a) {
 // Adds the groups' compensated sums of a warp (every group then holds the
 // total): error-free two-sums of the leading parts, corrections added.
 template <int KS>
-__device__ __forceinline__ float4 groups_total(Sum4 a) {
+__device__ __forceinline__ Sum4 groups_sum(Sum4 a) {
 #pragma unroll
     for (int o = Lanes<KS>::LPR; o < 32; o <<= 1) {
 #pragma unroll
@@ -241,7 +241,11 @@ __device__ __forceinline__ float4 groups_total(Sum4 a) {
             a.lo[i] = add2(add2(a.lo[i], olo), err);
         }
     }
-    return value4(a);
+    return a;
+}
+template <int KS>
+__device__ __forceinline__ float4 groups_total(const Sum4 &a) {
+    return value4(groups_sum<KS>(a));
 }
 
 // The columns one PageRank job iterates: a slice of a graph's own iterates
@@ -266,9 +270,30 @@ struct PView {
 struct PCols {
     __align__(16) int col[BT_MAX_KS], seed[BT_MAX_KS], kbase[BT_MAX_KS], active[BT_MAX_KS];
     int next[2];                              // by sweep parity: the block's next unit
-    float res[BT_THREADS / 32][32][4];        // per lane: |y - x| of its four columns
-    double wres[BT_THREADS / 32][8];          // narrow jobs: a warp's sums
+    // per lane: |y - x| of its four columns in the present unit, and in those before as hi + lo (see
+    // res_unit), pairs as packed values
+    __align__(16) float res[BT_THREADS / 32][32][4];
+    uint64_t hi[BT_THREADS / 32][32][2], lo[BT_THREADS / 32][32][2];
 };
+
+// The lane's sums of one unit into its hi + lo, error-free but for the roundings
+// of lo (2^-48 of the sum each).  Warps draw their units in no fixed order, so a
+// column's change is summed in another order in every run; that precisely, and
+// the sweep in which it falls below the tolerance is the same one.  (A unit's
+// rows have their order, so plain sums do there.)
+__device__ __forceinline__ void res_unit(PCols &C, int wib, int lane) {
+    float4 &r = *reinterpret_cast<float4 *>(C.res[wib][lane]);
+    const uint64_t x[2] = {pk(r.x, r.y), pk(r.z, r.w)};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        uint64_t &hi = C.hi[wib][lane][q], &lo = C.lo[wib][lane][q];
+        const uint64_t h = hi, t = add2(h, x[q]);
+        const uint64_t bp = sub2(t, h);
+        lo = add2(lo, add2(sub2(h, sub2(t, bp)), sub2(x[q], bp)));
+        hi = t;
+    }
+    r = make_float4(0.f, 0.f, 0.f, 0.f);
+}
 
 // Writes the lane's four columns of row v of the slice of Y from the gathered
 // sum and the row x of the current iterate, carrying stopped columns forward;
@@ -442,6 +467,8 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
         float *my_res = C.res[wib][lane];
 #pragma unroll
         for (int q = 0; q < 4; ++q) my_res[q] = 0.f;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) C.hi[wib][lane][q] = C.lo[wib][lane][q] = 0;
         if (threadIdx.x == 0) C.next[(k + 1) & 1] = 0;
         // The block's units, each to the warp that is free (equal shares of them left the warps
         // waiting for one another most of the time on small graphs): chunks of big vertices,
@@ -475,6 +502,7 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
                 if (grp == 0) {
                     const float4 x = __ldcg(reinterpret_cast<const float4 *>(Xc + o));
                     finish_seg(B, Y, o, v, c4, x, sum, my_res, C);
+                    res_unit(C, wib, lane);
                 }
             } else {
                 const int64_t v0 = (few ? u : u - G.nchunk) * seg;
@@ -501,31 +529,43 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
                     const float4 x = __ldcg(reinterpret_cast<const float4 *>(Xc + o));
                     finish_seg(B, Y, o, v, c4, x, sum, my_res, C);
                 }
+                res_unit(C, wib, lane);
             }
         }
         // the block's column residuals: the slots of every warp and group added
         // in a fixed order, then one FP64 atomic per column into the sweep's ring slot
-        if (KS < 32) {  // many groups per column: a warp's are added first
+        constexpr int SLOTS = KS < 32 ? 1 : NG;
+        if (KS < 32) {  // many groups per column: a warp's are added first, by the same sums
+            // (in FP64 six R-MAT graphs of up to 2^17 vertices, 256 columns, took 24.7 ms instead of 24.4)
+            Sum4 a;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                double r = my_res[q];
-#pragma unroll
-                for (int o = LPR; o < 32; o <<= 1) r += __shfl_xor_sync(FULL, r, o);
-                if (grp == 0) C.wres[wib][(4 * c4 + q) % 8] = r;
+            for (int q = 0; q < 2; ++q) {
+                a.hi[q] = C.hi[wib][lane][q];
+                a.lo[q] = C.lo[wib][lane][q];
             }
+            a = groups_sum<KS>(a);
+            __syncwarp();
+            if (grp == 0)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    C.hi[wib][lane][q] = a.hi[q];
+                    C.lo[wib][lane][q] = a.lo[q];
+                }
         }
         __syncthreads();
         for (int c = threadIdx.x; c < KS; c += blockDim.x) {
             if (!C.active[c]) continue;
-            double r = 0.0;
-            if (KS < 32) {
-                for (int i = 0; i < wpb; ++i) r += C.wres[i][c % 8];
-            } else {
-                ResSum t;
-                for (int i = 0; i < wpb; ++i)
-                    for (int g = 0; g < NG; ++g) t.push(C.res[i][g * LPR + c / 4][c % 4]);
-                r = t.get();
-            }
+            float t = 0.f, e = 0.f;  // as res_unit
+            for (int i = 0; i < wpb; ++i)
+                for (int g = 0; g < SLOTS; ++g) {
+                    const float hi = reinterpret_cast<const float *>(C.hi[i][g * LPR + c / 4])[c % 4];
+                    const float lo = reinterpret_cast<const float *>(C.lo[i][g * LPR + c / 4])[c % 4];
+                    const float s = t + hi;
+                    const float bp = s - t;
+                    e += (t - (s - bp)) + (hi - bp) + lo;
+                    t = s;
+                }
+            const double r = (double)t + (double)e;
             if (r != 0.0) atomicAdd(racc + c, r);
         }
         if (!grid_sync(B.sync, gridDim.x)) return false;
