@@ -496,6 +496,7 @@ __device__ __noinline__ bool ppr_job(const BatchDev &B, const PView &J, PCols &C
                         __threadfence();
                     }
                     if (__shfl_sync(FULL, done, 0) != (unsigned)ch.nch - 1u) continue;
+                    __syncwarp();  // what lane 0's fence has ordered is ordered for the warp (a shuffle orders no memory)
                     const int64_t cb = B.bcstart[ch.r] - G.chunk0;
                     sum = sum_parts<KS>(B.part + 4 * c4, cb + grp, cb + ch.nch);
                 }
