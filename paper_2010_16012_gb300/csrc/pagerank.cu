@@ -376,7 +376,8 @@ __device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread
         pull_write<HOT>(a, v, row, sum, res);
     }
     const int lane = lane_id();
-    for (int64_t i = thread >> 5; i < a.nlong; i += nthreads >> 5) {
+    // (neighbouring long rows to different blocks: in a power-law graph the longest are neighbours)
+    for (int64_t i = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < a.nlong; i += nthreads >> 5) {
         const int32_t r = a.long_rows[i];
         const int64_t v = (uint32_t)a.rows[r] & ~HOT_BIT;
         const int64_t t0 = a.off[v] / TILE_EDGES, t1 = (a.off[v + 1] - 1) / TILE_EDGES;

@@ -779,6 +779,28 @@ int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s) {
         if (e == cudaSuccess) e = read_mapped(&hl, nl, sizeof(hl), s);
         if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "edge tiles: %s", cudaGetErrorString(e));
     }
+    if (st == GP_OK && hl > 1) {  // in ascending order, whatever the order of the atomics: the residual is a sum by place
+        const int64_t words = (nfull + 31) >> 5;
+        uint32_t *bits = nullptr;
+        int64_t *counts = nullptr;
+        int32_t *prefix = nullptr;
+        st = tmp.alloc(bits, (size_t)words, s);
+        if (st == GP_OK) st = tmp.alloc(counts, (size_t)words + 1, s);
+        if (st == GP_OK) st = tmp.alloc(prefix, (size_t)words, s);
+        cudaError_t e = st == GP_OK ? cudaMemsetAsync(bits, 0, (size_t)words * sizeof(uint32_t), s) : cudaSuccess;
+        if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "edge tiles: %s", cudaGetErrorString(e));
+        if (st == GP_OK) {
+            const int lb = (int)std::min<int64_t>(((int64_t)hl + 255) / 256, 1024);
+            const int wb = (int)std::min<int64_t>((words + 255) / 256, (int64_t)g->num_sms * 8);
+            GP_LAUNCH("mark_long", s, (k_hot_mark<<<lb, 256, 0, s>>>(t.long_rows, (int64_t)hl, bits)));
+            GP_LAUNCH("long_counts", s, (k_hot_counts<<<wb, 256, 0, s>>>(bits, words, counts)));
+            st = exclusive_scan(counts, counts, words, tmp, s);
+            if (st == GP_OK) {
+                GP_LAUNCH("long_order", s, (k_hot_slots<<<wb, 256, 0, s>>>(bits, words, counts, prefix, t.long_rows)));
+                st = check_launch("long_order");
+            }
+        }
+    }
     tmp.release(s);
     if (st != GP_OK) {
         t.mem.release(s);
