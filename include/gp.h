@@ -503,9 +503,10 @@ typedef struct gp_sssp_stats {
  *               the same distance can be each other's predecessor.
  *   stats       NULL or filled on return.
  * Weights: the graph's weights as uploaded (csr_w for out-edges, csc_w for
- * in-edges; weights must be >= 0, else GP_ERR_INVALID; checked once per graph),
- * 1 for every edge of an unweighted graph.  FP32 distances: sums along a path
- * are rounded as they are formed (exact while they are integers below 2^24).
+ * in-edges; weights must be >= 0, else GP_ERR_INVALID; checked by the graph's
+ * first search and the first after gp_graph_set_weights), 1 for every edge of an
+ * unweighted graph.  FP32 distances: sums along a path are rounded as they are
+ * formed (exact while they are integers below 2^24).
  * Synchronisation as gp_bfs: with stats == NULL and device outputs the call
  * only enqueues the search; a grid-barrier timeout is then reported by the next
  * gp_sssp call on the graph.  GP_ERR_INVALID for a bad source, delta, mode or

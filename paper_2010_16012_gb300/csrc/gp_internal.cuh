@@ -277,6 +277,7 @@ int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, i
 // of m entries) with each of them replaced by HOT_BIT | slot.
 int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, const int32_t *enc_src, int min_share,
               cudaStream_t s);
+void sssp_new_weights(gp_graph *g);
 // inv_deg of a graph with normalised weights, from its current csr_w.
 int weight_scale(gp_graph *g, cudaStream_t s);
 int build_tiles(gp_graph *g, EdgeTiles &t, const int64_t *off, cudaStream_t s);

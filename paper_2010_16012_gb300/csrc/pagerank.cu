@@ -1724,6 +1724,7 @@ extern "C" int gp_graph_set_weights(gp_graph *g, const float *csr_w, const float
     cudaStream_t s = (cudaStream_t)stream;
     g->csr_w = csr_w;
     g->csc_w = shared ? csr_w : csc_w;
+    sssp_new_weights(g);
     // weights as given: the scale is 1 (0 where there are no edges) whatever they are
     return g->normalized ? weight_scale(g, s) : GP_OK;
 }

@@ -709,7 +709,7 @@ struct gp_sssp_work {
     int32_t *pred_dev = nullptr;
     void *host = nullptr;  // pinned: summary, iteration stats, barrier word
     int grid = 0;
-    int weights_ok = -1;  // -1 unknown, 0 negative or NaN weight, 1 checked
+    int weights_ok = -1;  // of the present weights: -1 unknown, 0 negative or NaN weight, 1 checked
     cudaEvent_t done_ev = nullptr;  // end of the last asynchronous search
     bool pending = false;           // its barrier status not yet checked
     Arena mem;
@@ -730,6 +730,11 @@ void release_sssp_work(gp_graph *g, cudaStream_t s) {
     g->sssp->mem.release(s);
     delete g->sssp;
     g->sssp = nullptr;
+}
+
+// The graph has other weights: the next search checks them.
+void sssp_new_weights(gp_graph *g) {
+    if (g->sssp) g->sssp->weights_ok = -1;
 }
 
 }  // namespace gp
