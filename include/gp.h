@@ -158,7 +158,8 @@ typedef struct gp_graph_info {
     int64_t push_big_chunks;
     int64_t isolated; /* vertices with no in- and no out-edges */
     int32_t symmetric, weighted;
-    int64_t device_bytes; /* library-owned device memory held by the handle */
+    int64_t device_bytes; /* library-owned device memory held by the handle: its arrays and what
+                             the calls so far have left with it (work areas, plans, hot sets) */
 } gp_graph_info;
 
 int gp_graph_info_get(const gp_graph *g, gp_graph_info *info);
@@ -596,6 +597,10 @@ typedef struct gp_bc_stats {
  *               throughout (path counts, coefficients, sums); results differ
  *               from a sequential FP64 evaluation only by summation order.
  *   stats       NULL or filled on return.
+ * Up to 16 sources run side by side (8 above 2^24 edges), each in a workspace of
+ * about 81 bytes per vertex.  The workspaces stay with the handle: as many as the
+ * calls so far could use, 4 GB of them at most, fewer where memory is short (one
+ * is enough).
  * Synchronisation as gp_sssp: with stats == NULL and device memory for
  * sources and bc_out the call only enqueues the work; a grid-barrier timeout is
  * then reported by the next gp_bc call on the graph.  GP_ERR_INVALID for a

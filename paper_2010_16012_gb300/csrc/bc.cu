@@ -924,6 +924,10 @@ void release_bc_work(gp_graph *g, cudaStream_t s) {
     g->bc = nullptr;
 }
 
+size_t bc_work_bytes(const gp_graph *g) {
+    return g->bc ? g->bc->mem.total + g->bc->hub_out.mem.total + g->bc->hub_in.mem.total + g->bc->hot.mem.total : 0;
+}
+
 }  // namespace gp
 
 static int ensure_bc_work(gp_graph *g, cudaStream_t s) {

@@ -420,6 +420,8 @@ void release_fe_work(gp_graph *g, cudaStream_t s) {
     g->fe = nullptr;
 }
 
+size_t fe_work_bytes(const gp_graph *g) { return g->fe ? g->fe->mem.total : 0; }
+
 }  // namespace gp
 
 static int ensure_fe_work(gp_graph *g, cudaStream_t s) {

@@ -939,6 +939,10 @@ void release_sssp_work(gp_graph *g, cudaStream_t s);
 void release_fe_work(gp_graph *g, cudaStream_t s);
 void release_bc_work(gp_graph *g, cudaStream_t s);
 void release_tc_work(gp_graph *g, cudaStream_t s);
+size_t sssp_work_bytes(const gp_graph *g);
+size_t fe_work_bytes(const gp_graph *g);
+size_t bc_work_bytes(const gp_graph *g);
+size_t tc_work_bytes(const gp_graph *g);
 }  // namespace gp
 
 using namespace gp;
@@ -1332,8 +1336,10 @@ int gp_graph_info_get(const gp_graph *g, gp_graph_info *info) {
     info->symmetric = g->symmetric;
     info->weighted = g->weighted;
     info->device_bytes = (int64_t)(g->mem.total + g->pull_bins.mem.total + g->push_bins.mem.total +
-                                   g->bfs_bins.mem.total + g->tiles.mem.total + g->out_tiles.mem.total + g->pr.mem.total +
-                                   g->bfs.mem.total + g->bfs.mmem.total);
+                                   g->bfs_bins.mem.total + g->pull_hot.mem.total + g->push_hot.mem.total +
+                                   g->tiles.mem.total + g->out_tiles.mem.total + g->pr.mem.total + g->bfs.mem.total +
+                                   g->bfs.mmem.total + sssp_work_bytes(g) + fe_work_bytes(g) + bc_work_bytes(g) +
+                                   tc_work_bytes(g));
     return GP_OK;
 }
 

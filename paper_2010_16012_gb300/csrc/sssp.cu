@@ -732,6 +732,8 @@ void release_sssp_work(gp_graph *g, cudaStream_t s) {
     g->sssp = nullptr;
 }
 
+size_t sssp_work_bytes(const gp_graph *g) { return g->sssp ? g->sssp->mem.total : 0; }
+
 // The graph has other weights: the next search checks them.
 void sssp_new_weights(gp_graph *g) {
     if (g->sssp) g->sssp->weights_ok = -1;

@@ -716,6 +716,8 @@ void release_tc_work(gp_graph *g, cudaStream_t s) {
     g->tc = nullptr;
 }
 
+size_t tc_work_bytes(const gp_graph *g) { return g->tc ? g->tc->mem.total : 0; }
+
 // The directed lists; general = true where the listing has to be run instead.
 static int build_tc(gp_graph *g, gp_tc_work &w, cudaStream_t s) {
     if (w.ready) return GP_OK;
