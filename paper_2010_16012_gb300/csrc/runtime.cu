@@ -1284,7 +1284,12 @@ int gp_graph_upload(gp_graph **out, int64_t n, int64_t m, const int64_t *csr_off
     }
     st = build_bins(g, g->pull_bins, g->csc_off, g->opt.pull_light_max, g->opt.chunk_edges, s);
     if (st == GP_OK) st = build_bins(g, g->push_bins, g->csr_off, g->opt.push_light_max, g->opt.chunk_edges, s);
-    if (st == GP_OK && g->normalized) st = weight_scale(g, s);
+    if (st == GP_OK && g->normalized) {
+        st = weight_scale(g, s);
+        // the scale is there when the call returns, whatever stream uses it
+        cudaError_t e = st == GP_OK ? cudaStreamSynchronize(s) : cudaSuccess;
+        if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "weight sums: %s", cudaGetErrorString(e));
+    }
     if (st != GP_OK) return upload_fail(g, s, st);
     *out = g;
     return GP_OK;
