@@ -358,8 +358,12 @@ __device__ __forceinline__ void pull_write(const PrArgs &a, int64_t v, const Pul
 // Bound by memory, and short of it by latency: the next row's number and a row's
 // operands are fetched before they are needed (n = 8.0M, 36 bytes a row: 68 -> 61
 // us; R-MAT 22: 26 -> 22.5; four rows a thread were slower than one).
+// long_warp: this warp's place among those that deal out the long rows.  A launch
+// of its own deals them over the blocks, the sweeps in one launch over few blocks
+// (R-MAT 2^18, directed, 40 sweeps and 40 of the adjoint: 2.45 ms, 2.48 the other way).
 template <bool HOT>
-__device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread, int64_t nthreads, ResSum &res) {
+__device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread, int64_t nthreads, int64_t long_warp,
+                                                 ResSum &res) {
     const int64_t count = a.k <= 2 ? a.n : a.nrows;
     uint32_t next = thread < count ? (uint32_t)a.rows[thread] : 0u;
     for (int64_t r = thread; r < count; r += nthreads) {
@@ -376,8 +380,7 @@ __device__ __forceinline__ void pull_finish_step(const PrArgs &a, int64_t thread
         pull_write<HOT>(a, v, row, sum, res);
     }
     const int lane = lane_id();
-    // (neighbouring long rows to different blocks: in a power-law graph the longest are neighbours)
-    for (int64_t i = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < a.nlong; i += nthreads >> 5) {
+    for (int64_t i = long_warp; i < a.nlong; i += nthreads >> 5) {
         const int32_t r = a.long_rows[i];
         const int64_t v = (uint32_t)a.rows[r] & ~HOT_BIT;
         const int64_t t0 = a.off[v] / TILE_EDGES, t1 = (a.off[v + 1] - 1) / TILE_EDGES;
@@ -393,7 +396,9 @@ __global__ void __launch_bounds__(256) k_pull_finish(PrArgs a) {
     __shared__ double sm[32];
     if (pr_stopped(a.status)) return;
     ResSum res;
-    pull_finish_step<HOT>(a, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, res);
+    // (neighbouring long rows to different blocks: in a power-law graph the longest are neighbours)
+    pull_finish_step<HOT>(a, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x,
+                          (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, res);
     const double r = block_residual(res, sm);
     if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
 }
@@ -447,7 +452,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_loop(const __grid_cons
         pull_tiles_step<W, false, true>(a, nullptr, (int)(thread >> 5), (int)(nthreads >> 5));
         if (!grid_sync(P.sync, gridDim.x)) return;
         ResSum res;
-        pull_finish_step<false>(a, thread, nthreads, res);
+        pull_finish_step<false>(a, thread, nthreads, thread >> 5, res);
         const double r = block_residual(res, sm);
         if (threadIdx.x == 0) a.partials[blockIdx.x] = r;
         if (!grid_sync(P.sync, gridDim.x)) return;
