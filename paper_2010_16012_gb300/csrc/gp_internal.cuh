@@ -271,8 +271,9 @@ struct gp_graph {
 
 namespace gp {
 
+// (sums: with room for the chunks' weight sums, so that new weights need no allocation)
 int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, int32_t chunk_edges,
-               cudaStream_t s);
+               cudaStream_t s, bool sums = false);
 // The `slots` vertices of largest degree by sel_off, and enc_src (an index array
 // of m entries) with each of them replaced by HOT_BIT | slot.
 int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, const int32_t *enc_src, int min_share,

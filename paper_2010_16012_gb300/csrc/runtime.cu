@@ -833,7 +833,7 @@ int grid_blocks(const gp_graph *g, int threads_per_block) {
 }
 
 int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, int32_t chunk_edges,
-               cudaStream_t s) {
+               cudaStream_t s, bool sums) {
     b.mem.release(s);
     b.nbig = b.nchunks = 0;
     b.big = nullptr;
@@ -872,9 +872,8 @@ int build_bins(gp_graph *g, BigBins &b, const int64_t *off, int32_t light_max, i
         if (e != cudaSuccess) st = set_error(GP_ERR_CUDA, "memset: %s", cudaGetErrorString(e));
     }
     tmp.release(s);
+    if (st == GP_OK && sums) st = b.mem.alloc(b.sums, (size_t)std::max<int64_t>(nchunks, 1), s);
     if (st != GP_OK) return st;
-    // (here, so that new weights need no allocation)
-    if (&b == &g->push_bins && g->normalized) GP_TRY(b.mem.alloc(b.sums, (size_t)std::max<int64_t>(nchunks, 1), s));
     b.nbig = nbig;
     b.nchunks = nchunks;
     return GP_OK;
@@ -918,8 +917,6 @@ __global__ void k_weight_scale(const int64_t *off, const float *w, int64_t n, co
 int weight_scale(gp_graph *g, cudaStream_t s) {
     if (g->n == 0) return GP_OK;
     const BigBins &b = g->push_bins;
-    if (!b.sums)  // a rebuild found no memory
-        GP_TRY(build_bins(g, g->push_bins, g->csr_off, g->opt.push_light_max, g->opt.chunk_edges, s));
     if (b.nchunks > 0) {
         const int cb = (int)std::min<int64_t>((b.nchunks + 7) / 8, (int64_t)g->num_sms * 8);
         GP_LAUNCH("weight_chunks", s, (k_weight_chunks<<<cb, 256, 0, s>>>(b.chunks, b.nchunks, g->csr_w, b.sums)));
@@ -1283,7 +1280,7 @@ int gp_graph_upload(gp_graph **out, int64_t n, int64_t m, const int64_t *csr_off
         g->isolated = (int64_t)hs.isolated;
     }
     st = build_bins(g, g->pull_bins, g->csc_off, g->opt.pull_light_max, g->opt.chunk_edges, s);
-    if (st == GP_OK) st = build_bins(g, g->push_bins, g->csr_off, g->opt.push_light_max, g->opt.chunk_edges, s);
+    if (st == GP_OK) st = build_bins(g, g->push_bins, g->csr_off, g->opt.push_light_max, g->opt.chunk_edges, s, g->normalized);
     if (st == GP_OK && g->normalized) {
         st = weight_scale(g, s);
         // the scale is there when the call returns, whatever stream uses it
@@ -1368,13 +1365,20 @@ int gp_graph_set_options(gp_graph *g, const gp_options *opt, void *stream) {
         return set_error(GP_ERR_INVALID, "gp_graph_set_options: option out of range");
     cudaStream_t s = (cudaStream_t)stream;
     const gp_options old = g->opt;
-    g->opt = *opt;
+    // the new chunk tables beside the old ones, which stay, with the old options, if there is no room for them
+    const bool new_pull = old.pull_light_max != opt->pull_light_max || old.chunk_edges != opt->chunk_edges;
+    const bool new_push = old.push_light_max != opt->push_light_max || old.chunk_edges != opt->chunk_edges;
+    BigBins pull, push;
     int st = GP_OK;
-    if (old.pull_light_max != opt->pull_light_max || old.chunk_edges != opt->chunk_edges)
-        st = build_bins(g, g->pull_bins, g->csc_off, opt->pull_light_max, opt->chunk_edges, s);
-    if (st == GP_OK && (old.push_light_max != opt->push_light_max || old.chunk_edges != opt->chunk_edges))
-        st = build_bins(g, g->push_bins, g->csr_off, opt->push_light_max, opt->chunk_edges, s);
-    if (st == GP_OK && (old.blocks_per_sm != opt->blocks_per_sm || old.chunk_edges != opt->chunk_edges ||
+    if (new_pull) st = build_bins(g, pull, g->csc_off, opt->pull_light_max, opt->chunk_edges, s);
+    if (st == GP_OK && new_push) st = build_bins(g, push, g->csr_off, opt->push_light_max, opt->chunk_edges, s, g->normalized);
+    if (st != GP_OK) {
+        pull.mem.release(s);
+        push.mem.release(s);
+        return st;
+    }
+    g->opt = *opt;
+    if ((old.blocks_per_sm != opt->blocks_per_sm || old.chunk_edges != opt->chunk_edges ||
                         old.pull_light_max != opt->pull_light_max || old.bfs_light_max != opt->bfs_light_max ||
                         old.push_light_max != opt->push_light_max)) {
         // workspace sizes depend on the grid and the chunk count: rebuild lazily
@@ -1383,12 +1387,16 @@ int gp_graph_set_options(gp_graph *g, const gp_options *opt, void *stream) {
         release_sssp_work(g, s);
         release_fe_work(g, s);
         release_bc_work(g, s);
-    } else if (st == GP_OK && old.bfs_groups != opt->bfs_groups) {
+    } else if (old.bfs_groups != opt->bfs_groups) {
         release_bfs_multi(g, s);  // sized for the old group count
     }
-    if (st != GP_OK) {
-        g->opt = old;
-        return st;
+    if (new_pull) {
+        g->pull_bins.mem.release(s);
+        g->pull_bins = std::move(pull);
+    }
+    if (new_push) {
+        g->push_bins.mem.release(s);
+        g->push_bins = std::move(push);
     }
     return GP_OK;
 }

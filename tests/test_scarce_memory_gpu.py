@@ -1,0 +1,99 @@
+"""Allocations that fail, each in turn: gp_graph_set_options then leaves the
+graph as it was (its chunk tables, work areas and options, and so its results)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+CALLBACKS = []  # kept: what they allocated is released through them, whenever that is
+
+
+@pytest.fixture()
+def scarce():
+    """gp, and a context in which the allocation of the given number fails."""
+    import contextlib
+
+    import torch
+
+    import paper_2010_16012_gb300 as gp
+
+    lib = gp.load()
+    left = [-1]
+
+    @gp.ALLOC_FN
+    def alloc(nbytes, stream, ctx):
+        left[0] -= 1
+        return None if left[0] == -1 else torch.cuda.caching_allocator_alloc(nbytes)
+
+    @gp.FREE_FN
+    def free(p, nbytes, stream, ctx):
+        torch.cuda.synchronize()
+        torch.cuda.caching_allocator_delete(p)
+
+    CALLBACKS.extend((alloc, free))
+
+    @contextlib.contextmanager
+    def failing(k):
+        left[0] = k
+        try:
+            yield
+        finally:
+            left[0] = -1
+
+    assert lib.gp_set_allocator(alloc, free, None) == gp.OK
+    yield gp, failing
+    assert lib.gp_set_allocator(gp.ALLOC_FN(), gp.FREE_FN(), ctypes.c_void_p()) == gp.OK
+
+
+def results(gp, G, w):
+    import torch
+
+    x, _ = gp.pagerank(G, gp.PULL, iters=5)
+    gw, gs, _ = gp.pagerank_backward(G, x, torch.ones_like(x), iters=5)
+    level, parent, _ = gp.bfs(G, 1)
+    dist, pred, _ = gp.sssp(G, 1, 0.5)
+    fe, _ = gp.pagerank_fe(G, gp.PULL, eps=-1.0, iters=5)
+    G.set_weights(*w)  # the sums of new weights use the chunk tables too
+    y, _ = gp.pagerank(G, gp.PULL, iters=5)
+    return [t.cpu().numpy() for t in (x, gw, gs, level, dist, pred, fe, y)]
+
+
+def test_options_without_memory(scarce):
+    import torch
+
+    gp, failing = scarce
+    g = gg.rmat(12, 16, seed=3, symmetrize=False)
+    rng = np.random.default_rng(0)
+    w = rng.uniform(0.1, 1.0, g.m).astype(np.float32)
+    src = np.repeat(np.arange(g.n), np.diff(g.csr_off))
+    order = np.lexsort((src, g.csr_idx))
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    G = gp.Graph(g.n, t(g.csr_off), t(g.csr_idx), t(g.csc_off), t(g.csc_idx), t(w), t(w[order]), normalize=True,
+                 validate=True)
+    both = t(w), t(w[order])
+    want = results(gp, G, both)
+    old, new = gp.options_dict(G.options()), dict(pull_light_max=8, push_light_max=4, chunk_edges=64)
+    k = 0
+    while True:
+        try:
+            with failing(k):
+                G.set_options(**new)
+            break
+        except gp.GpError as e:
+            assert e.status == gp.ERR_OOM
+        assert gp.options_dict(G.options()) == old
+        for a, b in zip(want, results(gp, G, both)):
+            assert np.array_equal(a, b)
+        k += 1
+    assert k >= 10 and G.options().chunk_edges == 64
+    for a, b in zip(want, results(gp, G, both)):  # the same but for the order of sums
+        if a.dtype == np.int32:
+            assert np.array_equal(a, b)
+        else:
+            assert np.allclose(a, b, rtol=1e-4, atol=1e-6 * np.abs(a[np.isfinite(a)]).max())
+    G.free()
