@@ -679,6 +679,7 @@ int build_hot(gp_graph *g, HotSet &h, int32_t slots, const int64_t *sel_off, con
     }
     if (st != GP_OK || edges < m / min_share) {
         tmp.release(s);
+        if (st != GP_OK) h = HotSet();  // the next call tries again
         return st;
     }
     const int64_t nhot = above + ntie, nwords = (n + 31) >> 5;

@@ -1,5 +1,6 @@
 """Allocations that fail, each in turn: gp_graph_set_options then leaves the
-graph as it was (its chunk tables, work areas and options, and so its results)."""
+graph as it was (its chunk tables, work areas and options, and so its results),
+and a hot set that found no memory is built by the next call."""
 import ctypes
 
 import numpy as np
@@ -97,3 +98,28 @@ def test_options_without_memory(scarce):
         else:
             assert np.allclose(a, b, rtol=1e-4, atol=1e-6 * np.abs(a[np.isfinite(a)]).max())
     G.free()
+
+
+def test_hot_set_without_memory(scarce):
+    gp, failing = scarce
+    g = gg.rmat(12, 16, seed=3)
+    graphs = [gp.Graph.from_graphgen(g) for _ in range(2)]
+    for G in graphs:
+        gp.pagerank(G, gp.PULL, iters=2)
+    want, _ = gp.pagerank(graphs[0], gp.PUSH, iters=5)
+    held = graphs[0].info()["device_bytes"]
+    k = 0
+    while True:
+        try:
+            with failing(k):
+                gp.pagerank(graphs[1], gp.PUSH, iters=5)
+            break
+        except gp.GpError as e:
+            assert e.status == gp.ERR_OOM
+        k += 1
+    assert k >= 8
+    x, _ = gp.pagerank(graphs[1], gp.PUSH, iters=5)
+    assert graphs[1].info()["device_bytes"] == held
+    assert np.allclose(x.cpu().numpy(), want.cpu().numpy(), rtol=1e-5)
+    for G in graphs:
+        G.free()
