@@ -784,13 +784,13 @@ static int build_tc(gp_graph *g, gp_tc_work &w, cudaStream_t s) {
         while (w.table < 2 * TC_MAX_OUT && w.table < 4 * (int64_t)hs.max_out) w.table *= 2;
     }
     tmp.release(s);
-    if (r == GP_ERR_OOM) {  // no room for the lists: the listing needs none
+    w.ready = r == GP_OK;
+    if (r == GP_ERR_OOM) {  // no room for the lists: the listing needs none, and the next call tries again
         clear_error();
         r = GP_OK;
         w.general = true;
     }
     if (w.general || r != GP_OK) w.mem.release(s);
-    w.ready = r == GP_OK;
     return r;
 }
 

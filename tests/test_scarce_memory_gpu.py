@@ -1,6 +1,7 @@
 """Allocations that fail, each in turn: gp_graph_set_options then leaves the
 graph as it was (its chunk tables, work areas and options, and so its results),
-and a hot set that found no memory is built by the next call."""
+and a hot set or the triangle counts' directed lists that found no memory are
+built by the next call."""
 import ctypes
 
 import numpy as np
@@ -123,3 +124,27 @@ def test_hot_set_without_memory(scarce):
     assert np.allclose(x.cpu().numpy(), want.cpu().numpy(), rtol=1e-5)
     for G in graphs:
         G.free()
+
+
+def test_directed_lists_without_memory(scarce):
+    gp, failing = scarce
+    g = gg.rmat(12, 16, seed=3)
+    G = gp.Graph.from_graphgen(g)
+    want, total, _ = gp.triangles(G)
+    held = G.info()["device_bytes"]
+    k, last = 0, None
+    while last != held:  # (the first call in which nothing fails leaves the lists)
+        H = gp.Graph.from_graphgen(g)
+        try:
+            with failing(k):
+                tc, t, _ = gp.triangles(H)
+            assert t == total and (tc == want).all()
+        except gp.GpError as e:
+            assert e.status == gp.ERR_OOM
+        last = H.info()["device_bytes"]
+        tc, t, _ = gp.triangles(H)  # with memory again
+        assert t == total and (tc == want).all() and H.info()["device_bytes"] == held
+        H.free()
+        k += 1
+    assert k > 3  # the offsets, the lists and a temporary list, each without memory once
+    G.free()
