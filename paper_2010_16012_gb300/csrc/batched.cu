@@ -56,8 +56,7 @@ struct BGraph {  // per-graph device descriptor
     float *X0, *X1;          // PPR iterates [n][K]; X0 doubles as the output
     uint64_t *F, *V, *N;     // MS-BFS masks
     int32_t *levels;         // MS-BFS output [n][64]
-    int64_t big0, nbig;      // big in-degree vertices of this graph in the big list
-    int64_t chunk0, nchunk;  // their in-edge chunks in the chunk list
+    int64_t chunk0, nchunk;  // in-edge chunks of its vertices of big in-degree in the chunk list
     int64_t ochunk0, nochunk;  // out-edge chunks of the vertices of big out-degree (the in-edge ones where the orders are one)
 };
 
@@ -94,10 +93,9 @@ struct BatchDev {
     const BGraph *graphs;
     const BJob *jobs;
     int njobs;
-    const int32_t *big;     // [nbig_total] vertex ids, grouped by graph
-    const int64_t *bcstart; // [nbig_total + 1] chunk range of each big vertex
+    const int64_t *bcstart; // [big vertices + 1] chunk range of each big vertex, grouped by graph
     const BChunk *chunks;
-    unsigned *bdone;        // [nbig_total] chunks of each big vertex summed in this sweep
+    unsigned *bdone;        // [big vertices] chunks of each big vertex summed in this sweep
     float *part;            // [max chunks of one graph][K] chunk partial rows
     double *res_acc;        // [3][K] per-sweep column residuals (a ring)
     const int32_t *seeds;   // [ngraphs][K]
@@ -1033,7 +1031,7 @@ static int64_t chunk_size(const gp_batch *b, int64_t m) {
 static int batch_layout(gp_batch *b, cudaStream_t s) {
     const int K = b->K;
     const int64_t big_min = b->opt.big_in_degree;
-    std::vector<int32_t> big;
+    int32_t nbig = 0;
     std::vector<int64_t> bcstart(1, 0);
     std::vector<BChunk> chunks;
     int64_t max_chunks = 1;
@@ -1047,18 +1045,15 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
         if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout: %s", cudaGetErrorString(e));
         const int64_t C = chunk_size(b, g->m);
         BGraph &G = b->hg[gi];
-        G.big0 = (int64_t)big.size();
         G.chunk0 = (int64_t)chunks.size();
         for (int64_t v = 0; v < g->n; ++v) {
             const int64_t d = off[v + 1] - off[v];
             if (d <= big_min) continue;
-            const int32_t r = (int32_t)big.size(), nch = (int32_t)((d + C - 1) / C);
-            big.push_back((int32_t)v);
+            const int32_t r = nbig++, nch = (int32_t)((d + C - 1) / C);
             for (int64_t p = off[v]; p < off[v + 1]; p += C)
                 chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v, r, nch});
             bcstart.push_back((int64_t)chunks.size());
         }
-        G.nbig = (int64_t)big.size() - G.big0;
         G.nchunk = (int64_t)chunks.size() - G.chunk0;
         max_chunks = std::max(max_chunks, G.nchunk);
         G.ochunk0 = G.chunk0;
@@ -1087,28 +1082,24 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
     }
     b->layout.release(s);
     BatchDev &D = b->dev;
-    int32_t *dbig = nullptr;
     int64_t *dbc = nullptr;
     BChunk *dch = nullptr;
     BJob *djobs = nullptr;
     int st = GP_OK;
-    if (st == GP_OK) st = b->layout.alloc(dbig, std::max<size_t>(big.size(), 1), s);
     if (st == GP_OK) st = b->layout.alloc(dbc, bcstart.size(), s);
     if (st == GP_OK) st = b->layout.alloc(dch, std::max<size_t>(chunks.size(), 1), s);
     if (st == GP_OK) st = b->layout.alloc(djobs, b->jobs.size(), s);
     if (st == GP_OK) st = b->layout.alloc(D.part, (size_t)max_chunks * K, s);
-    if (st == GP_OK) st = b->layout.alloc(D.bdone, std::max<size_t>(big.size(), 1), s);
+    if (st == GP_OK) st = b->layout.alloc(D.bdone, (size_t)std::max(nbig, 1), s);
     if (st != GP_OK) return st;
-    b->nbig = (int64_t)big.size();
+    b->nbig = nbig;
     cudaError_t e = cudaMemcpyAsync(b->dgraphs, b->hg.data(), b->ngraphs * sizeof(BGraph), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !big.empty()) e = cudaMemcpyAsync(dbig, big.data(), big.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dbc, bcstart.data(), bcstart.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && !chunks.empty()) e = cudaMemcpyAsync(dch, chunks.data(), chunks.size() * sizeof(BChunk), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(djobs, b->jobs.data(), b->jobs.size() * sizeof(BJob), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout copy: %s", cudaGetErrorString(e));
     D.big_min = big_min;
-    D.big = dbig;
     D.bcstart = dbc;
     D.chunks = dch;
     D.jobs = djobs;

@@ -65,7 +65,7 @@ struct PrArgs {
     float base_uniform;  // base term when s is nullptr: (1-d)/n
     const float *post_scale;  // factor of the gathered sum per owner (adjoint: inv_deg), or nullptr
     const float *cmul;        // c_next = y * cmul (forward: inv_deg), or nullptr (c_next = y)
-    float one_minus_d, d;
+    float d;
     double tol;
     int32_t k;  // sweep number, 1-based
     int32_t nprev;
@@ -1227,7 +1227,6 @@ static int pr_iterate(gp_graph *g, const IterSpec &sp, float *out, PrStatus &fin
     a.base_uniform = sp.base_uniform;
     a.post_scale = sp.post_scale;
     a.cmul = sp.cmul;
-    a.one_minus_d = 1.0f - sp.d;
     a.d = sp.d;
     a.tol = sp.tol;
     a.partials = w.partials;

@@ -158,7 +158,7 @@ __device__ __forceinline__ void ss_offers(const SsRun &R, uint32_t *act_next, fl
     bool same[U], later[U];
 #pragma unroll
     for (int q = 0; q < U; ++q) {
-        const bool better = old[q] != 0 && nd[q] < ss_dist(old[q]);  // (a reached key is never 0 off the source)
+        const bool better = old[q] != 0 && nd[q] < ss_dist(old[q]);  // (from a key of 0, the least, nothing is better)
         same[q] = better && nd[q] < end;
         later[q] = better && !same[q];
         const uint32_t bit = 1u << (w[q] & 31);

@@ -794,7 +794,7 @@ static int build_tc(gp_graph *g, gp_tc_work &w, cudaStream_t s) {
     return r;
 }
 
-// Counts by the directed lists into tc (nullptr: only the total, scal[0] = triangles).
+// Counts by the directed lists into tc, the number of triangles into scal[0].
 static int run_tc(gp_graph *g, const gp_tc_work &w, bool push, unsigned long long *tc, unsigned long long *scal,
                   cudaStream_t s) {
     TcRun R;
