@@ -1027,7 +1027,8 @@ static int64_t chunk_size(const gp_batch *b, int64_t m) {
 
 // Work lists for the current options: big in-degree vertices and their chunks,
 // big out-degree vertices, and the PPR jobs (column slices sized to the L2
-// budget).  Reads the offsets once; synchronises the stream.
+// budget).  Reads the offsets once; synchronises the stream.  Where something
+// fails the batch keeps the lists it had.
 static int batch_layout(gp_batch *b, cudaStream_t s) {
     const int K = b->K;
     const int64_t big_min = b->opt.big_in_degree;
@@ -1035,7 +1036,8 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
     std::vector<int64_t> bcstart(1, 0);
     std::vector<BChunk> chunks;
     int64_t max_chunks = 1;
-    b->jobs.clear();
+    std::vector<BJob> jobs;
+    std::vector<BGraph> hg = b->hg;
     const int64_t budget = (int64_t)b->opt.l2_budget_mb << 20;
     for (int gi = 0; gi < b->ngraphs; ++gi) {
         gp_graph *g = b->graphs[gi];
@@ -1044,7 +1046,7 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout: %s", cudaGetErrorString(e));
         const int64_t C = chunk_size(b, g->m);
-        BGraph &G = b->hg[gi];
+        BGraph &G = hg[gi];
         G.chunk0 = (int64_t)chunks.size();
         for (int64_t v = 0; v < g->n; ++v) {
             const int64_t d = off[v + 1] - off[v];
@@ -1061,7 +1063,7 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
         // the widest slice whose two iterates fit the budget (at least 32 columns)
         int ks = std::min(K, BT_MAX_KS);
         while (ks > 32 && 2 * g->n * (int64_t)ks * 4 > budget) ks /= 2;
-        for (int c0 = 0; c0 < K; c0 += ks) b->jobs.push_back(BJob{gi, c0, ks / 32, 0});
+        for (int c0 = 0; c0 < K; c0 += ks) jobs.push_back(BJob{gi, c0, ks / 32, 0});
     }
     // after every graph's in-edge chunks (bcstart numbers those): the out-edge ones where the orders differ
     for (int gi = 0; gi < b->ngraphs; ++gi) {
@@ -1072,7 +1074,7 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout: %s", cudaGetErrorString(e));
         const int64_t C = chunk_size(b, g->m);
-        BGraph &G = b->hg[gi];
+        BGraph &G = hg[gi];
         G.ochunk0 = (int64_t)chunks.size();
         for (int64_t v = 0; v < g->n; ++v)
             if (off[v + 1] - off[v] > big_min)
@@ -1080,34 +1082,45 @@ static int batch_layout(gp_batch *b, cudaStream_t s) {
                     chunks.push_back(BChunk{p, (int32_t)std::min<int64_t>(C, off[v + 1] - p), (int32_t)v, 0, 0});
         G.nochunk = (int64_t)chunks.size() - G.ochunk0;
     }
-    b->layout.release(s);
-    BatchDev &D = b->dev;
+    Arena layout;
+    BatchDev D = b->dev;
     int64_t *dbc = nullptr;
     BChunk *dch = nullptr;
     BJob *djobs = nullptr;
     int st = GP_OK;
-    if (st == GP_OK) st = b->layout.alloc(dbc, bcstart.size(), s);
-    if (st == GP_OK) st = b->layout.alloc(dch, std::max<size_t>(chunks.size(), 1), s);
-    if (st == GP_OK) st = b->layout.alloc(djobs, b->jobs.size(), s);
-    if (st == GP_OK) st = b->layout.alloc(D.part, (size_t)max_chunks * K, s);
-    if (st == GP_OK) st = b->layout.alloc(D.bdone, (size_t)std::max(nbig, 1), s);
-    if (st != GP_OK) return st;
-    b->nbig = nbig;
-    cudaError_t e = cudaMemcpyAsync(b->dgraphs, b->hg.data(), b->ngraphs * sizeof(BGraph), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dbc, bcstart.data(), bcstart.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
+    if (st == GP_OK) st = layout.alloc(dbc, bcstart.size(), s);
+    if (st == GP_OK) st = layout.alloc(dch, std::max<size_t>(chunks.size(), 1), s);
+    if (st == GP_OK) st = layout.alloc(djobs, jobs.size(), s);
+    if (st == GP_OK) st = layout.alloc(D.part, (size_t)max_chunks * K, s);
+    if (st == GP_OK) st = layout.alloc(D.bdone, (size_t)std::max(nbig, 1), s);
+    if (st != GP_OK) {
+        layout.release(s);
+        return st;
+    }
+    cudaError_t e = cudaMemcpyAsync(dbc, bcstart.data(), bcstart.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && !chunks.empty()) e = cudaMemcpyAsync(dch, chunks.data(), chunks.size() * sizeof(BChunk), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(djobs, b->jobs.data(), b->jobs.size() * sizeof(BJob), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(djobs, jobs.data(), jobs.size() * sizeof(BJob), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dgraphs, hg.data(), b->ngraphs * sizeof(BGraph), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return set_error(GP_ERR_CUDA, "batch layout copy: %s", cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        layout.release(s);
+        return set_error(GP_ERR_CUDA, "batch layout copy: %s", cudaGetErrorString(e));
+    }
     D.big_min = big_min;
     D.bcstart = dbc;
     D.chunks = dch;
     D.jobs = djobs;
-    D.njobs = (int)b->jobs.size();
+    D.njobs = (int)jobs.size();
     D.alpha = b->opt.msbfs_alpha;
     D.beta = b->opt.msbfs_beta;
     D.one_hot_start = b->opt.ppr_start;
     D.pack_max = b->opt.ppr_pack;
+    b->dev = D;
+    b->nbig = nbig;
+    b->hg = std::move(hg);
+    b->jobs = std::move(jobs);
+    b->layout.release(s);
+    b->layout = std::move(layout);
     b->ppr_stale = b->bfs_stale = true;  // captured launches hold the old arguments
     return GP_OK;
 }
@@ -1236,8 +1249,11 @@ extern "C" int gp_batch_set_options(gp_batch *b, const gp_batch_options *opt, vo
     const gp_batch_options old = b->opt;
     b->opt = *opt;
     if (old.big_in_degree != opt->big_in_degree || old.chunk_edges != opt->chunk_edges ||
-        old.l2_budget_mb != opt->l2_budget_mb)
-        return batch_layout(b, (cudaStream_t)stream);
+        old.l2_budget_mb != opt->l2_budget_mb) {
+        const int st = batch_layout(b, (cudaStream_t)stream);
+        if (st != GP_OK) b->opt = old;
+        return st;
+    }
     b->dev.alpha = opt->msbfs_alpha;
     b->dev.beta = opt->msbfs_beta;
     b->dev.one_hot_start = opt->ppr_start;

@@ -1,5 +1,6 @@
-"""Allocations that fail, each in turn: gp_graph_set_options then leaves the
-graph as it was (its chunk tables, work areas and options, and so its results),
+"""Allocations that fail, each in turn: gp_graph_set_options and
+gp_batch_set_options then leave the graph and the batch as they were (chunk
+tables, work areas and options, and so the results),
 and a hot set or the triangle counts' directed lists that found no memory are
 built by the next call."""
 import ctypes
@@ -148,3 +149,34 @@ def test_directed_lists_without_memory(scarce):
         k += 1
     assert k > 3  # the offsets, the lists and a temporary list, each without memory once
     G.free()
+
+
+def test_batch_options_without_memory(scarce):
+    gp, failing = scarce
+    graphs = [gp.Graph.from_graphgen(gg.rmat(s, 16, seed=s)) for s in (10, 11)]
+    B = gp.Batch(graphs, k_ppr=32)
+    rng = np.random.default_rng(2)
+    seeds, sources = rng.integers(0, 1024, (2, 32)), rng.integers(0, 1024, (2, 9))
+
+    def results():
+        outs, done, _ = B.ppr(seeds, iters=40, tol=1e-6)
+        return [t.cpu().numpy() for t in outs] + [done] + [t.cpu().numpy() for t in B.msbfs(sources)[0]]
+
+    want, old, k = results(), B.options(), 0
+    while True:
+        try:
+            with failing(k):
+                B.set_options(big_in_degree=8, chunk_edges=64, l2_budget_mb=1)
+            break
+        except gp.GpError as e:
+            assert e.status == gp.ERR_OOM
+        assert B.options() == old
+        for a, b in zip(want, results()):
+            assert np.array_equal(a, b)
+        k += 1
+    assert k > 4  # the five lists
+    for a, b in zip(want, results()):  # the same but for the order of sums
+        assert np.array_equal(a, b) if a.shape[1] == 64 else np.allclose(a, b, rtol=1e-4, atol=1e-6)
+    B.free()
+    for G in graphs:
+        G.free()
