@@ -314,7 +314,8 @@ int gp_pagerank_backward(const gp_graph *g, int mode, float damping, const float
 /* Replace the edge weights of a weighted graph (device arrays, caller-owned,
  * kept alive until the next call or gp_graph_free; csc_w may be NULL for a
  * symmetric graph whose CSC shares the CSR arrays).  The per-source normaliser
- * of a GP_UPLOAD_NORMALIZE graph is recomputed on `stream`.  Used by training
+ * of a GP_UPLOAD_NORMALIZE graph is recomputed on `stream`.  Later calls on the
+ * graph, and on batches that it is in, use the new weights.  Used by training
  * loops that update weights between forward passes. */
 int gp_graph_set_weights(gp_graph *g, const float *csr_w, const float *csc_w, void *stream);
 

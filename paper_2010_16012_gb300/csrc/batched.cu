@@ -1306,6 +1306,13 @@ extern "C" int gp_ppr_batched(gp_batch *b, const int32_t *seeds, float damping, 
         GP_CUDA(cudaEventCreate(&ev1));
     }
     GP_CUDA(cudaMemcpyAsync(b->seeds, seeds, (size_t)b->ngraphs * K * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    bool other_weights = false;  // since the batch was made, or the last call
+    for (int gi = 0; gi < b->ngraphs; ++gi) {
+        other_weights |= b->hg[gi].csc_w != b->graphs[gi]->csc_w;
+        b->hg[gi].csc_w = b->graphs[gi]->csc_w;
+    }
+    if (other_weights)
+        GP_CUDA(cudaMemcpyAsync(b->dgraphs, b->hg.data(), b->ngraphs * sizeof(BGraph), cudaMemcpyHostToDevice, s));
     const void *kernel = (const void *)k_ppr_persistent;
     const bool rebuild = b->ppr_stale || b->ppr_iters != iters || b->ppr_tol != tol || b->ppr_d != damping;
     if (rebuild) {
