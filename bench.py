@@ -202,8 +202,7 @@ def pick_sources(g, count: int):
     return gg.pick_vertices(g, count, seed=2)
 
 
-KERNEL_SOURCE = {"pull_tiles": "pagerank.cu", "pull_finish": "pagerank.cu", "pull_big": "pagerank.cu",
-                 "pull_light": "pagerank.cu", "push_tiles": "pagerank.cu", "push_scatter": "pagerank.cu",
+KERNEL_SOURCE = {"pull_tiles": "pagerank.cu", "pull_finish": "pagerank.cu", "push_tiles": "pagerank.cu",
                  "push_epilogue": "pagerank.cu", "bfs_persistent": "bfs.cu", "bfs_multi": "bfs.cu"}
 
 
@@ -271,14 +270,14 @@ def kernel_bytes(g, opt, l2_bytes=None) -> dict:
         "pull_tiles": 4 * m + m // 8 + 4 * n + 4 * rows + 8 * tiles,
         # per row: vertex, sum, x and inv_deg read, y and c' written
         "pull_finish": 24 * rows + 4 * tiles,
-        # a sweep split by degree at pull_light_max (the shape of the adjoint's sweep);
+        # for comparison, no launch has these names: a sweep split by degree at pull_light_max;
         # big in-edge lists: indices + chunk table + chunk partials written
         "pull_big": 4 * e_big_in + 16 * ch_in + 4 * ch_in,
         # light in-edge lists + offsets + c (once) + x, inv_deg read + y, c' written + big-vertex combine
         "pull_light": 4 * (m - e_big_in) + 8 * (n + 1) + 4 * n * 5 + 4 * ch_in + 12 * nb_in,
         # out-edge indices + source bits + sources + c + y read-modify-write
         "push_tiles": 4 * m + m // 8 + 4 * tiles + 8 * sources + 8 * n,
-        # the same with sources found from the offsets and a chunk table (the lists split by degree)
+        # for comparison as well: sources found from the offsets and a chunk table (the lists split by degree)
         "push_scatter": 4 * m + 8 * (n + 1) + 4 * n + 8 * n + 16 * ch_out,
         # FP64: the accumulator read and reset, x and inv_deg read, y and c' written;
         # FP32: y, x, inv_deg read, y, c' and the next accumulator (x) written

@@ -672,7 +672,7 @@ int gp_batch_autotune(gp_batch *b, const int32_t *seeds, const int32_t *sources,
  * by the caller and must outlive the batch).  k_ppr in {32, 64, 128, 256} is the
  * number of personalised PageRank vectors per graph.  Reads the in-degrees once
  * to lay out the work (vertex tiles per graph, warp chunks of in-edge lists
- * longer than 256) and allocates, per graph, two n x k_ppr iterates and the
+ * longer than big_in_degree) and allocates, per graph, two n x k_ppr iterates and the
  * n x 64 BFS level array.  Synchronises the stream.
  */
 int gp_batch_create(gp_batch **out, gp_graph *const *graphs, int ngraphs, int k_ppr, void *stream);

@@ -324,8 +324,8 @@ __device__ __forceinline__ void pull_tiles_step(const PrArgs &a, const float *sh
 // ~300 G/s from L2).  Equal tiles keep every lane's eight gathers in use at any
 // degree, where a warp per long list and a lane per short one left most of them
 // idle at degrees near 16: a sweep of a uniform graph (n = 8.0M, m = 128M) took
-// 555 + 335 us split that way and takes 462 + 61 us; R-MAT 22 (m = 128M) 295 +
-// 84 + 4 us, now 252 + 22 us (40 or 32 registers, 768 or 1024 threads a block:
+// 555 + 335 us split that way and takes 462 + 55 us; R-MAT 22 (m = 128M) 295 +
+// 84 + 4 us, now 286 + 26 us (40 or 32 registers, 768 or 1024 threads a block:
 // within 1% there; 768 is 10% faster on a graph of 16K vertices).
 template <bool W, bool HOT>
 __global__ void __launch_bounds__(TILE_THREADS, 2) k_pull_tiles(PrArgs a) {
@@ -356,8 +356,8 @@ __device__ __forceinline__ void pull_write(const PrArgs &a, int64_t v, const Pul
 // Rows, then, in the first two sweeps, the vertices without in-edges: theirs is
 // the base term in every sweep, so both iterate buffers hold it from then on.
 // Bound by memory, and short of it by latency: the next row's number and a row's
-// operands are fetched before they are needed (n = 8.0M, 36 bytes a row: 68 -> 61
-// us; R-MAT 22: 26 -> 22.5; four rows a thread were slower than one).
+// operands are fetched before they are needed (n = 8.0M, 36 bytes a row: 68 -> 55
+// us; R-MAT 22: 26; four rows a thread were slower than one).
 // long_warp: this warp's place among those that deal out the long rows.  A launch
 // of its own deals them over the blocks, the sweeps in one launch over few blocks
 // (R-MAT 2^18, directed, 40 sweeps and 40 of the adjoint: 2.45 ms, 2.48 the other way).
